@@ -60,9 +60,12 @@ struct CompactParams {
   float* patch_key;               // [max_frames][S][C]
   int* patch_cnt;                 // [max_frames][S]
   int pool_always;                // segment_kernel: pool whatever the flagged count says (the entries of an earlier call)
-  // compact_kernel: with prev.n_frames > 0 the grid has one more row of blocks (the second one), which pools
-  // the segment entries the previous call left to this one
+  // compact_kernel: with prev.n_frames > 0 the grid has prev_rows more rows of blocks (behind the first one), which
+  // pool the segment entries the previous call left to this one.  prev_rows = ceil(2L / n_frames), one (layer, K|V)
+  // plane per block: a plane is a chain of L2 round trips of about 5 us, so that a single row of n_frames blocks
+  // with several planes each kept one-frame calls waiting for 70 us (28 layers) behind 8 us of copying
   SegmentArgs prev;
+  int prev_rows;
   int sel_mode;                   // 0: kept ids are in the store; 1: select here from the partial sums;
                                   // 2: select here by the caller's scores; 3: ids and counts are in the store
                                   // (segment-level selection)
@@ -536,12 +539,13 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const Compa
   // in the first wave beside the copy blocks instead of alone at the end
   int row = blockIdx.y;
   if (p.prev.n_frames > 0) {
-    if (row == 1) {
+    if (row >= 1 && row <= p.prev_rows) {
       // nothing of this call is needed for the entries of the previous one: no wait for the scoring kernel
-      for (int pl = blockIdx.x; pl < 2 * p.prev.L; pl += gridDim.x) compact_segment_plane(p.prev, pl >> 1, pl & 1);
+      const int pl = (row - 1) * gridDim.x + blockIdx.x;
+      if (pl < 2 * p.prev.L) compact_segment_plane(p.prev, pl >> 1, pl & 1);
       return;
     }
-    if (row > 1) --row;
+    if (row > p.prev_rows) row -= p.prev_rows;
   }
   const int plane = p.patch_split > 0 && row >= 1 ? (row == 1 ? 2 * p.L : row - 1) : row;
   pdl_wait();

@@ -715,7 +715,7 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
   cp.ps_grid = ps_grid; cp.ps_items = ps_items; cp.ps_ipf = ps_ipf;
   cp.sp = sp;
   if (ps_grid > 0) cp.sp.colsum_part = ctx->ws + ctx->wl.colsum_p;
-  // segment entries the previous call left behind: one more row of blocks (with per-kernel timing on,
+  // segment entries the previous call left behind: more rows of blocks (with per-kernel timing on,
   // a launch of their own, so that each kernel is timed doing its own work only)
   if (ctx->seg_pending && ctx->prof_on) {
     ProfScope ps(ctx, 3, st);
@@ -723,10 +723,13 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
     if (e != cudaSuccess) return broke_off(ctx, "segment kernel", e);
     ++n_launch;
   }
-  if (ctx->seg_pending) cp.prev = segment_args_of(ctx, ctx->seg_first, ctx->seg_n);
+  if (ctx->seg_pending) {
+    cp.prev = segment_args_of(ctx, ctx->seg_first, ctx->seg_n);
+    cp.prev_rows = (2 * L + n - 1) / n;
+  }
   {
     ProfScope ps(ctx, 2, st);
-    e = launch_k(compact_kernel<T>, dim3(n, L * 2 + (c.patch_split > 0 ? 1 : 0) + (ctx->seg_pending ? 1 : 0)),
+    e = launch_k(compact_kernel<T>, dim3(n, L * 2 + (c.patch_split > 0 ? 1 : 0) + cp.prev_rows),
                  kCompactThreads, 0, st, !ctx->prof_on, cp);
   }
   if (e != cudaSuccess) return broke_off(ctx, "compact kernel", e);
