@@ -540,7 +540,9 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const Compa
   int row = blockIdx.y;
   if (p.prev.n_frames > 0) {
     if (row >= 1 && row <= p.prev_rows) {
-      // nothing of this call is needed for the entries of the previous one: no wait for the scoring kernel
+      // nothing of this call is needed for the entries of the previous one: no wait for the scoring kernel (which has
+      // itself waited for the previous call's kernels; without a scoring kernel the wait is here)
+      if (p.sel_mode == 2) pdl_wait();
       const int pl = (row - 1) * gridDim.x + blockIdx.x;
       if (pl < 2 * p.prev.L) compact_segment_plane(p.prev, pl >> 1, pl & 1);
       return;
@@ -648,6 +650,7 @@ __global__ void __launch_bounds__(kScoreThreads, 2) tail_kernel(const ScoreParam
   __shared__ CompactScratch cs;
   __shared__ int s_ok;
   const int tid = threadIdx.x;
+  pdl_trigger();                                // the next call's scoring kernel may be scheduled (it waits for this one itself)
   pdl_wait();
   const int n_fl = *sp.n_flagged;
   if (n_fl == 0) return;                        // the common case: the next call pools this chunk's segment entries

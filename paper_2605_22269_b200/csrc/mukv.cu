@@ -536,18 +536,18 @@ cudaError_t launch_score_ps(mukv_ctx* ctx, const ScoreParams& sp, const void* d_
   pp.tiles = t.tiles; pp.tpt = t.tpt; pp.npad = t.npad; pp.n_mt = t.n_mt; pp.n_stages = t.ps_stages;
   pp.own_rows = t.own_rows; pp.n_past = sp.n_past_frames; pp.past_pad = t.past_pad; pp.kappa = c.keep_per_frame;
   pp.past_plane0 = 2 * sp.first_score_layer; pp.past_first = sp.past_first;
-  pp.n_items = n * ctx->Ls * c.n_kv_heads * (t.n_mt + t.tiles);
+  pp.ipu = t.n_mt + t.tiles;
+  pp.ipf = ctx->Ls * c.n_kv_heads * pp.ipu;
+  pp.n_items = n * pp.ipf;
   pp.exp2_scale = (float)(1.4426950408889634 / std::sqrt((double)D));
   pp.status = reinterpret_cast<int*>(ctx->ws + ctx->wl.dev_status);
   int blocks = ctx->n_sms < kPsMaxBlocks ? ctx->n_sms : kPsMaxBlocks;
   if (blocks > pp.n_items) blocks = pp.n_items;
-  *ps_grid = blocks; *ps_items = pp.n_items; *ps_ipf = ctx->Ls * c.n_kv_heads * (t.n_mt + t.tiles);
-  if (sp.n_past_frames)
-    score_ps_kernel<true><<<blocks, kPsThreads, t.smem_ps, st>>>(pp, qmap, kmap, ctx->wmap, ctx->pmap);
-  else
-    score_ps_kernel<false><<<blocks, kPsThreads, t.smem_ps, st>>>(pp, qmap, kmap, ctx->wmap, kmap);
+  *ps_grid = blocks; *ps_items = pp.n_items; *ps_ipf = pp.ipf;
   *why = "score_ps kernel";
-  return cudaGetLastError();
+  const bool past = sp.n_past_frames > 0;
+  return launch_k(past ? score_ps_kernel<true> : score_ps_kernel<false>, dim3(blocks), kPsThreads, t.smem_ps, st,
+                  !ctx->prof_on, pp, qmap, kmap, ctx->wmap, past ? ctx->pmap : kmap);
 }
 
 template <typename T>

@@ -61,7 +61,8 @@ struct ScorePsParams {
   int past_plane0;           // plane (layer * 2) of the first scoring layer's keys in a page
   long long past_first;
   int n_stages;              // operand stages in the ring (2 .. kPsMaxStages)
-  int n_items;               // n_frames * Ls * Hkv * (n_mt + tiles)
+  int n_items;               // n_frames * ipf
+  int ipu, ipf;              // items per (frame, layer, key head): n_mt + tiles; items per frame: ipu * Hkv * Ls
   float exp2_scale;          // log2(e) / sqrt(D)
   int* status;
 };
@@ -170,7 +171,7 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
   const uint32_t raw = tc::smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   unsigned char* sm = smem_raw + (base - raw);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(kFull, tid >> 5, 0);   // (known to be uniform)
   const ScoreParams& sp = p.sp;
   const int P = sp.P, D = sp.D, G = sp.G, Hkv = sp.Hkv, KB = D >> 6, Ls = sp.Ls;
   // a unit is (frame, scoring layer, key head), in that order; its rows in the K / Q maps (layer-major tensors)
@@ -179,7 +180,7 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
     return ((fl % Ls) * sp.n_frames + fl / Ls) * P;
   };
   const int NS = p.n_stages;
-  const int ipu = p.n_mt + p.tiles;                      // items per (frame, key head)
+  const int ipu = p.ipu;
   const int n_cta = gridDim.x, cta = blockIdx.x;
   // contiguous shares [c*n/nb, (c+1)*n/nb); the compaction kernel finds the blocks of a frame from the same rule
   const int i0 = (int)((unsigned)cta * (unsigned)p.n_items / (unsigned)n_cta);
@@ -229,7 +230,8 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
   // operand stage are requested here, before the block-wide barrier and with as little code in
   // front of them as possible (the first instructions of a launch come from device memory), so
   // that they are on their way while tensor memory is being allocated; produce() issues the rest.
-  int pr_i = i0, pr_t = 0, pr_nk = 0, pr_ns = 0, pr_unit = -1;
+  int pr_i = i0, pr_t = 0, pr_nk = 0, pr_ns = 0, pr_unit = -1, pr_s = 0;   // pr_s, pr_par: the ring's next stage, its phase
+  uint32_t pr_par = 0;
   bool pr_ok = true;
   // the key tile of a unit into key buffer kb_i: the frame's own keys, then the cached keys of the past frames
   const uint32_t k_tx = (uint32_t)KB * 128u * (uint32_t)(p.own_rows + (PAST ? p.n_past * p.kappa : 0));
@@ -246,8 +248,11 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
                           (int)(p.past_first + w), bar);
     }
   };
+  // (A dependent launch: up to here the block may run beside the kernel in front of it in the stream.  The inputs may be
+  // that kernel's output, and every write of this kernel follows from a load that is issued here.)
   if (tid == 0) {
     const int unit0 = i0 / ipu, x0 = i0 - unit0 * ipu;
+    pdl_wait();
     const int g0 = unit0 % Hkv, r0 = unit_row(unit0);
     load_keys(unit0, 0);
     if (x0 < p.n_mt) {
@@ -258,13 +263,13 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
       for (int kb = 0; kb < KB; ++kb)
         tc::tma_load_3d(sS + kb * st_kb, &qmap, kb * 64, g0 * G, r0 + (x0 - p.n_mt) * p.tpt, PS_BAR_SF(0));
     }
-    pr_nk = 1; pr_unit = unit0; pr_ns = 1; pr_t = 1;
+    pr_nk = 1; pr_unit = unit0; pr_ns = 1; pr_s = 1; pr_t = 1;             // (the ring has at least two stages)
     if (x0 >= p.n_mt) { pr_i = i0 + 1; pr_t = 0; }         // an attention item has this one operand load
   }
+  // (one thread: no divisions in its loop, their latency would be exposed)
   auto produce = [&]() {
-    while (pr_i < i1 && pr_ok) {
-      const int unit = pr_i / ipu, x = pr_i % ipu;
-      const int g = unit % Hkv, urow = unit_row(unit);
+    int x = pr_i % ipu, unit = pr_i / ipu, g = unit % Hkv, urow = unit_row(unit);
+    while (pr_i < i1) {
       if (unit != pr_unit) {
         const int kb_i = pr_nk & 1;
         pr_ok = tc::mbar_wait(PS_BAR_KE(kb_i), (uint32_t)(((pr_nk >> 1) & 1) ^ 1));
@@ -275,25 +280,31 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
       }
       const int n_ld = x < p.n_mt ? 3 : 1;               // DFT item: the three matrix terms, smallest first
       while (pr_t < n_ld) {
-        const int s = pr_ns % NS;
-        pr_ok = tc::mbar_wait(PS_BAR_SE(s), (uint32_t)(((pr_ns / NS) & 1) ^ 1));
+        pr_ok = tc::mbar_wait(PS_BAR_SE(pr_s), pr_par ^ 1u);
         if (!pr_ok) break;
-        const uint32_t dst = sS + (uint32_t)s * st_buf;
+        const uint32_t dst = sS + (uint32_t)pr_s * st_buf;
         if (x < p.n_mt) {
-          tc::mbar_expect_tx(PS_BAR_SF(s), (uint32_t)KB * (uint32_t)D * 128u);
+          tc::mbar_expect_tx(PS_BAR_SF(pr_s), (uint32_t)KB * (uint32_t)D * 128u);
           for (int kb = 0; kb < KB; ++kb)
-            tc::tma_load_2d(dst + kb * st_kb, &wmap, kb * 64, (2 - pr_t) * D, PS_BAR_SF(s));
+            tc::tma_load_2d(dst + kb * st_kb, &wmap, kb * 64, (2 - pr_t) * D, PS_BAR_SF(pr_s));
         } else {
-          tc::mbar_expect_tx(PS_BAR_SF(s), (uint32_t)KB * (uint32_t)rows_q * 128u);
+          tc::mbar_expect_tx(PS_BAR_SF(pr_s), (uint32_t)KB * (uint32_t)rows_q * 128u);
           for (int kb = 0; kb < KB; ++kb)
-            tc::tma_load_3d(dst + kb * st_kb, &qmap, kb * 64, g * G, urow + (x - p.n_mt) * p.tpt, PS_BAR_SF(s));
+            tc::tma_load_3d(dst + kb * st_kb, &qmap, kb * 64, g * G, urow + (x - p.n_mt) * p.tpt, PS_BAR_SF(pr_s));
         }
         ++pr_ns;
+        if (++pr_s == NS) { pr_s = 0; pr_par ^= 1u; }
         ++pr_t;
       }
       if (!pr_ok) break;
       ++pr_i;
       pr_t = 0;
+      if (++x == ipu) {
+        x = 0;
+        ++unit;
+        g = unit % Hkv;
+        urow = unit_row(unit);
+      }
     }
   };
   if (warp == 1) {
@@ -329,55 +340,62 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
     }
   } else if (warp == 1) {
     // ================================================================== MMA issuer
-    if (lane == 0) {
-      bool ok = true;
-      const uint32_t idesc_att = tc::idesc_bf16_f32(128, p.npad), idesc_dft = tc::idesc_bf16_f32(128, D);
-      int nk = 0, ns = 0, it = 0, last_unit = -1, kb_i = 0;
-      for (int i = i0; i < i1 && ok; ++i, ++it) {
-        const int unit = i / ipu, x = i % ipu;
-        if (unit != last_unit) {
-          kb_i = nk & 1;
-          ok = tc::mbar_wait(PS_BAR_KF(kb_i), (uint32_t)((nk >> 1) & 1));
-          if (!ok) break;
-          ++nk;
-          last_unit = unit;
-        }
-        const int b = it & 1;
-        ok = tc::mbar_wait(PS_BAR_AE(b), (uint32_t)(((it >> 1) & 1) ^ 1));
+    // (The whole warp walks the items, so that descriptors and addresses stay in uniform registers, and one lane issues;
+    // no divisions.  With a division per item and descriptors built per instruction this loop took 1,900 clocks an item
+    // of the 4,200 that the epilogue needs, and the accumulators came late.)
+    const bool elected = tc::elect_one();
+    bool ok = true;
+    const uint32_t idesc_att = tc::idesc_bf16_f32(128, p.npad), idesc_dft = tc::idesc_bf16_f32(128, D);
+    const uint64_t desc0 = tc::smem_desc_sw128(0u);      // an operand's descriptor is this plus its address / 16
+    int x = i0 % ipu, kb_i = 1;
+    uint32_t k_par = 1u, st = 0u, st_par = 0u, a_par = 1u;   // phases of the key buffers, the ring and the accumulators
+    bool new_keys = true;
+    for (int i = i0; i < i1; ++i) {
+      if (new_keys) {
+        kb_i ^= 1;
+        k_par ^= (uint32_t)(kb_i ^ 1);
+        ok = __all_sync(kFull, tc::mbar_wait(PS_BAR_KF(kb_i), k_par));
+        if (!ok) break;
+        new_keys = false;
+      }
+      const uint32_t b = (uint32_t)(i - i0) & 1u;
+      ok = __all_sync(kFull, tc::mbar_wait(PS_BAR_AE(b), a_par));
+      if (!ok) break;
+      a_par ^= b;
+      const uint32_t d_tmem = tmem + b * 256u;
+      const uint64_t kdesc = desc0 + ((sK + (uint32_t)kb_i * k_buf) >> 4);
+      const bool dft = x < p.n_mt;
+      const int n_ld = dft ? 3 : 1;
+      for (int t = 0; t < n_ld; ++t) {
+        ok = __all_sync(kFull, tc::mbar_wait(PS_BAR_SF(st), st_par));
         if (!ok) break;
         tc::tc_fence_after_sync();
-        const uint32_t d_tmem = tmem + (uint32_t)b * 256u;
-        const uint32_t kbase = sK + (uint32_t)kb_i * k_buf;
-        const int n_ld = x < p.n_mt ? 3 : 1;
-        for (int t = 0; t < n_ld && ok; ++t) {
-          const int s = ns % NS;
-          ok = tc::mbar_wait(PS_BAR_SF(s), (uint32_t)((ns / NS) & 1));
-          if (!ok) break;
-          tc::tc_fence_after_sync();
-          const uint32_t sbase = sS + (uint32_t)s * st_buf;
-          if (x < p.n_mt) {
-            // rows x*128 .. of the key tile times one term of the DFT matrix
-            for (int kb = 0; kb < KB; ++kb)
+        const uint64_t sdesc = desc0 + ((sS + st * st_buf) >> 4);
+        // DFT: rows x*128 .. of the key tile times one term of the matrix; attention: query rows times keys
+        uint64_t a = dft ? kdesc + (((uint32_t)x * st_kb) >> 4) : sdesc, bd = dft ? sdesc : kdesc;
+        const uint32_t a_kb = (dft ? k_kb : st_kb) >> 4, b_kb = (dft ? st_kb : k_kb) >> 4;
+        const uint32_t idesc = dft ? idesc_dft : idesc_att;
+        if (elected) {
+          for (int kb = 0; kb < KB; ++kb) {
 #pragma unroll
-              for (int k = 0; k < 4; ++k)
-                tc::mma_bf16_ss(d_tmem, tc::smem_desc_sw128(kbase + kb * k_kb + (uint32_t)x * st_kb + k * 32),
-                                tc::smem_desc_sw128(sbase + kb * st_kb + k * 32), idesc_dft, (t | kb | k) != 0);
-          } else {
-            for (int kb = 0; kb < KB; ++kb)
-#pragma unroll
-              for (int k = 0; k < 4; ++k)
-                tc::mma_bf16_ss(d_tmem, tc::smem_desc_sw128(sbase + kb * st_kb + k * 32),
-                                tc::smem_desc_sw128(kbase + kb * k_kb + k * 32), idesc_att, (kb | k) != 0);
+            for (int k = 0; k < 4; ++k) tc::mma_bf16_ss(d_tmem, a + 2 * k, bd + 2 * k, idesc, (t | kb | k) != 0);
+            a += a_kb;
+            bd += b_kb;
           }
-          tc::mma_commit(PS_BAR_SE(s));
-          ++ns;
+          tc::mma_commit(PS_BAR_SE(st));
         }
-        if (!ok) break;
-        tc::mma_commit(PS_BAR_AF(b));
-        if (i + 1 == i1 || (i + 1) / ipu != unit) tc::mma_commit(PS_BAR_KE(kb_i));
+        __syncwarp();
+        if (++st == (uint32_t)NS) { st = 0u; st_par ^= 1u; }
       }
-      if (!ok) atomicCAS(p.status, 0, 4);
+      if (!ok) break;
+      if (++x == ipu) { x = 0; new_keys = true; }
+      if (elected) {
+        tc::mma_commit(PS_BAR_AF(b));
+        if (new_keys || i + 1 == i1) tc::mma_commit(PS_BAR_KE(kb_i));
+      }
+      __syncwarp();
     }
+    if (!ok && lane == 0) atomicCAS(p.status, 0, 4);
   }
   } else {
     // ================================================================== epilogue
