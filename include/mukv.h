@@ -362,13 +362,14 @@ mukv_status mukv_profile_read(mukv_ctx* ctx, double* ms, int64_t* launches);
  *   d_kept_out [n_frames][kappa] int32 ascending kept token ids, or NULL;
  *   d_scores_out [3][n_frames][P] float (I_att, I_fft, fused I), or NULL; not both NULL.
  *
- * The scratch (about 1.9 MB: per-head partial sums in float and double, arrival counters, the
- * list of frames that need the double-precision pass) is a fixed array inside the library; every
- * device that loads the library holds it until the process exits.  The call performs no
- * cudaMalloc / cudaFree and uses no allocating routine; it enqueues one small memset (the
- * counters must start at zero, the rest of the array is overwritten before it is read) and two
- * kernels on `stream`.  The first call on each device also looks up the array's device address
- * and raises the kernels' shared-memory limit; make that first call outside any stream capture.
+ * The scratch (about 2 MB: per-head partial sums in float and double, arrival counters, the
+ * list of frames that need the double-precision pass, the DFT matrix terms) is a fixed array inside the
+ * library; every device that loads the library holds it until the process exits.  The call performs no
+ * cudaMalloc / cudaFree and uses no allocating routine.  A bf16 call is scored on the tensor cores and
+ * enqueues three kernels on `stream`; an fp32 call one small memset (the counters must start at zero,
+ * the rest of the array is overwritten before it is read) and two kernels.  The first call on each device
+ * also looks up the array's device address, copies the matrix terms into it and raises the kernels'
+ * shared-memory limit; make that first call outside any stream capture.
  * All calls on a device share the one array: two calls whose kernels may overlap on the device
  * (different streams without an ordering between them) race.  Messages of failures are read
  * with mukv_last_error(NULL). */

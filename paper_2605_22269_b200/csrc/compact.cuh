@@ -610,6 +610,15 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const Compa
   else pool_patches<T>(p, f, &cs);
 }
 
+// Selection alone (scoring without a store): one block per frame, behind the persistent scoring kernel.
+__global__ void __launch_bounds__(kCompactThreads) select_kernel(const CompactParams p) {
+  __shared__ SelectScratch ss;
+  __shared__ int s_kept[MUKV_MAX_TOKENS];
+  pdl_wait();
+  pdl_trigger();
+  select_from_partials(p, blockIdx.x, true, s_kept, &ss);
+}
+
 // Bounded wait until *ctr reaches `target` (other blocks of the same grid add to it; the grid is
 // sized so that all its blocks are resident).  False after about 1.5 s.
 __device__ inline bool wait_counter(const int* ctr, int target) {
@@ -658,7 +667,8 @@ __global__ void __launch_bounds__(kScoreThreads, 2) tail_kernel(const ScoreParam
   const int units = sp.Ls * sp.Hq * sp.row_split;
   for (int w = blockIdx.x; w < n_fl * units; w += gridDim.x) {
     const int u = w % units;
-    score_frame_block<T, double, NC>(sp, u / sp.row_split, u % sp.row_split, sp.flagged[w / units], smem_raw);
+    const int fl = sp.flagged[w / units];
+    score_frame_block<T, double, NC>(sp, u / sp.row_split, u % sp.row_split, sp.row_split, fl, fl, smem_raw);
     __syncthreads();
   }
   // ---- every block waits for all selections

@@ -515,39 +515,62 @@ cudaError_t flush_segments(const mukv_ctx* ctx, cudaStream_t st) {
   return e;
 }
 
+// What a launch of the persistent scoring kernel needs beside the scoring parameters.
+struct PsLaunch {
+  const TcShape* t;
+  int n_sms;
+  const CUtensorMap* wmap;
+  const CUtensorMap* pmap;       // stored pages (past keys), or null
+  void* colsum;                  // float [blocks + frames][P]
+  int* status;
+  int* clear;                    // see ScorePsParams
+  int kappa;
+  bool dependent;
+  // out: what the selection needs to find a frame's partial sums
+  int grid, items, ipf;
+};
+
 // Scores a bf16 chunk on the tensor cores (Eq. 1-3; Eq. 4 and the selection follow in compact_kernel).
-cudaError_t launch_score_ps(mukv_ctx* ctx, const ScoreParams& sp, const void* d_q, const void* k_last, int n,
-                            cudaStream_t st, const char** why, int* ps_grid, int* ps_items, int* ps_ipf) {
-  *ps_grid = 0;
-  const mukv_config& c = ctx->cfg;
-  const TcShape& t = ctx->tcs;
-  const int P = c.tokens_per_frame, D = c.head_dim;
+cudaError_t launch_score_ps(PsLaunch& l, const ScoreParams& sp, cudaStream_t st, const char** why) {
+  const TcShape& t = *l.t;
+  const int P = sp.P, D = sp.D, n = sp.n_frames;
   CUtensorMap qmap, kmap;
-  const long long rows = (long long)ctx->Ls * n * P;
-  if (!encode_map3(&qmap, d_q, D, c.n_q_heads, rows, ctx->G, t.tpt) ||
-      !encode_map3(&kmap, k_last, D, c.n_kv_heads, rows, 1, t.own_rows)) {
+  const long long rows = (long long)sp.Ls * n * P;
+  if (!encode_map3(&qmap, sp.q, D, sp.Hq, rows, sp.G, t.tpt) || !encode_map3(&kmap, sp.k_last, D, sp.Hkv, rows, 1, t.own_rows)) {
     *why = "cuTensorMapEncodeTiled failed";
     return cudaErrorInvalidValue;
   }
   ScorePsParams pp;
   memset(&pp, 0, sizeof pp);
   pp.sp = sp;
-  pp.sp.colsum_part = ctx->ws + ctx->wl.colsum_p;
+  pp.sp.colsum_part = l.colsum;
   pp.tiles = t.tiles; pp.tpt = t.tpt; pp.npad = t.npad; pp.n_mt = t.n_mt; pp.n_stages = t.ps_stages;
-  pp.own_rows = t.own_rows; pp.n_past = sp.n_past_frames; pp.past_pad = t.past_pad; pp.kappa = c.keep_per_frame;
+  pp.own_rows = t.own_rows; pp.n_past = sp.n_past_frames; pp.past_pad = t.past_pad; pp.kappa = l.kappa;
   pp.past_plane0 = 2 * sp.first_score_layer; pp.past_first = sp.past_first;
   pp.ipu = t.n_mt + t.tiles;
-  pp.ipf = ctx->Ls * c.n_kv_heads * pp.ipu;
+  pp.ipf = sp.Ls * sp.Hkv * pp.ipu;
   pp.n_items = n * pp.ipf;
   pp.exp2_scale = (float)(1.4426950408889634 / std::sqrt((double)D));
-  pp.status = reinterpret_cast<int*>(ctx->ws + ctx->wl.dev_status);
-  int blocks = ctx->n_sms < kPsMaxBlocks ? ctx->n_sms : kPsMaxBlocks;
+  pp.status = l.status;
+  pp.clear = l.clear;
+  int blocks = l.n_sms < kPsMaxBlocks ? l.n_sms : kPsMaxBlocks;
   if (blocks > pp.n_items) blocks = pp.n_items;
-  *ps_grid = blocks; *ps_items = pp.n_items; *ps_ipf = pp.ipf;
+  l.grid = blocks; l.items = pp.n_items; l.ipf = pp.ipf;
   *why = "score_ps kernel";
   const bool past = sp.n_past_frames > 0;
-  return launch_k(past ? score_ps_kernel<true> : score_ps_kernel<false>, dim3(blocks), kPsThreads, t.smem_ps, st,
-                  !ctx->prof_on, pp, qmap, kmap, ctx->wmap, past ? ctx->pmap : kmap);
+  return launch_k(past ? score_ps_kernel<true> : score_ps_kernel<false>, dim3(blocks), kPsThreads, t.smem_ps, st, l.dependent,
+                  pp, qmap, kmap, *l.wmap, past ? *l.pmap : kmap);
+}
+
+PsLaunch ps_launch_of(mukv_ctx* ctx) {
+  PsLaunch l;
+  memset(&l, 0, sizeof l);
+  l.t = &ctx->tcs; l.n_sms = ctx->n_sms; l.wmap = &ctx->wmap; l.pmap = &ctx->pmap;
+  l.colsum = ctx->ws + ctx->wl.colsum_p;
+  l.status = reinterpret_cast<int*>(ctx->ws + ctx->wl.dev_status);
+  l.kappa = ctx->cfg.keep_per_frame;
+  l.dependent = !ctx->prof_on;
+  return l;
 }
 
 template <typename T>
@@ -627,17 +650,17 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
     }
     gp.stat_refined = reinterpret_cast<unsigned long long*>(ctx->ws + ctx->wl.stat_refined);
     if (tc_first) {
-      int ps_grid1 = 0, ps_items1 = 0, ps_ipf1 = 0;
+      PsLaunch pl = ps_launch_of(ctx);
       {
         ProfScope ps(ctx, 0, st);
-        e = launch_score_ps(ctx, sp, d_q, sp.k_last, n, st, &what, &ps_grid1, &ps_items1, &ps_ipf1);
+        e = launch_score_ps(pl, sp, st, &what);
       }
       if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "%s: %s", what, cudaGetErrorString(e));
       n_launch += 2;
       gp.sp = sp;
       gp.sp.colsum_part = ctx->ws + ctx->wl.colsum_p;
       gp.src32 = 1;
-      gp.ps_grid = ps_grid1; gp.ps_items = ps_items1; gp.ps_ipf = ps_ipf1;
+      gp.ps_grid = pl.grid; gp.ps_items = pl.items; gp.ps_ipf = pl.ipf;
       {
         ProfScope ps(ctx, 1, st);
         e = launch_k(segsel_kernel, dim3(n_seg + extra), kSegSelThreads, segsel_smem_bytes(seg_tokens), st, dep, gp);
@@ -680,9 +703,11 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
     n_launch += 2;
   } else if (!d_ext) {
     ProfScope ps(ctx, 0, st);
-    if (ctx->tcs.ok && !ctx->force_fma)
-      e = launch_score_ps(ctx, sp, d_q, sp.k_last, n, st, &what, &ps_grid, &ps_items, &ps_ipf);
-    else
+    if (ctx->tcs.ok && !ctx->force_fma) {
+      PsLaunch pl = ps_launch_of(ctx);
+      e = launch_score_ps(pl, sp, st, &what);
+      ps_grid = pl.grid; ps_items = pl.items; ps_ipf = pl.ipf;
+    } else
       e = launch_score<T, float>(sp, ctx->nc, grid, score_smem_bytes<T, float>(ctx->key_rows, c.head_dim), st);
     ++n_launch;
   }
@@ -1340,28 +1365,52 @@ constexpr size_t kNaFftD = kNaColD + (size_t)kNaFrames * kNaHq * kNaP * sizeof(d
 constexpr size_t kNaKept = kNaFftD + (size_t)kNaFrames * kNaHkv * kNaP * sizeof(double);
 constexpr size_t kNaTs = kNaKept + (size_t)kNaFrames * kNaP * sizeof(int);
 constexpr size_t kNaPt = kNaTs + 256;
-constexpr size_t kNaCtrl = kNaPt + 256;                  // frame_counter[16], flagged[16], n_flagged
+constexpr size_t kNaCtrl = kNaPt + 256;                  // frame_counter[16], flagged[16], n_flagged, status
 constexpr size_t kNaCtrlBytes = 256;
-constexpr size_t kNaTotal = kNaCtrl + kNaCtrlBytes;
+constexpr size_t kNaW128 = kNaCtrl + kNaCtrlBytes;       // DFT matrix terms, D = 128 and D = 64
+constexpr size_t kNaW64 = kNaW128 + 3 * 128 * 128 * 2;
+constexpr size_t kNaTotal = kNaW64 + 3 * 64 * 64 * 2;
+// the tensor-core path keeps its column sums where the multiply-add path has them
+static_assert((size_t)(kPsMaxBlocks + kNaFrames) * kNaP * sizeof(float) <= kNaFftF - kNaColF, "column-sum slots do not fit");
 
 // In host code this name is only a handle for cudaGetSymbolAddress, never a device address.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaTotal];
 
-unsigned char* g_noalloc_ptr[kMaxDevices];               // device address of the array, per device
+struct NoallocDevice {
+  unsigned char* ptr;                                    // device address of the array
+  int n_sms;
+  CUtensorMap wmap128, wmap64;
+};
+NoallocDevice g_noalloc[kMaxDevices];
 
 // Once per device, with that device current: resolves the array's device address and makes sure the
 // scoring kernels may use the shared memory the largest supported frame needs.  Allocates nothing.
-cudaError_t noalloc_setup(int dev, unsigned char** out) {
-  cudaError_t e = raise_kernel_limits(nullptr);
+cudaError_t noalloc_setup(int dev, const NoallocDevice** out) {
+  NoallocDevice& d = g_noalloc[dev];
+  {
+    std::lock_guard<std::mutex> lock(g_dev_mutex);
+    if (d.ptr) { *out = &d; return cudaSuccess; }
+  }
+  int n_sms = 0;
+  cudaError_t e = raise_kernel_limits(&n_sms);
   if (e != cudaSuccess) return e;
   std::lock_guard<std::mutex> lock(g_dev_mutex);
-  if (!g_noalloc_ptr[dev]) {
+  if (!d.ptr) {
     void* ptr = nullptr;
     e = cudaGetSymbolAddress(&ptr, g_noalloc_scratch);
     if (e != cudaSuccess) return e;
-    g_noalloc_ptr[dev] = static_cast<unsigned char*>(ptr);
+    unsigned char* base = static_cast<unsigned char*>(ptr);
+    for (int D : {64, 128}) {
+      const std::vector<uint16_t> w = dft_terms(D);
+      unsigned char* dst = base + (D == 128 ? kNaW128 : kNaW64);
+      e = cudaMemcpy(dst, w.data(), w.size() * 2, cudaMemcpyHostToDevice);
+      if (e == cudaSuccess && !encode_map2(D == 128 ? &d.wmap128 : &d.wmap64, dst, D, 3LL * D, D)) e = cudaErrorInvalidValue;
+      if (e != cudaSuccess) return e;
+    }
+    d.n_sms = n_sms;
+    d.ptr = base;
   }
-  *out = g_noalloc_ptr[dev];
+  *out = &d;
   return cudaSuccess;
 }
 
@@ -1373,18 +1422,19 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
   if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
   if (dev < 0 || dev >= kMaxDevices) return fail(nullptr, MUKV_E_CAPACITY, "device index %d not supported", dev);
   const int P = c.tokens_per_frame, D = c.head_dim, nc = pick_nc(P);
-  unsigned char* base = nullptr;
-  e = noalloc_setup(dev, &base);
+  const NoallocDevice* nd = nullptr;
+  e = noalloc_setup(dev, &nd);
   if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "set-up of the static scratch: %s", cudaGetErrorString(e));
-  // the array keeps what the last call left: the arrival counters and the flagged list start at zero
-  e = cudaMemsetAsync(base + kNaCtrl, 0, kNaCtrlBytes, st);
-  if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
+  unsigned char* base = nd->ptr;
+  const TcShape ts = tc_shape(c);
   ScoreParams sp;
   memset(&sp, 0, sizeof sp);
   sp.P = P; sp.Hq = c.n_q_heads; sp.Hkv = c.n_kv_heads; sp.D = D; sp.G = c.n_q_heads / c.n_kv_heads;
   sp.kappa = c.keep_per_frame; sp.n_frames = n; sp.causal = c.attn_causal; sp.keep_low = c.keep_low_freq;
   sp.alpha = c.alpha; sp.tie_eps = c.tie_eps; sp.flag_margin = kFlagMargin; sp.flat_ratio = kFlatRatio;
   sp.Ls = 1;                                             // one scoring layer: the one the caller passes
+  sp.q_layer_stride = (long long)n * P * c.n_q_heads * D;
+  sp.k_layer_stride = (long long)n * P * c.n_kv_heads * D;
   sp.first_frame = 0;
   sp.q = d_q;
   sp.k_last = d_k_last;
@@ -1400,13 +1450,43 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
   sp.page_table = reinterpret_cast<long long*>(base + kNaPt);
   sp.refine = 0;
   sp.row_split = 1;
-  const dim3 grid(c.n_q_heads, n);
-  e = launch_score<T, float>(sp, nc, grid, score_smem_bytes<T, float>(P, D), st);
-  if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "score kernel: %s", cudaGetErrorString(e));
+  if (ts.ok) {
+    // bf16: scored on the tensor cores like a chunk of a context (16 frames of 196 tokens, 28 heads: 338 us on the
+    // multiply-add kernel, 29.4 us here), then one block per frame selects.  The scoring kernel clears the flagged count.
+    PsLaunch pl;
+    memset(&pl, 0, sizeof pl);
+    pl.t = &ts; pl.n_sms = nd->n_sms; pl.wmap = D == 128 ? &nd->wmap128 : &nd->wmap64;
+    pl.colsum = base + kNaColF;
+    pl.status = sp.n_flagged + 1;
+    pl.clear = sp.n_flagged;
+    pl.kappa = c.keep_per_frame;
+    pl.dependent = true;
+    const char* why = "";
+    e = launch_score_ps(pl, sp, st, &why);
+    if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "%s: %s", why, cudaGetErrorString(e));
+    CompactParams cp;
+    memset(&cp, 0, sizeof cp);
+    cp.sp = sp;
+    cp.ps_grid = pl.grid; cp.ps_items = pl.items; cp.ps_ipf = pl.ipf;
+    e = launch_k(select_kernel, dim3(n), kCompactThreads, 0, st, true, cp);
+    if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "select kernel: %s", cudaGetErrorString(e));
+  } else {
+    // the array keeps what the last call left: the arrival counters and the flagged count start at zero
+    e = cudaMemsetAsync(base + kNaCtrl, 0, kNaCtrlBytes, st);
+    if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
+    e = launch_score<T, float>(sp, nc, dim3(c.n_q_heads, n), score_smem_bytes<T, float>(P, D), st);
+    if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "score kernel: %s", cudaGetErrorString(e));
+  }
+  // Flagged frames in double precision.  The scratch holds the partial sums of 16 frames with one block per head; while
+  // few frames are flagged the same room lets four blocks share a head.
   sp.refine = 1;
+  sp.row_split = kRefineSplit;
+  sp.scratch_units = kNaFrames * kNaHq;
   sp.colsum_part = base + kNaColD;
   sp.ifft_part = base + kNaFftD;
-  e = launch_score<T, double>(sp, nc, grid, score_smem_bytes<T, double>(P, D), st);
+  int grid_r = c.n_q_heads * kRefineSplit * (n < 2 ? n : 2);
+  if (grid_r > 2 * nd->n_sms) grid_r = 2 * nd->n_sms;
+  e = launch_score<T, double>(sp, nc, dim3(grid_r), score_smem_bytes<T, double>(P, D), st, true);
   if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "refine kernel: %s", cudaGetErrorString(e));
   return MUKV_OK;
 }

@@ -56,6 +56,10 @@ struct ScoreParams {
   int no_select;                // 1: only the partial sums are wanted (the selection runs over a whole segment elsewhere)
   int refine;                   // 1: frames come from the flagged list, no further flagging
   int row_split;                // blocks that share a query head, each a range of query rows (>= 1)
+  // double-precision pass with room for the partial sums of `scratch_units` / (Ls * Hq) frames only: they are indexed by
+  // the place in the flagged list, and a head is split over row_split blocks while that fits, else not split; 0: one
+  // place per frame of the chunk
+  int scratch_units;
   // segment-level selection, double-precision pass: only the frames of segments whose word is non-zero
   // are scored (segment of chunk frame f: f / gate_fseg); null: every frame
   const int* seg_gate;
@@ -267,10 +271,11 @@ __device__ inline void select_frame(const ScoreParams& p, int f, const double (&
   }
 }
 
-// The work of one block: part q (of p.row_split) of the query rows of head hv of frame f (a frame
-// slot of the chunk); hv counts the query heads of all scoring layers, layer-major.
+// The work of one block: part q (of RS) of the query rows of head hv of frame f (a frame
+// slot of the chunk); hv counts the query heads of all scoring layers, layer-major.  The partial sums go to
+// place sf of the scratch.
 template <typename T, typename A, int NC>
-__device__ __forceinline__ void score_frame_block(const ScoreParams& p, int hv, int q, int f,
+__device__ __forceinline__ void score_frame_block(const ScoreParams& p, int hv, int q, int RS, int f, int sf,
                                                   unsigned char* smem_raw) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int P = p.P, D = p.D, Hq = p.Hq, Hkv = p.Hkv, G = p.G;
@@ -347,7 +352,6 @@ __device__ __forceinline__ void score_frame_block(const ScoreParams& p, int hv, 
 #pragma unroll
   for (int c = 0; c < NC; ++c) jrow[c] = min(lane + 32 * c, Pk - 1) * WS;
 
-  const int RS = p.row_split;
   const int n_steps = (P + kRowsPerStep - 1) / kRowsPerStep;
   const int n_per = (n_steps + RS - 1) / RS;
   const int rb_end = (q + 1) * n_per < n_steps ? (q + 1) * n_per : n_steps;
@@ -409,7 +413,7 @@ __device__ __forceinline__ void score_frame_block(const ScoreParams& p, int hv, 
   if (tid < P) {                                       // the importance is that of the frame's own tokens
     A t = (A)0;
     for (int w = 0; w < kScoreWarps; ++w) t += red[w * 256 + n_past + tid];
-    reinterpret_cast<A*>(p.colsum_part)[(((long long)f * HqV + hv) * RS + q) * P + tid] = t;
+    reinterpret_cast<A*>(p.colsum_part)[(((long long)sf * HqV + hv) * RS + q) * P + tid] = t;
   }
 
   // ---- Eq. 2-3: sum over the D bins of |DFT(k_j)| for this block's share of head g's tokens
@@ -440,7 +444,7 @@ __device__ __forceinline__ void score_frame_block(const ScoreParams& p, int hv, 
       total = warp_sum(total);
       alt = warp_sum(alt);
       if (lane == 0)
-        reinterpret_cast<A*>(p.ifft_part)[((long long)f * HkvV + layer * Hkv + g) * P + j] = total + (alt < (A)0 ? -alt : alt);
+        reinterpret_cast<A*>(p.ifft_part)[((long long)sf * HkvV + layer * Hkv + g) * P + j] = total + (alt < (A)0 ? -alt : alt);
     }
   }
 
@@ -457,10 +461,10 @@ __device__ __forceinline__ void score_frame_block(const ScoreParams& p, int hv, 
   __threadfence();
   double att[1] = {0.0}, fft[1] = {0.0};
   if (tid < P) {
-    const A* cp = reinterpret_cast<const A*>(p.colsum_part) + (long long)f * HqV * RS * P + tid;
+    const A* cp = reinterpret_cast<const A*>(p.colsum_part) + (long long)sf * HqV * RS * P + tid;
     for (int hh = 0; hh < HqV * RS; ++hh) att[0] += (double)__ldcg(cp + (long long)hh * P);
     att[0] = att[0] / (double)((long long)HqV * P);
-    const A* fp = reinterpret_cast<const A*>(p.ifft_part) + (long long)f * HkvV * P + tid;
+    const A* fp = reinterpret_cast<const A*>(p.ifft_part) + (long long)sf * HkvV * P + tid;
     for (int gg = 0; gg < HkvV; ++gg) fft[0] += (double)__ldcg(fp + (long long)gg * P);
     fft[0] = fft[0] / (double)((long long)HkvV * D);
   }
@@ -469,8 +473,8 @@ __device__ __forceinline__ void score_frame_block(const ScoreParams& p, int hv, 
 }
 
 // Grid (Hq * row_split, frames).  Normal pass: block row = frame slot of the chunk.  Double-precision
-// pass (p.refine): the grid has few rows of blocks, which walk the list of flagged frames; with
-// nothing flagged they return at once.
+// pass (p.refine): a one-dimensional grid walks the (flagged frame, head, part) units; with
+// nothing flagged its blocks return at once.
 template <typename T, typename A, int NC>
 __global__ void __launch_bounds__(kScoreThreads) score_kernel(const ScoreParams p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -483,18 +487,21 @@ __global__ void __launch_bounds__(kScoreThreads) score_kernel(const ScoreParams 
       for (int f = 0; f < p.n_frames; ++f) {
         if (__ldcg(p.seg_gate + f / p.gate_fseg) == 0) continue;
         for (int u = blockIdx.x; u < units; u += gridDim.x) {
-          score_frame_block<T, A, NC>(p, u / p.row_split, u % p.row_split, f, smem_raw);
+          score_frame_block<T, A, NC>(p, u / p.row_split, u % p.row_split, p.row_split, f, f, smem_raw);
           __syncthreads();
         }
       }
       return;
     }
-    score_frame_block<T, A, NC>(p, blockIdx.x / p.row_split, blockIdx.x % p.row_split, blockIdx.y, smem_raw);
+    score_frame_block<T, A, NC>(p, blockIdx.x / p.row_split, blockIdx.x % p.row_split, p.row_split, blockIdx.y, blockIdx.y,
+                                smem_raw);
     return;
   }
-  const int n = *p.n_flagged;
-  for (int slot = blockIdx.y; slot < n; slot += gridDim.y) {
-    score_frame_block<T, A, NC>(p, blockIdx.x / p.row_split, blockIdx.x % p.row_split, p.flagged[slot], smem_raw);
+  const int n = *p.n_flagged, heads = p.Ls * p.Hq;
+  const int rs = n * heads * p.row_split <= p.scratch_units ? p.row_split : 1, units = heads * rs;
+  for (int w = blockIdx.x; w < n * units; w += gridDim.x) {
+    const int slot = w / units, u = w - slot * units;
+    score_frame_block<T, A, NC>(p, u / rs, u % rs, rs, p.flagged[slot], slot, smem_raw);
     __syncthreads();
   }
 }

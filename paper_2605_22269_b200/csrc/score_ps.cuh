@@ -64,6 +64,7 @@ struct ScorePsParams {
   int n_items;               // n_frames * ipf
   int ipu, ipf;              // items per (frame, layer, key head): n_mt + tiles; items per frame: ipu * Hkv * Ls
   float exp2_scale;          // log2(e) / sqrt(D)
+  int* clear;                // word that has to be zero when the next kernel starts, or null
   int* status;
 };
 
@@ -253,6 +254,7 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
   if (tid == 0) {
     const int unit0 = i0 / ipu, x0 = i0 - unit0 * ipu;
     pdl_wait();
+    if (cta == 0 && p.clear) *p.clear = 0;
     const int g0 = unit0 % Hkv, r0 = unit_row(unit0);
     load_keys(unit0, 0);
     if (x0 < p.n_mt) {
