@@ -39,6 +39,7 @@ struct StoreLayout {
 };
 
 struct WorkLayout {
+  size_t q_terms, k_terms; // fp32 chunks: queries and keys of the scoring layers as three bf16 terms
   size_t colsum_f, colsum_p, ifft_f, colsum_d, ifft_d, frame_counter, flagged, n_flagged, tail_ctr, sel_flag,
       seg_flag, stat_refined, dev_status;
   size_t q64, qnorm, s_frm, s_seg, s_pat, wtab, total;
@@ -51,6 +52,9 @@ struct TcShape {
   int tpt, tiles, npad, n_mt, ps_stages;
   int own_rows, past_pad;  // key-tile rows of the frame's own keys; rows reserved per cached past frame (0: none)
   size_t smem_ps;
+  bool split;              // fp32 chunk scored on the tensor cores in three bf16 terms (ok is false: it has a path of its own)
+  int split_frames;        // most frames of a call for that (what the terms of a call may take is limited)
+  int n_a, n_b, b_slot;    // its operand rings
 };
 
 thread_local std::string g_create_error;
@@ -214,7 +218,7 @@ TcShape tc_shape(const mukv_config& c) {
   TcShape t;
   memset(&t, 0, sizeof t);
   const int G = c.n_q_heads / c.n_kv_heads;
-  if (c.dtype != MUKV_BF16 || G > 128) return t;
+  if (G > 128) return t;
   t.tpt = 128 / G;
   t.tiles = (c.tokens_per_frame + t.tpt - 1) / t.tpt;
   t.npad = (c.tokens_per_frame + 15) / 16 * 16;
@@ -228,6 +232,19 @@ TcShape tc_shape(const mukv_config& c) {
     if (c.keep_per_segment > 0) return t;               // pages of different lengths are not one regular tensor
   }
   t.n_mt = (c.tokens_per_frame + 127) / 128;
+  if (c.dtype != MUKV_BF16) {
+    // fp32: frame-level selection without past keys.  (Segment-level selection ranks fp32 chunks in double precision,
+    // and past keys are stored as fp32 rows.)  The terms of a call take 6 bytes per value of the scoring layers' queries
+    // and keys, 4.8 MB per frame of 28 x 196 x 128 queries; longer chunks than fit 256 MB keep the multiply-add kernel.
+    if (c.past_frames > 0 || c.keep_per_segment > 0) return t;
+    const long long ls = c.n_score_layers > 1 ? c.n_score_layers : 1;
+    const long long per_frame = 6LL * ls * c.tokens_per_frame * (c.n_q_heads + c.n_kv_heads) * c.head_dim;
+    const long long most = (256LL << 20) / per_frame;
+    t.split_frames = (int)(most < c.max_frames_per_chunk ? most : c.max_frames_per_chunk);
+    t.split = t.split_frames > 0 && t.npad <= kPsSplit * kPsAccCols &&
+              score_ps_split_rings(t.npad, c.head_dim, 227 * 1024, &t.n_a, &t.n_b, &t.b_slot, &t.smem_ps);
+    return t;
+  }
   t.ps_stages = score_ps_stages(t.npad, c.head_dim, 227 * 1024);
   t.smem_ps = score_ps_smem_bytes(t.npad, c.head_dim, t.ps_stages < 2 ? 2 : t.ps_stages);
   t.ok = t.ps_stages >= 2 && t.npad <= kPsSplit * kPsAccCols;
@@ -251,7 +268,7 @@ WorkLayout work_layout(const mukv_config& c) {
   const TcShape ts = tc_shape(c);
   const size_t Ls = c.n_score_layers > 1 ? c.n_score_layers : 1;
   w.colsum_f = off;       off = align_up(off + F * Ls * (size_t)c.n_q_heads * P * sizeof(float));
-  w.colsum_p = off;       off = align_up(off + (ts.ok ? (kPsMaxBlocks + F) * P * sizeof(float) : 0));
+  w.colsum_p = off;       off = align_up(off + (ts.ok || ts.split ? (kPsMaxBlocks + F) * P * sizeof(float) : 0));
   w.ifft_f = off;         off = align_up(off + F * Ls * c.n_kv_heads * P * sizeof(float));
   w.colsum_d = off;       off = align_up(off + F * Ls * c.n_q_heads * kRefineSplit * P * sizeof(double));
   w.ifft_d = off;         off = align_up(off + F * Ls * c.n_kv_heads * P * sizeof(double));
@@ -271,7 +288,10 @@ WorkLayout work_layout(const mukv_config& c) {
   w.s_seg = off;          off = align_up(off + (size_t)MUKV_MAX_QUESTIONS * max_segs * sizeof(double));
   w.s_pat = off;          off = align_up(off + (size_t)MUKV_MAX_QUESTIONS * c.max_frames * c.patch_split * c.patch_split *
                                                sizeof(double));
-  w.wtab = off;           off = align_up(off + (ts.ok ? (size_t)3 * c.head_dim * c.head_dim * 2 : 0));
+  w.wtab = off;           off = align_up(off + (ts.ok || ts.split ? (size_t)3 * c.head_dim * c.head_dim * 2 : 0));
+  const size_t tf = ts.split ? (size_t)ts.split_frames * Ls * P * 6 : 0;
+  w.q_terms = off;        off = align_up(off + tf * c.n_q_heads * c.head_dim);
+  w.k_terms = off;        off = align_up(off + tf * C);
   w.total = off;
   return w;
 }
@@ -379,8 +399,9 @@ cudaError_t raise_kernel_limits(int* n_sms) {
   }
   if (e == cudaSuccess) e = raise_smem_limit((const void*)rank_kernel, optin);
   if (e == cudaSuccess) e = raise_smem_limit((const void*)segsel_kernel, optin);
-  if (e == cudaSuccess) e = raise_smem_limit((const void*)score_ps_kernel<false>, optin);
-  if (e == cudaSuccess) e = raise_smem_limit((const void*)score_ps_kernel<true>, optin);
+  if (e == cudaSuccess) e = raise_smem_limit((const void*)score_ps_kernel<false, false>, optin);
+  if (e == cudaSuccess) e = raise_smem_limit((const void*)score_ps_kernel<true, false>, optin);
+  if (e == cudaSuccess) e = raise_smem_limit((const void*)score_ps_kernel<false, true>, optin);
   if (e == cudaSuccess) g_limits_raised[dev] = true;
   return e;
 }
@@ -526,6 +547,7 @@ struct PsLaunch {
   int* clear;                    // see ScorePsParams
   int kappa;
   bool dependent;
+  __nv_bfloat16 *q_terms, *k_terms;   // SPLIT: room for the terms of an fp32 chunk
   // out: what the selection needs to find a frame's partial sums
   int grid, items, ipf;
 };
@@ -534,9 +556,26 @@ struct PsLaunch {
 cudaError_t launch_score_ps(PsLaunch& l, const ScoreParams& sp, cudaStream_t st, const char** why) {
   const TcShape& t = *l.t;
   const int P = sp.P, D = sp.D, n = sp.n_frames;
-  CUtensorMap qmap, kmap;
+  CUtensorMap qmap, kmap, kmap128;
   const long long rows = (long long)sp.Ls * n * P;
-  if (!encode_map3(&qmap, sp.q, D, sp.Hq, rows, sp.G, t.tpt) || !encode_map3(&kmap, sp.k_last, D, sp.Hkv, rows, 1, t.own_rows)) {
+  const void *q = sp.q, *k = sp.k_last;
+  bool maps = true;
+  if (t.split) {
+    SplitParams s;
+    s.src[0] = reinterpret_cast<const float*>(sp.q); s.src[1] = reinterpret_cast<const float*>(sp.k_last);
+    s.dst[0] = l.q_terms; s.dst[1] = l.k_terms;
+    s.n[0] = rows * sp.Hq * D; s.n[1] = rows * sp.Hkv * D;
+    const long long blocks = ((s.n[0] + s.n[1]) / 8 + 255) / 256, most = 8LL * l.n_sms;   // eight blocks per SM are resident
+    *why = "split_terms kernel";
+    const cudaError_t e = launch_k(split_terms_kernel, dim3((unsigned)(blocks < most ? blocks : most)), 256u, 0, st, l.dependent, s);
+    if (e != cudaSuccess) return e;
+    q = l.q_terms;
+    k = l.k_terms;
+    maps = encode_map3(&kmap128, k, D, sp.Hkv, 3 * rows, 1, 128);
+  }
+  const long long map_rows = t.split ? 3 * rows : rows;
+  if (!maps || !encode_map3(&qmap, q, D, sp.Hq, map_rows, sp.G, t.tpt) ||
+      !encode_map3(&kmap, k, D, sp.Hkv, map_rows, 1, t.own_rows)) {
     *why = "cuTensorMapEncodeTiled failed";
     return cudaErrorInvalidValue;
   }
@@ -558,8 +597,13 @@ cudaError_t launch_score_ps(PsLaunch& l, const ScoreParams& sp, cudaStream_t st,
   l.grid = blocks; l.items = pp.n_items; l.ipf = pp.ipf;
   *why = "score_ps kernel";
   const bool past = sp.n_past_frames > 0;
-  return launch_k(past ? score_ps_kernel<true> : score_ps_kernel<false>, dim3(blocks), kPsThreads, t.smem_ps, st, l.dependent,
-                  pp, qmap, kmap, *l.wmap, past ? *l.pmap : kmap);
+  if (t.split) {
+    pp.n_a = t.n_a; pp.n_b = t.n_b; pp.b_slot = t.b_slot; pp.term_rows = (int)rows;
+    return launch_k(score_ps_kernel<false, true>, dim3(blocks), kPsThreads, t.smem_ps, st, l.dependent, pp, qmap, kmap,
+                    *l.wmap, kmap128);
+  }
+  return launch_k(past ? score_ps_kernel<true, false> : score_ps_kernel<false, false>, dim3(blocks), kPsThreads, t.smem_ps,
+                  st, l.dependent, pp, qmap, kmap, *l.wmap, past ? *l.pmap : kmap);
 }
 
 PsLaunch ps_launch_of(mukv_ctx* ctx) {
@@ -570,6 +614,8 @@ PsLaunch ps_launch_of(mukv_ctx* ctx) {
   l.status = reinterpret_cast<int*>(ctx->ws + ctx->wl.dev_status);
   l.kappa = ctx->cfg.keep_per_frame;
   l.dependent = !ctx->prof_on;
+  l.q_terms = reinterpret_cast<__nv_bfloat16*>(ctx->ws + ctx->wl.q_terms);
+  l.k_terms = reinterpret_cast<__nv_bfloat16*>(ctx->ws + ctx->wl.k_terms);
   return l;
 }
 
@@ -703,7 +749,8 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
     n_launch += 2;
   } else if (!d_ext) {
     ProfScope ps(ctx, 0, st);
-    if (ctx->tcs.ok && !ctx->force_fma) {
+    if ((ctx->tcs.ok || (ctx->tcs.split && n <= ctx->tcs.split_frames)) && !ctx->force_fma) {
+      n_launch += ctx->tcs.split ? 1 : 0;
       PsLaunch pl = ps_launch_of(ctx);
       e = launch_score_ps(pl, sp, st, &what);
       ps_grid = pl.grid; ps_items = pl.items; ps_ipf = pl.ipf;
@@ -1021,11 +1068,11 @@ mukv_status create_impl(const mukv_config* cfg, void* d_store, size_t store_byte
     if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
     ctx->tail_capacity = per_sm * ctx->n_sms;
   }
-  if (e == cudaSuccess && ctx->tcs.ok) {
+  if (e == cudaSuccess && (ctx->tcs.ok || ctx->tcs.split)) {
     const std::vector<uint16_t> w = dft_terms(D);
     e = cudaMemcpy(ctx->ws + ctx->wl.wtab, w.data(), w.size() * 2, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !encode_map2(&ctx->wmap, ctx->ws + ctx->wl.wtab, D, 3LL * D, D)) e = cudaErrorInvalidValue;
-    if (e == cudaSuccess && cfg->past_frames > 0 &&
+    if (e == cudaSuccess && ctx->tcs.ok && cfg->past_frames > 0 &&
         !encode_map_pages(&ctx->pmap, ctx->store + ctx->sl.pages, D, cfg->n_kv_heads, cfg->keep_per_frame, 2 * cfg->n_layers,
                           cfg->max_frames, (long long)ctx->sl.page_bytes))
       e = cudaErrorInvalidValue;

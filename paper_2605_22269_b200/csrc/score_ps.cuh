@@ -28,6 +28,14 @@
 // All mbarrier waits are bounded; a wait that runs out makes the role record a code in the status
 // word; the producer and the MMA issuer then leave their loops, the epilogue warps go on without
 // waiting (their reads stay inside the accumulators).
+//
+// fp32 chunks (SPLIT): split_terms_kernel writes queries and keys as three bf16 terms each, x = hi + mid + lo (exact:
+// 3 x 8 significant bits), and a product of two values is summed over the six pairs of terms that reach 2^-24 of it
+// (hi hi, hi mid, mid hi, mid mid, hi lo, lo hi), every product exact and added in single precision.  The operands of
+// an item do not fit beside those of the next one as a whole, so blocks of 64 channels of one term travel through two
+// rings (query side, key side).  Six times the matrix instructions still cost less than the epilogue's exponentials;
+// what the multiply-add kernel took 473 us for (16 frames, 28 heads, 196 tokens: its floor at the fp32 rate is 60)
+// takes 72 here, split_terms_kernel included.
 #pragma once
 #include "common.cuh"
 #include "score.cuh"
@@ -64,11 +72,16 @@ struct ScorePsParams {
   int n_items;               // n_frames * ipf
   int ipu, ipf;              // items per (frame, layer, key head): n_mt + tiles; items per frame: ipu * Hkv * Ls
   float exp2_scale;          // log2(e) / sqrt(D)
+  // SPLIT: slots of the two operand rings, bytes of a key-side slot, rows of one term's plane of queries / keys
+  int n_a, n_b, b_slot;
+  int term_rows;
   int* clear;                // word that has to be zero when the next kernel starts, or null
   int* status;
 };
 
 constexpr int kPsMaxStages = 6;
+constexpr int kPsMaxA = 8;                 // SPLIT: most query-side slots (128 rows x 64 channels, 16 KB each)
+constexpr uint32_t kPsASlot = 128u * 128u;
 // two key buffers + n_stages operand stages + scratch (+ slack to align the tiles to 1024 bytes)
 __host__ inline size_t score_ps_smem_bytes(int npad, int D, int n_stages) {
   const size_t KB = D / 64;
@@ -78,6 +91,59 @@ __host__ inline int score_ps_stages(int npad, int D, size_t limit) {
   int n = kPsMaxStages;
   while (n >= 2 && score_ps_smem_bytes(npad, D, n) > limit) --n;
   return n;                  // < 2: the kernel does not fit
+}
+
+// SPLIT: the rings that fit: key-side slots (npad keys or D rows of the DFT matrix x 64 channels) and query-side slots.
+// Three of each are in use at a time; the fourth is what lets the next block's loads run ahead.
+__host__ inline bool score_ps_split_rings(int npad, int D, size_t limit, int* n_a, int* n_b, int* b_slot, size_t* smem) {
+  *b_slot = (npad > D ? npad : D) * 128;
+  const size_t fixed = kPsMiscBytes + 1024;
+  *n_b = kPsMaxStages;
+  for (; *n_b >= 4; --*n_b) {
+    const long long rest = (long long)limit - (long long)fixed - (long long)*n_b * *b_slot;
+    *n_a = rest > 0 ? (int)(rest / kPsASlot) : 0;
+    if (*n_a > kPsMaxA) *n_a = kPsMaxA;
+    if (*n_a >= 4) {
+      *smem = fixed + (size_t)*n_b * *b_slot + (size_t)*n_a * kPsASlot;
+      return true;
+    }
+  }
+  return false;
+}
+
+// An fp32 array as three arrays of bf16 terms, [3][n]: hi = bf16(x), mid = bf16(x - hi), lo = x - hi - mid (all
+// differences are exact).  Two arrays per launch, queries and keys; n a multiple of eight.  Bound by memory: 10 bytes
+// moved per value.
+struct SplitParams {
+  const float* src[2];
+  __nv_bfloat16* dst[2];
+  long long n[2];
+};
+__global__ void __launch_bounds__(256) split_terms_kernel(const SplitParams p) {
+  pdl_wait();
+  pdl_trigger();
+  const long long v0 = p.n[0] >> 3, v1 = v0 + (p.n[1] >> 3);
+  for (long long v = (long long)blockIdx.x * 256 + threadIdx.x; v < v1; v += (long long)gridDim.x * 256) {
+    const int a = v >= v0;
+    const long long i = (a ? v - v0 : v) << 3;
+    const uint4 x0 = ld_stream(p.src[a] + i), x1 = ld_stream(p.src[a] + i + 4);
+    const uint32_t x[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+    uint32_t t[3][4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      float r0 = __uint_as_float(x[2 * k]), r1 = __uint_as_float(x[2 * k + 1]);
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(r0, r1);
+        t[e][k] = *reinterpret_cast<const uint32_t*>(&h);
+        r0 -= bf16_lo(t[e][k]);
+        r1 -= bf16_hi(t[e][k]);
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 3; ++e)
+      *reinterpret_cast<uint4*>(p.dst[a] + e * p.n[a] + i) = make_uint4(t[e][0], t[e][1], t[e][2], t[e][3]);
+  }
 }
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -162,7 +228,9 @@ __device__ __forceinline__ float ps_chunk_exp(uint32_t (&r)[16], float c, float 
 
 // PAST: the key tile also holds cached keys of past frames (a second instantiation, so that the common
 // case keeps its shorter inner loop: the epilogue is bound by instruction issue)
-template <bool PAST>
+// SPLIT: operands in three bf16 terms (see the head of this file); pmap is then the map of the key terms with boxes of
+// 128 rows (the DFT items' row tiles)
+template <bool PAST, bool SPLIT>
 __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
                                                  const __grid_constant__ CUtensorMap qmap,
                                                  const __grid_constant__ CUtensorMap kmap,
@@ -190,16 +258,16 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
 
   const uint32_t k_kb = (uint32_t)p.npad * 128u, st_kb = 128u * 128u;
   const uint32_t k_buf = (uint32_t)KB * k_kb, st_buf = (uint32_t)KB * st_kb;
-  const uint32_t sK = base;                              // two key buffers
-  const uint32_t sS = sK + 2u * k_buf;                   // NS operand stages
-  const uint32_t misc_off = 2u * k_buf + (uint32_t)NS * st_buf;
+  const uint32_t sK = base;                              // two key buffers (SPLIT: the key-side ring)
+  const uint32_t sS = sK + (SPLIT ? (uint32_t)(p.n_b * p.b_slot) : 2u * k_buf);   // NS operand stages (the query-side ring)
+  const uint32_t misc_off = sS - sK + (SPLIT ? (uint32_t)p.n_a * kPsASlot : (uint32_t)NS * st_buf);
   float* s_col = reinterpret_cast<float*>(sm + misc_off);                     // [4][256]
   // (reference, sum) of a row's four warps, one copy per accumulator: a copy is rewritten two items
   // later, after the row's warps have met again at the barrier of the item in between
   float* s_mx = reinterpret_cast<float*>(sm + misc_off + 4096);               // [2][kPsSplit][128]
   float* s_sum = s_mx + 2 * kPsSplit * 128;                                   // [2][kPsSplit][128]
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + misc_off + 12288);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + misc_off + 12288 + 192);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + misc_off + 12288 + 480);
   float* s_mref = reinterpret_cast<float*>(sm + misc_off + 12800);            // [4 chunks][512 threads]
   const uint32_t b0 = tc::smem_u32(bars);
   // key buffer full / empty, accumulator full / empty (2 each), stage full / empty (kPsMaxStages each)
@@ -209,6 +277,9 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
 #define PS_BAR_AE(s) (b0 + 48u + 8u * (uint32_t)(s))
 #define PS_BAR_SF(s) (b0 + 64u + 8u * (uint32_t)(s))
 #define PS_BAR_SE(s) (b0 + 64u + 8u * (uint32_t)kPsMaxStages + 8u * (uint32_t)(s))
+  // SPLIT: key-side slots use SF / SE, query-side slots have these
+#define PS_BAR_QF(s) (b0 + 64u + 16u * (uint32_t)kPsMaxStages + 8u * (uint32_t)(s))
+#define PS_BAR_QE(s) (b0 + 64u + 16u * (uint32_t)kPsMaxStages + 8u * (uint32_t)kPsMaxA + 8u * (uint32_t)(s))
 
   if (tid == 0) {
     for (int s = 0; s < 2; ++s) {
@@ -221,11 +292,17 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
       tc::mbar_init(PS_BAR_SF(s), 1);
       tc::mbar_init(PS_BAR_SE(s), 1);
     }
+    if constexpr (SPLIT) {
+      for (int s = 0; s < kPsMaxA; ++s) {
+        tc::mbar_init(PS_BAR_QF(s), 1);
+        tc::mbar_init(PS_BAR_QE(s), 1);
+      }
+    }
     tc::fence_mbar_init();
     tc::prefetch_tmap(&qmap);
     tc::prefetch_tmap(&kmap);
     tc::prefetch_tmap(&wmap);
-    if (PAST) tc::prefetch_tmap(&pmap);
+    if (PAST || SPLIT) tc::prefetch_tmap(&pmap);
   }
   // ---- TMA producer (thread 0).  The key tile of the block's first (frame, head) and its first
   // operand stage are requested here, before the block-wide barrier and with as little code in
@@ -252,9 +329,11 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
   // (A dependent launch: up to here the block may run beside the kernel in front of it in the stream.  The inputs may be
   // that kernel's output, and every write of this kernel follows from a load that is issued here.)
   if (tid == 0) {
-    const int unit0 = i0 / ipu, x0 = i0 - unit0 * ipu;
     pdl_wait();
     if (cta == 0 && p.clear) *p.clear = 0;
+  }
+  if (!SPLIT && tid == 0) {
+    const int unit0 = i0 / ipu, x0 = i0 - unit0 * ipu;
     const int g0 = unit0 % Hkv, r0 = unit_row(unit0);
     load_keys(unit0, 0);
     if (x0 < p.n_mt) {
@@ -309,6 +388,51 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
       }
     }
   };
+  // SPLIT: per item and 64 channels the three terms of both sides, in the order in which the issuer needs them; then
+  // the hi terms once more
+  auto produce_split = [&]() {
+    int x = i0 % ipu, unit = i0 / ipu, g = unit % Hkv, urow = unit_row(unit), sa = 0, sb = 0;
+    uint32_t pa = 1u, pb = 1u;
+    for (int i = i0; i < i1; ++i) {
+      const bool dft = x < p.n_mt;
+      for (int step = 0; step < 2 * KB; ++step) {
+        const int kb = step < KB ? step : step - KB;
+        auto key_side = [&](int term) {
+          if (!pr_ok) return;
+          pr_ok = tc::mbar_wait(PS_BAR_SE(sb), pb);
+          if (!pr_ok) return;
+          const uint32_t dst = sK + (uint32_t)sb * (uint32_t)p.b_slot;
+          tc::mbar_expect_tx(PS_BAR_SF(sb), (uint32_t)(dft ? D : p.npad) * 128u);
+          if (dft) tc::tma_load_2d(dst, &wmap, kb * 64, term * D, PS_BAR_SF(sb));
+          else tc::tma_load_3d(dst, &kmap, kb * 64, g, term * p.term_rows + urow, PS_BAR_SF(sb));
+          ++pr_nk;
+          if (++sb == p.n_b) { sb = 0; pb ^= 1u; }
+        };
+        auto query_side = [&](int term) {
+          if (!pr_ok) return;
+          pr_ok = tc::mbar_wait(PS_BAR_QE(sa), pa);
+          if (!pr_ok) return;
+          const uint32_t dst = sS + (uint32_t)sa * kPsASlot;
+          tc::mbar_expect_tx(PS_BAR_QF(sa), (uint32_t)(dft ? 128 : rows_q) * 128u);
+          if (dft) tc::tma_load_3d(dst, &pmap, kb * 64, g, term * p.term_rows + urow + x * 128, PS_BAR_QF(sa));
+          else tc::tma_load_3d(dst, &qmap, kb * 64, g * G, term * p.term_rows + urow + (x - p.n_mt) * p.tpt, PS_BAR_QF(sa));
+          ++pr_ns;
+          if (++sa == p.n_a) { sa = 0; pa ^= 1u; }
+        };
+        key_side(0);
+        if (step < KB) { query_side(2); query_side(1); key_side(1); }
+        query_side(0);
+        if (step < KB) key_side(2);
+        if (!pr_ok) return;
+      }
+      if (++x == ipu) {
+        x = 0;
+        ++unit;
+        g = unit % Hkv;
+        urow = unit_row(unit);
+      }
+    }
+  };
   if (warp == 1) {
     __syncwarp();
     tc::tmem_alloc(tc::smem_u32(tmem_slot), 512u);
@@ -327,17 +451,19 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
   if (warp == 0) {
     // ================================================================== TMA producer (continued)
     if (lane == 0) {
-      produce();
+      if constexpr (SPLIT) produce_split();
+      else produce();
       if (!pr_ok) atomicCAS(p.status, 0, 3);
       pdl_trigger();                                     // the next kernel of the call may be scheduled
       // copies of this thread still in flight land before the block goes away
-      for (int s = 0; s < 2; ++s) {
-        const int cnt = (pr_nk + 1 - s) >> 1;
-        if (cnt) tc::mbar_wait(PS_BAR_KF(s), (uint32_t)((cnt - 1) & 1));
+      const int nk = SPLIT ? p.n_b : 2, ns = SPLIT ? p.n_a : NS;
+      for (int s = 0; s < nk; ++s) {
+        const int cnt = (pr_nk + nk - 1 - s) / nk;
+        if (cnt) tc::mbar_wait(SPLIT ? PS_BAR_SF(s) : PS_BAR_KF(s), (uint32_t)((cnt - 1) & 1));
       }
-      for (int s = 0; s < NS; ++s) {
-        const int cnt = (pr_ns + NS - 1 - s) / NS;
-        if (cnt) tc::mbar_wait(PS_BAR_SF(s), (uint32_t)((cnt - 1) & 1));
+      for (int s = 0; s < ns; ++s) {
+        const int cnt = (pr_ns + ns - 1 - s) / ns;
+        if (cnt) tc::mbar_wait(SPLIT ? PS_BAR_QF(s) : PS_BAR_SF(s), (uint32_t)((cnt - 1) & 1));
       }
     }
   } else if (warp == 1) {
@@ -352,7 +478,73 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
     int x = i0 % ipu, kb_i = 1;
     uint32_t k_par = 1u, st = 0u, st_par = 0u, a_par = 1u;   // phases of the key buffers, the ring and the accumulators
     bool new_keys = true;
-    for (int i = i0; i < i1; ++i) {
+    if constexpr (SPLIT) {
+      uint32_t sa = 0u, sb = 0u, pa = 0u, pb = 0u;
+      // the next slot of a ring, once its load has landed
+      auto take_a = [&]() {
+        const uint32_t s = sa;
+        if (ok) ok = __all_sync(kFull, tc::mbar_wait(PS_BAR_QF(s), pa));
+        if (++sa == (uint32_t)p.n_a) { sa = 0u; pa ^= 1u; }
+        return s;
+      };
+      auto take_b = [&]() {
+        const uint32_t s = sb;
+        if (ok) ok = __all_sync(kFull, tc::mbar_wait(PS_BAR_SF(s), pb));
+        if (++sb == (uint32_t)p.n_b) { sb = 0u; pb ^= 1u; }
+        return s;
+      };
+      for (int i = i0; i < i1; ++i) {
+        const uint32_t b = (uint32_t)(i - i0) & 1u;
+        ok = __all_sync(kFull, tc::mbar_wait(PS_BAR_AE(b), a_par));
+        if (!ok) break;
+        a_par ^= b;
+        const uint32_t d_tmem = tmem + b * 256u;
+        const uint32_t idesc = x < p.n_mt ? idesc_dft : idesc_att;
+        // one pair of terms over 64 channels
+        auto pair = [&](uint32_t a, uint32_t k, bool first) {
+          if (!ok || !elected) return;
+          tc::tc_fence_after_sync();
+          const uint64_t ad = desc0 + ((sS + a * kPsASlot) >> 4), bd = desc0 + ((sK + k * (uint32_t)p.b_slot) >> 4);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) tc::mma_bf16_ss(d_tmem, ad + 2 * j, bd + 2 * j, idesc, !first || j != 0);
+        };
+        auto free_a = [&](uint32_t s) { if (ok && elected) tc::mma_commit(PS_BAR_QE(s)); };
+        auto free_b = [&](uint32_t s) { if (ok && elected) tc::mma_commit(PS_BAR_SE(s)); };
+        for (int kb = 0; kb < KB && ok; ++kb) {
+          // The five small products of every block of channels come first, then hi hi: an addition loses up to 2^-24 of
+          // the sum it goes to, so all but the 4 KB last ones should go to a small sum.  (hi hi with the others of its
+          // block left an error of 8.8e-7 in the fused scores, this order 2.8e-7 and the multiply-add kernel 1.7e-7; loading
+          // the hi terms twice costs 4 us of 44.)  Both rings are given back in the order in which they were filled.
+          const uint32_t b_hi = take_b(), a_lo = take_a();
+          pair(a_lo, b_hi, kb == 0);
+          free_a(a_lo);
+          const uint32_t a_mid = take_a(), b_mid = take_b();
+          pair(a_mid, b_mid, false);
+          pair(a_mid, b_hi, false);
+          free_a(a_mid);
+          const uint32_t a_hi = take_a(), b_lo = take_b();
+          pair(a_hi, b_lo, false);
+          pair(a_hi, b_mid, false);
+          free_a(a_hi);
+          free_b(b_hi);
+          free_b(b_mid);
+          free_b(b_lo);
+          __syncwarp();
+        }
+        for (int kb = 0; kb < KB && ok; ++kb) {
+          const uint32_t b_hi = take_b(), a_hi = take_a();
+          pair(a_hi, b_hi, false);
+          free_a(a_hi);
+          free_b(b_hi);
+          __syncwarp();
+        }
+        if (!ok) break;
+        if (++x == ipu) x = 0;
+        if (elected) tc::mma_commit(PS_BAR_AF(b));
+        __syncwarp();
+      }
+    }
+    for (int i = i0; !SPLIT && i < i1; ++i) {
       if (new_keys) {
         kb_i ^= 1;
         k_par ^= (uint32_t)(kb_i ^ 1);
@@ -572,6 +764,8 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
 #undef PS_BAR_AE
 #undef PS_BAR_SF
 #undef PS_BAR_SE
+#undef PS_BAR_QF
+#undef PS_BAR_QE
 
   tc::tc_fence_before_sync();
   __syncthreads();
