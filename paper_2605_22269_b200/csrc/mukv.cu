@@ -888,16 +888,19 @@ mukv_status retrieve_impl(mukv_ctx* ctx, const void* d_qtok, const int32_t* h_q_
     const float* seg_key = reinterpret_cast<const float*>(ctx->store + ctx->sl.seg_key);
     const long long n_frm = ctx->frames;
     const long long n_seg = (n_frm + c.frames_per_segment - 1) / c.frames_per_segment;
+    const bool few = nq <= kScanFew;                       // see scan_few_kernel
+    cudaError_t e = cudaSuccess;
     {
       ProfScope ps(ctx, 4, st);
+      const dim3 grid(nq, c.n_kv_heads);
+      const int cs = few ? 1 : MUKV_MAX_QUESTIONS, qs = few ? C : 1;
       if (c.dtype == MUKV_BF16)
-        qpool_kernel<__nv_bfloat16><<<dim3(nq, c.n_kv_heads), kPoolThreads, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(d_qtok), meta,
-                                                       c.n_q_heads, c.n_kv_heads, c.head_dim, q64, qnorm);
+        e = launch_k(qpool_kernel<__nv_bfloat16>, grid, kPoolThreads, 0, st, !ctx->prof_on,
+                     reinterpret_cast<const __nv_bfloat16*>(d_qtok), meta, c.n_q_heads, c.n_kv_heads, c.head_dim, q64, cs, qs, qnorm);
       else
-        qpool_kernel<float><<<dim3(nq, c.n_kv_heads), kPoolThreads, 0, st>>>(reinterpret_cast<const float*>(d_qtok), meta, c.n_q_heads,
-                                               c.n_kv_heads, c.head_dim, q64, qnorm);
+        e = launch_k(qpool_kernel<float>, grid, kPoolThreads, 0, st, !ctx->prof_on, reinterpret_cast<const float*>(d_qtok), meta,
+                     c.n_q_heads, c.n_kv_heads, c.head_dim, q64, cs, qs, qnorm);
     }
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "qpool kernel: %s", cudaGetErrorString(e));
     const int S = c.patch_split * c.patch_split;
     const long long n_pat = k_pat > 0 ? n_frm * S : 0;
@@ -914,7 +917,13 @@ mukv_status retrieve_impl(mukv_ctx* ctx, const void* d_qtok, const int32_t* h_q_
       sc.C = C; sc.nq = nq; sc.Hkv = c.n_kv_heads; sc.q64t = q64; sc.qn2 = qnorm;
       sc.s_frm = s_frm; sc.s_seg = s_seg; sc.s_pat = s_pat;
       sc.frm_stride = c.max_frames; sc.seg_stride = ctx->sl.max_segs; sc.pat_stride = (long long)c.max_frames * S;
-      e = launch_k(scan_kernel, dim3(blocks), 256, 0, st, !ctx->prof_on, sc);
+      if (few) {
+        const long long want = (rows + 7) / 8, most = 8LL * ctx->n_sms;     // a warp per row, eight blocks per SM
+        const dim3 grid((unsigned)(want < most ? want : most));
+        e = launch_k(nq == 1 ? scan_few_kernel<1> : nq <= 4 ? scan_few_kernel<4> : scan_few_kernel<kScanFew>, grid, 256, 0, st,
+                     !ctx->prof_on, sc);
+      } else
+        e = launch_k(scan_kernel, dim3(blocks), 256, 0, st, !ctx->prof_on, sc);
     }
     if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "scan kernel: %s", cudaGetErrorString(e));
     RankParams rp;
@@ -934,9 +943,14 @@ mukv_status retrieve_impl(mukv_ctx* ctx, const void* d_qtok, const int32_t* h_q_
     {
       ProfScope ps(ctx, 6, st);
       size_t rank_smem = (size_t)C * sizeof(double);
-      const size_t staged = rank_smem + (size_t)(n_frm + n_seg) * sizeof(double);
-      rp.stage = staged <= (size_t)kRankStageBytes ? 1 : 0;
-      if (rp.stage) rank_smem = staged;
+      // single-precision copies of one granularity's scores at a time, if they fit
+      const size_t room = (size_t)kRankStageBytes - rank_smem - 16;
+      long long most = n_frm > n_seg ? n_frm : n_seg;
+      if (n_pat > most && (size_t)n_pat * sizeof(float) <= room) most = n_pat;
+      if ((size_t)most * sizeof(float) <= room) {
+        rp.stage = (int)most;
+        rank_smem += (size_t)most * sizeof(float) + 16;
+      }
       e = launch_k(rank_kernel, dim3(nq), kRankThreads, rank_smem, st, !ctx->prof_on, rp, meta);
     }
     if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "rank kernel: %s", cudaGetErrorString(e));
@@ -1274,12 +1288,12 @@ mukv_status mukv_gather3(mukv_ctx* ctx, const int32_t* d_seg_idx, const int32_t*
     const long long units = (long long)nq * c.n_layers * 2 * (k_frm + 1);
     const unsigned blocks = (unsigned)(units < 148 * 8 ? units : 148 * 8);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    cudaError_t e = cudaSuccess;
     {
       ProfScope ps(ctx, 7, st);
-      if (c.dtype == MUKV_BF16) gather3_kernel<__nv_bfloat16><<<blocks, 256, 0, st>>>(gp);
-      else gather3_kernel<float><<<blocks, 256, 0, st>>>(gp);
+      e = launch_k(c.dtype == MUKV_BF16 ? gather3_kernel<__nv_bfloat16> : gather3_kernel<float>, dim3(blocks), 256, 0, st,
+                   !ctx->prof_on, gp);
     }
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "gather3 kernel: %s", cudaGetErrorString(e));
     ctx->launches += 1;
     return MUKV_OK;
@@ -1320,11 +1334,12 @@ mukv_status mukv_gather(mukv_ctx* ctx, const int32_t* d_frm_idx, const int32_t* 
     gp.tok_meta = d_tok_meta;
     const long long units = (long long)nq * c.n_layers * 2 * k_frm;
     const unsigned blocks = (unsigned)(units < 148 * 8 ? units : 148 * 8);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    cudaError_t e = cudaSuccess;
     {
-      ProfScope ps(ctx, 7, static_cast<cudaStream_t>(stream));
-      gather_kernel<<<blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(gp);
+      ProfScope ps(ctx, 7, st);
+      e = launch_k(gather_kernel, dim3(blocks), 256, 0, st, !ctx->prof_on, gp);
     }
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "gather kernel: %s", cudaGetErrorString(e));
     ctx->launches += 1;
     return MUKV_OK;

@@ -23,21 +23,23 @@ struct QMeta {
 // One block per (question, key head).  Thread (slice, vector) sums one 16-byte vector of the head's
 // channels over the tokens n = slice, slice + slices, ... and the G query heads of the group: every
 // load is a full 16-byte vector and all of a thread's loads are independent.  The slices are added
-// in a fixed order.  The pooled query is written transposed, q64t[c][question] (row stride
-// MUKV_MAX_QUESTIONS), the layout scan_kernel stages; the head's share of the squared norm goes to
-// qn2[question][key head] (scan_kernel adds the shares in head order).
+// in a fixed order.  Channel c of question i is written to q64[c * cs + i * qs]: transposed (qs = 1) for
+// scan_kernel, which stages it, a row per question (cs = 1) for scan_few_kernel; the head's share of the squared
+// norm goes to qn2[question][key head] (the scans add the shares in head order).
 constexpr int kPoolThreads = 512;
 constexpr int kPoolSmemDoubles = 4096;
 
 template <typename T>
 __global__ void __launch_bounds__(kPoolThreads) qpool_kernel(const T* __restrict__ qtok, const QMeta meta, int Hq,
-                                                             int Hkv, int D, double* __restrict__ q64t,
+                                                             int Hkv, int D, double* __restrict__ q64, int cs, int qs,
                                                              double* __restrict__ qn2) {
   constexpr int VE = 16 / sizeof(T);
   __shared__ double s_acc[kPoolSmemDoubles];
   __shared__ double s_part[kPoolThreads / 32];
   const int qi = blockIdx.x, g = blockIdx.y;
   const int G = Hq / Hkv;
+  pdl_wait();
+  pdl_trigger();
   const int n0 = meta.off[qi], n1 = meta.off[qi + 1];
   const int DV = D / VE;                                    // vectors per head
   int nsl = kPoolThreads / DV;                              // token slices whose partial sums fit
@@ -77,7 +79,7 @@ __global__ void __launch_bounds__(kPoolThreads) qpool_kernel(const T* __restrict
     double t = 0.0;
     for (int k = 0; k < nsl; ++k) t += s_acc[k * D + col];
     t = t / (double)((long long)(n1 - n0) * G);
-    q64t[(long long)(g * D + col) * MUKV_MAX_QUESTIONS + qi] = t;
+    q64[(long long)(g * D + col) * cs + (long long)qi * qs] = t;
     sq += t * t;
   }
   sq = warp_sum(sq);
@@ -224,6 +226,73 @@ __global__ void __launch_bounds__(256) scan_kernel(const ScanParams sp) {
   }
 }
 
+// The same for at most kScanFew questions: a warp per row, plain double-precision multiply-adds.  The product is then
+// too thin for the tile above (64 questions wide, 32 rows in a block: 60 blocks of mostly padding for one question
+// and an hour of frames, 18 us); a row is one round trip to memory, its 16 doubles per lane and a butterfly: 4 us.
+// At eight questions and 9,100 rows the two take about the same time, which is where the line lies.
+constexpr int kScanFew = 8;
+
+template <int NQ>
+__global__ void __launch_bounds__(256) scan_few_kernel(const ScanParams sp) {
+  const int lane = threadIdx.x & 31;
+  const int C = sp.C, nq = sp.nq;
+  pdl_wait();                                                // the pooled questions are complete
+  pdl_trigger();
+  double qn = 0.0;                                           // lane i: norm of question i
+  if (lane < nq) {
+    for (int g = 0; g < sp.Hkv; ++g) qn += sp.qn2[(long long)lane * sp.Hkv + g];
+    qn = sqrt(qn);
+  }
+  const long long n_rows = sp.n_frm + sp.n_seg + sp.n_pat;
+  for (long long row = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); row < n_rows; row += (long long)gridDim.x * 8) {
+    const float* src = row < sp.n_frm ? sp.frame_key + row * C
+                       : (row < sp.n_frm + sp.n_seg ? sp.seg_key + (row - sp.n_frm) * C
+                                                    : sp.patch_key + (row - sp.n_frm - sp.n_seg) * C);
+    double dot[NQ], kk = 0.0;
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) dot[i] = 0.0;
+    for (int c0 = 0; c0 < C; c0 += 512) {
+      float4 x[4];                                           // (C is a multiple of 32, not always of 512)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c = c0 + 128 * j + 4 * lane;
+        x[j] = c < C ? __ldg(reinterpret_cast<const float4*>(src + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c = c0 + 128 * j + 4 * lane;
+        const double a0 = (double)x[j].x, a1 = (double)x[j].y, a2 = (double)x[j].z, a3 = (double)x[j].w;
+        kk = fma(a0, a0, fma(a1, a1, fma(a2, a2, fma(a3, a3, kk))));
+        if (c < C) {
+#pragma unroll
+          for (int i = 0; i < NQ; ++i) {
+            if (i < nq) {
+              const double2* q = reinterpret_cast<const double2*>(sp.q64t + (long long)i * C + c);
+              const double2 q0 = q[0], q1 = q[1];
+              dot[i] = fma(a0, q0.x, fma(a1, q0.y, fma(a2, q1.x, fma(a3, q1.y, dot[i]))));
+            }
+          }
+        }
+      }
+    }
+    const double knorm = sqrt(warp_sum(kk));
+    double mine = 0.0;
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+      const double d = warp_sum(dot[i]);
+      if (lane == i) mine = d;
+    }
+    if (lane < nq) {
+      double den = knorm * qn;
+      den = den > 1e-12 ? den : 1e-12;
+      const double sc = mine / den;
+      if (row < sp.n_frm) sp.s_frm[(long long)lane * sp.frm_stride + row] = sc;
+      else if (row < sp.n_frm + sp.n_seg) sp.s_seg[(long long)lane * sp.seg_stride + (row - sp.n_frm)] = sc;
+      else sp.s_pat[(long long)lane * sp.pat_stride + (row - sp.n_frm - sp.n_seg)] = sc;
+    }
+  }
+}
+
 // ------------------------------------------------------------------------------ ranking
 __device__ __forceinline__ unsigned long long order_key(double x) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
@@ -235,19 +304,31 @@ __device__ __forceinline__ double order_key_inv(unsigned long long k) {
 }
 
 constexpr int kRankList = 64;      // keys left in the radix select below which they are ranked directly
-constexpr int kRankCand = 256;     // scores at or above the tie band that the short emission path can hold
+constexpr int kRankCand = 512;     // candidates that are ranked among themselves (at most one per thread)
+constexpr int kRankBins = 512;     // bins of the linear histogram
+constexpr int kRankFew = 128;      // scores that are all candidates at once (the histogram costs as much as ranking that many)
 
 struct RankScratch {
-  unsigned int hist[256];
+  unsigned int hist[kRankBins];
+  unsigned int wmin[32], wmax[32];
+  int wcnt[32];
   int scan[40];
   unsigned long long prefix;
+  double tau;
   int remaining;
-  int bin_count, list_n, cand_n;
+  int bin, bin_count, list_n, cand_n;
   unsigned long long list[kRankList];
-  int cand_idx[kRankCand];
-  double cand_s[kRankCand];
-  unsigned char cand_band[kRankCand], cand_keep[kRankCand];
+  __align__(16) unsigned long long cand_key[kRankCand];      // order keys, padded with 0 to a multiple of four
+  __align__(16) int cand_idx[kRankCand];
+  __align__(16) int kept_idx[kRankCand];                     // cand_idx of what is kept, INT_MAX of the rest
 };
+
+// order-preserving bits of a float and back
+__device__ __forceinline__ unsigned order_key32(float x) {
+  const unsigned b = __float_as_uint(x);
+  return (b >> 31) ? ~b : (b | 0x80000000u);
+}
+__device__ __forceinline__ float order_key32_inv(unsigned k) { return __uint_as_float((k >> 31) ? (k & 0x7fffffffu) : ~k); }
 
 // Indices of the k highest scores among i in [0,n) with member(i) true, ascending by index, with
 // the tie band: tau = k-th largest; scores above tau+delta are taken; those within delta of tau
@@ -260,31 +341,187 @@ struct ArrScore {
   const double* p;
   __device__ double operator()(int i) const { return p[i]; }
 };
-struct AllMembers {
-  __device__ bool operator()(int) const { return true; }
+// every index takes part, or (patch-level blocks) those that hold tokens
+struct Members {
+  const int* cnt;
+  __device__ bool operator()(int i) const { return !cnt || cnt[i] > 0; }
 };
+
+// The k best of the n_cand candidates in sc->cand_key / cand_idx (all: every one), with the tie band, ascending by
+// index to out_idx / out_score; returns k.  n_cand <= kRankCand <= threads of the block.  Up to a quarter of the
+// threads' number of candidates, four threads share one (the counting loops are what takes the time).
+__device__ __noinline__ int rank_candidates(int n_cand, int k, bool all, double delta, int* out_idx, double* out_score,
+                                            RankScratch* sc) {
+  const int tid = threadIdx.x;
+  const int sh = n_cand <= (int)blockDim.x / 4 ? 2 : 0, parts = 1 << sh, part = tid & (parts - 1), me = tid >> sh;
+  const bool in = me < n_cand, first = part == 0;
+  const unsigned long long key = in ? sc->cand_key[me] : 0ull;
+  const int my_idx = in ? sc->cand_idx[me] : 0x7fffffff;
+  const int n4 = (n_cand + 3) & ~3;
+  if (tid >= n_cand && tid < n4) { sc->cand_key[tid] = 0ull; sc->kept_idx[tid] = 0x7fffffff; }
+  __syncthreads();
+  double tau = -1.0e300;
+  if (!all) {
+    int gt = 0, ge = 0;                                      // (the padding counts in neither: no score has key 0)
+    for (int t = 4 * part; in && t < n_cand; t += 4 * parts) {
+      const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(sc->cand_key + t);
+      const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(sc->cand_key + t + 2);
+      gt += (a.x > key) + (a.y > key) + (b.x > key) + (b.y > key);
+      ge += (a.x >= key) + (a.y >= key) + (b.x >= key) + (b.y >= key);
+    }
+    __syncwarp();
+    if (sh) {                                                // (sh is the same in every thread)
+      gt += __shfl_xor_sync(kFull, gt, 1);
+      gt += __shfl_xor_sync(kFull, gt, 2);
+      ge += __shfl_xor_sync(kFull, ge, 1);
+      ge += __shfl_xor_sync(kFull, ge, 2);
+    }
+    if (in && gt < k && k <= ge) sc->tau = order_key_inv(key);   // every writer holds the same value
+    __syncthreads();
+    tau = sc->tau;
+  }
+  const double s = order_key_inv(key);
+  const bool sure = in && (all || s > tau + delta);
+  const bool band = in && !sure && s >= tau - delta;
+  const int n_sure = __syncthreads_count(sure && first), n_band = __syncthreads_count(band && first);
+  bool keep = sure || band;
+  if (n_sure + n_band > k) {                                 // places inside the band go to the lowest indices
+    if (in && first) sc->kept_idx[me] = band ? my_idx : 0x7fffffff;
+    __syncthreads();
+    if (band) {
+      int before = 0;
+      for (int t = 0; t < n_cand; ++t) before += sc->kept_idx[t] < my_idx ? 1 : 0;
+      keep = before < k - n_sure;
+    }
+    __syncthreads();
+  }
+  if (in && first) sc->kept_idx[me] = keep ? my_idx : 0x7fffffff;
+  __syncthreads();
+  int pos = 0;
+  for (int t = 4 * part; in && t < n_cand; t += 4 * parts) {
+    const int4 a = *reinterpret_cast<const int4*>(sc->kept_idx + t);
+    pos += (a.x < my_idx) + (a.y < my_idx) + (a.z < my_idx) + (a.w < my_idx);
+  }
+  __syncwarp();
+  if (sh) {
+    pos += __shfl_xor_sync(kFull, pos, 1);
+    pos += __shfl_xor_sync(kFull, pos, 2);
+  }
+  if (keep && first) {
+    out_idx[pos] = my_idx;
+    if (out_score) out_score[pos] = s;
+  }
+  __syncthreads();
+  return k;
+}
+
+// bins of the linear histogram: the bin number does not decrease with s, whatever is rounded
+struct RankBins {
+  float lo, scale;
+  __device__ int operator()(float s) const {
+    const int b = (int)((s - lo) * scale);
+    return b < 0 ? 0 : (b < kRankBins ? b : kRankBins - 1);
+  }
+};
+__device__ __forceinline__ RankBins rank_bins(const RankScratch* sc, int nwarp) {
+  const int lane = threadIdx.x & 31, wl = lane < nwarp ? lane : 0;
+  const float lo = order_key32_inv(__reduce_min_sync(kFull, sc->wmin[wl]));
+  const float hi = order_key32_inv(__reduce_max_sync(kFull, sc->wmax[wl]));
+  return {lo, hi > lo ? fminf((float)kRankBins / (hi - lo), 1e35f) : 0.f};
+}
+// the bin that holds the k-th largest score (the histogram is complete); two barriers
+__device__ __forceinline__ int rank_find_bin(int k, RankScratch* sc) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int c = tid < kRankBins ? (int)sc->hist[kRankBins - 1 - tid] : 0;       // thread t: the bin t places from the top
+  int incl = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) sc->scan[warp] = incl;
+  __syncthreads();
+  const int above = __reduce_add_sync(kFull, lane < warp ? sc->scan[lane] : 0) + incl - c;
+  if (above < k && k <= above + c) sc->bin = kRankBins - 1 - tid;               // true for exactly one thread
+  __syncthreads();
+  return sc->bin;
+}
 
 template <typename ScoreFn, typename MemberFn>
 __device__ __noinline__ int block_topk_set(ScoreFn score, MemberFn member, int n, int k, double delta, int* out_idx,
                               double* out_score, RankScratch* sc) {
-  const int tid = threadIdx.x, nt = blockDim.x;
-  // how many members are there at all
-  int local = 0;
-  for (int i = tid; i < n; i += nt) local += member(i) ? 1 : 0;
-  __syncthreads();
-  if (tid == 0) sc->remaining = 0;
-  __syncthreads();
-  local = warp_sum(local);
-  if ((tid & 31) == 0 && local) atomicAdd(&sc->remaining, local);
-  __syncthreads();
-  const int n_mem = sc->remaining;
-  __syncthreads();
-  if (k > n_mem) k = n_mem;
-  if (k <= 0) return 0;
-  double tau;
-  if (k == n_mem) {
-    tau = -1.0e300;     // everything is taken; handled below by the "all" flag
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nt >> 5;
+  bool all = false, odd = false;
+  int n_mem = 0, bin = 0;
+  RankBins bin_of{0.f, 0.f};
+  __syncthreads();                                           // the scratch may still be read from a previous call
+  if (tid == 0) sc->cand_n = 0;
+  if (n > kRankFew) {
+    // The k-th largest score tau lies in one bin of a linear histogram.  Whatever could be above it or within the tie
+    // band of it is collected (any order) and ranked exactly: three sweeps over the scores instead of two for every
+    // eight bits of a radix select, whose first passes see nothing but the common exponent.
+    // ---- how many members, and the range of their scores (in single precision: it only places the bins)
+    unsigned kmin = 0xffffffffu, kmax = 0u;
+    int local = 0;
+    for (int i = tid; i < n; i += nt) {
+      if (!member(i)) continue;
+      const float s = (float)score(i);
+      const unsigned key = order_key32(s);
+      odd |= !(fabsf(s) < 1e30f);
+      kmin = min(kmin, key);
+      kmax = max(kmax, key);
+      ++local;
+    }
+    __syncwarp();
+    kmin = __reduce_min_sync(kFull, kmin);
+    kmax = __reduce_max_sync(kFull, kmax);
+    local = __reduce_add_sync(kFull, local);
+    if (lane == 0) { sc->wmin[warp] = kmin; sc->wmax[warp] = kmax; sc->wcnt[warp] = local; }
+    for (int b = tid; b < kRankBins; b += nt) sc->hist[b] = 0u;
+    odd = __syncthreads_or(odd) != 0;
+    n_mem = __reduce_add_sync(kFull, lane < nwarp ? sc->wcnt[lane] : 0);
+    if (k > n_mem) k = n_mem;
+    if (k <= 0) return 0;
+    all = (k == n_mem);
+    if (!odd) {
+      bin_of = rank_bins(sc, nwarp);
+      if (!all) {
+        for (int i = tid; i < n; i += nt)
+          if (member(i)) atomicAdd(&sc->hist[bin_of((float)score(i))], 1u);
+        __syncthreads();
+        bin = rank_find_bin(k, sc);
+      }
+    }
   } else {
+    __syncthreads();
+  }
+  if (!odd) {
+    const double slack = 2.0 * delta + 1e-12;
+    for (int i = tid; i < n; i += nt) {
+      if (!member(i)) continue;
+      const double s = score(i);
+      if (bin == 0 || bin_of((float)(s + slack)) >= bin) {
+        const int c = atomicAdd(&sc->cand_n, 1);
+        if (c < kRankCand) {
+          sc->cand_idx[c] = i;
+          sc->cand_key[c] = order_key(s);
+        }
+      }
+    }
+    __syncthreads();
+    const int n_cand = sc->cand_n;
+    if (n <= kRankFew) {
+      n_mem = n_cand;
+      if (k > n_mem) k = n_mem;
+      if (k <= 0) return 0;
+      all = (k == n_mem);
+    }
+    if (n_cand <= kRankCand) return rank_candidates(n_cand, k, all, delta, out_idx, out_score, sc);
+  }
+  // ---- too many candidates (a large k, a crowded bin), or scores that are not finite: radix select and an ordered walk
+  double tau = -1.0e300;                                     // (all: everything is taken)
+  __syncthreads();
+  if (!all) {
     // radix select of the k-th largest order key, 8 bits per pass from the top
     if (tid == 0) { sc->prefix = 0ull; sc->remaining = k; }
     for (int pass = 0; pass < 8; ++pass) {
@@ -352,52 +589,6 @@ __device__ __noinline__ int block_topk_set(ScoreFn score, MemberFn member, int n
     }
     tau = order_key_inv(sc->prefix);
   }
-  const bool all = (k == n_mem);
-  // Everything at or above the tie band, collected in any order.  When that is a short list (it
-  // holds k entries plus the ties), the band rule and the ascending output order are worked out
-  // on the list; the ordered walk over all n scores below is the fallback for a crowded band.
-  if (tid == 0) sc->cand_n = 0;
-  __syncthreads();
-  for (int i = tid; i < n; i += nt) {
-    if (!member(i)) continue;
-    const double s = score(i);
-    const bool sure = all || s > tau + delta;
-    const bool band = !sure && s >= tau - delta;
-    if (sure || band) {
-      const int c = atomicAdd(&sc->cand_n, 1);
-      if (c < kRankCand) {
-        sc->cand_idx[c] = i;
-        sc->cand_s[c] = s;
-        sc->cand_band[c] = band ? 1 : 0;
-      }
-    }
-  }
-  __syncthreads();
-  const int n_cand = sc->cand_n;
-  if (n_cand <= kRankCand) {
-    bool keep = false;
-    int my_idx = 0;
-    if (tid < n_cand) {
-      my_idx = sc->cand_idx[tid];
-      int n_sure = 0, band_before = 0;
-      for (int t = 0; t < n_cand; ++t) {
-        const bool bt = sc->cand_band[t] != 0;
-        n_sure += bt ? 0 : 1;
-        band_before += (bt && sc->cand_idx[t] < my_idx) ? 1 : 0;
-      }
-      keep = !sc->cand_band[tid] || band_before < k - n_sure;
-      sc->cand_keep[tid] = keep ? 1 : 0;
-    }
-    __syncthreads();
-    if (keep) {
-      int pos = 0;
-      for (int t = 0; t < n_cand; ++t) pos += (sc->cand_keep[t] && sc->cand_idx[t] < my_idx) ? 1 : 0;
-      out_idx[pos] = my_idx;
-      if (out_score) out_score[pos] = sc->cand_s[tid];
-    }
-    __syncthreads();
-    return k;
-  }
   // count the sure ones
   int cnt = 0;
   for (int i = tid; i < n; i += nt)
@@ -439,6 +630,102 @@ __device__ __noinline__ int block_topk_set(ScoreFn score, MemberFn member, int n
   return k;
 }
 
+// block_topk_set for scores in global memory, as many as `buf` holds: one pass reads them, keeps them in single
+// precision in shared memory and finds their range; the histogram and the collection run on those, four at a time,
+// and only the candidates' doubles are read again.  (On doubles in shared memory the three sweeps were bound by
+// instruction issue: 12 us for 10,800 scores.)
+__device__ __noinline__ int staged_topk_set(const double* scores, const int* cnt, int n, int k, double delta, int* out_idx,
+                                            double* out_score, float* buf, RankScratch* sc) {
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nt >> 5;
+  unsigned kmin = 0xffffffffu, kmax = 0u;
+  int local = 0;
+  bool odd = false;
+  __syncthreads();                                           // buffer and scratch may still be read from a previous call
+  const int n4 = (n + 3) & ~3;
+  for (int i0 = tid; i0 < n4; i0 += 8 * nt) {
+    double x[8];
+    int c[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 + u * nt;
+      x[u] = i < n ? scores[i] : 0.0;
+      c[u] = i < n ? (cnt ? cnt[i] : 1) : 0;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 + u * nt;
+      if (i < n4) {
+        const float s = (float)x[u];
+        if (c[u] > 0) {
+          const unsigned key = order_key32(s);
+          odd |= !(fabsf(s) < 1e30f);
+          kmin = min(kmin, key);
+          kmax = max(kmax, key);
+          ++local;
+        }
+        buf[i] = c[u] > 0 ? s : -INFINITY;                   // absent (it falls into bin 0, which may hold any number)
+      }
+    }
+  }
+  __syncwarp();
+  kmin = __reduce_min_sync(kFull, kmin);
+  kmax = __reduce_max_sync(kFull, kmax);
+  local = __reduce_add_sync(kFull, local);
+  if (lane == 0) { sc->wmin[warp] = kmin; sc->wmax[warp] = kmax; sc->wcnt[warp] = local; }
+  for (int b = tid; b < kRankBins; b += nt) sc->hist[b] = 0u;
+  if (tid == 0) sc->cand_n = 0;
+  odd = __syncthreads_or(odd) != 0;
+  const int n_mem = __reduce_add_sync(kFull, lane < nwarp ? sc->wcnt[lane] : 0);
+  if (k > n_mem) k = n_mem;
+  if (k <= 0) return 0;
+  const bool all = (k == n_mem);
+  if (!odd) {
+    const RankBins bin_of = rank_bins(sc, nwarp);
+    int bin = 0;
+    if (!all) {
+      for (int v = tid; v < n4 >> 2; v += nt) {
+        const float4 s = reinterpret_cast<const float4*>(buf)[v];
+        atomicAdd(&sc->hist[bin_of(s.x)], 1u);
+        atomicAdd(&sc->hist[bin_of(s.y)], 1u);
+        atomicAdd(&sc->hist[bin_of(s.z)], 1u);
+        atomicAdd(&sc->hist[bin_of(s.w)], 1u);
+      }
+      __syncthreads();
+      bin = rank_find_bin(k, sc);
+    }
+    // within delta of a score of that bin, and what single precision may have moved (scores of magnitude 1 or less
+    // by 6e-8; the range serves for others)
+    const float span = bin_of.scale > 0.f ? (float)kRankBins / bin_of.scale : 0.f;
+    const float slack = 2.f * (float)delta + 1e-6f * fmaxf(1.f, fmaxf(fabsf(bin_of.lo), fabsf(bin_of.lo + span)));
+    for (int v = tid; v < n4 >> 2; v += nt) {
+      const float4 q = reinterpret_cast<const float4*>(buf)[v];
+      const float s[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (bin_of(s[u] + slack) >= bin && s[u] > -INFINITY) {
+          const int c = atomicAdd(&sc->cand_n, 1);
+          if (c < kRankCand) sc->cand_idx[c] = 4 * v + u;
+        }
+      }
+    }
+    __syncthreads();
+    const int n_cand = sc->cand_n;
+    if (n_cand <= kRankCand) {
+      if (tid < n_cand) sc->cand_key[tid] = order_key(scores[sc->cand_idx[tid]]);
+      __syncthreads();
+      return rank_candidates(n_cand, k, all, delta, out_idx, out_score, sc);
+    }
+  }
+  return block_topk_set(ArrScore{scores}, Members{cnt}, n, k, delta, out_idx, out_score, sc);
+}
+
+// the one of the two that fits
+__device__ __forceinline__ int topk_set(const double* scores, const int* cnt, int n, int k, double delta, int* out_idx,
+                                        double* out_score, float* buf, int cap, RankScratch* sc) {
+  if (n > kRankFew && n <= cap) return staged_topk_set(scores, cnt, n, k, delta, out_idx, out_score, buf, sc);
+  return block_topk_set(ArrScore{scores}, Members{cnt}, n, k, delta, out_idx, out_score, sc);
+}
+
 struct RankParams {
   int nq, C, fseg;
   int k_seg, k_frm, k_pat, top_n, mode;
@@ -455,7 +742,7 @@ struct RankParams {
   const int* patch_cnt;                   // [frames][S]
   int* seg_idx; int* frm_idx; int* pat_idx; float* seg_score; float* frm_score; float* pat_score;
   int* counts; int counts_stride;         // 2 or 3 ints per question
-  int stage;                              // 1: the question's frame and segment scores are copied to shared memory first
+  int stage;                              // scores that the buffer of staged_topk_set holds
 };
 
 constexpr int kRankThreads = 512;
@@ -472,31 +759,39 @@ struct RankShared {
   double s_new[kMaxCand];
   int pick[MUKV_MAX_TOPK];
   double pick_score[MUKV_MAX_TOPK];
-  double gn;
+  double gn[kRankThreads / 32];
 };
 
 // Stage 1 + stage 2 of one granularity for one question, run by the whole block: top-2k candidates
 // by cosine among the members, Eq. 8 against the global query gq (norm gnorm; have_g false: gamma = 0),
 // then the k best by the calibrated score.  PARALLEL / HIER callers pass semi = false: the k best by
 // cosine among the members.  Results (ascending ids) in sh->pick / sh->pick_score; returns the count.
-template <typename MemberFn>
-__device__ __noinline__ int rank_level(const double* scores, MemberFn member, int n, int k, bool semi, double lambda,
+__device__ __noinline__ int rank_level(const double* scores, const int* cnt, int n, int k, bool semi, double lambda,
                                        double delta, const float* keys, int C, const double* gq, double gnorm,
-                                       bool have_g, RankShared* sh) {
+                                       bool have_g, RankShared* sh, float* buf, int cap) {
   const int tid = threadIdx.x;
-  const ArrScore s1{scores};
-  if (!semi) return block_topk_set(s1, member, n, k, delta, sh->pick, sh->pick_score, &sh->sc);
-  const int n_cand = block_topk_set(s1, member, n, 2 * k, delta, sh->cand, sh->cand_score, &sh->sc);
+  const int n_cand = topk_set(scores, cnt, n, semi ? 2 * k : k, delta, semi ? sh->cand : sh->pick,
+                              semi ? sh->cand_score : sh->pick_score, buf, cap, &sh->sc);
+  if (!semi) return n_cand;
   // Eq. 8 for every candidate: one warp per candidate
   const int lane = tid & 31, warp = tid >> 5;
   for (int ci = warp; ci < n_cand; ci += kRankThreads / 32) {
     const float* kr = keys + (long long)sh->cand[ci] * C;
     double dot = 0.0, kk = 0.0;
-    for (int c = lane; c < C; c += 32) {
-      const double x = (double)kr[c];
-      dot = fma(x, gq[c], dot);
-      kk = fma(x, x, kk);
+    for (int c0 = lane; c0 < C; c0 += 16 * 32) {             // (sixteen loads in flight)
+      float x[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) x[u] = c0 + u * 32 < C ? __ldg(kr + c0 + u * 32) : 0.f;
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        if (c0 + u * 32 < C) {
+          const double y = (double)x[u];
+          dot = fma(y, gq[c0 + u * 32], dot);
+          kk = fma(y, y, kk);
+        }
+      }
     }
+    __syncwarp();
     dot = warp_sum(dot);
     kk = warp_sum(kk);
     if (lane == 0) {
@@ -510,9 +805,7 @@ __device__ __noinline__ int rank_level(const double* scores, MemberFn member, in
     }
   }
   __syncthreads();
-  const ArrScore new_score{sh->s_new};
-  const AllMembers always;
-  const int c = block_topk_set(new_score, always, n_cand, k, delta, sh->pick, sh->pick_score, &sh->sc);
+  const int c = topk_set(sh->s_new, nullptr, n_cand, k, delta, sh->pick, sh->pick_score, buf, 0, &sh->sc);
   // pick holds positions in the candidate list (ascending position = ascending block id)
   for (int i = tid; i < c; i += kRankThreads) sh->pick[i] = sh->cand[sh->pick[i]];
   __syncthreads();
@@ -533,6 +826,7 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
 
   const int qi = blockIdx.x, tid = threadIdx.x;
   pdl_wait();                                                // the scores of the scan are complete
+  if (p.nq <= kScanFew) pdl_trigger();                       // (many of these blocks would leave the gather an uneven start)
   const int C = p.C;
   long long tl = meta.t_limit[qi];
   if (tl > p.n_frm) tl = p.n_frm;
@@ -544,46 +838,50 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
   if (n_seg > p.n_seg) n_seg = (int)p.n_seg;
   const double* sf = p.s_frm + (long long)qi * p.frm_stride;
   const double* ss = p.s_seg + (long long)qi * p.seg_stride;
-  if (p.stage) {
-    // every selection below scans the scores several times: do that out of shared memory
-    double* st_f = gq + C;
-    double* st_s = st_f + n_frm;
-    for (int i = tid; i < n_frm; i += kRankThreads) st_f[i] = sf[i];
-    for (int i = tid; i < n_seg; i += kRankThreads) st_s[i] = ss[i];
-    __syncthreads();
-    sf = st_f;
-    ss = st_s;
-  }
-  const ArrScore seg_score{ss};
-  const AllMembers always;
+  const double* sp = p.s_pat + (long long)qi * p.pat_stride;
+  float* buf = reinterpret_cast<float*>(gq + C);             // [p.stage], 16-byte aligned (C is even)
   const bool semi = p.mode == MUKV_RETR_SEMI;
 
   // ---- global query = mean of the top-N segment keys (stage 1 order)
   bool have_g = false;
   double gnorm = 0.0;
+  int c_seg = -1;
   if (semi) {
     const int N = p.top_n > 0 ? p.top_n : p.k_seg;
-    const int n_top = block_topk_set(seg_score, always, n_seg, N, p.delta, sh.top, (double*)nullptr, &sh.sc);
+    // (without a lambda for segments the N = k_seg best are also the result: one ranking serves both)
+    const bool same = N == p.k_seg && !(p.lam_seg > 0.0);
+    int* top = same ? sh.pick : sh.top;
+    const int n_top = topk_set(ss, nullptr, n_seg, N, p.delta, top, same ? sh.pick_score : (double*)nullptr, buf, p.stage, &sh.sc);
+    if (same) c_seg = n_top;
     double part = 0.0;
     for (int c = tid; c < C; c += kRankThreads) {
       double t = 0.0;
-      for (int i = 0; i < n_top; ++i) t += (double)p.seg_key[(long long)sh.top[i] * C + c];
+      for (int i = 0; i < n_top; i += 8) {                   // (eight loads in flight, added in order)
+        float x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = i + u < n_top ? p.seg_key[(long long)top[i + u] * C + c] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) t += (double)x[u];
+      }
       t = n_top > 0 ? t / (double)n_top : 0.0;
       gq[c] = t;
       part += t * t;
     }
-    if (tid == 0) sh.gn = 0.0;
-    __syncthreads();
+    __syncwarp();
     part = warp_sum(part);
-    if ((tid & 31) == 0) atomicAdd(&sh.gn, part);
+    if ((tid & 31) == 0) sh.gn[tid >> 5] = part;
     __syncthreads();
-    gnorm = sqrt(sh.gn);
+    double gn = 0.0;
+#pragma unroll
+    for (int w = 0; w < kRankThreads / 32; ++w) gn += sh.gn[w];
+    gnorm = sqrt(gn);
     have_g = n_top > 0;
   }
 
   // ---- segments (the paper's lambda for them is 0: final = stage-1 top-k)
-  const int c_seg = rank_level(ss, always, n_seg, p.k_seg, semi && p.lam_seg > 0.0, p.lam_seg, p.delta, p.seg_key, C, gq,
-                               gnorm, have_g, &sh);
+  if (c_seg < 0)
+    c_seg = rank_level(ss, nullptr, n_seg, p.k_seg, semi && p.lam_seg > 0.0, p.lam_seg, p.delta, p.seg_key, C, gq, gnorm,
+                       have_g, &sh, buf, p.stage);
   rank_emit(p.seg_idx, p.seg_score, (long long)qi * p.k_seg, p.k_seg, c_seg, &sh);
   for (int i = tid; i < c_seg; i += kRankThreads) sh.sel_seg[i] = sh.pick[i];
   __syncthreads();
@@ -602,7 +900,8 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
     for (int i = tid; i < c_frm; i += kRankThreads) sh.pick[i] = frame_of(sh.pick[i]);
     __syncthreads();
   } else {
-    c_frm = rank_level(sf, always, n_frm, p.k_frm, semi, p.lam_frm, p.delta, p.frame_key, C, gq, gnorm, have_g, &sh);
+    c_frm = rank_level(sf, nullptr, n_frm, p.k_frm, semi, p.lam_frm, p.delta, p.frame_key, C, gq, gnorm, have_g, &sh, buf,
+                       p.stage);
   }
   rank_emit(p.frm_idx, p.frm_score, (long long)qi * p.k_frm, p.k_frm, c_frm, &sh);
   __syncthreads();
@@ -612,12 +911,11 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
   if (p.k_pat > 0) {
     const int S = p.S;
     const int* cnt = p.patch_cnt;
-    const double* spat = p.s_pat + (long long)qi * p.pat_stride;
     if (S > 0) {
       if (p.mode == MUKV_RETR_HIER) {
         const int per_seg = fseg * S;
         auto block_of = [&](int i) { return sh.sel_seg[i / per_seg] * per_seg + i % per_seg; };
-        auto score_h = [&](int i) { return spat[block_of(i)]; };
+        auto score_h = [&](int i) { return sp[block_of(i)]; };
         auto member_h = [&](int i) {
           const int b = block_of(i);
           return b < n_frm * S && cnt[b] > 0;
@@ -626,9 +924,8 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
         for (int i = tid; i < c_pat; i += kRankThreads) sh.pick[i] = block_of(sh.pick[i]);
         __syncthreads();
       } else {
-        auto member = [&](int b) { return cnt[b] > 0; };
-        c_pat = rank_level(spat, member, n_frm * S, p.k_pat, semi, p.lam_pat, p.delta, p.patch_key, C, gq, gnorm, have_g,
-                           &sh);
+        c_pat = rank_level(sp, cnt, n_frm * S, p.k_pat, semi, p.lam_pat, p.delta, p.patch_key, C, gq, gnorm, have_g, &sh, buf,
+                           p.stage);
       }
     }
     rank_emit(p.pat_idx, p.pat_score, (long long)qi * p.k_pat, p.k_pat, c_pat, &sh);
@@ -653,6 +950,7 @@ struct GatherParams {
 // unit = (question, plane = l*2+kv, slot): one contiguous run of the page goes to one contiguous
 // run of the decode buffer.
 __global__ void __launch_bounds__(256) gather_kernel(const GatherParams p) {
+  pdl_wait();                                              // the selection may be the work of the kernel in front
   const long long planes = (long long)p.L * 2;
   const long long n_units = (long long)p.nq * planes * p.k_frm;
   for (long long u = blockIdx.x; u < n_units; u += gridDim.x) {
@@ -731,6 +1029,7 @@ __global__ void __launch_bounds__(256) gather3_kernel(const Gather3Params p) {
   __shared__ int s_off[MUKV_MAX_TOPK + 1];                 // first row of each selected patch block
   __shared__ long long s_src[kGatherListCap];              // byte offset in the store of each listed row
   __shared__ int s_row0;
+  pdl_wait();
   const long long planes = (long long)p.L * 2;
   const int upp = p.k_frm + 1;                             // units per (question, plane)
   const long long n_units = (long long)p.nq * planes * upp;

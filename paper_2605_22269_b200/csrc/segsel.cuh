@@ -438,9 +438,7 @@ __global__ void __launch_bounds__(kSegSelThreads) segsel_kernel(const SegSelPara
     if (tid == 0 && any_bad && sp.status) atomicCAS(sp.status, 0, kStatusNonFinite);
     __syncthreads();
     // ---- ascending
-    const ArrScore score{sa};
-    const AllMembers always;
-    n_kept = block_topk_set(score, always, O, k, (double)sp.tie_eps, oi, (double*)nullptr, &sc);
+    n_kept = block_topk_set(ArrScore{sa}, Members{nullptr}, O, k, (double)sp.tie_eps, oi, (double*)nullptr, &sc);
     __syncthreads();
   }
   // first kept token of every frame: lower bound of f * P in the ascending list
