@@ -42,7 +42,7 @@ struct WorkLayout {
   size_t q_terms, k_terms; // fp32 chunks: queries and keys of the scoring layers as three bf16 terms
   size_t colsum_f, colsum_p, ifft_f, colsum_d, ifft_d, frame_counter, flagged, n_flagged, tail_ctr, sel_flag,
       seg_flag, stat_refined, dev_status;
-  size_t q64, qnorm, s_frm, s_seg, s_pat, wtab, total;
+  size_t q64, qnorm, s_frm, s_seg, s_pat, f_frm, f_seg, f_pat, wtab, total;
   size_t zero_begin, zero_end;          // region that must start as zeros
 };
 
@@ -259,6 +259,9 @@ constexpr int kRefineSplit = 4;     // blocks per query head in the double-preci
 constexpr float kFlagMargin = 3e-6f;
 constexpr float kFlatRatio = 1e-3f;
 
+// rows of single-precision scores start on 16 bytes
+inline long long pad4(long long n) { return (n + 3) / 4 * 4; }
+
 WorkLayout work_layout(const mukv_config& c) {
   WorkLayout w;
   const size_t F = c.max_frames_per_chunk, P = c.tokens_per_frame;
@@ -288,6 +291,10 @@ WorkLayout work_layout(const mukv_config& c) {
   w.s_seg = off;          off = align_up(off + (size_t)MUKV_MAX_QUESTIONS * max_segs * sizeof(double));
   w.s_pat = off;          off = align_up(off + (size_t)MUKV_MAX_QUESTIONS * c.max_frames * c.patch_split * c.patch_split *
                                                sizeof(double));
+  w.f_frm = off;          off = align_up(off + (size_t)MUKV_MAX_QUESTIONS * pad4(c.max_frames) * sizeof(float));
+  w.f_seg = off;          off = align_up(off + (size_t)MUKV_MAX_QUESTIONS * pad4(max_segs) * sizeof(float));
+  w.f_pat = off;          off = align_up(off + (size_t)MUKV_MAX_QUESTIONS * pad4(c.max_frames * c.patch_split * c.patch_split) *
+                                               sizeof(float));
   w.wtab = off;           off = align_up(off + (ts.ok || ts.split ? (size_t)3 * c.head_dim * c.head_dim * 2 : 0));
   const size_t tf = ts.split ? (size_t)ts.split_frames * Ls * P * 6 : 0;
   w.q_terms = off;        off = align_up(off + tf * c.n_q_heads * c.head_dim);
@@ -917,8 +924,13 @@ mukv_status retrieve_impl(mukv_ctx* ctx, const void* d_qtok, const int32_t* h_q_
       sc.C = C; sc.nq = nq; sc.Hkv = c.n_kv_heads; sc.q64t = q64; sc.qn2 = qnorm;
       sc.s_frm = s_frm; sc.s_seg = s_seg; sc.s_pat = s_pat;
       sc.frm_stride = c.max_frames; sc.seg_stride = ctx->sl.max_segs; sc.pat_stride = (long long)c.max_frames * S;
+      sc.f_frm = reinterpret_cast<float*>(ctx->ws + ctx->wl.f_frm); sc.f_frm_stride = pad4(c.max_frames);
+      sc.f_seg = reinterpret_cast<float*>(ctx->ws + ctx->wl.f_seg); sc.f_seg_stride = pad4(ctx->sl.max_segs);
+      sc.f_pat = reinterpret_cast<float*>(ctx->ws + ctx->wl.f_pat); sc.f_pat_stride = pad4((long long)c.max_frames * S);
+      sc.patch_cnt = reinterpret_cast<const int*>(ctx->store + ctx->sl.patch_cnt);
       if (few) {
-        const long long want = (rows + 7) / 8, most = 8LL * ctx->n_sms;     // a warp per row, eight blocks per SM
+        const int per_block = nq > 1 ? 16 : 8;                 // a row or two per warp, up to eight blocks per SM
+        const long long want = (rows + per_block - 1) / per_block, most = 8LL * ctx->n_sms;
         const dim3 grid((unsigned)(want < most ? want : most));
         e = launch_k(nq == 1 ? scan_few_kernel<1> : nq <= 4 ? scan_few_kernel<4> : scan_few_kernel<kScanFew>, grid, 256, 0, st,
                      !ctx->prof_on, sc);
@@ -943,13 +955,14 @@ mukv_status retrieve_impl(mukv_ctx* ctx, const void* d_qtok, const int32_t* h_q_
     {
       ProfScope ps(ctx, 6, st);
       size_t rank_smem = (size_t)C * sizeof(double);
-      // single-precision copies of one granularity's scores at a time, if they fit
-      const size_t room = (size_t)kRankStageBytes - rank_smem - 16;
-      long long most = n_frm > n_seg ? n_frm : n_seg;
-      if (n_pat > most && (size_t)n_pat * sizeof(float) <= room) most = n_pat;
-      if ((size_t)most * sizeof(float) <= room) {
-        rp.stage = (int)most;
-        rank_smem += (size_t)most * sizeof(float) + 16;
+      rp.f_frm = reinterpret_cast<const float*>(ctx->ws + ctx->wl.f_frm); rp.f_frm_stride = pad4(c.max_frames);
+      rp.f_seg = reinterpret_cast<const float*>(ctx->ws + ctx->wl.f_seg); rp.f_seg_stride = pad4(ctx->sl.max_segs);
+      rp.f_pat = reinterpret_cast<const float*>(ctx->ws + ctx->wl.f_pat); rp.f_pat_stride = pad4((long long)c.max_frames * S);
+      const size_t room = (size_t)kRankStageBytes - rank_smem;
+      const size_t b1 = (size_t)(pad4(n_frm) + pad4(n_seg)) * sizeof(float), b2 = (size_t)pad4(n_pat) * sizeof(float);
+      if (b1 <= room) {
+        rp.stage = n_pat == 0 ? 1 : b1 + b2 <= room ? 2 : b2 <= room ? 3 : 1;
+        rank_smem += rp.stage == 2 ? b1 + b2 : rp.stage == 3 && b2 > b1 ? b2 : b1;
       }
       e = launch_k(rank_kernel, dim3(nq), kRankThreads, rank_smem, st, !ctx->prof_on, rp, meta);
     }

@@ -11,6 +11,7 @@
 //   gather_kernel   Eq. 9   copies the selected pages into the per-question decode buffers
 #pragma once
 #include "common.cuh"
+#include "tc.cuh"
 
 namespace mukv {
 
@@ -119,7 +120,27 @@ struct ScanParams {
   const double* q64t; const double* qn2;
   double* s_frm; double* s_seg; double* s_pat;
   long long frm_stride, seg_stride, pat_stride;
+  // the scores in single precision, which rank_kernel sifts; a patch-level block without tokens is marked kScanAbsent
+  float* f_frm; float* f_seg; float* f_pat;
+  long long f_frm_stride, f_seg_stride, f_pat_stride;         // multiples of four
+  const int* patch_cnt;
 };
+#define kScanAbsent (-INFINITY)
+
+__device__ __forceinline__ void scan_store(const ScanParams& sp, int qi, long long row, double sc) {
+  if (row < sp.n_frm) {
+    sp.s_frm[(long long)qi * sp.frm_stride + row] = sc;
+    sp.f_frm[(long long)qi * sp.f_frm_stride + row] = (float)sc;
+  } else if (row < sp.n_frm + sp.n_seg) {
+    row -= sp.n_frm;
+    sp.s_seg[(long long)qi * sp.seg_stride + row] = sc;
+    sp.f_seg[(long long)qi * sp.f_seg_stride + row] = (float)sc;
+  } else {
+    row -= sp.n_frm + sp.n_seg;
+    sp.s_pat[(long long)qi * sp.pat_stride + row] = sc;
+    sp.f_pat[(long long)qi * sp.f_pat_stride + row] = sp.patch_cnt[row] > 0 ? (float)sc : kScanAbsent;
+  }
+}
 
 __global__ void __launch_bounds__(256) scan_kernel(const ScanParams sp) {
   const float* __restrict__ frame_key = sp.frame_key;
@@ -128,9 +149,6 @@ __global__ void __launch_bounds__(256) scan_kernel(const ScanParams sp) {
   const int C = sp.C, nq = sp.nq, Hkv = sp.Hkv;
   const double* __restrict__ q64t = sp.q64t;
   const double* __restrict__ qn2 = sp.qn2;
-  double* __restrict__ s_frm = sp.s_frm;
-  double* __restrict__ s_seg = sp.s_seg;
-  const long long frm_stride = sp.frm_stride, seg_stride = sp.seg_stride;
   __shared__ float rows[kScanRows][kScanCC + 1];
   __shared__ __align__(16) double qs[kScanCC][kScanQPad];
   __shared__ double s_knorm[kScanRows];
@@ -217,9 +235,7 @@ __global__ void __launch_bounds__(256) scan_kernel(const ScanParams sp) {
           double den = knorm * s_qn[qi];
           den = den > 1e-12 ? den : 1e-12;
           const double sc = acc[nt][j] / den;
-          if (row < n_frm) s_frm[(long long)qi * frm_stride + row] = sc;
-          else if (row < n_frm + n_seg) s_seg[(long long)qi * seg_stride + (row - n_frm)] = sc;
-          else sp.s_pat[(long long)qi * sp.pat_stride + (row - n_frm - n_seg)] = sc;
+          scan_store(sp, qi, row, sc);
         }
       }
     }
@@ -244,51 +260,70 @@ __global__ void __launch_bounds__(256) scan_few_kernel(const ScanParams sp) {
     qn = sqrt(qn);
   }
   const long long n_rows = sp.n_frm + sp.n_seg + sp.n_pat;
-  for (long long row = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); row < n_rows; row += (long long)gridDim.x * 8) {
-    const float* src = row < sp.n_frm ? sp.frame_key + row * C
-                       : (row < sp.n_frm + sp.n_seg ? sp.seg_key + (row - sp.n_frm) * C
-                                                    : sp.patch_key + (row - sp.n_frm - sp.n_seg) * C);
-    double dot[NQ], kk = 0.0;
+  auto row_ptr = [&](long long row) {
+    return row < sp.n_frm ? sp.frame_key + row * C
+           : (row < sp.n_frm + sp.n_seg ? sp.seg_key + (row - sp.n_frm) * C
+                                        : sp.patch_key + (row - sp.n_frm - sp.n_seg) * C);
+  };
+  constexpr int RW = NQ > 1 ? 2 : 1;                         // rows of a warp (they share the loads of the questions)
+  for (long long row = ((long long)blockIdx.x * 8 + (threadIdx.x >> 5)) * RW; row < n_rows; row += (long long)gridDim.x * 8 * RW) {
+    const float* src[RW];
+    double dot[RW][NQ], kk[RW];
 #pragma unroll
-    for (int i = 0; i < NQ; ++i) dot[i] = 0.0;
+    for (int r = 0; r < RW; ++r) {
+      src[r] = row_ptr(row + r < n_rows ? row + r : row);
+      kk[r] = 0.0;
+#pragma unroll
+      for (int i = 0; i < NQ; ++i) dot[r][i] = 0.0;
+    }
     for (int c0 = 0; c0 < C; c0 += 512) {
-      float4 x[4];                                           // (C is a multiple of 32, not always of 512)
+      float4 x[RW][4];                                       // (C is a multiple of 32, not always of 512)
+#pragma unroll
+      for (int r = 0; r < RW; ++r)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int c = c0 + 128 * j + 4 * lane;
+          x[r][j] = c < C ? __ldg(reinterpret_cast<const float4*>(src[r] + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int c = c0 + 128 * j + 4 * lane;
-        x[j] = c < C ? __ldg(reinterpret_cast<const float4*>(src + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
+        double a[RW][4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int c = c0 + 128 * j + 4 * lane;
-        const double a0 = (double)x[j].x, a1 = (double)x[j].y, a2 = (double)x[j].z, a3 = (double)x[j].w;
-        kk = fma(a0, a0, fma(a1, a1, fma(a2, a2, fma(a3, a3, kk))));
+        for (int r = 0; r < RW; ++r) {
+          a[r][0] = (double)x[r][j].x; a[r][1] = (double)x[r][j].y; a[r][2] = (double)x[r][j].z; a[r][3] = (double)x[r][j].w;
+          kk[r] = fma(a[r][0], a[r][0], fma(a[r][1], a[r][1], fma(a[r][2], a[r][2], fma(a[r][3], a[r][3], kk[r]))));
+        }
         if (c < C) {
 #pragma unroll
           for (int i = 0; i < NQ; ++i) {
             if (i < nq) {
               const double2* q = reinterpret_cast<const double2*>(sp.q64t + (long long)i * C + c);
               const double2 q0 = q[0], q1 = q[1];
-              dot[i] = fma(a0, q0.x, fma(a1, q0.y, fma(a2, q1.x, fma(a3, q1.y, dot[i]))));
+#pragma unroll
+              for (int r = 0; r < RW; ++r)
+                dot[r][i] = fma(a[r][0], q0.x, fma(a[r][1], q0.y, fma(a[r][2], q1.x, fma(a[r][3], q1.y, dot[r][i]))));
             }
           }
         }
       }
     }
-    const double knorm = sqrt(warp_sum(kk));
-    double mine = 0.0;
+    __syncwarp();
 #pragma unroll
-    for (int i = 0; i < NQ; ++i) {
-      const double d = warp_sum(dot[i]);
-      if (lane == i) mine = d;
-    }
-    if (lane < nq) {
-      double den = knorm * qn;
-      den = den > 1e-12 ? den : 1e-12;
-      const double sc = mine / den;
-      if (row < sp.n_frm) sp.s_frm[(long long)lane * sp.frm_stride + row] = sc;
-      else if (row < sp.n_frm + sp.n_seg) sp.s_seg[(long long)lane * sp.seg_stride + (row - sp.n_frm)] = sc;
-      else sp.s_pat[(long long)lane * sp.pat_stride + (row - sp.n_frm - sp.n_seg)] = sc;
+    for (int r = 0; r < RW; ++r) {
+      const double knorm = sqrt(warp_sum(kk[r]));
+      double mine = 0.0;
+#pragma unroll
+      for (int i = 0; i < NQ; ++i) {
+        const double d = warp_sum(dot[r][i]);
+        if (lane == i) mine = d;
+      }
+      if (lane < nq && row + r < n_rows) {
+        double den = knorm * qn;
+        den = den > 1e-12 ? den : 1e-12;
+        scan_store(sp, lane, row + r, mine / den);
+      }
+      __syncwarp();
     }
   }
 }
@@ -630,44 +665,33 @@ __device__ __noinline__ int block_topk_set(ScoreFn score, MemberFn member, int n
   return k;
 }
 
-// block_topk_set for scores in global memory, as many as `buf` holds: one pass reads them, keeps them in single
-// precision in shared memory and finds their range; the histogram and the collection run on those, four at a time,
-// and only the candidates' doubles are read again.  (On doubles in shared memory the three sweeps were bound by
-// instruction issue: 12 us for 10,800 scores.)
+// block_topk_set for scores whose single-precision copies lie in shared memory (buf, 16-byte aligned, kScanAbsent where a
+// score takes no part; up to three values behind the n-th are overwritten): range, histogram and collection run on the
+// copies, four at a time, and only the candidates' doubles are read.  (On doubles the three sweeps were bound by
+// instruction issue: 12 us for 10,800 scores; loading and converting them here took another 7.)
 __device__ __noinline__ int staged_topk_set(const double* scores, const int* cnt, int n, int k, double delta, int* out_idx,
                                             double* out_score, float* buf, RankScratch* sc) {
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nt >> 5;
-  unsigned kmin = 0xffffffffu, kmax = 0u;
   int local = 0;
   bool odd = false;
-  __syncthreads();                                           // buffer and scratch may still be read from a previous call
   const int n4 = (n + 3) & ~3;
-  for (int i0 = tid; i0 < n4; i0 += 8 * nt) {
-    double x[8];
-    int c[8];
+  if (tid < n4 - n) buf[n + tid] = kScanAbsent;
+  __syncthreads();                                           // (the scratch may still be read from a previous call, too)
+  float lo = INFINITY, hi = -INFINITY;
+  for (int v = tid; v < n4 >> 2; v += nt) {
+    const float4 q = reinterpret_cast<const float4*>(buf)[v];
+    const float s[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int i = i0 + u * nt;
-      x[u] = i < n ? scores[i] : 0.0;
-      c[u] = i < n ? (cnt ? cnt[i] : 1) : 0;
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int i = i0 + u * nt;
-      if (i < n4) {
-        const float s = (float)x[u];
-        if (c[u] > 0) {
-          const unsigned key = order_key32(s);
-          odd |= !(fabsf(s) < 1e30f);
-          kmin = min(kmin, key);
-          kmax = max(kmax, key);
-          ++local;
-        }
-        buf[i] = c[u] > 0 ? s : -INFINITY;                   // absent (it falls into bin 0, which may hold any number)
-      }
+    for (int u = 0; u < 4; ++u) {
+      const bool absent = s[u] == kScanAbsent;
+      lo = fminf(lo, absent ? INFINITY : s[u]);
+      hi = fmaxf(hi, s[u]);
+      odd |= !absent && !(fabsf(s[u]) < 1e30f);
+      local += absent ? 0 : 1;
     }
   }
   __syncwarp();
+  unsigned kmin = order_key32(lo), kmax = order_key32(hi);
   kmin = __reduce_min_sync(kFull, kmin);
   kmax = __reduce_max_sync(kFull, kmax);
   local = __reduce_add_sync(kFull, local);
@@ -702,7 +726,7 @@ __device__ __noinline__ int staged_topk_set(const double* scores, const int* cnt
       const float s[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        if (bin_of(s[u] + slack) >= bin && s[u] > -INFINITY) {
+        if (bin_of(s[u] + slack) >= bin && s[u] != kScanAbsent) {
           const int c = atomicAdd(&sc->cand_n, 1);
           if (c < kRankCand) sc->cand_idx[c] = 4 * v + u;
         }
@@ -719,10 +743,10 @@ __device__ __noinline__ int staged_topk_set(const double* scores, const int* cnt
   return block_topk_set(ArrScore{scores}, Members{cnt}, n, k, delta, out_idx, out_score, sc);
 }
 
-// the one of the two that fits
+// the one of the two that fits (buf: null where there are no copies)
 __device__ __forceinline__ int topk_set(const double* scores, const int* cnt, int n, int k, double delta, int* out_idx,
-                                        double* out_score, float* buf, int cap, RankScratch* sc) {
-  if (n > kRankFew && n <= cap) return staged_topk_set(scores, cnt, n, k, delta, out_idx, out_score, buf, sc);
+                                        double* out_score, float* buf, RankScratch* sc) {
+  if (n > kRankFew && buf) return staged_topk_set(scores, cnt, n, k, delta, out_idx, out_score, buf, sc);
   return block_topk_set(ArrScore{scores}, Members{cnt}, n, k, delta, out_idx, out_score, sc);
 }
 
@@ -742,7 +766,10 @@ struct RankParams {
   const int* patch_cnt;                   // [frames][S]
   int* seg_idx; int* frm_idx; int* pat_idx; float* seg_score; float* frm_score; float* pat_score;
   int* counts; int counts_stride;         // 2 or 3 ints per question
-  int stage;                              // scores that the buffer of staged_topk_set holds
+  const float* f_frm; const float* f_seg; const float* f_pat;     // single-precision copies of the scores
+  long long f_frm_stride, f_seg_stride, f_pat_stride;
+  int stage;                              // 1: the copies of segments and frames fit in shared memory; 2: those of the
+                                          // patch-level blocks beside them; 3: those in place of them, afterwards
 };
 
 constexpr int kRankThreads = 512;
@@ -768,10 +795,10 @@ struct RankShared {
 // cosine among the members.  Results (ascending ids) in sh->pick / sh->pick_score; returns the count.
 __device__ __noinline__ int rank_level(const double* scores, const int* cnt, int n, int k, bool semi, double lambda,
                                        double delta, const float* keys, int C, const double* gq, double gnorm,
-                                       bool have_g, RankShared* sh, float* buf, int cap) {
+                                       bool have_g, RankShared* sh, float* buf) {
   const int tid = threadIdx.x;
   const int n_cand = topk_set(scores, cnt, n, semi ? 2 * k : k, delta, semi ? sh->cand : sh->pick,
-                              semi ? sh->cand_score : sh->pick_score, buf, cap, &sh->sc);
+                              semi ? sh->cand_score : sh->pick_score, buf, &sh->sc);
   if (!semi) return n_cand;
   // Eq. 8 for every candidate: one warp per candidate
   const int lane = tid & 31, warp = tid >> 5;
@@ -805,7 +832,7 @@ __device__ __noinline__ int rank_level(const double* scores, const int* cnt, int
     }
   }
   __syncthreads();
-  const int c = topk_set(sh->s_new, nullptr, n_cand, k, delta, sh->pick, sh->pick_score, buf, 0, &sh->sc);
+  const int c = topk_set(sh->s_new, nullptr, n_cand, k, delta, sh->pick, sh->pick_score, (float*)nullptr, &sh->sc);
   // pick holds positions in the candidate list (ascending position = ascending block id)
   for (int i = tid; i < c; i += kRankThreads) sh->pick[i] = sh->cand[sh->pick[i]];
   __syncthreads();
@@ -821,6 +848,7 @@ __device__ __forceinline__ void rank_emit(int* idx, float* score, long long base
 
 __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, const QMeta meta) {
   __shared__ RankShared sh;
+  __shared__ __align__(8) uint64_t s_bar[3];
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* gq = reinterpret_cast<double*>(smem_raw);               // [C] global query
 
@@ -839,7 +867,37 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
   const double* sf = p.s_frm + (long long)qi * p.frm_stride;
   const double* ss = p.s_seg + (long long)qi * p.seg_stride;
   const double* sp = p.s_pat + (long long)qi * p.pat_stride;
-  float* buf = reinterpret_cast<float*>(gq + C);             // [p.stage], 16-byte aligned (C is even)
+  // Single-precision copies of the scores, on their way while the segments are ranked.  (n4 values each: what lies
+  // behind the n-th belongs to this question's row, too)
+  float *buf_s = nullptr, *buf_f = nullptr, *buf_p = nullptr;
+  const int s4 = (n_seg + 3) & ~3, f4 = (n_frm + 3) & ~3, p4 = (n_frm * p.S + 3) & ~3;
+  const uint32_t bar0 = tc::smem_u32(s_bar);
+  auto load = [&](float* dst, const float* src, int n4, int bar) {
+    tc::mbar_expect_tx(bar0 + 8u * bar, 4u * (uint32_t)n4);
+    tc::bulk_load(tc::smem_u32(dst), src, 4u * (uint32_t)n4, bar0 + 8u * bar);
+  };
+  if (p.stage) {
+    buf_s = reinterpret_cast<float*>(gq + C);
+    buf_f = buf_s + s4;
+    if (p.stage == 2) buf_p = buf_f + f4;
+    if (p.stage == 3) buf_p = buf_s;
+    if (tid == 0) {
+      for (int b = 0; b < 3; ++b) tc::mbar_init(bar0 + 8u * b, 1);
+      tc::fence_mbar_init();
+      tc::fence_proxy_async_smem();
+      if (s4) load(buf_s, p.f_seg + (long long)qi * p.f_seg_stride, s4, 0);
+      if (f4) load(buf_f, p.f_frm + (long long)qi * p.f_frm_stride, f4, 1);
+      if (p.stage == 2 && p4) load(buf_p, p.f_pat + (long long)qi * p.f_pat_stride, p4, 2);
+    }
+    __syncthreads();
+  }
+  // a wait that runs out (it cannot, the copies need nothing else) leaves the doubles in global memory to rank by
+  auto landed = [&](float* buf, int n4, int bar) -> float* {
+    if (!buf || !n4) return nullptr;
+    const bool ok = tc::mbar_wait(bar0 + 8u * bar, 0u);
+    return __syncthreads_and(ok) ? buf : nullptr;
+  };
+  float* const seg_buf = landed(buf_s, s4, 0);
   const bool semi = p.mode == MUKV_RETR_SEMI;
 
   // ---- global query = mean of the top-N segment keys (stage 1 order)
@@ -851,7 +909,7 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
     // (without a lambda for segments the N = k_seg best are also the result: one ranking serves both)
     const bool same = N == p.k_seg && !(p.lam_seg > 0.0);
     int* top = same ? sh.pick : sh.top;
-    const int n_top = topk_set(ss, nullptr, n_seg, N, p.delta, top, same ? sh.pick_score : (double*)nullptr, buf, p.stage, &sh.sc);
+    const int n_top = topk_set(ss, nullptr, n_seg, N, p.delta, top, same ? sh.pick_score : (double*)nullptr, seg_buf, &sh.sc);
     if (same) c_seg = n_top;
     double part = 0.0;
     for (int c = tid; c < C; c += kRankThreads) {
@@ -881,7 +939,7 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
   // ---- segments (the paper's lambda for them is 0: final = stage-1 top-k)
   if (c_seg < 0)
     c_seg = rank_level(ss, nullptr, n_seg, p.k_seg, semi && p.lam_seg > 0.0, p.lam_seg, p.delta, p.seg_key, C, gq, gnorm,
-                       have_g, &sh, buf, p.stage);
+                       have_g, &sh, seg_buf);
   rank_emit(p.seg_idx, p.seg_score, (long long)qi * p.k_seg, p.k_seg, c_seg, &sh);
   for (int i = tid; i < c_seg; i += kRankThreads) sh.sel_seg[i] = sh.pick[i];
   __syncthreads();
@@ -892,6 +950,7 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
   // winners back (ascending position = ascending frame).
   const int fseg = p.fseg;
   int c_frm;
+  float* const frm_buf = landed(buf_f, f4, 1);               // (waited for in every mode: the copy must land before the block leaves)
   if (p.mode == MUKV_RETR_HIER) {
     auto frame_of = [&](int i) { return sh.sel_seg[i / fseg] * fseg + i % fseg; };
     auto score_h = [&](int i) { return sf[frame_of(i)]; };
@@ -900,14 +959,22 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
     for (int i = tid; i < c_frm; i += kRankThreads) sh.pick[i] = frame_of(sh.pick[i]);
     __syncthreads();
   } else {
-    c_frm = rank_level(sf, nullptr, n_frm, p.k_frm, semi, p.lam_frm, p.delta, p.frame_key, C, gq, gnorm, have_g, &sh, buf,
-                       p.stage);
+    c_frm = rank_level(sf, nullptr, n_frm, p.k_frm, semi, p.lam_frm, p.delta, p.frame_key, C, gq, gnorm, have_g, &sh,
+                       frm_buf);
   }
   rank_emit(p.frm_idx, p.frm_score, (long long)qi * p.k_frm, p.k_frm, c_frm, &sh);
   __syncthreads();
 
   // ---- patch-level blocks: (frame, super patch) pairs that kept at least one token
   int c_pat = 0;
+  if (p.stage == 3 && p4) {
+    __syncthreads();                                         // the frames' copies are no longer read
+    if (tid == 0) {
+      tc::fence_proxy_async_smem();
+      load(buf_p, p.f_pat + (long long)qi * p.f_pat_stride, p4, 2);
+    }
+  }
+  float* const pat_buf = landed(buf_p, p4, 2);
   if (p.k_pat > 0) {
     const int S = p.S;
     const int* cnt = p.patch_cnt;
@@ -924,8 +991,8 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
         for (int i = tid; i < c_pat; i += kRankThreads) sh.pick[i] = block_of(sh.pick[i]);
         __syncthreads();
       } else {
-        c_pat = rank_level(sp, cnt, n_frm * S, p.k_pat, semi, p.lam_pat, p.delta, p.patch_key, C, gq, gnorm, have_g, &sh, buf,
-                           p.stage);
+        c_pat = rank_level(sp, cnt, n_frm * S, p.k_pat, semi, p.lam_pat, p.delta, p.patch_key, C, gq, gnorm, have_g, &sh,
+                           pat_buf);
       }
     }
     rank_emit(p.pat_idx, p.pat_score, (long long)qi * p.k_pat, p.k_pat, c_pat, &sh);
