@@ -101,10 +101,10 @@ def load_library(path: str | None = None) -> C.CDLL:
     lib.mukv_import.restype = i32
     lib.mukv_import.argtypes = [C.POINTER(MukvStoreHeader), vp, C.c_size_t, vp, C.c_size_t, C.POINTER(vp)]
     lib.mukv_retrieve.restype = i32
-    lib.mukv_retrieve.argtypes = [vp, vp, C.POINTER(i32), C.POINTER(i64), i32, i32, i32, i32, f32, i32,
+    lib.mukv_retrieve.argtypes = [vp, vp, vp, vp, i32, i32, i32, i32, f32, i32,
                                   vp, vp, vp, vp, vp, vp]
     lib.mukv_retrieve3.restype = i32
-    lib.mukv_retrieve3.argtypes = [vp, vp, C.POINTER(i32), C.POINTER(i64), i32, C.POINTER(MukvRetrParams),
+    lib.mukv_retrieve3.argtypes = [vp, vp, vp, vp, i32, C.POINTER(MukvRetrParams),
                                    vp, vp, vp, vp, vp, vp, vp, vp]
     lib.mukv_decode3_tokens.restype = i64
     lib.mukv_decode3_tokens.argtypes = [vp, i32, i32, i32]
@@ -133,9 +133,24 @@ def _ptr(t) -> int | None:
     return None if t is None else t.data_ptr()
 
 
+# Handle of the current stream.  (torch.cuda.current_stream() builds a Stream object, 3 us of the 5 that the marshalling
+# of a call took; the raw getter gives the handle in 0.1.)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream) -> int:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None and _raw_device is not None and torch.cuda.is_initialized():
+        return _raw_stream(_raw_device())
+    return torch.cuda.current_stream().cuda_stream
+
+
+def _host_array(x, dtype) -> tuple[np.ndarray, int]:
+    """x as a contiguous array, and its address (valid while the array lives)."""
+    a = x if type(x) is np.ndarray and x.dtype == dtype and x.flags.c_contiguous else np.ascontiguousarray(x, dtype=dtype)
+    return a, a.ctypes.data
 
 
 def make_config(*, n_layers, n_q_heads, n_kv_heads, head_dim, tokens_per_frame, keep_per_frame,
@@ -231,23 +246,20 @@ class MukvContext:
 
     def mukv_retrieve(self, qtok, q_offsets, t_limit, k_seg: int, k_frm: int, top_n: int, lambda_frm: float,
                       mode: int, seg_idx, frm_idx, seg_score, frm_score, counts, stream=None):
-        offs = np.ascontiguousarray(q_offsets, dtype=np.int32)
+        offs, p_offs = _host_array(q_offsets, np.int32)
         nq = offs.shape[0] - 1
-        tl = None if t_limit is None else np.ascontiguousarray(t_limit, dtype=np.int64)
+        tl, p_tl = (None, None) if t_limit is None else _host_array(t_limit, np.int64)
         self._check(self.lib.mukv_retrieve(
-            self.handle, _ptr(qtok), offs.ctypes.data_as(C.POINTER(C.c_int32)),
-            None if tl is None else tl.ctypes.data_as(C.POINTER(C.c_int64)),
-            nq, k_seg, k_frm, top_n, lambda_frm, mode, _ptr(seg_idx), _ptr(frm_idx), _ptr(seg_score),
+            self.handle, _ptr(qtok), p_offs, p_tl, nq, k_seg, k_frm, top_n, lambda_frm, mode, _ptr(seg_idx), _ptr(frm_idx), _ptr(seg_score),
             _ptr(frm_score), _ptr(counts), _stream(stream)))
 
     def mukv_retrieve3(self, qtok, q_offsets, t_limit, params: MukvRetrParams, seg_idx, frm_idx, patch_idx,
                        seg_score, frm_score, patch_score, counts, stream=None):
-        offs = np.ascontiguousarray(q_offsets, dtype=np.int32)
+        offs, p_offs = _host_array(q_offsets, np.int32)
         nq = offs.shape[0] - 1
-        tl = None if t_limit is None else np.ascontiguousarray(t_limit, dtype=np.int64)
+        tl, p_tl = (None, None) if t_limit is None else _host_array(t_limit, np.int64)
         self._check(self.lib.mukv_retrieve3(
-            self.handle, _ptr(qtok), offs.ctypes.data_as(C.POINTER(C.c_int32)),
-            None if tl is None else tl.ctypes.data_as(C.POINTER(C.c_int64)), nq, C.byref(params),
+            self.handle, _ptr(qtok), p_offs, p_tl, nq, C.byref(params),
             _ptr(seg_idx), _ptr(frm_idx), _ptr(patch_idx), _ptr(seg_score), _ptr(frm_score), _ptr(patch_score),
             _ptr(counts), _stream(stream)))
 
