@@ -66,6 +66,7 @@ struct CompactParams {
   // with several planes each kept one-frame calls waiting for 70 us (28 layers) behind 8 us of copying
   SegmentArgs prev;
   int prev_rows;
+  int parts;                      // compact_kernel: blocks that share a (layer, K|V) plane of a frame, by columns
   int sel_mode;                   // 0: kept ids are in the store; 1: select here from the partial sums;
                                   // 2: select here by the caller's scores; 3: ids and counts are in the store
                                   // (segment-level selection)
@@ -115,23 +116,31 @@ __device__ inline bool select_from_partials(const CompactParams& p, int f, bool 
     const int c_last = share_owner((unsigned)((f + 1) * p.ps_ipf - 1), (unsigned)p.ps_items, (unsigned)p.ps_grid);
     const float* cp = reinterpret_cast<const float*>(sp.colsum_part) + tid;
     const float* fp = reinterpret_cast<const float*>(sp.ifft_part) + (long long)f * Hkv * P + tid;
-    // all loads of the common case (up to 16 blocks per frame, up to 8 key heads) are in flight together
-    float x[16], y[8];
+    // Sixteen blocks' sums and eight key heads are in flight together, which is all of a frame in the common case.  (A
+    // frame of a short call is spread over up to 52 blocks, five scoring layers have 20 heads: one load after the other
+    // behind the first batch took 10 us of a one-frame call.)
+    float a32 = 0.f, f32 = 0.f;
+    int cc = c_first, g = 0;
+#pragma unroll 1
+    do {
+      float x[16], y[8];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) x[i] = c_first + i <= c_last ? __ldcg(cp + (long long)(c_first + i + f) * P) : 0.f;
+      for (int i = 0; i < 16; ++i) x[i] = cc + i <= c_last ? __ldcg(cp + (long long)(cc + i + f) * P) : 0.f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) y[i] = i < Hkv ? __ldcg(fp + (long long)i * P) : 0.f;
+      for (int i = 0; i < 8; ++i) y[i] = g + i < Hkv ? __ldcg(fp + (long long)(g + i) * P) : 0.f;
 #pragma unroll
-    for (int w = 8; w >= 1; w >>= 1)
+      for (int w = 8; w >= 1; w >>= 1)
 #pragma unroll
-      for (int i = 0; i < w; ++i) x[i] += x[i + w];
+        for (int i = 0; i < w; ++i) x[i] += x[i + w];
 #pragma unroll
-    for (int w = 4; w >= 1; w >>= 1)
+      for (int w = 4; w >= 1; w >>= 1)
 #pragma unroll
-      for (int i = 0; i < w; ++i) y[i] += y[i + w];
-    float a32 = x[0], f32 = y[0];
-    for (int cc = c_first + 16; cc <= c_last; ++cc) a32 += __ldcg(cp + (long long)(cc + f) * P);
-    for (int g = 8; g < Hkv; ++g) f32 += __ldcg(fp + (long long)g * P);
+        for (int i = 0; i < w; ++i) y[i] += y[i + w];
+      a32 += x[0];
+      f32 += y[0];
+      cc += 16;
+      g += 8;
+    } while (cc <= c_last || g < Hkv);
     att = a32 * (1.f / (float)((long long)sp.Hq * sp.Ls * P));
     fft = f32 * (1.f / (float)((long long)Hkv * sp.D));
   }
@@ -376,19 +385,21 @@ struct CompactScratch {
 // Copies the kappa kept rows (ids in sc->kept, ascending) of plane (l, kv) of chunk frame f to the
 // frame's page (planes of kappa rows each, starting at `page`) and writes the plane's frame entry
 // (Eq. 5; zeros for a frame that keeps nothing).  Run by a whole block.
-// NV = 16-byte vectors per row; the block covers 256/NV rows per pass.
+// NV = 16-byte vectors per row; the block covers 256/NV rows per pass.  With `parts` > 1 the block copies part `part` of
+// the columns only (NV / parts vectors), so that more rows are in flight at a time: see compact_kernel.
 template <typename T>
 __device__ inline void compact_plane(const CompactParams& p, int plane, int f, CompactScratch* sc, int kappa,
-                                     unsigned char* page) {
+                                     unsigned char* page, int part, int parts) {
   constexpr int VE = 16 / sizeof(T);
   const int tid = threadIdx.x;
   const int l = plane >> 1, kv = plane & 1;
   const long long f_abs = p.first_frame + f;
   const int C = p.C;
-  const int NV = C / VE;                        // vectors per row (power of two, <= 256)
+  const int NV = C / VE / parts;                // vectors per row (power of two, <= 256)
+  const int c_off = part * NV * VE;             // first column
   const int rows_per_pass = kCompactThreads / NV;
-  const T* src_base = reinterpret_cast<const T*>(kv ? p.v : p.k) + ((long long)l * p.n_frames + f) * p.P * C;
-  T* dst_base = reinterpret_cast<T*>(page) + (long long)plane * kappa * C;
+  const T* src_base = reinterpret_cast<const T*>(kv ? p.v : p.k) + ((long long)l * p.n_frames + f) * p.P * C + c_off;
+  T* dst_base = reinterpret_cast<T*>(page) + (long long)plane * kappa * C + c_off;
   const int c = tid % NV, r0 = tid / NV;
   const bool exact = (l == p.L - 1) && (kv == 0);
   float acc[VE];
@@ -439,16 +450,16 @@ __device__ inline void compact_plane(const CompactParams& p, int plane, int f, C
     for (int i = 0; i < VE; ++i) sc->red[tid * VE + i] = acc[i];
   }
   __syncthreads();
-  float* fe = p.frame_entry + ((f_abs * p.L + l) * 2 + kv) * C;
-  for (int col = tid; col < C; col += kCompactThreads) {
+  float* fe = p.frame_entry + ((f_abs * p.L + l) * 2 + kv) * C + c_off;
+  for (int col = tid; col < NV * VE; col += kCompactThreads) {
     const int cv = col / VE, ce = col % VE;
     if (exact) {
       double t = 0.0;
       for (int g = 0; g < rows_per_pass; ++g) t += sc->red64[(g * NV + cv) * VE + ce];
-      p.frame_ksum[f_abs * C + col] = t;
+      p.frame_ksum[f_abs * C + c_off + col] = t;
       const float m = kappa ? (float)(t / (double)kappa) : 0.f;
       fe[col] = m;
-      p.frame_key[f_abs * C + col] = m;
+      p.frame_key[f_abs * C + c_off + col] = m;
     } else {
       float t = 0.f;
       for (int g = 0; g < rows_per_pass; ++g) t += sc->red[(g * NV + cv) * VE + ce];
@@ -549,7 +560,10 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const Compa
     }
     if (row > p.prev_rows) row -= p.prev_rows;
   }
-  const int plane = p.patch_split > 0 && row >= 1 ? (row == 1 ? 2 * p.L : row - 1) : row;
+  const bool patches = p.patch_split > 0 && row == 1;
+  if (p.patch_split > 0 && row > 1) --row;
+  const int plane = patches ? 2 * p.L : row / p.parts, part = patches ? 0 : row % p.parts;
+  const bool writes = plane == 0 && part == 0;           // this block writes the ids and the index of its frame
   pdl_wait();
   pdl_trigger();
   if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *p.n_flagged_next = 0;
@@ -562,7 +576,7 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const Compa
     // the first wave do) reads them; every other block selects itself.  Nobody waits.
     if (tid == 0) {
       unsigned v = 0u;
-      if (plane != 0) {
+      if (!writes) {
         v = *reinterpret_cast<volatile unsigned*>(p.sel_flag + f);
         __threadfence();
       }
@@ -575,8 +589,8 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const Compa
       for (int r = tid; r < p.kappa; r += kCompactThreads) cs.kept[r] = token_id(__ldcg(p.sp.kept_store + f_abs * p.kappa + r), p.P);
       __syncthreads();
     } else {
-      risky = select_from_partials(p, f, plane == 0, cs.kept, &ss);
-      if (plane == 0) {
+      risky = select_from_partials(p, f, writes, cs.kept, &ss);
+      if (writes) {
         __threadfence();                        // this thread's ids are visible before the flag is
         __syncthreads();
         if (tid == 0) *reinterpret_cast<volatile unsigned*>(p.sel_flag + f) = (p.epoch << 1) | (risky ? 1u : 0u);
@@ -589,8 +603,8 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const Compa
     const bool bad = __syncthreads_or(tid < p.P && !isfinite(sx[0])) != 0;
     if (bad) sx[0] = 0.0;
     bool keep[1];
-    select_by_score<1>(p.sp, f, sx, plane == 0, cs.kept, keep, ss.sc64, ss.cnt64, ss.misc64);
-    if (bad && plane == 0 && tid == 0 && p.sp.status) atomicCAS(p.sp.status, 0, kStatusNonFinite);
+    select_by_score<1>(p.sp, f, sx, writes, cs.kept, keep, ss.sc64, ss.cnt64, ss.misc64);
+    if (bad && writes && tid == 0 && p.sp.status) atomicCAS(p.sp.status, 0, kStatusNonFinite);
     risky = false;
     __syncthreads();
   } else if (p.sel_mode == 3) {
@@ -606,7 +620,7 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const Compa
     __syncthreads();
   }
   if (risky) return;
-  if (plane < 2 * p.L) compact_plane<T>(p, plane, f, &cs, kappa_f, page);
+  if (plane < 2 * p.L) compact_plane<T>(p, plane, f, &cs, kappa_f, page, part, p.parts);
   else pool_patches<T>(p, f, &cs);
 }
 
@@ -692,7 +706,7 @@ __global__ void __launch_bounds__(kScoreThreads, 2) tail_kernel(const ScoreParam
         __syncthreads();
         for (int r = tid; r < p.kappa; r += kCompactThreads) cs.kept[r] = token_id(__ldcg(sp.kept_store + f_abs * p.kappa + r), p.P);
         __syncthreads();
-        if (plane < 2 * p.L) compact_plane<T>(p, plane, f, &cs, p.kappa, p.store + sp.pages_off + f_abs * sp.page_bytes);
+        if (plane < 2 * p.L) compact_plane<T>(p, plane, f, &cs, p.kappa, p.store + sp.pages_off + f_abs * sp.page_bytes, 0, 1);
         else pool_patches<T>(p, f, &cs);
       }
       if (plane >= 2 * p.L) continue;

@@ -806,9 +806,14 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
     cp.prev = segment_args_of(ctx, ctx->seg_first, ctx->seg_n);
     cp.prev_rows = (2 * L + n - 1) / n;
   }
+  // A plane of a frame is three round trips of rows for one block.  While the planes of a short call leave most of the
+  // device idle (three blocks per SM are resident), two or four blocks share one by columns, which leaves one trip; a part
+  // of a row stays at least 256 bytes.
+  cp.parts = 1;
+  while (cp.parts < 4 && 4LL * n * L * cp.parts <= 3LL * ctx->n_sms && C * ctx->esize / (2 * cp.parts) >= 256) cp.parts *= 2;
   {
     ProfScope ps(ctx, 2, st);
-    e = launch_k(compact_kernel<T>, dim3(n, L * 2 + (c.patch_split > 0 ? 1 : 0) + cp.prev_rows),
+    e = launch_k(compact_kernel<T>, dim3(n, L * 2 * cp.parts + (c.patch_split > 0 ? 1 : 0) + cp.prev_rows),
                  kCompactThreads, 0, st, !ctx->prof_on, cp);
   }
   if (e != cudaSuccess) return broke_off(ctx, "compact kernel", e);
