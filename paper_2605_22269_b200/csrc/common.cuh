@@ -135,9 +135,18 @@ __device__ __forceinline__ int super_patch_index(int j, int P, int grid_width, i
   return (j / grid_width) / rh * split + (j % grid_width) / cw;
 }
 
-// owner of item i when n items are split into contiguous shares [c*n/nb, (c+1)*n/nb) (the blocks of
-// the persistent scoring kernel take such shares of its item list)
-__device__ __forceinline__ int share_owner(unsigned i, unsigned n, unsigned nb) { return (int)(((i + 1u) * nb - 1u) / n); }
+// Column sums of the softmax (Eq. 1), as the blocks of the persistent scoring kernel add them up: 24.40 fixed point in 64
+// bits, so that the result does not depend on the order of the additions.  A column sum is at most the number of query
+// rows that see the frame (layers x heads x tokens: 2^20 at the supported shapes), a block's share has 24 significant
+// bits, and 2^-40 is 2^-17 of the last of them at a sum of 1.  Bit 63 marks a share that is not a number.
+constexpr unsigned long long kAttPoison = 1ull << 63;
+__device__ __forceinline__ void att_add(unsigned long long* acc, float v) {
+  if (!(v < 1e30f)) atomicOr(acc, kAttPoison);
+  else if (v > 0.f) atomicAdd(acc, __float2ull_rn(v * 1099511627776.f));
+}
+__device__ __forceinline__ float att_value(unsigned long long acc) {
+  return (acc & kAttPoison) ? __int_as_float(0x7fffffff) : __ull2float_rn(acc) * (1.f / 1099511627776.f);
+}
 
 // ---------------------------------------------------------------- segment entries (Eq. 5 at segment level)
 // What the pooling of segment entries needs, small enough to travel in registers (compact_segment_plane

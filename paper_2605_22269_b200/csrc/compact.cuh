@@ -8,8 +8,8 @@
 // later ranks blocks, so it is kept free of accumulation-order noise.
 //
 // Where do the kept ids come from?  After the persistent tensor-core scoring kernel every block
-// works them out itself (sel_mode 1): it adds the scoring blocks' partial column sums of its frame
-// in a fixed order, applies Eq. 4 and selects, all in single precision; the blocks of a frame run
+// works them out itself (sel_mode 1): it reads the column sums of its frame, adds the key heads'
+// frequency sums in a fixed order, applies Eq. 4 and selects, all in single precision; the blocks of a frame run
 // the same arithmetic on the same numbers, so they agree, and the one with plane 0 writes the ids
 // and the index.  That costs a few microseconds at the start of each block, in parallel on the
 // whole device, where a selection inside the scoring kernel left one block per frame working while
@@ -73,7 +73,9 @@ struct CompactParams {
   const float* ext_scores;        // [n_frames][P] (sel_mode 2)
   const int* kept_count;          // [max_frames] (sel_mode 3: a frame's page holds that many tokens; ids in
                                   // kept_store with a stride of P), else null
-  int ps_grid, ps_items, ps_ipf;  // the scoring launch: blocks, items, items per frame
+  const unsigned long long* att_acc;  // [F][P] column sums of the persistent scoring kernel (sel_mode 1)
+  unsigned long long* att_clear;  // sums of the call before, cleared for the next one
+  long long n_clear;
   unsigned* sel_flag;             // [F] (epoch << 1 | risky) once the plane-0 block has published its frame's ids
   unsigned epoch;                 // number of this call, never repeated
   ScoreParams sp;                 // partial sums, Eq. 4 parameters, index and flag outputs
@@ -111,36 +113,20 @@ __device__ inline bool select_from_partials(const CompactParams& p, int f, bool 
   const bool valid = tid < P;
   float att = 0.f, fft = 0.f;
   if (valid) {
-    // the scoring blocks' column sums, added in block order
-    const int c_first = share_owner((unsigned)(f * p.ps_ipf), (unsigned)p.ps_items, (unsigned)p.ps_grid);
-    const int c_last = share_owner((unsigned)((f + 1) * p.ps_ipf - 1), (unsigned)p.ps_items, (unsigned)p.ps_grid);
-    const float* cp = reinterpret_cast<const float*>(sp.colsum_part) + tid;
     const float* fp = reinterpret_cast<const float*>(sp.ifft_part) + (long long)f * Hkv * P + tid;
-    // Sixteen blocks' sums and eight key heads are in flight together, which is all of a frame in the common case.  (A
-    // frame of a short call is spread over up to 52 blocks, five scoring layers have 20 heads: one load after the other
-    // behind the first batch took 10 us of a one-frame call.)
-    float a32 = 0.f, f32 = 0.f;
-    int cc = c_first, g = 0;
+    const float a32 = att_value(__ldcg(p.att_acc + (long long)f * P + tid));
+    float f32 = 0.f;
 #pragma unroll 1
-    do {
-      float x[16], y[8];
-#pragma unroll
-      for (int i = 0; i < 16; ++i) x[i] = cc + i <= c_last ? __ldcg(cp + (long long)(cc + i + f) * P) : 0.f;
+    for (int g = 0; g < Hkv; g += 8) {                     // (eight key heads in flight)
+      float y[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) y[i] = g + i < Hkv ? __ldcg(fp + (long long)(g + i) * P) : 0.f;
-#pragma unroll
-      for (int w = 8; w >= 1; w >>= 1)
-#pragma unroll
-        for (int i = 0; i < w; ++i) x[i] += x[i + w];
 #pragma unroll
       for (int w = 4; w >= 1; w >>= 1)
 #pragma unroll
         for (int i = 0; i < w; ++i) y[i] += y[i + w];
-      a32 += x[0];
       f32 += y[0];
-      cc += 16;
-      g += 8;
-    } while (cc <= c_last || g < Hkv);
+    }
     att = a32 * (1.f / (float)((long long)sp.Hq * sp.Ls * P));
     fft = f32 * (1.f / (float)((long long)Hkv * sp.D));
   }
@@ -567,6 +553,8 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const Compa
   pdl_wait();
   pdl_trigger();
   if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *p.n_flagged_next = 0;
+  if (writes)
+    for (long long i = (long long)f * kCompactThreads + tid; i < p.n_clear; i += (long long)gridDim.x * kCompactThreads) p.att_clear[i] = 0ull;
   const long long f_abs = p.first_frame + f;
   int kappa_f = p.kappa;
   unsigned char* page = p.store + p.sp.pages_off + f_abs * p.sp.page_bytes;
@@ -631,6 +619,8 @@ __global__ void __launch_bounds__(kCompactThreads) select_kernel(const CompactPa
   pdl_wait();
   pdl_trigger();
   select_from_partials(p, blockIdx.x, true, s_kept, &ss);
+  // the only reader of the frame's sums leaves them cleared
+  for (int t = threadIdx.x; t < p.sp.P; t += kCompactThreads) p.att_clear[(long long)blockIdx.x * p.sp.P + t] = 0ull;
 }
 
 // Bounded wait until *ctr reaches `target` (other blocks of the same grid add to it; the grid is

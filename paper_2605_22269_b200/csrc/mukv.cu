@@ -40,10 +40,10 @@ struct StoreLayout {
 
 struct WorkLayout {
   size_t q_terms, k_terms; // fp32 chunks: queries and keys of the scoring layers as three bf16 terms
-  size_t colsum_f, colsum_p, ifft_f, colsum_d, ifft_d, frame_counter, flagged, n_flagged, tail_ctr, sel_flag,
-      seg_flag, stat_refined, dev_status;
+  size_t colsum_f, ifft_f, colsum_d, ifft_d, frame_counter, flagged, n_flagged, tail_ctr, sel_flag,
+      seg_flag, stat_refined, dev_status, att_acc;
   size_t q64, qnorm, s_frm, s_seg, s_pat, f_frm, f_seg, f_pat, wtab, total;
-  size_t zero_begin, zero_end;          // region that must start as zeros
+  size_t zero_begin, zero_end;          // region that must start as zeros: counters up to att_acc, then att_acc
 };
 
 // Tiling of the tensor-core scoring kernel (bf16 inputs only).
@@ -69,7 +69,8 @@ struct mukv_ctx {
   unsigned char* ws;
   long long frames;
   long long launches;
-  int parity = 0;                        // which of the two flagged counters this chunk uses
+  int parity = 0;                        // which of the two flagged counters and sets of column sums this chunk uses
+  long long att_dirty[2] = {0, 0};       // values of a set that the last call on it has written
   unsigned epoch = 0;                    // compress calls so far (tags the per-frame selection flags)
   int C, G, esize, nc, Ls;
   int key_rows;                          // key rows of the multiply-add scoring kernel: P + past_frames * kappa
@@ -271,7 +272,6 @@ WorkLayout work_layout(const mukv_config& c) {
   const TcShape ts = tc_shape(c);
   const size_t Ls = c.n_score_layers > 1 ? c.n_score_layers : 1;
   w.colsum_f = off;       off = align_up(off + F * Ls * (size_t)c.n_q_heads * P * sizeof(float));
-  w.colsum_p = off;       off = align_up(off + (ts.ok || ts.split ? (kPsMaxBlocks + F) * P * sizeof(float) : 0));
   w.ifft_f = off;         off = align_up(off + F * Ls * c.n_kv_heads * P * sizeof(float));
   w.colsum_d = off;       off = align_up(off + F * Ls * c.n_q_heads * kRefineSplit * P * sizeof(double));
   w.ifft_d = off;         off = align_up(off + F * Ls * c.n_kv_heads * P * sizeof(double));
@@ -284,6 +284,7 @@ WorkLayout work_layout(const mukv_config& c) {
   w.seg_flag = off;       off = align_up(off + F * sizeof(int));
   w.stat_refined = off;   off = align_up(off + sizeof(long long));
   w.dev_status = off;     off = align_up(off + sizeof(int));
+  w.att_acc = off;        off = align_up(off + (ts.ok || ts.split ? 2 * F * P * sizeof(unsigned long long) : 0));   // alternate, too
   w.zero_end = off;
   w.q64 = off;            off = align_up(off + (size_t)MUKV_MAX_QUESTIONS * C * sizeof(double));
   w.qnorm = off;          off = align_up(off + (size_t)MUKV_MAX_QUESTIONS * c.n_kv_heads * sizeof(double));
@@ -549,14 +550,12 @@ struct PsLaunch {
   int n_sms;
   const CUtensorMap* wmap;
   const CUtensorMap* pmap;       // stored pages (past keys), or null
-  void* colsum;                  // float [blocks + frames][P]
+  unsigned long long* att_acc;   // [frames][P], zero
   int* status;
   int* clear;                    // see ScorePsParams
   int kappa;
   bool dependent;
   __nv_bfloat16 *q_terms, *k_terms;   // SPLIT: room for the terms of an fp32 chunk
-  // out: what the selection needs to find a frame's partial sums
-  int grid, items, ipf;
 };
 
 // Scores a bf16 chunk on the tensor cores (Eq. 1-3; Eq. 4 and the selection follow in compact_kernel).
@@ -589,7 +588,7 @@ cudaError_t launch_score_ps(PsLaunch& l, const ScoreParams& sp, cudaStream_t st,
   ScorePsParams pp;
   memset(&pp, 0, sizeof pp);
   pp.sp = sp;
-  pp.sp.colsum_part = l.colsum;
+  pp.att_acc = l.att_acc;
   pp.tiles = t.tiles; pp.tpt = t.tpt; pp.npad = t.npad; pp.n_mt = t.n_mt; pp.n_stages = t.ps_stages;
   pp.own_rows = t.own_rows; pp.n_past = sp.n_past_frames; pp.past_pad = t.past_pad; pp.kappa = l.kappa;
   pp.past_plane0 = 2 * sp.first_score_layer; pp.past_first = sp.past_first;
@@ -601,7 +600,6 @@ cudaError_t launch_score_ps(PsLaunch& l, const ScoreParams& sp, cudaStream_t st,
   pp.clear = l.clear;
   int blocks = l.n_sms < kPsMaxBlocks ? l.n_sms : kPsMaxBlocks;
   if (blocks > pp.n_items) blocks = pp.n_items;
-  l.grid = blocks; l.items = pp.n_items; l.ipf = pp.ipf;
   *why = "score_ps kernel";
   const bool past = sp.n_past_frames > 0;
   if (t.split) {
@@ -613,11 +611,16 @@ cudaError_t launch_score_ps(PsLaunch& l, const ScoreParams& sp, cudaStream_t st,
                   st, l.dependent, pp, qmap, kmap, *l.wmap, past ? *l.pmap : kmap);
 }
 
+unsigned long long* att_acc_of(const mukv_ctx* ctx, int parity) {
+  return reinterpret_cast<unsigned long long*>(ctx->ws + ctx->wl.att_acc) +
+         (size_t)parity * ctx->cfg.max_frames_per_chunk * ctx->cfg.tokens_per_frame;
+}
+
 PsLaunch ps_launch_of(mukv_ctx* ctx) {
   PsLaunch l;
   memset(&l, 0, sizeof l);
   l.t = &ctx->tcs; l.n_sms = ctx->n_sms; l.wmap = &ctx->wmap; l.pmap = &ctx->pmap;
-  l.colsum = ctx->ws + ctx->wl.colsum_p;
+  l.att_acc = att_acc_of(ctx, ctx->parity);
   l.status = reinterpret_cast<int*>(ctx->ws + ctx->wl.dev_status);
   l.kappa = ctx->cfg.keep_per_frame;
   l.dependent = !ctx->prof_on;
@@ -670,7 +673,7 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
   const dim3 grid(ctx->Ls * c.n_q_heads, n);
   cudaError_t e = cudaSuccess;
   const char* what = "score kernel";
-  int ps_grid = 0, ps_items = 0, ps_ipf = 0;
+  bool on_tc = false;                                    // scored by the persistent kernel, selected by compact_kernel
   int n_launch = 0;
   if (seg_scope) {
     // One block per segment ranks all its tokens.  A bf16 chunk is first scored on the tensor cores and
@@ -707,13 +710,13 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
       {
         ProfScope ps(ctx, 0, st);
         e = launch_score_ps(pl, sp, st, &what);
+        ctx->att_dirty[ctx->parity] = (long long)n * P;
       }
       if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "%s: %s", what, cudaGetErrorString(e));
       n_launch += 2;
       gp.sp = sp;
-      gp.sp.colsum_part = ctx->ws + ctx->wl.colsum_p;
+      gp.att_acc = pl.att_acc;
       gp.src32 = 1;
-      gp.ps_grid = pl.grid; gp.ps_items = pl.items; gp.ps_ipf = pl.ipf;
       {
         ProfScope ps(ctx, 1, st);
         e = launch_k(segsel_kernel, dim3(n_seg + extra), kSegSelThreads, segsel_smem_bytes(seg_tokens), st, dep, gp);
@@ -760,7 +763,8 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
       n_launch += ctx->tcs.split ? 1 : 0;
       PsLaunch pl = ps_launch_of(ctx);
       e = launch_score_ps(pl, sp, st, &what);
-      ps_grid = pl.grid; ps_items = pl.items; ps_ipf = pl.ipf;
+      ctx->att_dirty[ctx->parity] = (long long)n * P;
+      on_tc = true;
     } else
       e = launch_score<T, float>(sp, ctx->nc, grid, score_smem_bytes<T, float>(ctx->key_rows, c.head_dim), st);
     ++n_launch;
@@ -788,12 +792,14 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
   cp.patch_split = c.patch_split; cp.grid_width = c.grid_width;
   cp.patch_key = reinterpret_cast<float*>(ctx->store + ctx->sl.patch_key);
   cp.patch_cnt = reinterpret_cast<int*>(ctx->store + ctx->sl.patch_cnt);
-  cp.sel_mode = seg_scope ? 3 : d_ext ? 2 : ps_grid > 0 ? 1 : 0;
+  cp.sel_mode = seg_scope ? 3 : d_ext ? 2 : on_tc ? 1 : 0;
   cp.kept_count = seg_scope ? reinterpret_cast<const int*>(ctx->store + ctx->sl.kept_count) : nullptr;
   cp.ext_scores = d_ext;
-  cp.ps_grid = ps_grid; cp.ps_items = ps_items; cp.ps_ipf = ps_ipf;
+  cp.att_acc = att_acc_of(ctx, ctx->parity);
+  cp.att_clear = att_acc_of(ctx, ctx->parity ^ 1);       // (nobody reads the previous call's sums any more)
+  cp.n_clear = ctx->att_dirty[ctx->parity ^ 1];
+  ctx->att_dirty[ctx->parity ^ 1] = 0;
   cp.sp = sp;
-  if (ps_grid > 0) cp.sp.colsum_part = ctx->ws + ctx->wl.colsum_p;
   // segment entries the previous call left behind: more rows of blocks (with per-kernel timing on,
   // a launch of their own, so that each kernel is timed doing its own work only)
   if (ctx->seg_pending && ctx->prof_on) {
@@ -1155,11 +1161,13 @@ mukv_status mukv_profile_read(mukv_ctx* ctx, double* ms, int64_t* launches) {
 mukv_status mukv_reset(mukv_ctx* ctx, mukv_stream stream) {
   if (!ctx) return MUKV_E_INVALID;
   // arrival counters, flagged lists, selection flags, statistics and the event word start over
-  cudaError_t e = cudaMemsetAsync(ctx->ws + ctx->wl.zero_begin, 0, ctx->wl.zero_end - ctx->wl.zero_begin,
+  // (the column sums are clean where the next call needs them, unless a call broke off)
+  cudaError_t e = cudaMemsetAsync(ctx->ws + ctx->wl.zero_begin, 0,
+                                  (ctx->failed ? ctx->wl.zero_end : ctx->wl.att_acc) - ctx->wl.zero_begin,
                                   static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "mukv_reset: %s", cudaGetErrorString(e));
   ctx->frames = 0;
-  ctx->parity = 0;
+  if (ctx->failed) ctx->att_dirty[0] = ctx->att_dirty[1] = 0;
   ctx->failed = false;
   ctx->seg_pending = false;
   return MUKV_OK;
@@ -1449,9 +1457,8 @@ constexpr size_t kNaCtrl = kNaPt + 256;                  // frame_counter[16], f
 constexpr size_t kNaCtrlBytes = 256;
 constexpr size_t kNaW128 = kNaCtrl + kNaCtrlBytes;       // DFT matrix terms, D = 128 and D = 64
 constexpr size_t kNaW64 = kNaW128 + 3 * 128 * 128 * 2;
-constexpr size_t kNaTotal = kNaW64 + 3 * 64 * 64 * 2;
-// the tensor-core path keeps its column sums where the multiply-add path has them
-static_assert((size_t)(kPsMaxBlocks + kNaFrames) * kNaP * sizeof(float) <= kNaFftF - kNaColF, "column-sum slots do not fit");
+constexpr size_t kNaAtt = kNaW64 + 3 * 64 * 64 * 2;       // column sums of the tensor-core path, zero between calls
+constexpr size_t kNaTotal = kNaAtt + (size_t)kNaFrames * kNaP * sizeof(unsigned long long);
 
 // In host code this name is only a handle for cudaGetSymbolAddress, never a device address.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNaTotal];
@@ -1536,7 +1543,7 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
     PsLaunch pl;
     memset(&pl, 0, sizeof pl);
     pl.t = &ts; pl.n_sms = nd->n_sms; pl.wmap = D == 128 ? &nd->wmap128 : &nd->wmap64;
-    pl.colsum = base + kNaColF;
+    pl.att_acc = reinterpret_cast<unsigned long long*>(base + kNaAtt);
     pl.status = sp.n_flagged + 1;
     pl.clear = sp.n_flagged;
     pl.kappa = c.keep_per_frame;
@@ -1547,9 +1554,12 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
     CompactParams cp;
     memset(&cp, 0, sizeof cp);
     cp.sp = sp;
-    cp.ps_grid = pl.grid; cp.ps_items = pl.items; cp.ps_ipf = pl.ipf;
+    cp.att_acc = cp.att_clear = pl.att_acc;
     e = launch_k(select_kernel, dim3(n), kCompactThreads, 0, st, true, cp);
-    if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "select kernel: %s", cudaGetErrorString(e));
+    if (e != cudaSuccess) {
+      cudaMemsetAsync(base + kNaAtt, 0, kNaTotal - kNaAtt, st);
+      return fail(nullptr, MUKV_E_CUDA, "select kernel: %s", cudaGetErrorString(e));
+    }
   } else {
     // the array keeps what the last call left: the arrival counters and the flagged count start at zero
     e = cudaMemsetAsync(base + kNaCtrl, 0, kNaCtrlBytes, st);

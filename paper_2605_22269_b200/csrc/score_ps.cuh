@@ -21,10 +21,11 @@
 //               (shuffle butterfly), so the per-tile cost is one fused multiply-add per logit.
 //               DFT item: magnitudes of the D bins of each key vector, summed.
 //
-// Per frame, every block that worked on it stores its column sums in a slot of its own (slot
-// index = block + frame).  Eq. 4 and the selection are left to the kernel that follows
-// (compact_kernel adds the slots in a fixed order): done here, by the block that finishes a frame
-// last, they kept one block per frame busy for microseconds after all others had finished.
+// Every block adds its column sums of a frame to the frame's (att_add: one row of 64-bit sums per frame).  Eq. 4 and the
+// selection are left to the kernel that follows: done here, by the block that finishes a frame last, they kept one block
+// per frame busy for microseconds after all others had finished.  (A row per block and frame, added up by whoever selects,
+// was 10 rows a frame for 16 frames and 52 for one: hundreds of selecting blocks read the same few lines, which took 2 us
+// and 5 us of the selection.)
 // All mbarrier waits are bounded; a wait that runs out makes the role record a code in the status
 // word; the producer and the MMA issuer then leave their loops, the epilogue warps go on without
 // waiting (their reads stay inside the accumulators).
@@ -48,7 +49,7 @@ constexpr int kPsEpiThreads = 512;
 constexpr int kPsSplit = 4;                // warps that share a row (32-lane quarter), each a column range
 constexpr int kPsEpiOff = 128;             // first epilogue thread
 constexpr int kPsMiscBytes = 12800 + 8192;
-constexpr int kPsMaxBlocks = 256;          // bound on the grid (slots of partial sums)
+constexpr int kPsMaxBlocks = 256;          // bound on the grid
 constexpr int kPsAccCols = 64;             // accumulator columns per epilogue thread: P <= 4 * 64
 // Twenty warps put five on each scheduler, whose 16 K registers allow 96 per thread at launch.
 // The control warpgroup then gives registers back (setmaxnreg.dec) and the four epilogue warpgroups
@@ -60,7 +61,8 @@ static_assert(128 * (96 - kPsCtrlRegs) >= 512 * (kPsEpiRegs - 96), "register han
 typedef NamedGroup<5, kPsEpiThreads, kPsEpiOff> PsEpiGroup;
 
 struct ScorePsParams {
-  ScoreParams sp;            // colsum_part: float [grid + n_frames][P] slots, ifft_part: float [F][Hkv][P]
+  ScoreParams sp;            // ifft_part: float [F][Hkv][P]
+  unsigned long long* att_acc;  // [F][P], zero when the kernel starts
   int tiles, tpt, npad, n_mt;  // npad: rows of a key tile = columns of an attention product
   // cached keys the queries also attend to (Sec. 3.2): rows own_rows + w * past_pad .. + kappa of the key
   // tile hold the kept keys of frame past_first + w (w < n_past), read from that frame's page
@@ -251,7 +253,7 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
   const int NS = p.n_stages;
   const int ipu = p.ipu;
   const int n_cta = gridDim.x, cta = blockIdx.x;
-  // contiguous shares [c*n/nb, (c+1)*n/nb); the compaction kernel finds the blocks of a frame from the same rule
+  // contiguous shares [c*n/nb, (c+1)*n/nb)
   const int i0 = (int)((unsigned)cta * (unsigned)p.n_items / (unsigned)n_cta);
   const int i1 = (int)((unsigned)(cta + 1) * (unsigned)p.n_items / (unsigned)n_cta);
   const int rows_q = p.tpt * G;
@@ -743,9 +745,9 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
           if (pp * 32 + lane < my_nch * 16) s_col[q * 256 + my_c0 * 16 + pp * 32 + lane] = s;
         }
         PsEpiGroup::sync();
-        float* slot = reinterpret_cast<float*>(sp.colsum_part) + (long long)(cta + f) * P;
+        unsigned long long* row = p.att_acc + (long long)f * P;
         for (int t = et; t < P; t += kPsEpiThreads)
-          slot[t] = (s_col[t] + s_col[256 + t]) + (s_col[512 + t] + s_col[768 + t]);
+          att_add(row + t, (s_col[t] + s_col[256 + t]) + (s_col[512 + t] + s_col[768 + t]));
         PsEpiGroup::sync();                                // the sums may be overwritten
       }
       if (++x == ipu) {

@@ -39,7 +39,7 @@ struct SegSelParams {
   int src32;                    // see the head of this file
   int only_flagged;             // 1: segments whose seg_flag word is 0 are left alone
   int* seg_flag;                // [segments of the chunk]; written with src32 = 1, read with only_flagged
-  int ps_grid, ps_items, ps_ipf;  // the persistent scoring launch: blocks, items, items per frame (src32 = 1)
+  const unsigned long long* att_acc;  // [F][P] column sums of the persistent scoring kernel (src32 = 1)
   unsigned long long* stat_refined;  // frames ranked by the gated double-precision pass are added here
   // Blocks n_seg, n_seg + 1, ... of the grid (one per (layer, K|V) plane, present when prev.n_frames > 0)
   // pool the segment entries the previous call left to this one, on SMs this kernel leaves idle
@@ -86,7 +86,7 @@ __device__ inline int segment_select32(const SegSelParams& p, int f0, int O, int
   const ScoreParams& sp = p.sp;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int P = sp.P, HkvV = sp.Ls * sp.Hkv;
-  // ---- the indicators, from the scoring blocks' column sums (added in block order)
+  // ---- the indicators, from the scoring kernel's column sums
   const float na = 1.f / (float)((long long)sp.Ls * sp.Hq * P), nf = 1.f / (float)((long long)HkvV * sp.D);
   unsigned k0 = 0xffffffffu, k1 = 0u, k2 = 0xffffffffu, k3 = 0u;
   bool bad = false;
@@ -95,20 +95,11 @@ __device__ inline int segment_select32(const SegSelParams& p, int f0, int O, int
   const bool vec4 = (P & 3) == 0;
   for (int i = tid * 4; vec4 && i < O; i += 4 * kSegSelThreads) {
     const int f = f0 + i / P, j = i % P;
-    const int c_first = share_owner((unsigned)(f * p.ps_ipf), (unsigned)p.ps_items, (unsigned)p.ps_grid);
-    const int c_last = share_owner((unsigned)((f + 1) * p.ps_ipf - 1), (unsigned)p.ps_items, (unsigned)p.ps_grid);
-    const float* cp = reinterpret_cast<const float*>(sp.colsum_part) + j;
     const float* fp = reinterpret_cast<const float*>(sp.ifft_part) + (long long)f * HkvV * P + j;
-    float4 a4 = make_float4(0.f, 0.f, 0.f, 0.f), f4 = a4;
-    for (int c0 = c_first; c0 <= c_last; c0 += 8) {
-      float4 x[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        x[u] = c0 + u <= c_last ? __ldcg(reinterpret_cast<const float4*>(cp + (long long)(c0 + u + f) * P))
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int u = 0; u < 8; ++u) { a4.x += x[u].x; a4.y += x[u].y; a4.z += x[u].z; a4.w += x[u].w; }
-    }
+    const ulonglong2* ap = reinterpret_cast<const ulonglong2*>(p.att_acc + (long long)f * P + j);
+    const ulonglong2 a01 = __ldcg(ap), a23 = __ldcg(ap + 1);
+    const float4 a4 = make_float4(att_value(a01.x), att_value(a01.y), att_value(a23.x), att_value(a23.y));
+    float4 f4 = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int g0 = 0; g0 < HkvV; g0 += 8) {
       float4 y[8];
 #pragma unroll
@@ -131,23 +122,16 @@ __device__ inline int segment_select32(const SegSelParams& p, int f0, int O, int
   }
   for (int i = tid; !vec4 && i < O; i += kSegSelThreads) {
     const int f = f0 + i / P, j = i % P;
-    const int c_first = share_owner((unsigned)(f * p.ps_ipf), (unsigned)p.ps_items, (unsigned)p.ps_grid);
-    const int c_last = share_owner((unsigned)((f + 1) * p.ps_ipf - 1), (unsigned)p.ps_items, (unsigned)p.ps_grid);
-    const float* cp = reinterpret_cast<const float*>(sp.colsum_part) + j;
     const float* fp = reinterpret_cast<const float*>(sp.ifft_part) + (long long)f * HkvV * P + j;
-    // all loads of the common case (up to 16 blocks per frame, up to 8 key heads) are in flight together
-    float x[16], y[8];
+    const float a32 = att_value(__ldcg(p.att_acc + (long long)f * P + j));
+    float f32 = 0.f;
+    for (int g0 = 0; g0 < HkvV; g0 += 8) {                 // (eight key heads in flight)
+      float y[8];
 #pragma unroll
-    for (int u = 0; u < 16; ++u) x[u] = c_first + u <= c_last ? __ldcg(cp + (long long)(c_first + u + f) * P) : 0.f;
+      for (int u = 0; u < 8; ++u) y[u] = g0 + u < HkvV ? __ldcg(fp + (long long)(g0 + u) * P) : 0.f;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) y[u] = u < HkvV ? __ldcg(fp + (long long)u * P) : 0.f;
-    float a32 = 0.f, f32 = 0.f;
-#pragma unroll
-    for (int u = 0; u < 16; ++u) a32 += x[u];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) f32 += y[u];
-    for (int cc = c_first + 16; cc <= c_last; ++cc) a32 += __ldcg(cp + (long long)(cc + f) * P);
-    for (int gg = 8; gg < HkvV; ++gg) f32 += __ldcg(fp + (long long)gg * P);
+      for (int u = 0; u < 8; ++u) f32 += y[u];
+    }
     const float a = a32 * na, b = f32 * nf;
     att[i] = a;
     fft[i] = b;
