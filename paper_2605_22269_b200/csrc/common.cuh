@@ -148,6 +148,20 @@ __device__ __forceinline__ float att_value(unsigned long long acc) {
   return (acc & kAttPoison) ? __int_as_float(0x7fffffff) : __ull2float_rn(acc) * (1.f / 1099511627776.f);
 }
 
+// sum of n doubles `stride` apart, added in order, sixteen loads in flight (one after the other each is a round trip to L2)
+__device__ __forceinline__ double ordered_sum(const double* p, int n, long long stride) {
+  double t = 0.0;
+#pragma unroll 1
+  for (int i0 = 0; i0 < n; i0 += 16) {
+    double x[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) x[i] = i0 + i < n ? __ldcg(p + (i0 + i) * stride) : 0.0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) t += x[i];
+  }
+  return t;
+}
+
 // ---------------------------------------------------------------- segment entries (Eq. 5 at segment level)
 // What the pooling of segment entries needs, small enough to travel in registers (compact_segment_plane
 // is kept out of line so that its 32 loads in flight do not set the register count of the kernels that

@@ -114,7 +114,7 @@ __device__ inline bool select_from_partials(const CompactParams& p, int f, bool 
   float att = 0.f, fft = 0.f;
   if (valid) {
     const float* fp = reinterpret_cast<const float*>(sp.ifft_part) + (long long)f * Hkv * P + tid;
-    const float a32 = att_value(__ldcg(p.att_acc + (long long)f * P + tid));
+    const unsigned long long a64 = __ldcg(p.att_acc + (long long)f * P + tid);
     float f32 = 0.f;
 #pragma unroll 1
     for (int g = 0; g < Hkv; g += 8) {                     // (eight key heads in flight)
@@ -127,6 +127,7 @@ __device__ inline bool select_from_partials(const CompactParams& p, int f, bool 
         for (int i = 0; i < w; ++i) y[i] += y[i + w];
       f32 += y[0];
     }
+    const float a32 = att_value(a64);
     att = a32 * (1.f / (float)((long long)sp.Hq * sp.Ls * P));
     fft = f32 * (1.f / (float)((long long)Hkv * sp.D));
   }

@@ -381,11 +381,7 @@ __global__ void __launch_bounds__(kSegSelThreads) segsel_kernel(const SegSelPara
       const int f = f0 + i / P, j = i % P;
       const double* cp = reinterpret_cast<const double*>(sp.colsum_part) + (long long)f * HqV * P + j;
       const double* fp = reinterpret_cast<const double*>(sp.ifft_part) + (long long)f * HkvV * P + j;
-      double a = 0.0, b = 0.0;
-      for (int hh = 0; hh < HqV; ++hh) a += __ldcg(cp + (long long)hh * P);
-      for (int gg = 0; gg < HkvV; ++gg) b += __ldcg(fp + (long long)gg * P);
-      a *= na;
-      b *= nf;
+      const double a = ordered_sum(cp, HqV, P) * na, b = ordered_sum(fp, HkvV, P) * nf;
       sa[i] = a;
       sf[i] = b;
       bad |= !(isfinite(a) && isfinite(b));
