@@ -1312,7 +1312,7 @@ mukv_status mukv_gather3(mukv_ctx* ctx, const int32_t* d_seg_idx, const int32_t*
     gp.decode_stride = decode_stride_bytes;
     gp.ntok = d_ntok; gp.tok_meta = d_tok_meta;
     const long long units = (long long)nq * c.n_layers * 2 * (k_frm + 1);
-    const unsigned blocks = (unsigned)(units < 148 * 8 ? units : 148 * 8);
+    const unsigned blocks = (unsigned)(units < 0x7fffffffLL ? units : 0x7fffffffLL);   // one run per block, see gather_kernel
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaSuccess;
     {
@@ -1359,7 +1359,7 @@ mukv_status mukv_gather(mukv_ctx* ctx, const int32_t* d_frm_idx, const int32_t* 
     gp.decode_stride = decode_stride_bytes;
     gp.tok_meta = d_tok_meta;
     const long long units = (long long)nq * c.n_layers * 2 * k_frm;
-    const unsigned blocks = (unsigned)(units < 148 * 8 ? units : 148 * 8);
+    const unsigned blocks = (unsigned)(units < 0x7fffffffLL ? units : 0x7fffffffLL);   // one run per block, see gather_kernel
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaSuccess;
     {

@@ -1015,7 +1015,9 @@ struct GatherParams {
 };
 
 // unit = (question, plane = l*2+kv, slot): one contiguous run of the page goes to one contiguous
-// run of the decode buffer.
+// run of the decode buffer.  Bound by memory.  One block per unit: with eight blocks per SM that walked the units the blocks
+// drifted apart, and 64 questions (5.75 GB, 57,344 runs of 50 KB) took 1,002 us; blocks that start in the order of the
+// units keep to neighbouring pages: 867 us, 6.6 TB/s.  (A ring of bulk copies through shared memory: 961 us.)
 __global__ void __launch_bounds__(256) gather_kernel(const GatherParams p) {
   pdl_wait();                                              // the selection may be the work of the kernel in front
   const long long planes = (long long)p.L * 2;
