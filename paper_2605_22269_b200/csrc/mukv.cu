@@ -1364,7 +1364,8 @@ mukv_status mukv_gather(mukv_ctx* ctx, const int32_t* d_frm_idx, const int32_t* 
     cudaError_t e = cudaSuccess;
     {
       ProfScope ps(ctx, 7, st);
-      e = launch_k(gather_kernel, dim3(blocks), 256, 0, st, !ctx->prof_on, gp);
+      const bool wide = run >= 16 * 1024;
+      e = launch_k(wide ? gather_kernel<512> : gather_kernel<128>, dim3(blocks), wide ? 512u : 128u, 0, st, !ctx->prof_on, gp);
     }
     if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "gather kernel: %s", cudaGetErrorString(e));
     ctx->launches += 1;

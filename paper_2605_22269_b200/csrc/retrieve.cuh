@@ -1017,8 +1017,11 @@ struct GatherParams {
 // unit = (question, plane = l*2+kv, slot): one contiguous run of the page goes to one contiguous
 // run of the decode buffer.  Bound by memory.  One block per unit: with eight blocks per SM that walked the units the blocks
 // drifted apart, and 64 questions (5.75 GB, 57,344 runs of 50 KB) took 1,002 us; blocks that start in the order of the
-// units keep to neighbouring pages: 867 us, 6.6 TB/s.  (A ring of bulk copies through shared memory: 961 us.)
-__global__ void __launch_bounds__(256) gather_kernel(const GatherParams p) {
+// units keep to neighbouring pages: 867 us with 256 threads, 855 with 512 (two thirds as many runs open at a time; 128
+// threads: 904), 6.7 TB/s.  Runs below 16 KB would leave 512 threads idle and take 128.  (A ring of bulk copies through
+// shared memory: 961 us.)
+template <int NT>
+__global__ void __launch_bounds__(NT) gather_kernel(const GatherParams p) {
   pdl_wait();                                              // the selection may be the work of the kernel in front
   const long long planes = (long long)p.L * 2;
   const long long n_units = (long long)p.nq * planes * p.k_frm;
@@ -1034,19 +1037,16 @@ __global__ void __launch_bounds__(256) gather_kernel(const GatherParams p) {
                          ((long long)plane * p.k_frm + slot) * p.run_bytes;
     const long long nvec = p.run_bytes >> 4;
     long long v = threadIdx.x;
-    for (; v + 3 * 256 < nvec; v += 4 * 256) {
-      uint4 x0 = ld_stream(src + (v << 4));
-      uint4 x1 = ld_stream(src + ((v + 256) << 4));
-      uint4 x2 = ld_stream(src + ((v + 512) << 4));
-      uint4 x3 = ld_stream(src + ((v + 768) << 4));
-      st_stream(dst + (v << 4), x0);
-      st_stream(dst + ((v + 256) << 4), x1);
-      st_stream(dst + ((v + 512) << 4), x2);
-      st_stream(dst + ((v + 768) << 4), x3);
+    for (; v + 3 * NT < nvec; v += 4 * NT) {
+      uint4 x[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[i] = ld_stream(src + ((v + i * NT) << 4));
+#pragma unroll
+      for (int i = 0; i < 4; ++i) st_stream(dst + ((v + i * NT) << 4), x[i]);
     }
-    for (; v < nvec; v += 256) st_stream(dst + (v << 4), ld_stream(src + (v << 4)));
+    for (; v < nvec; v += NT) st_stream(dst + (v << 4), ld_stream(src + (v << 4)));
     if (plane == 0 && p.tok_meta) {
-      for (int t = threadIdx.x; t < p.kappa; t += 256) {
+      for (int t = threadIdx.x; t < p.kappa; t += NT) {
         int* m = p.tok_meta + (((long long)qi * p.k_frm + slot) * p.kappa + t) * 2;
         m[0] = f;
         m[1] = p.kept_store[(long long)f * p.kappa + t];
@@ -1089,43 +1089,45 @@ __device__ __forceinline__ void copy_run16(unsigned char* dst, const unsigned ch
 
 constexpr int kGatherListCap = 1024;       // rows of patch-level blocks listed at a time (>= MUKV_MAX_TOKENS)
 
-// Units, per question and (layer, K|V) plane: k_frm frame runs (one contiguous run of the page each),
-// then one unit for the summary tokens and the patch-level rows.  Token slots of a plane: summary
+// Units, one per block: first, for every question and (layer, K|V) plane, the summary tokens and the patch-level rows
+// (the longest ones: at the end of their plane's runs the last of them worked alone), then per question and plane k_frm
+// frame runs (one contiguous run of the page each).  Token slots of a plane: summary
 // tokens of the selected segments, kept tokens of the selected frames, kept tokens of the selected
 // patch-level blocks.
 template <typename T>
 __global__ void __launch_bounds__(256) gather3_kernel(const Gather3Params p) {
   __shared__ int s_off[MUKV_MAX_TOPK + 1];                 // first row of each selected patch block
   __shared__ long long s_src[kGatherListCap];              // byte offset in the store of each listed row
-  __shared__ int s_row0;
   pdl_wait();
   const long long planes = (long long)p.L * 2;
-  const int upp = p.k_frm + 1;                             // units per (question, plane)
-  const long long n_units = (long long)p.nq * planes * upp;
+  const long long n_rest = (long long)p.nq * planes;
+  const long long n_units = n_rest * (p.k_frm + 1);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   const long long row_bytes = (long long)p.C * p.esize;
   const long long run_bytes = (long long)p.kappa * row_bytes;
   for (long long u = blockIdx.x; u < n_units; u += gridDim.x) {
-    const int slot = (int)(u % upp);
-    const long long r = u / upp;
+    const bool run = u >= n_rest;
+    const int slot = run ? (int)((u - n_rest) % p.k_frm) : 0;
+    const long long r = run ? (u - n_rest) / p.k_frm : u;
     const int plane = (int)(r % planes);
     const int qi = (int)(r / planes);
     const int c_seg = p.counts[3 * qi], c_frm = p.counts[3 * qi + 1], c_pat = p.counts[3 * qi + 2];
     unsigned char* dplane = p.decode + (long long)qi * p.decode_stride + (long long)plane * p.tok_cap * row_bytes;
     int* meta = p.tok_meta ? p.tok_meta + (long long)qi * p.tok_cap * 2 : nullptr;
-    if (slot < p.k_frm) {
+    // kept tokens of the first n selected frames, with pages of different lengths (every warp adds them up itself)
+    auto kept_before = [&](int n) {
+      int t = 0;
+      for (int i = lane; i < n; i += 32) t += p.kept_count[p.frm_idx[(long long)qi * p.k_frm + i]];
+      __syncwarp();
+      return warp_sum(t);
+    };
+    if (run) {
       if (slot >= c_frm) continue;
       const int f = p.frm_idx[(long long)qi * p.k_frm + slot];
       int row0 = c_seg + slot * p.kappa, rows = p.kappa;
       if (p.kept_count) {
         // pages of different lengths: this frame's rows start behind those of the frames before it
-        __syncthreads();
-        if (threadIdx.x == 0) {
-          int off = c_seg;
-          for (int i = 0; i < slot; ++i) off += p.kept_count[p.frm_idx[(long long)qi * p.k_frm + i]];
-          s_row0 = off;
-        }
-        __syncthreads();
-        row0 = s_row0;
+        row0 = c_seg + kept_before(slot);
         rows = p.kept_count[f];
       }
       const long long fbytes = (long long)rows * row_bytes;
@@ -1151,23 +1153,21 @@ __global__ void __launch_bounds__(256) gather3_kernel(const Gather3Params p) {
     }
     // ---- patch-level rows: block b = frame * S + super patch holds the frame's kept rows inside it
     __syncthreads();
+    const int off0 = c_seg + (p.kept_count ? kept_before(c_frm) : c_frm * p.kappa);
+    for (int i = threadIdx.x; i < c_pat; i += blockDim.x) s_off[i + 1] = p.patch_cnt[p.pat_idx[(long long)qi * p.k_pat + i]];
+    __syncthreads();
     if (threadIdx.x == 0) {
-      int off = c_seg + c_frm * p.kappa;
-      if (p.kept_count) {
-        off = c_seg;
-        for (int i = 0; i < c_frm; ++i) off += p.kept_count[p.frm_idx[(long long)qi * p.k_frm + i]];
-      }
-      for (int i = 0; i < c_pat; ++i) {
+      int off = off0;
+      s_off[0] = off;
+      for (int i = 1; i <= c_pat; ++i) {
+        off += s_off[i];
         s_off[i] = off;
-        off += p.patch_cnt[p.pat_idx[(long long)qi * p.k_pat + i]];
       }
-      s_off[c_pat] = off;
       if (plane == 0 && p.ntok) p.ntok[qi] = off;
     }
     __syncthreads();
     // Patch blocks in batches whose rows fit the list.  One warp per block walks the frame's kept
     // list and notes where the rows of its super patch lie; then the whole block copies the rows.
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     const int vpr = (int)(row_bytes >> 4);                 // 16-byte vectors per row
     for (int b0 = 0; b0 < c_pat;) {
       int b1 = b0 + 1;                                     // (one block has at most kappa <= list capacity rows)
