@@ -970,12 +970,12 @@ mukv_status retrieve_impl(mukv_ctx* ctx, const void* d_qtok, const int32_t* h_q_
       rp.f_seg = reinterpret_cast<const float*>(ctx->ws + ctx->wl.f_seg); rp.f_seg_stride = pad4(ctx->sl.max_segs);
       rp.f_pat = reinterpret_cast<const float*>(ctx->ws + ctx->wl.f_pat); rp.f_pat_stride = pad4((long long)c.max_frames * S);
       const size_t room = (size_t)kRankStageBytes - rank_smem;
-      const size_t b1 = (size_t)(pad4(n_frm) + pad4(n_seg)) * sizeof(float), b2 = (size_t)pad4(n_pat) * sizeof(float);
-      if (b1 <= room) {
-        rp.stage = n_pat == 0 ? 1 : b1 + b2 <= room ? 2 : b2 <= room ? 3 : 1;
-        rank_smem += rp.stage == 2 ? b1 + b2 : rp.stage == 3 && b2 > b1 ? b2 : b1;
-      }
-      e = launch_k(rank_kernel, dim3(nq), kRankThreads, rank_smem, st, !ctx->prof_on, rp, meta);
+      const size_t b1 = (size_t)(pad4(n_seg) + pad4(n_frm)) * sizeof(float);
+      const size_t b2 = (size_t)(pad4(n_seg) + pad4(n_pat)) * sizeof(float);
+      if (b1 <= room) rp.stage |= 1;
+      if (n_pat > 0 && b2 <= room) rp.stage |= 2;
+      rank_smem += rp.stage == 3 ? (b1 > b2 ? b1 : b2) : rp.stage == 2 ? b2 : rp.stage == 1 ? b1 : 0;
+      e = launch_k(rank_kernel, dim3(nq, k_pat > 0 ? 2 : 1), kRankThreads, rank_smem, st, !ctx->prof_on, rp, meta);
     }
     if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "rank kernel: %s", cudaGetErrorString(e));
     ctx->launches += 4;

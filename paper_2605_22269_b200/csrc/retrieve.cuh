@@ -142,7 +142,7 @@ __device__ __forceinline__ void scan_store(const ScanParams& sp, int qi, long lo
   }
 }
 
-__global__ void __launch_bounds__(256) scan_kernel(const ScanParams sp) {
+__global__ void __launch_bounds__(256, 3) scan_kernel(const ScanParams sp) {
   const float* __restrict__ frame_key = sp.frame_key;
   const float* __restrict__ seg_key = sp.seg_key;
   const long long n_frm = sp.n_frm, n_seg = sp.n_seg;
@@ -768,8 +768,8 @@ struct RankParams {
   int* counts; int counts_stride;         // 2 or 3 ints per question
   const float* f_frm; const float* f_seg; const float* f_pat;     // single-precision copies of the scores
   long long f_frm_stride, f_seg_stride, f_pat_stride;
-  int stage;                              // 1: the copies of segments and frames fit in shared memory; 2: those of the
-                                          // patch-level blocks beside them; 3: those in place of them, afterwards
+  int stage;                              // bit 0: the copies of segments and frames fit in shared memory, bit 1: those of
+                                          // segments and patch-level blocks
 };
 
 constexpr int kRankThreads = 512;
@@ -846,6 +846,8 @@ __device__ __forceinline__ void rank_emit(int* idx, float* score, long long base
   }
 }
 
+// Grid (questions, 1 or 2): with patch-level blocks a second block per question ranks them beside the frames; it finds the
+// segments again, which both need.  (One block for all: 42 us for eight questions on 1,800 frames; so: 28.)
 __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, const QMeta meta) {
   __shared__ RankShared sh;
   __shared__ __align__(8) uint64_t s_bar[3];
@@ -853,6 +855,7 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
   double* gq = reinterpret_cast<double*>(smem_raw);               // [C] global query
 
   const int qi = blockIdx.x, tid = threadIdx.x;
+  const bool do_frm = blockIdx.y == 0, do_pat = p.k_pat > 0 && blockIdx.y + 1 == gridDim.y;
   pdl_wait();                                                // the scores of the scan are complete
   if (p.nq <= kScanFew) pdl_trigger();                       // (many of these blocks would leave the gather an uneven start)
   const int C = p.C;
@@ -870,7 +873,7 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
   // Single-precision copies of the scores, on their way while the segments are ranked.  (n4 values each: what lies
   // behind the n-th belongs to this question's row, too)
   float *buf_s = nullptr, *buf_f = nullptr, *buf_p = nullptr;
-  const int s4 = (n_seg + 3) & ~3, f4 = (n_frm + 3) & ~3, p4 = (n_frm * p.S + 3) & ~3;
+  const int s4 = (n_seg + 3) & ~3, f4 = do_frm ? (n_frm + 3) & ~3 : 0, p4 = do_pat ? (n_frm * p.S + 3) & ~3 : 0;
   const uint32_t bar0 = tc::smem_u32(s_bar);
   auto load = [&](float* dst, const float* src, int n4, int bar) {
     tc::mbar_expect_tx(bar0 + 8u * bar, 4u * (uint32_t)n4);
@@ -878,16 +881,15 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
   };
   if (p.stage) {
     buf_s = reinterpret_cast<float*>(gq + C);
-    buf_f = buf_s + s4;
-    if (p.stage == 2) buf_p = buf_f + f4;
-    if (p.stage == 3) buf_p = buf_s;
+    if (do_frm && (p.stage & 1)) buf_f = buf_s + s4;
+    if (do_pat && (p.stage & 2)) buf_p = buf_s + s4;       // (in a block of its own)
     if (tid == 0) {
       for (int b = 0; b < 3; ++b) tc::mbar_init(bar0 + 8u * b, 1);
       tc::fence_mbar_init();
       tc::fence_proxy_async_smem();
       if (s4) load(buf_s, p.f_seg + (long long)qi * p.f_seg_stride, s4, 0);
-      if (f4) load(buf_f, p.f_frm + (long long)qi * p.f_frm_stride, f4, 1);
-      if (p.stage == 2 && p4) load(buf_p, p.f_pat + (long long)qi * p.f_pat_stride, p4, 2);
+      if (buf_f && f4) load(buf_f, p.f_frm + (long long)qi * p.f_frm_stride, f4, 1);
+      if (buf_p && p4) load(buf_p, p.f_pat + (long long)qi * p.f_pat_stride, p4, 2);
     }
     __syncthreads();
   }
@@ -940,7 +942,7 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
   if (c_seg < 0)
     c_seg = rank_level(ss, nullptr, n_seg, p.k_seg, semi && p.lam_seg > 0.0, p.lam_seg, p.delta, p.seg_key, C, gq, gnorm,
                        have_g, &sh, seg_buf);
-  rank_emit(p.seg_idx, p.seg_score, (long long)qi * p.k_seg, p.k_seg, c_seg, &sh);
+  if (do_frm) rank_emit(p.seg_idx, p.seg_score, (long long)qi * p.k_seg, p.k_seg, c_seg, &sh);
   for (int i = tid; i < c_seg; i += kRankThreads) sh.sel_seg[i] = sh.pick[i];
   __syncthreads();
 
@@ -949,9 +951,10 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
   // runs over positions in the list "selected segments (ascending) x their frames" and maps the
   // winners back (ascending position = ascending frame).
   const int fseg = p.fseg;
-  int c_frm;
+  int c_frm = 0;
   float* const frm_buf = landed(buf_f, f4, 1);               // (waited for in every mode: the copy must land before the block leaves)
-  if (p.mode == MUKV_RETR_HIER) {
+  if (!do_frm) {
+  } else if (p.mode == MUKV_RETR_HIER) {
     auto frame_of = [&](int i) { return sh.sel_seg[i / fseg] * fseg + i % fseg; };
     auto score_h = [&](int i) { return sf[frame_of(i)]; };
     auto member_h = [&](int i) { return frame_of(i) < n_frm; };
@@ -962,20 +965,13 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
     c_frm = rank_level(sf, nullptr, n_frm, p.k_frm, semi, p.lam_frm, p.delta, p.frame_key, C, gq, gnorm, have_g, &sh,
                        frm_buf);
   }
-  rank_emit(p.frm_idx, p.frm_score, (long long)qi * p.k_frm, p.k_frm, c_frm, &sh);
+  if (do_frm) rank_emit(p.frm_idx, p.frm_score, (long long)qi * p.k_frm, p.k_frm, c_frm, &sh);
   __syncthreads();
 
   // ---- patch-level blocks: (frame, super patch) pairs that kept at least one token
   int c_pat = 0;
-  if (p.stage == 3 && p4) {
-    __syncthreads();                                         // the frames' copies are no longer read
-    if (tid == 0) {
-      tc::fence_proxy_async_smem();
-      load(buf_p, p.f_pat + (long long)qi * p.f_pat_stride, p4, 2);
-    }
-  }
   float* const pat_buf = landed(buf_p, p4, 2);
-  if (p.k_pat > 0) {
+  if (do_pat) {
     const int S = p.S;
     const int* cnt = p.patch_cnt;
     if (S > 0) {
@@ -998,9 +994,11 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
     rank_emit(p.pat_idx, p.pat_score, (long long)qi * p.k_pat, p.k_pat, c_pat, &sh);
   }
   if (tid == 0) {
-    p.counts[p.counts_stride * qi] = c_seg;
-    p.counts[p.counts_stride * qi + 1] = c_frm;
-    if (p.counts_stride > 2) p.counts[p.counts_stride * qi + 2] = c_pat;
+    if (do_frm) {
+      p.counts[p.counts_stride * qi] = c_seg;
+      p.counts[p.counts_stride * qi + 1] = c_frm;
+    }
+    if (p.counts_stride > 2 && blockIdx.y + 1 == gridDim.y) p.counts[p.counts_stride * qi + 2] = c_pat;
   }
 }
 
