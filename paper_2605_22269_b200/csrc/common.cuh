@@ -135,10 +135,16 @@ __device__ __forceinline__ int super_patch_index(int j, int P, int grid_width, i
   return (j / grid_width) / rh * split + (j % grid_width) / cw;
 }
 
-// Column sums of the softmax (Eq. 1), as the blocks of the persistent scoring kernel add them up: 24.40 fixed point in 64
+// Column sums of the softmax (Eq. 1), as the blocks of the persistent scoring kernel add them up: 23.40 fixed point in 64
 // bits, so that the result does not depend on the order of the additions.  A column sum is at most the number of query
-// rows that see the frame (layers x heads x tokens: 2^20 at the supported shapes), a block's share has 24 significant
-// bits, and 2^-40 is 2^-17 of the last of them at a sum of 1.  Bit 63 marks a share that is not a number.
+// rows that see the frame (layers x heads x tokens: 2^20 at the supported shapes).  Bit 63 marks a share that is not a
+// number.
+// A share is rounded to 2^-40, at most 256 blocks share a frame: a sum is off by 2^-33 at the most.  Eq. 4 divides by
+// the range of the frame's sums, so a range below kAttFine = 2^-10 sends the frame to the double-precision pass; above it the
+// rounding stays below 2^-23 of the range.  Without past keys the sums of a frame reach layers x heads at least, and the
+// test for a flat signal flags such a frame already; with them a strong cached key can leave the frame's own columns next
+// to nothing (at e^-30 of the mass every share rounds to 0).
+constexpr float kAttFine = 1.f / 1024.f;
 constexpr unsigned long long kAttPoison = 1ull << 63;
 __device__ __forceinline__ void att_add(unsigned long long* acc, float v) {
   if (!(v < 1e30f)) atomicOr(acc, kAttPoison);

@@ -239,6 +239,9 @@ __device__ inline bool select_from_partials(const CompactParams& p, int f, bool 
   const float aabs = fmaxf(amax, -amin), fabs_ = fmaxf(fmax_, -fmin_);
   if (amax != amin && (amax - amin) < sp.flat_ratio * aabs && sp.alpha != 0.f) risky = true;
   if (fmax_ != fmin_ && (fmax_ - fmin_) < sp.flat_ratio * fabs_ && sp.alpha != 1.f) risky = true;
+  // column sums too close together for their fixed-point step (see kAttFine); equal ones only when they are small as well
+  const float fine = kAttFine / (float)((long long)sp.Hq * sp.Ls * P);
+  if (amax - amin < fine && (amax != amin || amax < fine)) risky = true;
   if (bad) risky = false;                                 // double precision would not rank it either
   if (keep) s_kept[pos] = tid;
   if (write) {

@@ -211,3 +211,37 @@ def test_past_keys_in_the_attention(name, T, chunk, W, over, opts):
         # tensor-core path with cached keys in the tile: the headroom the single-precision selection rests on
         worst = max(float(np.max(np.abs(run.scores[2, t] - st.scores[t][2]))) for t in range(T))
         assert worst < H.FLAG_MARGIN / 2 and stats.refined_frames <= max(1, T // 8), (worst, stats.refined_frames)
+
+
+@pytest.mark.parametrize("gap", [6, 12, 20, 30, 45, 70])
+def test_past_keys_that_take_almost_all_the_attention(gap):
+    # Every cached key's logit lies about `gap` nats above the frame's own ones: the own column sums are then about e^-gap
+    # of a row each, down to far below what a sum near 1 resolves, and Eq. 4 divides by their range.
+    spec = H.StreamSpec(seed=77, n_layers=1, n_q_heads=8, n_kv_heads=2, head_dim=64, tokens_per_frame=64, bf16=True, n_outlier=0,
+                        n_frames=3, scene_sigma=1.0, frame_sigma=0.5, scene_min=2, scene_max=4)
+    run = H.GpuRun(dict(spec=spec, keep=16, fseg=2, chunk=2, alpha=0.7), past_frames=1)
+    rng = np.random.default_rng(5)
+    q = rng.standard_normal((3, 64, 8, 64)).astype(np.float32)
+    k = rng.standard_normal((1, 3, 64, 2, 64)).astype(np.float32)
+    q[..., 0], k[..., 0] = 8.0, 0.0
+    k[:, 0, ..., 0] = gap                                  # 8 * gap / sqrt(64) in the logits of frame 0's keys
+    q, k = (H.to_device(x, False, run.device).bfloat16() for x in (q, k))
+    qb, kb = H.to_numpy_bits(q), H.to_numpy_bits(k)
+    # frame 0 is ranked by given numbers: its own signals, all logits and every spectrum offset by `gap`, are not the subject
+    given = rng.random((1, 64)).astype(np.float32)
+    kept = torch.full((3, 16), -1, dtype=torch.int32, device=run.device)
+    sc = torch.zeros((3, 2, 64), dtype=torch.float32, device=run.device)
+    k0, k1 = k[:, :1].contiguous(), k[:, 1:].contiguous()
+    run.ctx.mukv_compress_chunk_scored(torch.from_numpy(given).to(run.device), k0, k0, 1, 0, kept[:1])
+    run.ctx.mukv_compress_chunk(q[1:], k1, k1, 2, 1, kept[1:], sc)
+    torch.cuda.synchronize()
+    st = O.Store(H.oracle_cfg(run.cfg))
+    O.compress_chunk(st, None, kb[:, :1], kb[:, :1], select_scores=given)
+    O.compress_chunk(st, qb[1:], kb[:, 1:], kb[:, 1:])
+    assert kept[0].tolist() == st.kept[0].tolist()
+    for f in (1, 2):
+        assert kept[f].tolist() == st.kept[f].tolist()
+        # the bound that the choice between single and double precision rests on holds at every distance
+        assert np.abs(sc[2, f - 1].cpu().numpy() - st.scores[f][2]).max() < H.FLAG_MARGIN / 2
+        assert np.abs(sc[0, f - 1].cpu().numpy() / st.scores[f][0] - 1.0).max() < 1e-5
+    assert st.scores[2][0].sum() < 2.0 * np.exp(5.0 - gap)  # (the own columns are what the name says)
