@@ -43,7 +43,7 @@ struct WorkLayout {
   size_t colsum_f, ifft_f, colsum_d, ifft_d, frame_counter, flagged, n_flagged, tail_ctr, sel_flag,
       seg_flag, stat_refined, dev_status, att_acc;
   size_t q64, qnorm, s_frm, s_seg, s_pat, f_frm, f_seg, f_pat, wtab, total;
-  size_t zero_begin, zero_end;          // region that must start as zeros: counters up to att_acc, then att_acc
+  size_t zero_begin, zero_end;          // region that must start as zeros
 };
 
 // Tiling of the tensor-core scoring kernel (bf16 inputs only).
@@ -1160,14 +1160,15 @@ mukv_status mukv_profile_read(mukv_ctx* ctx, double* ms, int64_t* launches) {
 
 mukv_status mukv_reset(mukv_ctx* ctx, mukv_stream stream) {
   if (!ctx) return MUKV_E_INVALID;
-  // arrival counters, flagged lists, selection flags, statistics and the event word start over
-  // (the column sums are clean where the next call needs them, unless a call broke off)
-  cudaError_t e = cudaMemsetAsync(ctx->ws + ctx->wl.zero_begin, 0,
-                                  (ctx->failed ? ctx->wl.zero_end : ctx->wl.att_acc) - ctx->wl.zero_begin,
+  // Arrival counters, flagged lists, selection flags, statistics, the event word and the column sums start over, and so does
+  // the alternation between the two sets: calls captured into a graph behind a reset are replayed with the sets that they were
+  // captured with, so the reset has to leave both in the same state every time.
+  cudaError_t e = cudaMemsetAsync(ctx->ws + ctx->wl.zero_begin, 0, ctx->wl.zero_end - ctx->wl.zero_begin,
                                   static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "mukv_reset: %s", cudaGetErrorString(e));
   ctx->frames = 0;
-  if (ctx->failed) ctx->att_dirty[0] = ctx->att_dirty[1] = 0;
+  ctx->parity = 0;
+  ctx->att_dirty[0] = ctx->att_dirty[1] = 0;
   ctx->failed = false;
   ctx->seg_pending = false;
   return MUKV_OK;
