@@ -226,6 +226,8 @@ mukv_status mukv_compress_chunk_scored(mukv_ctx* ctx, const float* d_select_scor
  *   d_seg_idx [nq][k_seg], d_frm_idx [nq][k_frm]: selected ids ascending, unused slots -1.
  *   d_seg_score / d_frm_score: matching scores (stage-1 cosine for segments, final score
  *               for frames), or NULL.   d_counts [nq][2]: number of valid (segments, frames).
+ * A block whose key holds Inf or NaN, and every block for a question whose tokens do, has no cosine: it ranks behind all
+ * others with the score -2 (ties to the lowest id, as always) and its key stays out of the global query.
  * Errors: INVALID, ALIGN, CAPACITY (nq, k, question length, workspace), STATE (empty store). */
 mukv_status mukv_retrieve(mukv_ctx* ctx, const void* d_qtok, const int32_t* h_q_offsets,
                           const int64_t* h_t_limit, int32_t nq,

@@ -28,6 +28,7 @@ import numpy as np
 
 TIE_EPS = 1e-6
 NORM_FLOOR = 1e-12
+NO_SCORE = -2.0                  # cosine of vectors that are not finite: behind every other
 
 
 # --------------------------------------------------------------------------
@@ -434,14 +435,25 @@ def pool_question(Qq, n_kv_heads: int) -> np.ndarray:
 
 
 def cosine(q, keys) -> np.ndarray:
-    """cos(q, keys[t]) for every row (Eq. 7); a zero-norm pair scores 0."""
+    """cos(q, keys[t]) for every row (Eq. 7); a zero-norm pair scores 0.
+
+    The paper does not say what a vector with an Inf or NaN scores.  Reading: NO_SCORE, which ranks behind every cosine.
+    """
     q = np.asarray(q, dtype=np.float64)
     keys = np.asarray(keys, dtype=np.float64)
     if keys.shape[0] == 0:
         return np.zeros(0, dtype=np.float64)
-    num = keys @ q
-    den = np.sqrt((keys * keys).sum(axis=1)) * np.sqrt((q * q).sum())
-    return num / np.maximum(den, NORM_FLOOR)
+    with np.errstate(invalid="ignore", over="ignore"):
+        num = keys @ q
+        den = np.sqrt((keys * keys).sum(axis=1)) * np.sqrt((q * q).sum())
+        s = num / np.maximum(den, NORM_FLOOR)
+    return np.where(np.isfinite(s), s, NO_SCORE)
+
+
+def global_query(s_seg, key_s, top):
+    """Mean of the keys of the segments `top` that have a score; None if none has."""
+    top = top[s_seg[top] != NO_SCORE]
+    return key_s[top].sum(axis=0) / float(top.shape[0]) if top.shape[0] > 0 else None
 
 
 MODE_PARALLEL, MODE_HIER, MODE_SEMI = 0, 1, 2
@@ -482,15 +494,8 @@ def retrieve(store: Store, Qq, k_seg: int, k_frm: int, top_n: int = 0, lam: floa
         cand = topk_set(s_frm, min(2 * k_frm, n_frm), delta)
         N = k_seg if top_n <= 0 else top_n
         top = topk_set(s_seg, min(N, n_seg), delta)
-        if top.shape[0] > 0:
-            g = key_s[top].sum(axis=0) / float(top.shape[0])
-            gamma = cosine(g, key_f[cand])
-        else:
-            gamma = np.zeros(cand.shape[0])
-        s_new = (1.0 - lam) * s_frm[cand] + lam * gamma
-        pick = topk_set(s_new, min(k_frm, cand.shape[0]), delta)
+        pick, final = _rerank(s_frm, key_f, cand, global_query(s_seg, key_s, top), lam, k_frm, delta)
         sel_frm = cand[pick]
-        final = s_new[pick]
     return {
         "q": q, "s_frm": s_frm, "s_seg": s_seg,
         "seg_idx": sel_seg, "seg_score": s_seg[sel_seg],
@@ -501,7 +506,7 @@ def retrieve(store: Store, Qq, k_seg: int, k_frm: int, top_n: int = 0, lam: floa
 def _rerank(s_stage1, keys, cand, g, lam, k, delta):
     """Eq. 8 on one granularity's candidates: returns (positions in cand, their calibrated scores)."""
     gamma = cosine(g, keys[cand]) if g is not None else np.zeros(cand.shape[0])
-    s_new = (1.0 - lam) * s_stage1[cand] + lam * gamma
+    s_new = np.where(s_stage1[cand] == NO_SCORE, NO_SCORE, (1.0 - lam) * s_stage1[cand] + lam * gamma)
     pick = topk_set(s_new, min(k, cand.shape[0]), delta)
     return pick, s_new[pick]
 
@@ -540,7 +545,7 @@ def retrieve3(store: Store, Qq, k_g, lambda_g, top_n: int = 0, mode: int = MODE_
     # segment level; its own lambda is applied too (the paper sets it to 0: the global query comes from them)
     N = k_seg if top_n <= 0 else top_n
     top = topk_set(s_seg, min(N, n_seg), delta)
-    g = key_s[top].sum(axis=0) / float(top.shape[0]) if top.shape[0] > 0 else None
+    g = global_query(s_seg, key_s, top)
     if mode == MODE_SEMI and lam_seg > 0.0:
         cand = topk_set(s_seg, min(2 * k_seg, n_seg), delta)
         pick, sc = _rerank(s_seg, key_s, cand, g, lam_seg, k_seg, delta)

@@ -126,8 +126,13 @@ struct ScanParams {
   const int* patch_cnt;
 };
 #define kScanAbsent (-INFINITY)
+// The score of a block whose key, or of a question whose pooled vector, holds Inf or NaN: below every cosine and every mix
+// of two.  Every score that is ranked is finite, so that a ranking of n members for k <= n places always fills all k (with a
+// NaN for the k-th largest score no comparison holds and nothing was kept; the ids were then whatever lay in shared memory).
+constexpr double kScoreNone = -2.0;
 
 __device__ __forceinline__ void scan_store(const ScanParams& sp, int qi, long long row, double sc) {
+  if (!(fabs(sc) < 2.0)) sc = kScoreNone;
   if (row < sp.n_frm) {
     sp.s_frm[(long long)qi * sp.frm_stride + row] = sc;
     sp.f_frm[(long long)qi * sp.f_frm_stride + row] = (float)sc;
@@ -486,7 +491,7 @@ template <typename ScoreFn, typename MemberFn>
 __device__ __noinline__ int block_topk_set(ScoreFn score, MemberFn member, int n, int k, double delta, int* out_idx,
                               double* out_score, RankScratch* sc) {
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nt >> 5;
-  bool all = false, odd = false;
+  bool all = false;
   int n_mem = 0, bin = 0;
   RankBins bin_of{0.f, 0.f};
   __syncthreads();                                           // the scratch may still be read from a previous call
@@ -502,7 +507,6 @@ __device__ __noinline__ int block_topk_set(ScoreFn score, MemberFn member, int n
       if (!member(i)) continue;
       const float s = (float)score(i);
       const unsigned key = order_key32(s);
-      odd |= !(fabsf(s) < 1e30f);
       kmin = min(kmin, key);
       kmax = max(kmax, key);
       ++local;
@@ -513,47 +517,43 @@ __device__ __noinline__ int block_topk_set(ScoreFn score, MemberFn member, int n
     local = __reduce_add_sync(kFull, local);
     if (lane == 0) { sc->wmin[warp] = kmin; sc->wmax[warp] = kmax; sc->wcnt[warp] = local; }
     for (int b = tid; b < kRankBins; b += nt) sc->hist[b] = 0u;
-    odd = __syncthreads_or(odd) != 0;
+    __syncthreads();
     n_mem = __reduce_add_sync(kFull, lane < nwarp ? sc->wcnt[lane] : 0);
     if (k > n_mem) k = n_mem;
     if (k <= 0) return 0;
     all = (k == n_mem);
-    if (!odd) {
-      bin_of = rank_bins(sc, nwarp);
-      if (!all) {
-        for (int i = tid; i < n; i += nt)
-          if (member(i)) atomicAdd(&sc->hist[bin_of((float)score(i))], 1u);
-        __syncthreads();
-        bin = rank_find_bin(k, sc);
-      }
+    bin_of = rank_bins(sc, nwarp);
+    if (!all) {
+      for (int i = tid; i < n; i += nt)
+        if (member(i)) atomicAdd(&sc->hist[bin_of((float)score(i))], 1u);
+      __syncthreads();
+      bin = rank_find_bin(k, sc);
     }
   } else {
     __syncthreads();
   }
-  if (!odd) {
-    const double slack = 2.0 * delta + 1e-12;
-    for (int i = tid; i < n; i += nt) {
-      if (!member(i)) continue;
-      const double s = score(i);
-      if (bin == 0 || bin_of((float)(s + slack)) >= bin) {
-        const int c = atomicAdd(&sc->cand_n, 1);
-        if (c < kRankCand) {
-          sc->cand_idx[c] = i;
-          sc->cand_key[c] = order_key(s);
-        }
+  const double slack = 2.0 * delta + 1e-12;
+  for (int i = tid; i < n; i += nt) {
+    if (!member(i)) continue;
+    const double s = score(i);
+    if (bin == 0 || bin_of((float)(s + slack)) >= bin) {
+      const int c = atomicAdd(&sc->cand_n, 1);
+      if (c < kRankCand) {
+        sc->cand_idx[c] = i;
+        sc->cand_key[c] = order_key(s);
       }
     }
-    __syncthreads();
-    const int n_cand = sc->cand_n;
-    if (n <= kRankFew) {
-      n_mem = n_cand;
-      if (k > n_mem) k = n_mem;
-      if (k <= 0) return 0;
-      all = (k == n_mem);
-    }
-    if (n_cand <= kRankCand) return rank_candidates(n_cand, k, all, delta, out_idx, out_score, sc);
   }
-  // ---- too many candidates (a large k, a crowded bin), or scores that are not finite: radix select and an ordered walk
+  __syncthreads();
+  const int n_cand = sc->cand_n;
+  if (n <= kRankFew) {
+    n_mem = n_cand;
+    if (k > n_mem) k = n_mem;
+    if (k <= 0) return 0;
+    all = (k == n_mem);
+  }
+  if (n_cand <= kRankCand) return rank_candidates(n_cand, k, all, delta, out_idx, out_score, sc);
+  // ---- too many candidates (a large k, a crowded bin): radix select and an ordered walk
   double tau = -1.0e300;                                     // (all: everything is taken)
   __syncthreads();
   if (!all) {
@@ -673,7 +673,6 @@ __device__ __noinline__ int staged_topk_set(const double* scores, const int* cnt
                                             double* out_score, float* buf, RankScratch* sc) {
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nt >> 5;
   int local = 0;
-  bool odd = false;
   const int n4 = (n + 3) & ~3;
   if (tid < n4 - n) buf[n + tid] = kScanAbsent;
   __syncthreads();                                           // (the scratch may still be read from a previous call, too)
@@ -686,7 +685,6 @@ __device__ __noinline__ int staged_topk_set(const double* scores, const int* cnt
       const bool absent = s[u] == kScanAbsent;
       lo = fminf(lo, absent ? INFINITY : s[u]);
       hi = fmaxf(hi, s[u]);
-      odd |= !absent && !(fabsf(s[u]) < 1e30f);
       local += absent ? 0 : 1;
     }
   }
@@ -698,47 +696,45 @@ __device__ __noinline__ int staged_topk_set(const double* scores, const int* cnt
   if (lane == 0) { sc->wmin[warp] = kmin; sc->wmax[warp] = kmax; sc->wcnt[warp] = local; }
   for (int b = tid; b < kRankBins; b += nt) sc->hist[b] = 0u;
   if (tid == 0) sc->cand_n = 0;
-  odd = __syncthreads_or(odd) != 0;
+  __syncthreads();
   const int n_mem = __reduce_add_sync(kFull, lane < nwarp ? sc->wcnt[lane] : 0);
   if (k > n_mem) k = n_mem;
   if (k <= 0) return 0;
   const bool all = (k == n_mem);
-  if (!odd) {
-    const RankBins bin_of = rank_bins(sc, nwarp);
-    int bin = 0;
-    if (!all) {
-      for (int v = tid; v < n4 >> 2; v += nt) {
-        const float4 s = reinterpret_cast<const float4*>(buf)[v];
-        atomicAdd(&sc->hist[bin_of(s.x)], 1u);
-        atomicAdd(&sc->hist[bin_of(s.y)], 1u);
-        atomicAdd(&sc->hist[bin_of(s.z)], 1u);
-        atomicAdd(&sc->hist[bin_of(s.w)], 1u);
-      }
-      __syncthreads();
-      bin = rank_find_bin(k, sc);
-    }
-    // within delta of a score of that bin, and what single precision may have moved (scores of magnitude 1 or less
-    // by 6e-8; the range serves for others)
-    const float span = bin_of.scale > 0.f ? (float)kRankBins / bin_of.scale : 0.f;
-    const float slack = 2.f * (float)delta + 1e-6f * fmaxf(1.f, fmaxf(fabsf(bin_of.lo), fabsf(bin_of.lo + span)));
+  const RankBins bin_of = rank_bins(sc, nwarp);
+  int bin = 0;
+  if (!all) {
     for (int v = tid; v < n4 >> 2; v += nt) {
-      const float4 q = reinterpret_cast<const float4*>(buf)[v];
-      const float s[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (bin_of(s[u] + slack) >= bin && s[u] != kScanAbsent) {
-          const int c = atomicAdd(&sc->cand_n, 1);
-          if (c < kRankCand) sc->cand_idx[c] = 4 * v + u;
-        }
-      }
+      const float4 s = reinterpret_cast<const float4*>(buf)[v];
+      atomicAdd(&sc->hist[bin_of(s.x)], 1u);
+      atomicAdd(&sc->hist[bin_of(s.y)], 1u);
+      atomicAdd(&sc->hist[bin_of(s.z)], 1u);
+      atomicAdd(&sc->hist[bin_of(s.w)], 1u);
     }
     __syncthreads();
-    const int n_cand = sc->cand_n;
-    if (n_cand <= kRankCand) {
-      if (tid < n_cand) sc->cand_key[tid] = order_key(scores[sc->cand_idx[tid]]);
-      __syncthreads();
-      return rank_candidates(n_cand, k, all, delta, out_idx, out_score, sc);
+    bin = rank_find_bin(k, sc);
+  }
+  // within delta of a score of that bin, and what single precision may have moved (scores of magnitude 1 or less
+  // by 6e-8; the range serves for others)
+  const float span = bin_of.scale > 0.f ? (float)kRankBins / bin_of.scale : 0.f;
+  const float slack = 2.f * (float)delta + 1e-6f * fmaxf(1.f, fmaxf(fabsf(bin_of.lo), fabsf(bin_of.lo + span)));
+  for (int v = tid; v < n4 >> 2; v += nt) {
+    const float4 q = reinterpret_cast<const float4*>(buf)[v];
+    const float s[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (bin_of(s[u] + slack) >= bin && s[u] != kScanAbsent) {
+        const int c = atomicAdd(&sc->cand_n, 1);
+        if (c < kRankCand) sc->cand_idx[c] = 4 * v + u;
+      }
     }
+  }
+  __syncthreads();
+  const int n_cand = sc->cand_n;
+  if (n_cand <= kRankCand) {
+    if (tid < n_cand) sc->cand_key[tid] = order_key(scores[sc->cand_idx[tid]]);
+    __syncthreads();
+    return rank_candidates(n_cand, k, all, delta, out_idx, out_score, sc);
   }
   return block_topk_set(ArrScore{scores}, Members{cnt}, n, k, delta, out_idx, out_score, sc);
 }
@@ -828,7 +824,8 @@ __device__ __noinline__ int rank_level(const double* scores, const int* cnt, int
         den = den > 1e-12 ? den : 1e-12;
         gamma = dot / den;
       }
-      sh->s_new[ci] = (1.0 - lambda) * sh->cand_score[ci] + lambda * gamma;
+      const double s1 = sh->cand_score[ci];
+      sh->s_new[ci] = s1 == kScoreNone ? kScoreNone : (1.0 - lambda) * s1 + lambda * gamma;
     }
   }
   __syncthreads();
@@ -911,19 +908,22 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
     // (without a lambda for segments the N = k_seg best are also the result: one ranking serves both)
     const bool same = N == p.k_seg && !(p.lam_seg > 0.0);
     int* top = same ? sh.pick : sh.top;
-    const int n_top = topk_set(ss, nullptr, n_seg, N, p.delta, top, same ? sh.pick_score : (double*)nullptr, seg_buf, &sh.sc);
+    double* top_score = same ? sh.pick_score : sh.cand_score;
+    const int n_top = topk_set(ss, nullptr, n_seg, N, p.delta, top, top_score, seg_buf, &sh.sc);
     if (same) c_seg = n_top;
+    const int n_use = __syncthreads_count(tid < n_top && top_score[tid] != kScoreNone);   // (N <= threads of the block)
     double part = 0.0;
     for (int c = tid; c < C; c += kRankThreads) {
       double t = 0.0;
       for (int i = 0; i < n_top; i += 8) {                   // (eight loads in flight, added in order)
         float x[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) x[u] = i + u < n_top ? p.seg_key[(long long)top[i + u] * C + c] : 0.f;
+        for (int u = 0; u < 8; ++u)
+          x[u] = i + u < n_top && top_score[i + u] != kScoreNone ? p.seg_key[(long long)top[i + u] * C + c] : 0.f;
 #pragma unroll
         for (int u = 0; u < 8; ++u) t += (double)x[u];
       }
-      t = n_top > 0 ? t / (double)n_top : 0.0;
+      t = n_use > 0 ? t / (double)n_use : 0.0;
       gq[c] = t;
       part += t * t;
     }
@@ -935,7 +935,7 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
 #pragma unroll
     for (int w = 0; w < kRankThreads / 32; ++w) gn += sh.gn[w];
     gnorm = sqrt(gn);
-    have_g = n_top > 0;
+    have_g = n_use > 0;
   }
 
   // ---- segments (the paper's lambda for them is 0: final = stage-1 top-k)

@@ -40,3 +40,42 @@ def test_sizes_of_a_retrieval(frames, fseg, n_q, k_seg, k_frm, mode):
         assert frm[i, :n_frm].tolist() == np.asarray(r["frm_idx"]).tolist() and (frm[i, n_frm:] == -1).all()
         ref, _ = O.gather(st, r["frm_idx"])
         assert bits[i][:, :, :n_frm * 4].tobytes() == ref.tobytes()
+
+
+@pytest.mark.parametrize("frames,n_q,k_seg,k_frm,mode", [
+    (60, 3, 2, 3, B.RETR_SEMI),                            # few blocks, all ranked directly
+    (60, 3, 12, 40, B.RETR_SEMI),                          # the segment without a score is among the top N; 60 candidates of 60
+    (300, 9, 70, 4, B.RETR_SEMI),                          # the histogram
+    (300, 2, 3, 8, B.RETR_PARALLEL),
+    (300, 2, 75, 256, B.RETR_HIER),                        # every segment selected
+])
+def test_blocks_and_questions_that_are_not_finite(frames, n_q, k_seg, k_frm, mode):
+    # An Inf among a frame's keys is accepted input (the frame keeps its lowest ids).  Its frame, segment and one patch-level
+    # block have no cosine: they rank last and stay out of the global query.  The last question holds a NaN: no block has a
+    # score for it, the lowest ids are taken.  Ids only: nothing is gathered.
+    wl = dict(spec=SPEC, keep=4, fseg=4, chunk=60, alpha=0.7)
+    run = H.GpuRun(wl, n_frames=frames, want_scores=False, patch_split=2, grid_width=4)
+    st = O.Store(H.oracle_cfg(run.cfg))
+    for t0 in range(0, frames, 60):
+        q, k, v = SPEC.chunk(t0, 60)
+        if t0 == 0:
+            k[0, 9, 2, 1, 5] = 0x7F80
+        run.ctx.mukv_compress_chunk(*(H.to_device(x, True, run.device) for x in (q, k, v)), 60, t0)
+        O.compress_chunk(st, q, k, v)
+    qtok, offs, _ = SPEC.questions(n_q, 1, 6)
+    qtok[offs[n_q - 1], 0, 0] = 0x7FC0
+    dev, i32 = run.device, H.torch.int32
+    k_pat = 2 * k_frm if k_frm < 128 else 256
+    seg, frm, pat = (H.torch.full((n_q, k), -9, dtype=i32, device=dev) for k in (k_seg, k_frm, k_pat))
+    sc = [H.torch.full(x.shape, float("nan"), device=dev) for x in (seg, frm, pat)]
+    counts = H.torch.zeros((n_q, 3), dtype=i32, device=dev)
+    omode = {B.RETR_SEMI: O.MODE_SEMI, B.RETR_PARALLEL: O.MODE_PARALLEL, B.RETR_HIER: O.MODE_HIER}[mode]
+    for lam_seg in (0.0, 0.3):
+        run.ctx.mukv_retrieve3(H.to_device(qtok, True, dev), offs, None,
+                               B.MukvRetrParams(k_pat, k_frm, k_seg, 0.3, 0.3, lam_seg, 0, mode), seg, frm, pat, *sc, counts)
+        for i in range(n_q):
+            r = O.retrieve3(st, qtok[offs[i]:offs[i + 1]], (k_pat, k_frm, k_seg), (0.3, 0.3, lam_seg), 0, omode)
+            for got, score, name, n in zip((seg, frm, pat), sc, ("seg", "frm", "patch"), counts[i].tolist()):
+                ref = np.asarray(r[name + "_idx"]).tolist()
+                assert n == len(ref) and got[i, :n].tolist() == ref and (got[i, n:] == -1).all(), (lam_seg, i, name)
+                H.close(score[i, :n].cpu().numpy(), r[name + "_score"], name)
