@@ -367,13 +367,15 @@ mukv_status mukv_profile_read(mukv_ctx* ctx, double* ms, int64_t* launches);
  * The scratch (about 2 MB: per-head partial sums in float and double, arrival counters, the
  * list of frames that need the double-precision pass, the DFT matrix terms) is a fixed array inside the
  * library; every device that loads the library holds it until the process exits.  The call performs no
- * cudaMalloc / cudaFree and uses no allocating routine.  A bf16 call is scored on the tensor cores and
- * enqueues three kernels on `stream`; an fp32 call one small memset (the counters must start at zero,
- * the rest of the array is overwritten before it is read) and two kernels.  The first call on each device
+ * cudaMalloc / cudaFree and uses no allocating routine.  A call enqueues one small memset on `stream` (counters and
+ * column sums must start at zero; the rest of the array is overwritten before it is read), then a bf16 call, scored on the
+ * tensor cores, three kernels and an fp32 call two.  The first call on each device
  * also looks up the array's device address, copies the matrix terms into it and raises the kernels'
  * shared-memory limit; make that first call outside any stream capture.
  * All calls on a device share the one array: two calls whose kernels may overlap on the device
- * (different streams without an ordering between them) race.  Messages of failures are read
+ * (different streams without an ordering between them) race; what such calls return is undefined, later calls
+ * are not affected.  If a bounded wait inside the tensor-core scoring kernel runs out (codes 3, 4, 5 of mukv_stats; never
+ * seen), every id of the call is -1 and every score NaN.  Messages of failures are read
  * with mukv_last_error(NULL). */
 #define MUKV_NOALLOC_MAX_FRAMES 16
 #define MUKV_NOALLOC_MAX_Q_HEADS 32

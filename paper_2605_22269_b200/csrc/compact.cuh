@@ -616,15 +616,23 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const Compa
   else pool_patches<T>(p, f, &cs);
 }
 
-// Selection alone (scoring without a store): one block per frame, behind the persistent scoring kernel.
-__global__ void __launch_bounds__(kCompactThreads) select_kernel(const CompactParams p) {
+// Selection alone (scoring without a store): one block per frame, behind the persistent scoring kernel.  A code in *scoring
+// (one of that kernel's bounded waits ran out) leaves no sums to trust: the ids are then -1 and the scores NaN.
+__global__ void __launch_bounds__(kCompactThreads) select_kernel(const CompactParams p, const int* scoring) {
   __shared__ SelectScratch ss;
   __shared__ int s_kept[MUKV_MAX_TOKENS];
   pdl_wait();
   pdl_trigger();
-  select_from_partials(p, blockIdx.x, true, s_kept, &ss);
-  // the only reader of the frame's sums leaves them cleared
-  for (int t = threadIdx.x; t < p.sp.P; t += kCompactThreads) p.att_clear[(long long)blockIdx.x * p.sp.P + t] = 0ull;
+  if (*scoring == 0) {
+    select_from_partials(p, blockIdx.x, true, s_kept, &ss);
+    return;
+  }
+  const ScoreParams& sp = p.sp;
+  const long long np = (long long)sp.n_frames * sp.P;
+  for (int t = threadIdx.x; t < sp.P; t += kCompactThreads) {
+    if (t < sp.kappa) sp.kept_store[(long long)blockIdx.x * sp.kappa + t] = -1;
+    for (int s = 0; s < 3 && sp.scores_out; ++s) sp.scores_out[s * np + (long long)blockIdx.x * sp.P + t] = __int_as_float(0x7fffffff);
+  }
 }
 
 // Bounded wait until *ctr reaches `target` (other blocks of the same grid add to it; the grid is

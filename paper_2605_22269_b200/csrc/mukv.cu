@@ -552,7 +552,6 @@ struct PsLaunch {
   const CUtensorMap* pmap;       // stored pages (past keys), or null
   unsigned long long* att_acc;   // [frames][P], zero
   int* status;
-  int* clear;                    // see ScorePsParams
   int kappa;
   bool dependent;
   __nv_bfloat16 *q_terms, *k_terms;   // SPLIT: room for the terms of an fp32 chunk
@@ -597,7 +596,6 @@ cudaError_t launch_score_ps(PsLaunch& l, const ScoreParams& sp, cudaStream_t st,
   pp.n_items = n * pp.ipf;
   pp.exp2_scale = (float)(1.4426950408889634 / std::sqrt((double)D));
   pp.status = l.status;
-  pp.clear = l.clear;
   int blocks = l.n_sms < kPsMaxBlocks ? l.n_sms : kPsMaxBlocks;
   if (blocks > pp.n_items) blocks = pp.n_items;
   *why = "score_ps kernel";
@@ -1455,11 +1453,11 @@ constexpr size_t kNaFftD = kNaColD + (size_t)kNaFrames * kNaHq * kNaP * sizeof(d
 constexpr size_t kNaKept = kNaFftD + (size_t)kNaFrames * kNaHkv * kNaP * sizeof(double);
 constexpr size_t kNaTs = kNaKept + (size_t)kNaFrames * kNaP * sizeof(int);
 constexpr size_t kNaPt = kNaTs + 256;
-constexpr size_t kNaCtrl = kNaPt + 256;                  // frame_counter[16], flagged[16], n_flagged, status
-constexpr size_t kNaCtrlBytes = 256;
-constexpr size_t kNaW128 = kNaCtrl + kNaCtrlBytes;       // DFT matrix terms, D = 128 and D = 64
+constexpr size_t kNaW128 = kNaPt + 256;                  // DFT matrix terms, D = 128 and D = 64
 constexpr size_t kNaW64 = kNaW128 + 3 * 128 * 128 * 2;
-constexpr size_t kNaAtt = kNaW64 + 3 * 64 * 64 * 2;       // column sums of the tensor-core path, zero between calls
+constexpr size_t kNaCtrl = kNaW64 + 3 * 64 * 64 * 2;     // frame_counter[16], flagged[16], n_flagged, status
+constexpr size_t kNaCtrlBytes = 256;
+constexpr size_t kNaAtt = kNaCtrl + kNaCtrlBytes;        // column sums of the tensor-core path: zeroed together with the words
 constexpr size_t kNaTotal = kNaAtt + (size_t)kNaFrames * kNaP * sizeof(unsigned long long);
 
 // In host code this name is only a handle for cudaGetSymbolAddress, never a device address.
@@ -1496,6 +1494,9 @@ cudaError_t noalloc_setup(int dev, const NoallocDevice** out) {
       if (e == cudaSuccess && !encode_map2(D == 128 ? &d.wmap128 : &d.wmap64, dst, D, 3LL * D, D)) e = cudaErrorInvalidValue;
       if (e != cudaSuccess) return e;
     }
+    // (a copy from pageable memory may return before it has arrived, and the caller's stream need not wait for it)
+    e = cudaStreamSynchronize(cudaStreamLegacy);
+    if (e != cudaSuccess) return e;
     d.n_sms = n_sms;
     d.ptr = base;
   }
@@ -1539,15 +1540,17 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
   sp.page_table = reinterpret_cast<long long*>(base + kNaPt);
   sp.refine = 0;
   sp.row_split = 1;
+  // The array keeps what the last call left, be it one that broke off or raced with another: the arrival counters, the flagged
+  // count, the status word and (tensor-core path) the column sums start at zero in every call.
+  e = cudaMemsetAsync(base + kNaCtrl, 0, kNaCtrlBytes + (ts.ok ? (size_t)n * P * sizeof(unsigned long long) : 0), st);
+  if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
   if (ts.ok) {
-    // bf16: scored on the tensor cores like a chunk of a context (16 frames of 196 tokens, 28 heads: 338 us on the
-    // multiply-add kernel, 29.4 us here), then one block per frame selects.  The scoring kernel clears the flagged count.
+    // bf16: scored on the tensor cores like a chunk of a context, then one block per frame selects.
     PsLaunch pl;
     memset(&pl, 0, sizeof pl);
     pl.t = &ts; pl.n_sms = nd->n_sms; pl.wmap = D == 128 ? &nd->wmap128 : &nd->wmap64;
     pl.att_acc = reinterpret_cast<unsigned long long*>(base + kNaAtt);
     pl.status = sp.n_flagged + 1;
-    pl.clear = sp.n_flagged;
     pl.kappa = c.keep_per_frame;
     pl.dependent = true;
     const char* why = "";
@@ -1556,16 +1559,10 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
     CompactParams cp;
     memset(&cp, 0, sizeof cp);
     cp.sp = sp;
-    cp.att_acc = cp.att_clear = pl.att_acc;
-    e = launch_k(select_kernel, dim3(n), kCompactThreads, 0, st, true, cp);
-    if (e != cudaSuccess) {
-      cudaMemsetAsync(base + kNaAtt, 0, kNaTotal - kNaAtt, st);
-      return fail(nullptr, MUKV_E_CUDA, "select kernel: %s", cudaGetErrorString(e));
-    }
+    cp.att_acc = pl.att_acc;
+    e = launch_k(select_kernel, dim3(n), kCompactThreads, 0, st, true, cp, (const int*)pl.status);
+    if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "select kernel: %s", cudaGetErrorString(e));
   } else {
-    // the array keeps what the last call left: the arrival counters and the flagged count start at zero
-    e = cudaMemsetAsync(base + kNaCtrl, 0, kNaCtrlBytes, st);
-    if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
     e = launch_score<T, float>(sp, nc, dim3(c.n_q_heads, n), score_smem_bytes<T, float>(P, D), st);
     if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "score kernel: %s", cudaGetErrorString(e));
   }

@@ -77,7 +77,6 @@ struct ScorePsParams {
   // SPLIT: slots of the two operand rings, bytes of a key-side slot, rows of one term's plane of queries / keys
   int n_a, n_b, b_slot;
   int term_rows;
-  int* clear;                // word that has to be zero when the next kernel starts, or null
   int* status;
 };
 
@@ -330,10 +329,7 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
   };
   // (A dependent launch: up to here the block may run beside the kernel in front of it in the stream.  The inputs may be
   // that kernel's output, and every write of this kernel follows from a load that is issued here.)
-  if (tid == 0) {
-    pdl_wait();
-    if (cta == 0 && p.clear) *p.clear = 0;
-  }
+  if (tid == 0) pdl_wait();
   if (!SPLIT && tid == 0) {
     const int unit0 = i0 / ipu, x0 = i0 - unit0 * ipu;
     const int g0 = unit0 % Hkv, r0 = unit_row(unit0);

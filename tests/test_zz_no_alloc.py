@@ -84,3 +84,52 @@ def test_noalloc_rejects_what_does_not_fit():
     with pytest.raises(B.MukvError) as e:
         B.mukv_score_frames_noalloc(cfg, x, x, 1, None, None)
     assert e.value.status == -1
+
+
+def _inputs(hq, hkv, d, tokens, n, bf16, seed):
+    spec = H.StreamSpec(seed=seed, n_layers=1, n_q_heads=hq, n_kv_heads=hkv, head_dim=d, tokens_per_frame=tokens, bf16=bf16,
+                        n_outlier=1, n_frames=n, scene_sigma=1.0, frame_sigma=0.5, scene_min=2, scene_max=4)
+    q, k, _ = spec.chunk(0, n)
+    return spec, q, k[0]
+
+
+def _against_oracle(spec, q, k, n, keep, exact=(), **over):
+    """exact: frames that go through the double-precision pass; their scores are the rounded exact ones."""
+    cfg = H.spec_config(spec, dict(keep=keep, fseg=1, chunk=n, alpha=0.7), **over)
+    kept = torch.full((n, keep), -2, dtype=torch.int32, device="cuda:0")
+    sc = torch.full((3, n, spec.tokens_per_frame), -2.0, dtype=torch.float32, device="cuda:0")
+    B.mukv_score_frames_noalloc(cfg, H.to_device(q, spec.bf16), H.to_device(k, spec.bf16), n, kept, sc)
+    kept, sc = kept.cpu().numpy(), sc.cpu().numpy()
+    for f in range(n):
+        ref = O.score_frame(q[f], k[f], float(cfg.alpha), bool(over.get("attn_causal")), bool(over.get("keep_low_freq")))
+        assert kept[f].tolist() == O.select_tokens(ref[2], keep).tolist(), f
+        assert np.abs(sc[2, f] - ref[2]).max() < H.FLAG_MARGIN / 2, f
+        for i in range(3):
+            H.close(sc[i, f], ref[i], f"score[{i}] frame {f}")
+            if f in exact:                                 # (one rounding to float: half a unit in the last place)
+                assert (np.abs(sc[i, f] - ref[i]) <= 2.0 ** -24 * np.abs(ref[i]) + 1e-12).all(), (i, f)
+
+
+def test_noalloc_shapes_back_to_back():
+    # other head sizes, tilings and matrix tables, each behind a call of another shape and length
+    for i, (hq, hkv, d, tokens, n, bf16, over) in enumerate([
+            (8, 8, 64, 130, 1, True, dict(attn_causal=1)),
+            (28, 4, 128, 196, 16, True, dict(keep_low_freq=1)),
+            (8, 8, 64, 130, 16, True, dict(attn_causal=1, keep_low_freq=1)),
+            (2, 1, 64, 17, 5, True, {}),
+            (32, 8, 128, 256, 16, True, {}),
+            (14, 2, 64, 77, 3, False, {}),
+            (14, 2, 64, 77, 16, True, dict(attn_causal=1))]):
+        spec, q, k = _inputs(hq, hkv, d, tokens, n, bf16, 90 + i)
+        _against_oracle(spec, q, k, n, max(1, tokens // 4), **over)
+
+
+@pytest.mark.parametrize("bf16", [True, False])
+@pytest.mark.parametrize("paired", [[3], [0, 5, 9, 15], [0, 1, 2, 5, 15], [0, 1, 2, 4, 5, 6, 8, 10, 12, 14]])
+def test_noalloc_frames_in_double_precision(bf16, paired):
+    # Every token of a paired frame stands there twice, and an odd number is kept: a pair lies across the boundary and the
+    # frame is scored again in double precision.  Up to four such frames of 28 heads share a head between blocks, more do not.
+    spec, q, k = _inputs(28, 4, 128, 196, 16, bf16, 97)
+    for f in paired:
+        q[f, 1::2], k[f, 1::2] = q[f, ::2], k[f, ::2]
+    _against_oracle(spec, q, k, 16, 49, exact=paired)
