@@ -432,6 +432,9 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
     }
   };
   if (warp == 1) {
+    // Behind the wait as well: the kernel in front may be a caller's, start this one early and ask for tensor memory only
+    // then.  A block that held all of it while it waits for that kernel to end would never see it end.
+    pdl_wait();
     __syncwarp();
     tc::tmem_alloc(tc::smem_u32(tmem_slot), 512u);
   }
