@@ -129,10 +129,15 @@ struct ScanParams {
 // The score of a block whose key, or of a question whose pooled vector, holds Inf or NaN: below every cosine and every mix
 // of two.  Every score that is ranked is finite, so that a ranking of n members for k <= n places always fills all k (with a
 // NaN for the k-th largest score no comparison holds and nothing was kept; the ids were then whatever lay in shared memory).
+// (Both tests look at the high words: a comparison of doubles is slow, and these sit in chains that a question waits for.)
 constexpr double kScoreNone = -2.0;
+__device__ __forceinline__ bool no_score(double sc) { return __double2hiint(sc) == (int)0xc0000000; }   // (-2, cosines are above it)
+__device__ __forceinline__ double finite_score(double sc) {
+  return (__double2hiint(sc) & 0x7ff00000) == 0x7ff00000 ? kScoreNone : sc;
+}
 
 __device__ __forceinline__ void scan_store(const ScanParams& sp, int qi, long long row, double sc) {
-  if (!(fabs(sc) < 2.0)) sc = kScoreNone;
+  sc = finite_score(sc);
   if (row < sp.n_frm) {
     sp.s_frm[(long long)qi * sp.frm_stride + row] = sc;
     sp.f_frm[(long long)qi * sp.f_frm_stride + row] = (float)sc;
@@ -825,7 +830,7 @@ __device__ __noinline__ int rank_level(const double* scores, const int* cnt, int
         gamma = dot / den;
       }
       const double s1 = sh->cand_score[ci];
-      sh->s_new[ci] = s1 == kScoreNone ? kScoreNone : (1.0 - lambda) * s1 + lambda * gamma;
+      sh->s_new[ci] = no_score(s1) ? kScoreNone : (1.0 - lambda) * s1 + lambda * gamma;
     }
   }
   __syncthreads();
@@ -911,15 +916,22 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
     double* top_score = same ? sh.pick_score : sh.cand_score;
     const int n_top = topk_set(ss, nullptr, n_seg, N, p.delta, top, top_score, seg_buf, &sh.sc);
     if (same) c_seg = n_top;
-    const int n_use = __syncthreads_count(tid < n_top && top_score[tid] != kScoreNone);   // (N <= threads of the block)
+    const int n_use = __syncthreads_count(tid < n_top && !no_score(top_score[tid]));      // (N <= threads of the block)
+    if (n_use < n_top) {                                     // the list without those that have no score
+      if (tid == 0)
+        for (int i = 0, c = 0; i < n_top; ++i)
+          if (!no_score(top_score[i])) sh.top[c++] = top[i];
+      __syncthreads();
+      top = sh.top;
+    }
     double part = 0.0;
     for (int c = tid; c < C; c += kRankThreads) {
       double t = 0.0;
-      for (int i = 0; i < n_top; i += 8) {                   // (eight loads in flight, added in order)
+      for (int i = 0; i < n_use; i += 8) {                   // (eight loads in flight, added in order)
         float x[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-          x[u] = i + u < n_top && top_score[i + u] != kScoreNone ? p.seg_key[(long long)top[i + u] * C + c] : 0.f;
+          x[u] = i + u < n_use ? p.seg_key[(long long)top[i + u] * C + c] : 0.f;
 #pragma unroll
         for (int u = 0; u < 8; ++u) t += (double)x[u];
       }
