@@ -263,6 +263,9 @@ constexpr float kFlatRatio = 1e-3f;
 // rows of single-precision scores start on 16 bytes
 inline long long pad4(long long n) { return (n + 3) / 4 * 4; }
 
+// the DFT matrix in three bf16 terms, see DftTerms
+constexpr size_t dft_bytes(int D) { return (size_t)3 * D * D * sizeof(uint16_t); }
+
 WorkLayout work_layout(const mukv_config& c) {
   WorkLayout w;
   const size_t F = c.max_frames_per_chunk, P = c.tokens_per_frame;
@@ -296,7 +299,7 @@ WorkLayout work_layout(const mukv_config& c) {
   w.f_seg = off;          off = align_up(off + (size_t)MUKV_MAX_QUESTIONS * pad4(max_segs) * sizeof(float));
   w.f_pat = off;          off = align_up(off + (size_t)MUKV_MAX_QUESTIONS * pad4(c.max_frames * c.patch_split * c.patch_split) *
                                                sizeof(float));
-  w.wtab = off;           off = align_up(off + (ts.ok || ts.split ? (size_t)3 * c.head_dim * c.head_dim * 2 : 0));
+  w.wtab = off;           off = align_up(off + (ts.ok || ts.split ? dft_bytes(c.head_dim) : 0));
   const size_t tf = ts.split ? (size_t)ts.split_frames * Ls * P * 6 : 0;
   w.q_terms = off;        off = align_up(off + tf * c.n_q_heads * c.head_dim);
   w.k_terms = off;        off = align_up(off + tf * C);
@@ -489,27 +492,37 @@ float bf16_val(uint16_t h) {
 // The D-point DFT as a matrix, rows = output column n, columns = input channel d (the layout of
 // a K-major B operand): n <= D/2 holds cos(2 pi n d / D), n > D/2 holds -sin(2 pi (n - D/2) d / D).
 // Each entry is split into three bf16 terms, hi + mid + lo, stored as [3][D][D].
-std::vector<uint16_t> dft_terms(int D) {
-  std::vector<uint16_t> w((size_t)3 * D * D);
-  const double pi = 3.14159265358979323846;
-  for (int n = 0; n < D; ++n)
-    for (int d = 0; d < D; ++d) {
-      const int b = n <= D / 2 ? n : n - D / 2;
-      const int m = (int)(((long long)b * d) % D);
-      const double ang = 2.0 * pi * (double)m / (double)D;
-      const double x = n <= D / 2 ? std::cos(ang) : -std::sin(ang);
-      const uint16_t hi = bf16_rne((float)x);
-      const double r1 = x - (double)bf16_val(hi);
-      const uint16_t mid = bf16_rne((float)r1);
-      const double r2 = r1 - (double)bf16_val(mid);
-      const uint16_t lo = bf16_rne((float)r2);
-      w[((size_t)0 * D + n) * D + d] = hi;
-      w[((size_t)1 * D + n) * D + d] = mid;
-      w[((size_t)2 * D + n) * D + d] = lo;
-    }
-  return w;
-}
+template <int D>
+struct DftTerms {
+  uint16_t w[3 * D * D];
+  DftTerms() {
+    const double pi = 3.14159265358979323846;
+    for (int n = 0; n < D; ++n)
+      for (int d = 0; d < D; ++d) {
+        const int b = n <= D / 2 ? n : n - D / 2;
+        const int m = (int)(((long long)b * d) % D);
+        const double ang = 2.0 * pi * (double)m / (double)D;
+        const double x = n <= D / 2 ? std::cos(ang) : -std::sin(ang);
+        const uint16_t hi = bf16_rne((float)x);
+        const double r1 = x - (double)bf16_val(hi);
+        const uint16_t mid = bf16_rne((float)r1);
+        const double r2 = r1 - (double)bf16_val(mid);
+        w[(0 * D + n) * D + d] = hi;
+        w[(1 * D + n) * D + d] = mid;
+        w[(2 * D + n) * D + d] = bf16_rne((float)r2);
+      }
+  }
+};
 
+// Worked out once per process and head size (for every context: 80 us of mukv_create at D = 64, 300 us at D = 128).
+const uint16_t* dft_terms(int D) {
+  if (D == 64) {
+    static const DftTerms<64> t;
+    return t.w;
+  }
+  static const DftTerms<128> t;
+  return t.w;
+}
 // The pooling of segment entries (Eq. 5 at segment level) for frames first .. first + n - 1.
 SegmentArgs segment_args_of(const mukv_ctx* ctx, long long first, int n) {
   const mukv_config& c = ctx->cfg;
@@ -1105,8 +1118,7 @@ mukv_status create_impl(const mukv_config* cfg, void* d_store, size_t store_byte
     ctx->tail_capacity = per_sm * ctx->n_sms;
   }
   if (e == cudaSuccess && (ctx->tcs.ok || ctx->tcs.split)) {
-    const std::vector<uint16_t> w = dft_terms(D);
-    e = cudaMemcpy(ctx->ws + ctx->wl.wtab, w.data(), w.size() * 2, cudaMemcpyHostToDevice);
+    e = cudaMemcpy(ctx->ws + ctx->wl.wtab, dft_terms(D), dft_bytes(D), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !encode_map2(&ctx->wmap, ctx->ws + ctx->wl.wtab, D, 3LL * D, D)) e = cudaErrorInvalidValue;
     if (e == cudaSuccess && ctx->tcs.ok && cfg->past_frames > 0 &&
         !encode_map_pages(&ctx->pmap, ctx->store + ctx->sl.pages, D, cfg->n_kv_heads, cfg->keep_per_frame, 2 * cfg->n_layers,
@@ -1488,9 +1500,8 @@ cudaError_t noalloc_setup(int dev, const NoallocDevice** out) {
     if (e != cudaSuccess) return e;
     unsigned char* base = static_cast<unsigned char*>(ptr);
     for (int D : {64, 128}) {
-      const std::vector<uint16_t> w = dft_terms(D);
       unsigned char* dst = base + (D == 128 ? kNaW128 : kNaW64);
-      e = cudaMemcpy(dst, w.data(), w.size() * 2, cudaMemcpyHostToDevice);
+      e = cudaMemcpy(dst, dft_terms(D), dft_bytes(D), cudaMemcpyHostToDevice);
       if (e == cudaSuccess && !encode_map2(D == 128 ? &d.wmap128 : &d.wmap64, dst, D, 3LL * D, D)) e = cudaErrorInvalidValue;
       if (e != cudaSuccess) return e;
     }
