@@ -366,49 +366,56 @@ __device__ __noinline__ void compact_segment_plane(const SegmentArgs p, int l, i
   }
 }
 
+// Rows in flight per thread.  With 4 row groups per pass, 5 covers the 49 kept rows of the 7B shape in
+// three trips (20 + 20 + 9) where 4 needs a fourth trip for a single row; the kernel then takes 80
+// registers and three blocks per SM instead of four, which measured faster all the same.
+constexpr int kRowsInFlight = 5;
+
 struct CompactScratch {
-  float red[kCompactThreads * 8];
-  double red64[kCompactThreads * 8];
+  union {
+    struct {
+      float red[kCompactThreads * 8];
+      double red64[kCompactThreads * 8];
+    };
+    struct {                                               // compact_plane_part
+      uint4 rows[kRowsInFlight * kCompactThreads];
+      double sums[kCompactThreads * 4];
+    };
+  };
   int kept[MUKV_MAX_TOKENS];
 };
 
 // Copies the kappa kept rows (ids in sc->kept, ascending) of plane (l, kv) of chunk frame f to the
 // frame's page (planes of kappa rows each, starting at `page`) and writes the plane's frame entry
 // (Eq. 5; zeros for a frame that keeps nothing).  Run by a whole block.
-// NV = 16-byte vectors per row; the block covers 256/NV rows per pass.  With `parts` > 1 the block copies part `part` of
-// the columns only (NV / parts vectors), so that more rows are in flight at a time: see compact_kernel.
+// NV = 16-byte vectors per row; the block covers 256/NV rows per pass.
 template <typename T>
 __device__ inline void compact_plane(const CompactParams& p, int plane, int f, CompactScratch* sc, int kappa,
-                                     unsigned char* page, int part, int parts) {
+                                     unsigned char* page) {
   constexpr int VE = 16 / sizeof(T);
   const int tid = threadIdx.x;
   const int l = plane >> 1, kv = plane & 1;
   const long long f_abs = p.first_frame + f;
   const int C = p.C;
-  const int NV = C / VE / parts;                // vectors per row (power of two, <= 256)
-  const int c_off = part * NV * VE;             // first column
+  const int NV = C / VE;                        // vectors per row (power of two, <= 256)
   const int rows_per_pass = kCompactThreads / NV;
-  const T* src_base = reinterpret_cast<const T*>(kv ? p.v : p.k) + ((long long)l * p.n_frames + f) * p.P * C + c_off;
-  T* dst_base = reinterpret_cast<T*>(page) + (long long)plane * kappa * C + c_off;
+  const T* src_base = reinterpret_cast<const T*>(kv ? p.v : p.k) + ((long long)l * p.n_frames + f) * p.P * C;
+  T* dst_base = reinterpret_cast<T*>(page) + (long long)plane * kappa * C;
   const int c = tid % NV, r0 = tid / NV;
   const bool exact = (l == p.L - 1) && (kv == 0);
   float acc[VE];
   double acc64[VE];
 #pragma unroll
   for (int e = 0; e < VE; ++e) { acc[e] = 0.f; acc64[e] = 0.0; }
-  // Rows in flight per thread.  With 4 row groups per pass, 5 covers the 49 kept rows of the 7B shape in
-  // three trips (20 + 20 + 9) where 4 needs a fourth trip for a single row; the kernel then takes 80
-  // registers and three blocks per SM instead of four, which measured faster all the same.
-  constexpr int kUnroll = 5;
-  for (int r = r0; r < kappa; r += rows_per_pass * kUnroll) {
-    uint4 x[kUnroll];
+  for (int r = r0; r < kappa; r += rows_per_pass * kRowsInFlight) {
+    uint4 x[kRowsInFlight];
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
+    for (int u = 0; u < kRowsInFlight; ++u) {
       const int rr = r + u * rows_per_pass;
       if (rr < kappa) x[u] = ld_stream(src_base + (long long)sc->kept[rr] * C + c * VE);
     }
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
+    for (int u = 0; u < kRowsInFlight; ++u) {
       const int rr = r + u * rows_per_pass;
       if (rr < kappa) {
         st_stream(dst_base + (long long)rr * C + c * VE, x[u]);
@@ -440,19 +447,113 @@ __device__ inline void compact_plane(const CompactParams& p, int plane, int f, C
     for (int i = 0; i < VE; ++i) sc->red[tid * VE + i] = acc[i];
   }
   __syncthreads();
-  float* fe = p.frame_entry + ((f_abs * p.L + l) * 2 + kv) * C + c_off;
-  for (int col = tid; col < NV * VE; col += kCompactThreads) {
+  float* fe = p.frame_entry + ((f_abs * p.L + l) * 2 + kv) * C;
+  for (int col = tid; col < C; col += kCompactThreads) {
     const int cv = col / VE, ce = col % VE;
     if (exact) {
       double t = 0.0;
       for (int g = 0; g < rows_per_pass; ++g) t += sc->red64[(g * NV + cv) * VE + ce];
+      p.frame_ksum[f_abs * C + col] = t;
+      const float m = kappa ? (float)(t / (double)kappa) : 0.f;
+      fe[col] = m;
+      p.frame_key[f_abs * C + col] = m;
+    } else {
+      float t = 0.f;
+      for (int g = 0; g < rows_per_pass; ++g) t += sc->red[(g * NV + cv) * VE + ce];
+      fe[col] = kappa ? t / (float)kappa : 0.f;
+    }
+  }
+}
+
+// The same for part `part` of `parts` (2 or 4) of the plane's columns: NV = C / VE / parts vectors per row, parts times the rows
+// per pass, which takes short calls from three round trips of rows to one or two (see compact_kernel).  The rows of a trip
+// go through shared memory and are added up in the order of compact_plane (256 / (C / VE) groups of rows, each ascending,
+// then the groups), so that a frame's entry is the same bit for bit however the stream is cut into calls.  (Adding them up in
+// the order of the copy was 0.6 us of 18 faster in a one-frame call; a thread per vector of 256 / parts threads, 13 rows each
+// in flight, 9 us slower: two warps then fetch all the code.)
+template <typename T>
+__device__ inline void compact_plane_part(const CompactParams& p, int plane, int f, CompactScratch* sc, int kappa,
+                                          unsigned char* page, int part, int parts) {
+  constexpr int VE = 16 / sizeof(T), WE = VE / 2;          // elements per vector, per half of one
+  const int tid = threadIdx.x;
+  const int l = plane >> 1, kv = plane & 1;
+  const long long f_abs = p.first_frame + f;
+  const int C = p.C;
+  const int NV = C / VE / parts, c_off = part * NV * VE;
+  const int groups = kCompactThreads / (C / VE), rows_per_pass = groups * parts;
+  const T* src_base = reinterpret_cast<const T*>(kv ? p.v : p.k) + ((long long)l * p.n_frames + f) * p.P * C + c_off;
+  T* dst_base = reinterpret_cast<T*>(page) + (long long)plane * kappa * C + c_off;
+  const int c = tid % NV, r0 = tid / NV;
+  const bool exact = (l == p.L - 1) && (kv == 0);
+  // sums: thread (row group, half vector)
+  const int halves = 2 * kCompactThreads / parts;          // of a group of rows
+  const int g = tid / (2 * NV);
+  float acc[WE];
+  double acc64[WE];
+#pragma unroll
+  for (int e = 0; e < WE; ++e) { acc[e] = 0.f; acc64[e] = 0.0; }
+  const uint2* half = reinterpret_cast<const uint2*>(sc->rows);
+  auto elem = [](const uint2& x, int e) {
+    const uint32_t w = WE == 4 ? (e < 2 ? x.x : x.y) : (e == 0 ? x.x : x.y);
+    return WE == 4 ? ((e & 1) ? bf16_hi(w) : bf16_lo(w)) : __uint_as_float(w);
+  };
+  for (int base = 0; base < kappa; base += rows_per_pass * kRowsInFlight) {
+    uint4 x[kRowsInFlight];
+#pragma unroll
+    for (int u = 0; u < kRowsInFlight; ++u) {
+      const int rr = base + u * rows_per_pass + r0;
+      if (rr < kappa) x[u] = ld_stream(src_base + (long long)sc->kept[rr] * C + c * VE);
+    }
+    if (base) __syncthreads();                             // the previous trip's rows have been added
+#pragma unroll
+    for (int u = 0; u < kRowsInFlight; ++u) {
+      const int rr = base + u * rows_per_pass + r0;
+      if (rr < kappa) {
+        st_stream(dst_base + (long long)rr * C + c * VE, x[u]);
+        sc->rows[u * kCompactThreads + tid] = x[u];
+      }
+    }
+    __syncthreads();
+    const int n = min(kappa - base, rows_per_pass * kRowsInFlight);
+    if (tid < halves) {
+      if (exact) {
+        for (int r = g, o = tid; r < n; r += groups, o += halves) {
+          const uint2 y = half[o];
+#pragma unroll
+          for (int e = 0; e < WE; ++e) acc64[e] += (double)elem(y, e);
+        }
+      } else {
+#pragma unroll 4
+        for (int r = g, o = tid; r < n; r += groups, o += halves) {
+          const uint2 y = half[o];
+#pragma unroll
+          for (int e = 0; e < WE; ++e) acc[e] += elem(y, e);
+        }
+      }
+    }
+  }
+  float* sums = reinterpret_cast<float*>(sc->sums);        // [groups][NV * VE]
+  if (tid < halves) {
+#pragma unroll
+    for (int e = 0; e < WE; ++e) {
+      if (exact) sc->sums[tid * WE + e] = acc64[e];
+      else sums[tid * WE + e] = acc[e];
+    }
+  }
+  __syncthreads();
+  const int cols = NV * VE;
+  float* fe = p.frame_entry + ((f_abs * p.L + l) * 2 + kv) * C + c_off;
+  for (int col = tid; col < cols; col += kCompactThreads) {
+    if (exact) {
+      double t = 0.0;
+      for (int g = 0; g < groups; ++g) t += sc->sums[g * cols + col];
       p.frame_ksum[f_abs * C + c_off + col] = t;
       const float m = kappa ? (float)(t / (double)kappa) : 0.f;
       fe[col] = m;
       p.frame_key[f_abs * C + c_off + col] = m;
     } else {
       float t = 0.f;
-      for (int g = 0; g < rows_per_pass; ++g) t += sc->red[(g * NV + cv) * VE + ce];
+      for (int g = 0; g < groups; ++g) t += sums[g * cols + col];
       fe[col] = kappa ? t / (float)kappa : 0.f;
     }
   }
@@ -612,8 +713,9 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const Compa
     __syncthreads();
   }
   if (risky) return;
-  if (plane < 2 * p.L) compact_plane<T>(p, plane, f, &cs, kappa_f, page, part, p.parts);
-  else pool_patches<T>(p, f, &cs);
+  if (plane >= 2 * p.L) pool_patches<T>(p, f, &cs);
+  else if (p.parts == 1) compact_plane<T>(p, plane, f, &cs, kappa_f, page);
+  else compact_plane_part<T>(p, plane, f, &cs, kappa_f, page, part, p.parts);
 }
 
 // Selection alone (scoring without a store): one block per frame, behind the persistent scoring kernel.  A code in *scoring
@@ -708,7 +810,7 @@ __global__ void __launch_bounds__(kScoreThreads, 2) tail_kernel(const ScoreParam
         __syncthreads();
         for (int r = tid; r < p.kappa; r += kCompactThreads) cs.kept[r] = token_id(__ldcg(sp.kept_store + f_abs * p.kappa + r), p.P);
         __syncthreads();
-        if (plane < 2 * p.L) compact_plane<T>(p, plane, f, &cs, p.kappa, p.store + sp.pages_off + f_abs * sp.page_bytes, 0, 1);
+        if (plane < 2 * p.L) compact_plane<T>(p, plane, f, &cs, p.kappa, p.store + sp.pages_off + f_abs * sp.page_bytes);
         else pool_patches<T>(p, f, &cs);
       }
       if (plane >= 2 * p.L) continue;

@@ -383,3 +383,20 @@ def test_stream_1h():
     assert H.to_numpy_bits(dec)[0].tobytes() == ref_dec.tobytes()
     assert meta.cpu().numpy()[0][:, 1].tolist() == ref_meta[:, 1].tolist()
     assert meta.cpu().numpy()[0][:, 0].tolist() == np.repeat(frm, cfg.keep_per_frame).tolist()
+
+
+@pytest.mark.parametrize("kv_heads,head_dim,keep,bf16", [(4, 128, 49, True), (4, 128, 49, False), (8, 64, 33, True), (2, 64, 16, False)])
+def test_entries_do_not_depend_on_how_the_stream_is_cut(kv_heads, head_dim, keep, bf16):
+    # short calls share a plane's columns among several blocks, calls that flag a frame redo it in another kernel: pages, ids,
+    # frame and segment entries and keys are the same bit for bit
+    spec = StreamSpec(seed=83, n_layers=5, n_q_heads=2 * kv_heads, n_kv_heads=kv_heads, head_dim=head_dim, tokens_per_frame=196,
+                      bf16=bf16, n_outlier=1, n_frames=16, scene_sigma=1.0, frame_sigma=0.5, scene_min=2, scene_max=4)
+    wl = dict(spec=spec, keep=keep, fseg=5, chunk=16, alpha=0.7)
+    got = []
+    for chunk, margin in ((16, None), (1, None), (5, None), (16, 4.0)):
+        run = H.GpuRun(wl, options=None if margin is None else {B.OPT_FLAG_MARGIN: margin}).compress(chunk)
+        got.append([run.ctx.region(i) for i in (0, 1, 2, 3, 4, 5)])
+        assert run.ctx.mukv_get_stats().refined_frames == (16 if margin else 0)
+    for other in got[1:]:
+        for x, y in zip(other, got[0]):
+            assert torch.equal(x, y)
