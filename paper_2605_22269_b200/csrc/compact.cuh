@@ -127,9 +127,9 @@ __device__ inline bool select_from_partials(const CompactParams& p, int f, bool 
         for (int i = 0; i < w; ++i) y[i] += y[i + w];
       f32 += y[0];
     }
-    const float a32 = att_value(a64);
-    att = a32 * (1.f / (float)((long long)sp.Hq * sp.Ls * P));
-    fft = f32 * (1.f / (float)((long long)Hkv * sp.D));
+    // (divisions: a rounded reciprocal would shift all scores of a frame alike, I_att of 28 heads x 196 tokens by 4e-8)
+    att = att_value(a64) / (float)((long long)sp.Hq * sp.Ls * P);
+    fft = f32 / (float)((long long)Hkv * sp.D);
   }
   // ---- min / max of both signals over the frame (both are sums of non-negative terms)
   {
