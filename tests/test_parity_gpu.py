@@ -190,8 +190,8 @@ def test_chunk7b_causal():
 
 @pytest.mark.parametrize("chunk", [1, 3])
 def test_chunk7b_small_chunks(chunk):
-    # a one-frame chunk spreads a frame over 52 scoring blocks (more partial sums than the selection
-    # loads in one batch); three-frame chunks leave block shares that straddle frames
+    # a one-frame chunk spreads a frame over 52 scoring blocks, which all add to its column sums;
+    # three-frame chunks leave block shares that straddle frames
     run = H.GpuRun("chunk7b", n_frames=4)
     full_compress_check(run, chunk=chunk)
     assert run.ctx.mukv_get_stats().device_status == 0
