@@ -46,7 +46,7 @@ struct WorkLayout {
   size_t zero_begin, zero_end;          // region that must start as zeros
 };
 
-// Tiling of the tensor-core scoring kernel (bf16 inputs only).
+// Tiling of the tensor-core scoring kernel.
 struct TcShape {
   bool ok;                 // bf16 chunk scored on the tensor cores (every supported bf16 shape fits)
   int tpt, tiles, npad, n_mt, ps_stages;
@@ -236,7 +236,8 @@ TcShape tc_shape(const mukv_config& c) {
   if (c.dtype != MUKV_BF16) {
     // fp32: frame-level selection without past keys.  (Segment-level selection ranks fp32 chunks in double precision,
     // and past keys are stored as fp32 rows.)  The terms of a call take 6 bytes per value of the scoring layers' queries
-    // and keys, 4.8 MB per frame of 28 x 196 x 128 queries; longer chunks than fit 256 MB keep the multiply-add kernel.
+    // and keys, 4.8 MB per frame of 28 x 196 x 128 queries.  256 MB is what a workspace is given for them (a choice, not a
+    // measurement: 55 such frames); longer calls keep the multiply-add kernel, about five times slower.
     if (c.past_frames > 0 || c.keep_per_segment > 0) return t;
     const long long ls = c.n_score_layers > 1 ? c.n_score_layers : 1;
     const long long per_frame = 6LL * ls * c.tokens_per_frame * (c.n_q_heads + c.n_kv_heads) * c.head_dim;
@@ -523,6 +524,7 @@ const uint16_t* dft_terms(int D) {
   static const DftTerms<128> t;
   return t.w;
 }
+
 // The pooling of segment entries (Eq. 5 at segment level) for frames first .. first + n - 1.
 SegmentArgs segment_args_of(const mukv_ctx* ctx, long long first, int n) {
   const mukv_config& c = ctx->cfg;
@@ -540,7 +542,7 @@ SegmentArgs segment_args_of(const mukv_ctx* ctx, long long first, int n) {
 
 // A compress call does not pool the segment entries of its chunk itself (unless frames were flagged:
 // tail_kernel then does): the next compress call does it with blocks that do not wait for that call's
-// scoring kernel (one more row in its compaction kernel; with segment-level selection, extra blocks of its
+// scoring kernel (more rows in its compaction kernel, one plane per block; with segment-level selection, extra blocks of its
 // first segsel_kernel launch).  Whoever else needs the entries first
 // (retrieval, a gather with summary tokens, a view of the store, an export) pools them with one launch here.
 cudaError_t flush_segments(const mukv_ctx* ctx, cudaStream_t st) {
@@ -570,7 +572,7 @@ struct PsLaunch {
   __nv_bfloat16 *q_terms, *k_terms;   // SPLIT: room for the terms of an fp32 chunk
 };
 
-// Scores a bf16 chunk on the tensor cores (Eq. 1-3; Eq. 4 and the selection follow in compact_kernel).
+// Scores a chunk on the tensor cores (Eq. 1-3; Eq. 4 and the selection follow in compact_kernel).
 cudaError_t launch_score_ps(PsLaunch& l, const ScoreParams& sp, cudaStream_t st, const char** why) {
   const TcShape& t = *l.t;
   const int P = sp.P, D = sp.D, n = sp.n_frames;

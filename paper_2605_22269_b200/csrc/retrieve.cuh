@@ -5,10 +5,13 @@
 // questions, tiny next to the gather, and it makes the selected indices independent of
 // summation order.  Kernels:
 //   qpool_kernel    Eq. 6   one block per (question, key head)
-//   scan_kernel     Eq. 7   cosine of every question with every frame key and segment key (a skinny
+//   scan_kernel     Eq. 7   cosine of every question with every frame, segment and patch-level key (a skinny
 //                           double-precision product on the fp64 tensor-core instruction)
-//   rank_kernel     stage-1 candidates, Eq. 8 rerank, final top-k; one block per question
+//   scan_few_kernel         the same for at most eight questions, a warp per row or two
+//   rank_kernel     stage-1 candidates, Eq. 8 rerank, final top-k; one block per question, a second one for its
+//                   patch-level blocks
 //   gather_kernel   Eq. 9   copies the selected pages into the per-question decode buffers
+//   gather3_kernel          the same with summary tokens and the rows of patch-level blocks
 #pragma once
 #include "common.cuh"
 #include "tc.cuh"
@@ -375,10 +378,6 @@ __device__ __forceinline__ unsigned order_key32(float x) {
 }
 __device__ __forceinline__ float order_key32_inv(unsigned k) { return __uint_as_float((k >> 31) ? (k & 0x7fffffffu) : ~k); }
 
-// Indices of the k highest scores among i in [0,n) with member(i) true, ascending by index, with
-// the tie band: tau = k-th largest; scores above tau+delta are taken; those within delta of tau
-// share the remaining places by lowest index.  Run by the whole block; returns the count
-// (= min(k, number of members)).  score(i) must be cheap and pure.
 // score(i) read from an array; every index a member.  One pair of types for the selections over
 // segments, frames and candidates, so that they share one copy of block_topk_set (kept out of
 // line: the ranking kernel is bound by instruction fetch, not by arithmetic).
@@ -492,6 +491,10 @@ __device__ __forceinline__ int rank_find_bin(int k, RankScratch* sc) {
   return sc->bin;
 }
 
+// Indices of the k highest scores among i in [0,n) with member(i) true, ascending by index, with
+// the tie band: tau = k-th largest; scores above tau+delta are taken; those within delta of tau
+// share the remaining places by lowest index.  Run by the whole block; returns the count
+// (= min(k, number of members)).  score(i) must be cheap, pure and finite.
 template <typename ScoreFn, typename MemberFn>
 __device__ __noinline__ int block_topk_set(ScoreFn score, MemberFn member, int n, int k, double delta, int* out_idx,
                               double* out_score, RankScratch* sc) {
@@ -1028,7 +1031,7 @@ struct GatherParams {
 // run of the decode buffer.  Bound by memory.  One block per unit: with eight blocks per SM that walked the units the blocks
 // drifted apart, and 64 questions (5.75 GB, 57,344 runs of 50 KB) took 1,002 us; blocks that start in the order of the
 // units keep to neighbouring pages: 867 us with 256 threads, 855 with 512 (two thirds as many runs open at a time; 128
-// threads: 904), 6.7 TB/s.  Runs below 16 KB would leave 512 threads idle and take 128.  (A ring of bulk copies through
+// threads: 904), 6.7 TB/s of algorithmic bytes; where two questions share a page its second reader finds it in L2.  Runs below 16 KB would leave 512 threads idle and take 128.  (A ring of bulk copies through
 // shared memory: 961 us.)
 template <int NT>
 __global__ void __launch_bounds__(NT) gather_kernel(const GatherParams p) {

@@ -56,9 +56,9 @@ struct ScoreParams {
   int no_select;                // 1: only the partial sums are wanted (the selection runs over a whole segment elsewhere)
   int refine;                   // 1: frames come from the flagged list, no further flagging
   int row_split;                // blocks that share a query head, each a range of query rows (>= 1)
-  // double-precision pass with room for the partial sums of `scratch_units` / (Ls * Hq) frames only: they are indexed by
-  // the place in the flagged list, and a head is split over row_split blocks while that fits, else not split; 0: one
-  // place per frame of the chunk
+  // score_kernel's double-precision pass: room for the partial sums of that many (frame, head, part) units.  They are
+  // indexed by the place in the flagged list, and a head is split over row_split blocks while that fits, else not split.
+  // (tail_kernel has one place per frame of the chunk and does not look at this.)
   int scratch_units;
   // segment-level selection, double-precision pass: only the frames of segments whose word is non-zero
   // are scored (segment of chunk frame f: f / gate_fseg); null: every frame
