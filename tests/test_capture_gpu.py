@@ -51,3 +51,32 @@ def test_replays_of_a_captured_stream(calls, bf16, over):
             for x, y in zip(outs, first):
                 assert torch.equal(x, y)
     assert ctx.mukv_get_stats().device_status == 0
+
+
+@pytest.mark.parametrize("bf16", [True, False])
+def test_replays_of_scoring_without_a_workspace(bf16):
+    # (the first call on a device is made outside the capture); a call of another length between two replays leaves its own scratch
+    spec = StreamSpec(seed=82, n_layers=1, n_q_heads=8, n_kv_heads=2, head_dim=64, tokens_per_frame=40, bf16=bf16, n_outlier=1,
+                      n_frames=5, scene_sigma=1.0, frame_sigma=0.5, scene_min=2, scene_max=4)
+    run = H.GpuRun(dict(spec=spec, keep=10, fseg=4, chunk=5, alpha=0.7))
+    q, k, _ = run.gs.chunk(0, 5)
+    kept = torch.full((5, 10), -1, dtype=torch.int32, device=run.device)
+    scores = torch.zeros((3, 5, 40), device=run.device)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        def call(n):
+            B.mukv_score_frames_noalloc(run.cfg, q, k[0], n, kept, scores)
+        call(5)
+        side.synchronize()
+        first = [kept.clone(), scores.clone()]
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side):
+            call(5)
+        for _ in range(3):
+            call(2)
+            kept.fill_(-1)
+            scores.zero_()
+            graph.replay()
+            side.synchronize()
+            assert torch.equal(kept, first[0]) and torch.equal(scores, first[1])
