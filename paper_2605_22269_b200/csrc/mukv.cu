@@ -1555,7 +1555,8 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
   sp.refine = 0;
   sp.row_split = 1;
   // The array keeps what the last call left, be it one that broke off or raced with another: the arrival counters, the flagged
-  // count, the status word and (tensor-core path) the column sums start at zero in every call.
+  // count, the status word and (tensor-core path) the column sums start at zero in every call.  (2.6 us of 30.7 for sixteen
+  // frames of 28 heads x 196 tokens; left clean by the call before, they cost nothing and could be spoilt for good.)
   e = cudaMemsetAsync(base + kNaCtrl, 0, kNaCtrlBytes + (ts.ok ? (size_t)n * P * sizeof(unsigned long long) : 0), st);
   if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
   if (ts.ok) {
