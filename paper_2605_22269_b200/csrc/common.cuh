@@ -33,32 +33,33 @@ template <> __device__ __forceinline__ float elem_to_float<__nv_bfloat16>(__nv_b
 }
 
 // acc += q.k over the elements packed in one 32-bit word
-template <typename T, typename A> __device__ __forceinline__ A dot_word(uint32_t q, uint32_t k, A acc);
-template <> __device__ __forceinline__ float dot_word<__nv_bfloat16, float>(uint32_t q, uint32_t k, float acc) {
+template <typename T> __device__ __forceinline__ float dot_word(uint32_t q, uint32_t k, float acc);
+template <> __device__ __forceinline__ float dot_word<__nv_bfloat16>(uint32_t q, uint32_t k, float acc) {
   acc = fmaf(bf16_lo(q), bf16_lo(k), acc);
   return fmaf(bf16_hi(q), bf16_hi(k), acc);
 }
-template <> __device__ __forceinline__ double dot_word<__nv_bfloat16, double>(uint32_t q, uint32_t k, double acc) {
-  acc = fma((double)bf16_lo(q), (double)bf16_lo(k), acc);
-  return fma((double)bf16_hi(q), (double)bf16_hi(k), acc);
-}
-template <> __device__ __forceinline__ float dot_word<float, float>(uint32_t q, uint32_t k, float acc) {
+template <> __device__ __forceinline__ float dot_word<float>(uint32_t q, uint32_t k, float acc) {
   return fmaf(__uint_as_float(q), __uint_as_float(k), acc);
 }
-template <> __device__ __forceinline__ double dot_word<float, double>(uint32_t q, uint32_t k, double acc) {
-  return fma((double)__uint_as_float(q), (double)__uint_as_float(k), acc);
+
+// C += A B on the double-precision tensor-core instruction, 8 x 8 x 4: lane l holds A[l / 4][l % 4], B[l % 4][l / 4] and
+// C[l / 4][2 (l % 4)], C[l / 4][2 (l % 4) + 1].  Measured: 64 multiply-adds per clock and SM, as its larger shapes and as
+// plain double-precision multiply-adds, with a quarter of the operands to fetch and convert.
+__device__ __forceinline__ void dmma_m8n8k4(double (&c)[2], double a, double b) {
+  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
+               : "+d"(c[0]), "+d"(c[1])
+               : "d"(a), "d"(b));
 }
 
-// ---------------------------------------------------------------- math in the accumulation type
-__device__ __forceinline__ float exp_acc(float x) { return expf(x); }
-__device__ __forceinline__ double exp_acc(double x) { return exp(x); }
-__device__ __forceinline__ float fma_acc(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double fma_acc(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float sqrt_acc(float x) { return sqrtf(x); }
-__device__ __forceinline__ double sqrt_acc(double x) { return sqrt(x); }
-template <typename A> __device__ __forceinline__ A neg_inf();
-template <> __device__ __forceinline__ float neg_inf<float>() { return -INFINITY; }
-template <> __device__ __forceinline__ double neg_inf<double>() { return -(double)INFINITY; }
+// order-preserving bits of a double and back
+__device__ __forceinline__ unsigned long long order_key(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
+}
+__device__ __forceinline__ double order_key_inv(unsigned long long k) {
+  const unsigned long long b = (k >> 63) ? (k & 0x7fffffffffffffffull) : ~k;
+  return __longlong_as_double((long long)b);
+}
 
 // ---------------------------------------------------------------- warp / block reductions
 template <typename A> __device__ __forceinline__ A warp_sum(A v) {

@@ -15,13 +15,12 @@
 // whole device, where a selection inside the scoring kernel left one block per frame working while
 // all others had finished.  After the other scoring kernels the ids are read from the store
 // (sel_mode 0).  Either way a frame whose lowest kept and highest dropped score are closer than
-// tie_eps + flag_margin is skipped here: tail_kernel decides it in double precision and compacts it.
+// tie_eps + flag_margin is skipped here: redo_flagged decides it in double precision and compacts it.
 //
-// What has to wait for every frame of the chunk:
-// tail_kernel<T, NC>, launched behind compact_kernel: returns at once unless frames were flagged (about
-// one chunk in fifty on the synthetic streams); then all its blocks first score those frames in double
-// precision and select; once every block has finished that, the flagged frames are compacted and then
-// the segment entries written, one plane per block.
+// Flagged frames (about one chunk in fifty on the synthetic streams): redo_flagged.  Blocks behind those of the copies (bf16
+// calls; p.redo_blocks of them) wait until the ids of every frame of the chunk are published or the frame is on the list, and
+// leave if the list is empty; else they score its frames in double precision (score64.cuh), and when the selections have all been
+// made they compact those frames.  fp32 calls have tail_kernel<T> for it, a launch behind compact_kernel.
 // The segment entries (Eq. 5 at segment level; one (layer, K|V) plane per block, mean over the frames
 // present) of the common case are not written by the call itself.  The next call pools them with a row
 // of compact_kernel blocks that does not wait for its scoring kernel (CompactParams::prev), or the first
@@ -30,12 +29,12 @@
 // then needs before it signs off costs more than a launch.)
 #pragma once
 #include "common.cuh"
-#include "score.cuh"
+#include "score64.cuh"
 
 namespace mukv {
 
 constexpr int kCompactThreads = 256;
-static_assert(kCompactThreads == kScoreThreads, "tail_kernel runs the scoring and the compaction code in one block");
+static_assert(kCompactThreads == kScoreThreads, "redo_flagged runs the scoring and the compaction code in one block");
 
 struct CompactParams {
   int L, kappa, C, P;             // C = Hkv*D elements per row
@@ -49,7 +48,9 @@ struct CompactParams {
   double* frame_ksum;             // [max_frames][C]  exact sums of the last-layer kept keys
   long long* stat_refined;        // device counter
   int* n_flagged_next;            // the flagged count of the next chunk (the two chunks' counts alternate)
-  int* tail_ctr;                  // [2] tail_kernel: blocks done with the double-precision scores / with everything
+  int* tail_ctr;                  // [2] redo_flagged: blocks done with the double-precision scores / with everything
+  int redo_blocks;                // compact_kernel: blocks at the end of the grid that redo flagged frames (0: none)
+  double *colsum_d, *ifft_d;      // their partial sums, see score64_frame_block
   // segment entries (Eq. 5 at segment level)
   int fseg;                       // frames per segment
   float* seg_entry;               // [max_segs][L][2][C]
@@ -59,7 +60,6 @@ struct CompactParams {
   int patch_split, grid_width;    // 0: no patch level
   float* patch_key;               // [max_frames][S][C]
   int* patch_cnt;                 // [max_frames][S]
-  int pool_always;                // segment_kernel: pool whatever the flagged count says (the entries of an earlier call)
   // compact_kernel: with prev.n_frames > 0 the grid has prev_rows more rows of blocks (behind the first one), which
   // pool the segment entries the previous call left to this one.  prev_rows = ceil(2L / n_frames), one (layer, K|V)
   // plane per block: a plane is a chain of L2 round trips of about 5 us, so that a single row of n_frames blocks
@@ -381,6 +381,7 @@ struct CompactScratch {
       uint4 rows[kRowsInFlight * kCompactThreads];
       double sums[kCompactThreads * 4];
     };
+    Score64Scratch s64;                                    // redo_flagged
   };
   int kept[MUKV_MAX_TOKENS];
 };
@@ -628,8 +629,81 @@ __device__ __forceinline__ bool frame_is_flagged(const int* flagged, int n, int 
   return hit;
 }
 
+// Bounded wait until done() holds (other blocks of the same grid bring it about).  False after about 1.5 s.
+template <typename Done>
+__device__ __forceinline__ bool wait_until(Done done) {
+  unsigned long long t0 = 0;
+  for (long long spin = 0;; ++spin) {
+    if (done()) return true;
+    if ((spin & 63) == 63) {
+      unsigned long long now;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+      if (t0 == 0) t0 = now;
+      else if (now - t0 > 1500000000ull) return false;
+    }
+    __nanosleep(100);
+  }
+}
+
+constexpr int kStatusTailWait = 6;   // the wait for another block's ids or double-precision scores ran out
+
+// The flagged frames of a call: block e of `blocks` that run this (no more than are resident at once, see mukv_create: they
+// wait for one another).
 template <typename T>
-__global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const CompactParams p) {
+__device__ __noinline__ void redo_flagged(const CompactParams& p, int e, int blocks, CompactScratch* cs) {
+  __shared__ int s_ok;
+  const ScoreParams& sp = p.sp;
+  const int tid = threadIdx.x;
+  const int n_fl = *reinterpret_cast<volatile int*>(sp.n_flagged);
+  // ---- scores in double precision; the block that finishes a frame last selects
+  const int heads = sp.Ls * sp.Hq, rs = score64_split(n_fl, heads, sp.P, blocks, sp.scratch_rows), units = heads * rs;
+  for (int w = e; w < n_fl * units; w += blocks) {
+    const int slot = w / units, u = w % units;
+    score64_frame_block<T>(sp, p.colsum_d, p.ifft_d, u / rs, u % rs, rs, __ldcg(sp.flagged + slot), slot, &cs->s64);
+    __syncthreads();
+  }
+  // ---- every block waits for all selections
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) {
+    atomicAdd(p.tail_ctr, 1);
+    const volatile int* ctr = p.tail_ctr;
+    s_ok = wait_until([&] { return *ctr >= blocks; }) ? 1 : 0;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!s_ok) {
+    if (tid == 0 && sp.status) atomicCAS(sp.status, 0, kStatusTailWait);
+  } else {
+    // ---- the flagged frames' compaction, plane by plane; two blocks share one by columns while there are enough
+    const int parts = n_fl * 4 * p.L <= blocks && p.C * (int)sizeof(T) >= 512 ? 2 : 1;
+    const int per = 2 * p.L * parts + (p.patch_split > 0 ? 1 : 0);
+    for (int u = e; u < n_fl * per; u += blocks) {
+      const int f = __ldcg(sp.flagged + u / per), x = u % per;
+      const long long f_abs = p.first_frame + f;
+      unsigned char* page = p.store + sp.pages_off + f_abs * sp.page_bytes;
+      __syncthreads();
+      for (int r = tid; r < p.kappa; r += kCompactThreads) cs->kept[r] = token_id(__ldcg(sp.kept_store + f_abs * p.kappa + r), p.P);
+      __syncthreads();
+      if (x >= 2 * p.L * parts) pool_patches<T>(p, f, cs);
+      else if (parts == 1) compact_plane<T>(p, x, f, cs, p.kappa, page);
+      else compact_plane_part<T>(p, x >> 1, f, cs, p.kappa, page, x & 1, 2);
+    }
+  }
+  // ---- the block that leaves last resets the counters and adds to the statistics
+  __syncthreads();
+  if (tid == 0) {
+    const int old = atomicAdd(p.tail_ctr + 1, 1);
+    if (old == blocks - 1) {
+      *p.stat_refined += n_fl;
+      p.tail_ctr[0] = 0;
+      p.tail_ctr[1] = 0;
+    }
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __grid_constant__ CompactParams p) {
   __shared__ CompactScratch cs;
   __shared__ SelectScratch ss;
   __shared__ unsigned s_seen;
@@ -650,6 +724,31 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const Compa
       return;
     }
     if (row > p.prev_rows) row -= p.prev_rows;
+  }
+  if constexpr (sizeof(T) == 2) {
+    const int first = 2 * p.L * p.parts + (p.patch_split > 0 ? 1 : 0);     // row of the first block for flagged frames
+    if (p.redo_blocks > 0 && row >= first) {
+      const int e = (row - first) * gridDim.x + blockIdx.x;
+      if (e >= p.redo_blocks) return;
+      pdl_wait();
+      pdl_trigger();
+      // Nothing is flagged any more once every frame's ids are out.  The blocks that publish them are earlier ones of the grid
+      // and wait for nobody.
+      if (p.sel_mode == 1) {
+        bool ok = true;
+        for (int i = tid; i < p.n_frames; i += kCompactThreads) {
+          const volatile unsigned* flag = p.sel_flag + i;
+          ok = wait_until([&] { return (*flag >> 1) == p.epoch; }) && ok;
+        }
+        __threadfence();
+        if (!__syncthreads_and(ok)) {
+          if (tid == 0 && p.sp.status) atomicCAS(p.sp.status, 0, kStatusTailWait);
+          return;
+        }
+      }
+      if (*reinterpret_cast<volatile int*>(p.sp.n_flagged) != 0) redo_flagged<T>(p, e, p.redo_blocks, &cs);
+      return;
+    }
   }
   const bool patches = p.patch_split > 0 && row == 1;
   if (p.patch_split > 0 && row > 1) --row;
@@ -737,98 +836,24 @@ __global__ void __launch_bounds__(kCompactThreads) select_kernel(const CompactPa
   }
 }
 
-// Bounded wait until *ctr reaches `target` (other blocks of the same grid add to it; the grid is
-// sized so that all its blocks are resident).  False after about 1.5 s.
-__device__ inline bool wait_counter(const int* ctr, int target) {
-  const volatile int* c = ctr;
-  unsigned long long t0 = 0;
-  for (long long spin = 0;; ++spin) {
-    if (*c >= target) return true;
-    if ((spin & 63) == 63) {
-      unsigned long long now;
-      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-      if (t0 == 0) t0 = now;
-      else if (now - t0 > 1500000000ull) return false;
-    }
-    __nanosleep(200);
-  }
-}
-
-constexpr int kStatusTailWait = 6;   // tail_kernel: the wait for the double-precision scores ran out
-
-// tail_kernel: see the head of this file.  sp is the scoring configuration of the double-precision
-// pass (its partial-sum buffers, refine = 1); the grid is a multiple of nothing in particular: blocks
-// stride over the work, and the host keeps the grid within what is resident at once.
 // segment_kernel: one block per (layer, K|V) plane writes that plane of every segment entry the frames
-// first_frame .. first_frame + n_frames - 1 touch.  Launched for the chunk of an earlier call when
-// something is about to read its segment entries (pool_always = 1); without pool_always it leaves
-// everything to tail_kernel when frames were flagged.
+// first_frame .. first_frame + n_frames - 1 touch.  Launched for the chunk of an earlier call when something is about to
+// read its segment entries.
 __global__ void __launch_bounds__(kCompactThreads) segment_kernel(const CompactParams p) {
   pdl_wait();
   pdl_trigger();
-  if (!p.pool_always && *p.sp.n_flagged != 0) return;
   for (int plane = blockIdx.x; plane < 2 * p.L; plane += gridDim.x)
     compact_segment_plane(segment_args(p), plane >> 1, plane & 1);
 }
 
-template <typename T, int NC>
-__global__ void __launch_bounds__(kScoreThreads, 2) tail_kernel(const ScoreParams sp, const CompactParams p) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+// The flagged frames as a launch of their own.
+template <typename T>
+__global__ void __launch_bounds__(kCompactThreads, 3) tail_kernel(const __grid_constant__ CompactParams p) {
   __shared__ CompactScratch cs;
-  __shared__ int s_ok;
-  const int tid = threadIdx.x;
   pdl_trigger();                                // the next call's scoring kernel may be scheduled (it waits for this one itself)
   pdl_wait();
-  const int n_fl = *sp.n_flagged;
-  if (n_fl == 0) return;                        // the common case: the next call pools this chunk's segment entries
-  // ---- scores of the flagged frames in double precision; the block that finishes a frame last selects
-  const int units = sp.Ls * sp.Hq * sp.row_split;
-  for (int w = blockIdx.x; w < n_fl * units; w += gridDim.x) {
-    const int u = w % units;
-    const int fl = sp.flagged[w / units];
-    score_frame_block<T, double, NC>(sp, u / sp.row_split, u % sp.row_split, sp.row_split, fl, fl, smem_raw);
-    __syncthreads();
-  }
-  // ---- every block waits for all selections
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) {
-    atomicAdd(p.tail_ctr, 1);
-    s_ok = wait_counter(p.tail_ctr, (int)gridDim.x) ? 1 : 0;
-    __threadfence();
-  }
-  __syncthreads();
-  if (!s_ok) {
-    if (tid == 0 && sp.status) atomicCAS(sp.status, 0, kStatusTailWait);
-  } else {
-    // ---- the flagged frames' compaction, then the segment entries, plane by plane
-    const int n_planes = 2 * p.L + (p.patch_split > 0 ? 1 : 0);
-    for (int plane = blockIdx.x; plane < n_planes; plane += gridDim.x) {
-      for (int i = 0; i < n_fl; ++i) {
-        const int f = sp.flagged[i];
-        const long long f_abs = p.first_frame + f;
-        __syncthreads();
-        for (int r = tid; r < p.kappa; r += kCompactThreads) cs.kept[r] = token_id(__ldcg(sp.kept_store + f_abs * p.kappa + r), p.P);
-        __syncthreads();
-        if (plane < 2 * p.L) compact_plane<T>(p, plane, f, &cs, p.kappa, p.store + sp.pages_off + f_abs * sp.page_bytes);
-        else pool_patches<T>(p, f, &cs);
-      }
-      if (plane >= 2 * p.L) continue;
-      __threadfence();                          // the frame entries just written are read below by other threads
-      __syncthreads();
-      compact_segment_plane(segment_args(p), plane >> 1, plane & 1);
-    }
-  }
-  // ---- the block that leaves last resets the counters and adds to the statistics
-  __syncthreads();
-  if (tid == 0) {
-    const int old = atomicAdd(p.tail_ctr + 1, 1);
-    if (old == (int)gridDim.x - 1) {
-      *p.stat_refined += n_fl;
-      p.tail_ctr[0] = 0;
-      p.tail_ctr[1] = 0;
-    }
-  }
+  if (*p.sp.n_flagged == 0) return;             // the common case
+  redo_flagged<T>(p, blockIdx.x, gridDim.x, &cs);
 }
 
 }  // namespace mukv

@@ -6,6 +6,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -20,6 +21,7 @@
 #include "compact.cuh"
 #include "retrieve.cuh"
 #include "score.cuh"
+#include "score64.cuh"
 #include "score_ps.cuh"
 #include "segsel.cuh"
 
@@ -79,7 +81,7 @@ struct mukv_ctx {
   bool failed = false;                   // a compress call broke off half way: only reset / stats / destroy
   TcShape tcs;                           // tcs.ok: the chunk is scored on the tensor cores
   int n_sms;
-  int tail_capacity = 1;                 // blocks of tail_kernel that are resident at once on this device
+  int redo_capacity = 1;                 // blocks of redo_flagged that are resident at once on this device
   CUtensorMap wmap;                      // DFT matrix terms [3*D][D] bf16
   CUtensorMap pmap;                      // the page region as [frame][plane][kept row][key head][D] (past_frames > 0)
   // Segment entries a compress call left to whoever comes next (see flush_segments): the frames whose
@@ -180,8 +182,8 @@ const char* check_config(const mukv_config* c) {
   if (!is_pow2(row_vec) || row_vec > 256) return "Hkv*D*sizeof(element)/16 must be a power of two <= 256";
   // the scoring kernel keeps one key head of a frame in shared memory
   const int key_rows = c->tokens_per_frame + c->past_frames * c->keep_per_frame;
-  const size_t smem = c->dtype == MUKV_BF16 ? score_smem_bytes<__nv_bfloat16, double>(key_rows, c->head_dim)
-                                            : score_smem_bytes<float, double>(key_rows, c->head_dim);
+  const size_t smem = c->dtype == MUKV_BF16 ? score_smem_bytes<__nv_bfloat16>(key_rows, c->head_dim)
+                                            : score_smem_bytes<float>(key_rows, c->head_dim);
   if (smem > 227 * 1024) return "tokens_per_frame * head_dim too large for shared memory";
   return nullptr;
 }
@@ -253,7 +255,13 @@ TcShape tc_shape(const mukv_config& c) {
   return t;
 }
 
-constexpr int kRefineSplit = 4;     // blocks per query head in the double-precision pass
+constexpr int kRefineSplit = 4;     // blocks per query head where whole segments are scored in double precision
+// Rows of P doubles that the column sums of the double-precision pass have room for: one for every (frame, head, part) of a
+// call of segment-level selection, and for a head of a single flagged frame to be split over the device (see score64_split).
+size_t refine_rows(const mukv_config& c) {
+  const size_t rows = (size_t)c.max_frames_per_chunk * (c.n_score_layers > 1 ? c.n_score_layers : 1) * c.n_q_heads * kRefineSplit;
+  return rows > 512 ? rows : 512;
+}
 // Single precision decides a frame only when its lowest kept and highest dropped fused score are
 // further apart than tie_eps + kFlagMargin; a signal whose range is below kFlatRatio of its
 // magnitude (the min-max division then amplifies rounding noise) also sends the frame to the
@@ -277,7 +285,7 @@ WorkLayout work_layout(const mukv_config& c) {
   const size_t Ls = c.n_score_layers > 1 ? c.n_score_layers : 1;
   w.colsum_f = off;       off = align_up(off + F * Ls * (size_t)c.n_q_heads * P * sizeof(float));
   w.ifft_f = off;         off = align_up(off + F * Ls * c.n_kv_heads * P * sizeof(float));
-  w.colsum_d = off;       off = align_up(off + F * Ls * c.n_q_heads * kRefineSplit * P * sizeof(double));
+  w.colsum_d = off;       off = align_up(off + refine_rows(c) * P * sizeof(double));
   w.ifft_d = off;         off = align_up(off + F * Ls * c.n_kv_heads * P * sizeof(double));
   w.zero_begin = off;
   w.frame_counter = off;  off = align_up(off + F * sizeof(int));
@@ -330,34 +338,12 @@ cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t
 }
 
 template <typename T>
-const void* tail_fn(int nc) {
+cudaError_t launch_score(const ScoreParams& sp, int nc, dim3 grid, size_t smem, cudaStream_t st) {
   switch (nc) {
-    case 2: return (const void*)tail_kernel<T, 2>;
-    case 4: return (const void*)tail_kernel<T, 4>;
-    case 7: return (const void*)tail_kernel<T, 7>;
-    default: return (const void*)tail_kernel<T, 8>;
-  }
-}
-
-template <typename T>
-cudaError_t launch_tail(const ScoreParams& sp, const CompactParams& cp, int nc, int grid, size_t smem, cudaStream_t st,
-                        bool dependent) {
-  switch (nc) {
-    case 2: return launch_k(tail_kernel<T, 2>, dim3(grid), kScoreThreads, smem, st, dependent, sp, cp);
-    case 4: return launch_k(tail_kernel<T, 4>, dim3(grid), kScoreThreads, smem, st, dependent, sp, cp);
-    case 7: return launch_k(tail_kernel<T, 7>, dim3(grid), kScoreThreads, smem, st, dependent, sp, cp);
-    default: return launch_k(tail_kernel<T, 8>, dim3(grid), kScoreThreads, smem, st, dependent, sp, cp);
-  }
-}
-
-template <typename T, typename A>
-cudaError_t launch_score(const ScoreParams& sp, int nc, dim3 grid, size_t smem, cudaStream_t st,
-                         bool dependent = false) {
-  switch (nc) {
-    case 2: return launch_k(score_kernel<T, A, 2>, grid, kScoreThreads, smem, st, dependent, sp);
-    case 4: return launch_k(score_kernel<T, A, 4>, grid, kScoreThreads, smem, st, dependent, sp);
-    case 7: return launch_k(score_kernel<T, A, 7>, grid, kScoreThreads, smem, st, dependent, sp);
-    default: return launch_k(score_kernel<T, A, 8>, grid, kScoreThreads, smem, st, dependent, sp);
+    case 2: return launch_k(score_kernel<T, 2>, grid, kScoreThreads, smem, st, false, sp);
+    case 4: return launch_k(score_kernel<T, 4>, grid, kScoreThreads, smem, st, false, sp);
+    case 7: return launch_k(score_kernel<T, 7>, grid, kScoreThreads, smem, st, false, sp);
+    default: return launch_k(score_kernel<T, 8>, grid, kScoreThreads, smem, st, false, sp);
   }
 }
 
@@ -370,12 +356,12 @@ cudaError_t raise_smem_limit(const void* fn, int optin) {
   return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
 }
 
-template <typename T, typename A>
+template <typename T>
 cudaError_t raise_score_limits(int optin) {
-  cudaError_t e = raise_smem_limit((const void*)score_kernel<T, A, 2>, optin);
-  if (e == cudaSuccess) e = raise_smem_limit((const void*)score_kernel<T, A, 4>, optin);
-  if (e == cudaSuccess) e = raise_smem_limit((const void*)score_kernel<T, A, 7>, optin);
-  if (e == cudaSuccess) e = raise_smem_limit((const void*)score_kernel<T, A, 8>, optin);
+  cudaError_t e = raise_smem_limit((const void*)score_kernel<T, 2>, optin);
+  if (e == cudaSuccess) e = raise_smem_limit((const void*)score_kernel<T, 4>, optin);
+  if (e == cudaSuccess) e = raise_smem_limit((const void*)score_kernel<T, 7>, optin);
+  if (e == cudaSuccess) e = raise_smem_limit((const void*)score_kernel<T, 8>, optin);
   return e;
 }
 
@@ -400,15 +386,8 @@ cudaError_t raise_kernel_limits(int* n_sms) {
   if (g_limits_raised[dev]) return cudaSuccess;
   int optin = 0;
   e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e == cudaSuccess) e = raise_score_limits<__nv_bfloat16, float>(optin);
-  if (e == cudaSuccess) e = raise_score_limits<__nv_bfloat16, double>(optin);
-  if (e == cudaSuccess) e = raise_score_limits<float, float>(optin);
-  if (e == cudaSuccess) e = raise_score_limits<float, double>(optin);
-  const int ncs[4] = {2, 4, 7, 8};
-  for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
-    e = raise_smem_limit(tail_fn<__nv_bfloat16>(ncs[i]), optin);
-    if (e == cudaSuccess) e = raise_smem_limit(tail_fn<float>(ncs[i]), optin);
-  }
+  if (e == cudaSuccess) e = raise_score_limits<__nv_bfloat16>(optin);
+  if (e == cudaSuccess) e = raise_score_limits<float>(optin);
   if (e == cudaSuccess) e = raise_smem_limit((const void*)rank_kernel, optin);
   if (e == cudaSuccess) e = raise_smem_limit((const void*)segsel_kernel, optin);
   if (e == cudaSuccess) e = raise_smem_limit((const void*)score_ps_kernel<false, false>, optin);
@@ -540,8 +519,8 @@ SegmentArgs segment_args_of(const mukv_ctx* ctx, long long first, int n) {
   return a;
 }
 
-// A compress call does not pool the segment entries of its chunk itself (unless frames were flagged:
-// tail_kernel then does): the next compress call does it with blocks that do not wait for that call's
+// A compress call does not pool the segment entries of its chunk itself: the next compress call does it with blocks that do
+// not wait for that call's
 // scoring kernel (more rows in its compaction kernel, one plane per block; with segment-level selection, extra blocks of its
 // first segsel_kernel launch).  Whoever else needs the entries first
 // (retrieval, a gather with summary tokens, a view of the store, an export) pools them with one launch here.
@@ -553,7 +532,6 @@ cudaError_t flush_segments(const mukv_ctx* ctx, cudaStream_t st) {
   cp.L = a.L; cp.kappa = a.kappa; cp.C = a.C; cp.fseg = a.fseg; cp.n_frames = a.n_frames; cp.first_frame = a.first_frame;
   cp.frame_entry = const_cast<float*>(a.frame_entry); cp.frame_ksum = const_cast<double*>(a.frame_ksum);
   cp.seg_entry = a.seg_entry; cp.seg_key = a.seg_key; cp.kept_count = a.kept_count;
-  cp.pool_always = 1;
   const cudaError_t e = launch_k(segment_kernel, dim3(2 * a.L), kCompactThreads, 0, st, false, cp);
   if (e == cudaSuccess) ctx->seg_pending = false;
   return e;
@@ -750,10 +728,9 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
     }
     {
       ProfScope ps(ctx, tc_first ? 1 : 0, st);
-      const int units = ctx->Ls * c.n_q_heads * kRefineSplit;
-      const dim3 grid_d = tc_first ? dim3(units < 2 * ctx->n_sms ? units : 2 * ctx->n_sms) : dim3(units, n);
-      e = launch_score<T, double>(sd, ctx->nc, grid_d,
-                                  score_smem_bytes<T, double>(P, c.head_dim), st, tc_first && dep);
+      const long long units = (long long)ctx->Ls * c.n_q_heads * kRefineSplit * (tc_first ? 1 : n), most = 3LL * ctx->n_sms;
+      const dim3 grid_d((unsigned)(units < most ? units : most));
+      e = launch_k(score64_kernel<T>, grid_d, kScoreThreads, 0, st, tc_first && dep, sd);
     }
     if (e != cudaSuccess) {
       if (tc_first) return broke_off(ctx, "score kernel", e);
@@ -779,7 +756,7 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
       ctx->att_dirty[ctx->parity] = (long long)n * P;
       on_tc = true;
     } else
-      e = launch_score<T, float>(sp, ctx->nc, grid, score_smem_bytes<T, float>(ctx->key_rows, c.head_dim), st);
+      e = launch_score<T>(sp, ctx->nc, grid, score_smem_bytes<T>(ctx->key_rows, c.head_dim), st);
     ++n_launch;
   }
   if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "%s: %s", what, cudaGetErrorString(e));
@@ -831,28 +808,33 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
   // 300 with parts; calls of 7 frames and 24 layers, which get two parts: no difference.)
   cp.parts = 1;
   while (cp.parts < 4 && 4LL * n * L * cp.parts <= 3LL * ctx->n_sms && C * ctx->esize / (2 * cp.parts) >= 256) cp.parts *= 2;
+  // Flagged frames (frame-level selection by Eq. 1-4 only): blocks that redo them, one per SM, fewer when a frame has less work.
+  // They are blocks of the compaction kernel, which spares the calls that flag nothing a launch.  fp32 calls keep the launch:
+  // a hundredth of their time, behind a kernel of twice the bytes.
+  int redo = 0;
+  if (!seg_scope && !d_ext) {
+    const int units = ctx->Ls * c.n_q_heads * ((P + 7) / 8), planes = 4 * L + 1;
+    redo = std::min(std::min(std::max(units, planes), ctx->redo_capacity), ctx->n_sms);
+    cp.colsum_d = reinterpret_cast<double*>(ctx->ws + ctx->wl.colsum_d);
+    cp.ifft_d = reinterpret_cast<double*>(ctx->ws + ctx->wl.ifft_d);
+    cp.sp.scratch_rows = (int)std::min<size_t>(refine_rows(c), 0x7fffffff);
+    if (sizeof(T) == 2) cp.redo_blocks = redo;
+  }
   {
     ProfScope ps(ctx, 2, st);
-    e = launch_k(compact_kernel<T>, dim3(n, L * 2 * cp.parts + (c.patch_split > 0 ? 1 : 0) + cp.prev_rows),
-                 kCompactThreads, 0, st, !ctx->prof_on, cp);
+    const int rows = L * 2 * cp.parts + (c.patch_split > 0 ? 1 : 0) + cp.prev_rows + (cp.redo_blocks + n - 1) / n;
+    e = launch_k(compact_kernel<T>, dim3(n, rows), kCompactThreads, 0, st, !ctx->prof_on, cp);
   }
   if (e != cudaSuccess) return broke_off(ctx, "compact kernel", e);
   ctx->seg_pending = false;
 
-  // The segment entries need every frame of the chunk.  They are left to the next call (flush_segments);
-  // when frames were flagged, tail_kernel pools them after it has redone those frames.
-  cp.sp.n_flagged = sp.n_flagged;
-  sp.refine = 1;
-  sp.row_split = kRefineSplit;
-  sp.colsum_part = ctx->ws + ctx->wl.colsum_d;
-  sp.ifft_part = ctx->ws + ctx->wl.ifft_d;
-  if (!seg_scope) {                                      // (segment-level selection flags nothing)
-    ProfScope ps(ctx, 1, st);
-    int grid_t = ctx->Ls * c.n_q_heads * kRefineSplit * (n < 2 ? n : 2);
-    if (grid_t < 2 * L + 1) grid_t = 2 * L + 1;
-    if (grid_t > ctx->tail_capacity) grid_t = ctx->tail_capacity;
-    e = launch_tail<T>(sp, cp, ctx->nc, grid_t, score_smem_bytes<T, double>(ctx->key_rows, c.head_dim), st, !ctx->prof_on);
-    ++n_launch;
+  // (The segment entries need every frame of the chunk.  They are left to the next call, see flush_segments.)
+  if constexpr (sizeof(T) == 4) {
+    if (redo > 0) {
+      ProfScope ps(ctx, 1, st);
+      e = launch_k(tail_kernel<T>, dim3(redo), kCompactThreads, 0, st, !ctx->prof_on, cp);
+      ++n_launch;
+    }
   }
   if (e != cudaSuccess) return broke_off(ctx, "tail kernel", e);
   ctx->seg_pending = true;
@@ -1110,15 +1092,12 @@ mukv_status create_impl(const mukv_config* cfg, void* d_store, size_t store_byte
   const int D = cfg->head_dim;
   cudaError_t e = raise_kernel_limits(&ctx->n_sms);
   if (e == cudaSuccess) {
-    // the blocks of tail_kernel wait for one another: its grid must be resident as a whole
+    // the blocks of redo_flagged wait for one another: all of them must be resident
     int per_sm = 0;
-    const bool bf = cfg->dtype == MUKV_BF16;
-    const size_t dyn = bf ? score_smem_bytes<__nv_bfloat16, double>(ctx->key_rows, D)
-                          : score_smem_bytes<float, double>(ctx->key_rows, D);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bf ? tail_fn<__nv_bfloat16>(ctx->nc) : tail_fn<float>(ctx->nc),
-                                                      kScoreThreads, dyn);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &per_sm, cfg->dtype == MUKV_BF16 ? (const void*)compact_kernel<__nv_bfloat16> : (const void*)tail_kernel<float>, kCompactThreads, 0);
     if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
-    ctx->tail_capacity = per_sm * ctx->n_sms;
+    ctx->redo_capacity = per_sm * ctx->n_sms;
   }
   if (e == cudaSuccess && (ctx->tcs.ok || ctx->tcs.split)) {
     e = cudaMemcpy(ctx->ws + ctx->wl.wtab, dft_terms(D), dft_bytes(D), cudaMemcpyHostToDevice);
@@ -1578,19 +1557,17 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
     e = launch_k(select_kernel, dim3(n), kCompactThreads, 0, st, true, cp, (const int*)pl.status);
     if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "select kernel: %s", cudaGetErrorString(e));
   } else {
-    e = launch_score<T, float>(sp, nc, dim3(c.n_q_heads, n), score_smem_bytes<T, float>(P, D), st);
+    e = launch_score<T>(sp, nc, dim3(c.n_q_heads, n), score_smem_bytes<T>(P, D), st);
     if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "score kernel: %s", cudaGetErrorString(e));
   }
   // Flagged frames in double precision.  The scratch holds the partial sums of 16 frames with one block per head; while
-  // few frames are flagged the same room lets four blocks share a head.
+  // few frames are flagged the same room lets several blocks share a head.
   sp.refine = 1;
-  sp.row_split = kRefineSplit;
-  sp.scratch_units = kNaFrames * kNaHq;
+  sp.scratch_rows = kNaFrames * kNaHq;
   sp.colsum_part = base + kNaColD;
   sp.ifft_part = base + kNaFftD;
-  int grid_r = c.n_q_heads * kRefineSplit * (n < 2 ? n : 2);
-  if (grid_r > 2 * nd->n_sms) grid_r = 2 * nd->n_sms;
-  e = launch_score<T, double>(sp, nc, dim3(grid_r), score_smem_bytes<T, double>(P, D), st, true);
+  const int units = n * c.n_q_heads * ((P + 7) / 8);
+  e = launch_k(score64_kernel<T>, dim3(std::min(units, nd->n_sms)), kScoreThreads, 0, st, true, sp);
   if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "refine kernel: %s", cudaGetErrorString(e));
   return MUKV_OK;
 }

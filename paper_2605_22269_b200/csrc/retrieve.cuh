@@ -110,12 +110,6 @@ constexpr int kScanCC = 64;
 constexpr int kScanQB = 64;
 constexpr int kScanQPad = kScanQB + 4;
 
-__device__ __forceinline__ void dmma_m8n8k4(double (&c)[2], double a, double b) {
-  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
-               : "+d"(c[0]), "+d"(c[1])
-               : "d"(a), "d"(b));
-}
-
 struct ScanParams {
   const float* frame_key; const float* seg_key; const float* patch_key;
   long long n_frm, n_seg, n_pat;
@@ -342,15 +336,6 @@ __global__ void __launch_bounds__(256) scan_few_kernel(const ScanParams sp) {
 }
 
 // ------------------------------------------------------------------------------ ranking
-__device__ __forceinline__ unsigned long long order_key(double x) {
-  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
-}
-__device__ __forceinline__ double order_key_inv(unsigned long long k) {
-  const unsigned long long b = (k >> 63) ? (k & 0x7fffffffffffffffull) : ~k;
-  return __longlong_as_double((long long)b);
-}
-
 constexpr int kRankList = 64;      // keys left in the radix select below which they are ranked directly
 constexpr int kRankCand = 512;     // candidates that are ranked among themselves (at most one per thread)
 constexpr int kRankBins = 512;     // bins of the linear histogram

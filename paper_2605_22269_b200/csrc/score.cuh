@@ -1,6 +1,7 @@
 // Per-frame token scoring and selection (Sec. 3.3, Eq. 1-4 and the top-kappa rule).
 //
-// score_kernel<T, A, NC>: one thread block per (query head h, frame f).
+// score_kernel<T, NC>: one thread block per (query head h, frame f), single precision on the multiply-add units (fp32 calls
+// that the tensor cores do not hold; MUKV_OPT_SCORE_PATH 1).  The double-precision pass is in score64.cuh.
 //   * Eq. 1: S = Q_h K_g^T / sqrt(D) over the frame's P tokens, row softmax, column sums.
 //     Lanes own key columns (j = lane + 32c), a warp walks the query rows four at a time, so
 //     the column sums stay in registers and only the row maximum / row sum cross lanes.
@@ -9,8 +10,7 @@
 //     transform each key vector along the feature axis; sum of the D bin magnitudes per token.
 //   * The block that finishes a frame last (arrival counter, nobody waits) reduces the
 //     per-head partials in a fixed order, applies Eq. 4 and selects the kappa tokens.
-// T is the input element type, A the arithmetic type: float for the normal path, double for
-// the frames whose selection is too close to a tie boundary to trust single precision.
+// T is the input element type.
 #pragma once
 #include "common.cuh"
 
@@ -56,28 +56,34 @@ struct ScoreParams {
   int no_select;                // 1: only the partial sums are wanted (the selection runs over a whole segment elsewhere)
   int refine;                   // 1: frames come from the flagged list, no further flagging
   int row_split;                // blocks that share a query head, each a range of query rows (>= 1)
-  // score_kernel's double-precision pass: room for the partial sums of that many (frame, head, part) units.  They are
-  // indexed by the place in the flagged list, and a head is split over row_split blocks while that fits, else not split.
-  // (tail_kernel has one place per frame of the chunk and does not look at this.)
-  int scratch_units;
+  int scratch_rows;             // double-precision pass over flagged frames: rows of P doubles that colsum_part has room for
+                                // (see score64_split; a flagged frame's place is its place in the list)
   // segment-level selection, double-precision pass: only the frames of segments whose word is non-zero
   // are scored (segment of chunk frame f: f / gate_fseg); null: every frame
   const int* seg_gate;
   int gate_fseg;
 };
 
+struct FinishScratch {
+  double part[kScoreWarps][256];
+  double sc[256];
+  double misc[64];
+  int ints[64];
+};
+
 template <typename T>
 __host__ __device__ constexpr int score_row_stride(int D) { return D + ElemTraits<T>::kPad; }
 
 // P: key rows held in shared memory (the frame's tokens plus the past keys)
-template <typename T, typename A>
+template <typename T>
 __host__ inline size_t score_smem_bytes(int P, int D) {
+  typedef float A;
   size_t ks = (size_t)P * score_row_stride<T>(D) * sizeof(T);
   size_t qs = (size_t)kScoreWarps * kRowsPerStep * D * sizeof(T);
   size_t tw = (size_t)D * 2 * sizeof(A);
   size_t red = (size_t)kScoreWarps * 256 * sizeof(A);
-  size_t sel = (size_t)256 * sizeof(double) + 64 * sizeof(double) + 64 * sizeof(int);
-  return ((ks + 15) / 16) * 16 + qs + tw + red + sel + 64;
+  const size_t all = ((ks + 15) / 16) * 16 + qs + tw + red;
+  return (all > sizeof(FinishScratch) ? all : sizeof(FinishScratch)) + 64;
 }
 
 // The top-kappa rule for one frame on final scores s (double), run by all threads of the group Grp.
@@ -93,13 +99,14 @@ __device__ inline void select_by_score(const ScoreParams& p, int f, const double
   const int tid = Grp::tid();
   const int nt = Grp::size();
   const int P = p.P;
+  unsigned long long* s_key = reinterpret_cast<unsigned long long*>(s_sc);
   int tok[TOK];
   bool valid[TOK];
 #pragma unroll
   for (int k = 0; k < TOK; ++k) {
     tok[k] = tid + k * nt;
     valid[k] = tok[k] < P;
-    if (valid[k]) s_sc[tok[k]] = s[k];
+    if (valid[k]) s_key[tok[k]] = order_key(s[k]);
   }
   Grp::sync();
   const int kappa = p.kappa;
@@ -107,10 +114,13 @@ __device__ inline void select_by_score(const ScoreParams& p, int f, const double
   for (int k = 0; k < TOK; ++k) {
     if (valid[k]) {
       int gt = 0, ge = 0;
+      // (on order-preserving integers: a comparison of doubles takes sixteen clocks of a scheduler)
+      const unsigned long long key = order_key(s[k]);
+#pragma unroll 4
       for (int i = 0; i < P; ++i) {
-        const double o = s_sc[i];
-        gt += (o > s[k]);
-        ge += (o >= s[k]);
+        const unsigned long long o = s_key[i];
+        gt += (o > key);
+        ge += (o >= key);
       }
       if (gt < kappa && kappa <= ge) s_misc[0] = s[k];      // every writer holds the same value
     }
@@ -160,11 +170,12 @@ __device__ inline void select_by_score(const ScoreParams& p, int f, const double
 // Eq. 4 and the top-kappa rule for one frame, run by all threads of the group Grp.  Thread tid owns
 // the tokens tid + k*size, k < TOK (TOK*size >= P); att_raw / fft_raw are their I_att and I_fft;
 // s_sc (P doubles), s_int (one int per warp + 1), s_misc (4 doubles per warp) are shared scratch.
+// With `refined` the frame is not put on the flagged list however close it is.
 // The arithmetic here is always double: it is a few hundred operations per frame and keeps
 // the normalisation from adding rounding noise of its own to the scores.
 template <int TOK, class Grp = BlockGroup>
 __device__ inline void select_frame(const ScoreParams& p, int f, const double (&att_raw)[TOK],
-                                    const double (&fft_raw)[TOK], double* s_sc, int* s_int, double* s_misc) {
+                                    const double (&fft_raw)[TOK], bool refined, double* s_sc, int* s_int, double* s_misc) {
   typedef double A;
   const int tid = Grp::tid(), lane = tid & 31, warp = tid >> 5;
   const int nt = Grp::size(), nwarp = nt >> 5;
@@ -236,7 +247,7 @@ __device__ inline void select_frame(const ScoreParams& p, int f, const double (&
   // perturbation of the scores below flag_margin / 2 as long as a - b > tie_eps + flag_margin: no
   // dropped token can then enter the tie band of the kappa-th score.  Anything closer is redone
   // in double precision.
-  if (!p.refine && !bad) {
+  if (!refined && !bad) {
     const int kappa = p.kappa;
     const A delta = (A)p.tie_eps;
     A a = big, b = -big;
@@ -271,12 +282,65 @@ __device__ inline void select_frame(const ScoreParams& p, int f, const double (&
   }
 }
 
-// The work of one block: part q (of RS) of the query rows of head hv of frame f (a frame
-// slot of the chunk); hv counts the query heads of all scoring layers, layer-major.  The partial sums go to
-// place sf of the scratch.
-template <typename T, typename A, int NC>
-__device__ __forceinline__ void score_frame_block(const ScoreParams& p, int hv, int q, int RS, int f, int sf,
-                                                  unsigned char* smem_raw) {
+// Sums over n rows of P values, rows in order inside an eighth, then the eighths in order: thread t < P of a block of
+// kScoreThreads gets column t.  A warp takes an eighth of the rows, a lane of it every 32nd column: all loads of a thread are
+// independent (one thread per column walks n round trips to L2: 6 us for 112 rows).  part: [kScoreWarps][256].
+template <typename A>
+__device__ inline double column_sums(const A* rows, int n, int P, double (*part)[256]) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int per = (n + kScoreWarps - 1) / kScoreWarps, r0 = min(n, warp * per), r1 = min(n, r0 + per);
+  for (int c0 = lane; c0 < P; c0 += 64) {                  // two columns at a time, eight rows in flight
+    double t0 = 0.0, t1 = 0.0;
+    const bool two = c0 + 32 < P;
+    for (int r = r0; r < r1; r += 8) {
+      A x0[8], x1[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        x0[i] = r + i < r1 ? __ldcg(rows + (long long)(r + i) * P + c0) : (A)0;
+        x1[i] = two && r + i < r1 ? __ldcg(rows + (long long)(r + i) * P + c0 + 32) : (A)0;
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) { t0 += (double)x0[i]; t1 += (double)x1[i]; }
+    }
+    part[warp][c0] = t0;
+    if (two) part[warp][c0 + 32] = t1;
+  }
+  __syncthreads();
+  double t = 0.0;
+  if (tid < P)
+    for (int w = 0; w < kScoreWarps; ++w) t += part[w][tid];
+  __syncthreads();
+  return t;
+}
+
+// Every block that has written its share of a frame's partial sums (column sums [heads * RS][P] and frequency sums [key
+// heads][P], at place sf) calls this; the one that arrives last finishes Eq. 1 / Eq. 3 and selects, unless no_select.  Run by
+// a whole block.  refined: the selection is final (see select_frame).
+template <typename A>
+__device__ inline void finish_frame(const ScoreParams& p, const A* colsum, const A* ifft, int f, int sf, int RS, bool refined,
+                                    FinishScratch* s) {
+  const int tid = threadIdx.x, P = p.P, HqV = p.Ls * p.Hq, HkvV = p.Ls * p.Hkv;
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) {
+    const int old = atomicAdd(p.frame_counter + f, 1);
+    s->ints[63] = (old == HqV * RS - 1);
+    if (old == HqV * RS - 1) p.frame_counter[f] = 0;  // ready for the next launch
+  }
+  __syncthreads();
+  if (!s->ints[63] || p.no_select) return;
+  __threadfence();
+  double att[1], fft[1];
+  att[0] = column_sums(colsum + (long long)sf * HqV * RS * P, HqV * RS, P, s->part) / (double)((long long)HqV * P);
+  fft[0] = column_sums(ifft + (long long)sf * HkvV * P, HkvV, P, s->part) / (double)((long long)HkvV * p.D);
+  select_frame<1>(p, f, att, fft, refined, s->sc, s->ints, s->misc);
+}
+
+// The work of one block: query head hv of frame f (a frame slot of the chunk); hv counts the query heads of all scoring
+// layers, layer-major.
+template <typename T, int NC>
+__device__ __forceinline__ void score_frame_block(const ScoreParams& p, int hv, int f, unsigned char* smem_raw) {
+  typedef float A;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int P = p.P, D = p.D, Hq = p.Hq, Hkv = p.Hkv, G = p.G;
   const int layer = hv / Hq, h = hv - layer * Hq;
@@ -299,12 +363,7 @@ __device__ __forceinline__ void score_frame_block(const ScoreParams& p, int hv, 
   A* tw = reinterpret_cast<A*>(smem_raw + off);
   off += (size_t)D * 2 * sizeof(A);
   A* red = reinterpret_cast<A*>(smem_raw + off);
-  off += (size_t)kScoreWarps * 256 * sizeof(A);
-  double* s_sc = reinterpret_cast<double*>(smem_raw + off);
-  off += (size_t)256 * sizeof(double);
-  double* s_misc = reinterpret_cast<double*>(smem_raw + off);
-  off += 64 * sizeof(double);
-  int* s_int = reinterpret_cast<int*>(smem_raw + off);
+  FinishScratch* fin = reinterpret_cast<FinishScratch*>(smem_raw);   // (in the place of the keys, when all is done with them)
 
   // ---- stage K_g of this frame (rows padded so that 32 consecutive rows hit 32 banks)
   const T* Kg = reinterpret_cast<const T*>(p.k_last) + layer * p.k_layer_stride + ((long long)f * P * Hkv + g) * D;
@@ -353,9 +412,7 @@ __device__ __forceinline__ void score_frame_block(const ScoreParams& p, int hv, 
   for (int c = 0; c < NC; ++c) jrow[c] = min(lane + 32 * c, Pk - 1) * WS;
 
   const int n_steps = (P + kRowsPerStep - 1) / kRowsPerStep;
-  const int n_per = (n_steps + RS - 1) / RS;
-  const int rb_end = (q + 1) * n_per < n_steps ? (q + 1) * n_per : n_steps;
-  for (int rb = q * n_per + warp; rb < rb_end; rb += kScoreWarps) {
+  for (int rb = warp; rb < n_steps; rb += kScoreWarps) {
     __syncwarp();
 #pragma unroll
     for (int r = 0; r < kRowsPerStep; ++r) {
@@ -378,26 +435,26 @@ __device__ __forceinline__ void score_frame_block(const ScoreParams& p, int hv, 
       for (int c = 0; c < NC; ++c) {
         const uint32_t kw = Kw[jrow[c] + w];
 #pragma unroll
-        for (int r = 0; r < kRowsPerStep; ++r) acc[r][c] = dot_word<T, A>(qw[r], kw, acc[r][c]);
+        for (int r = 0; r < kRowsPerStep; ++r) acc[r][c] = dot_word<T>(qw[r], kw, acc[r][c]);
       }
     }
 #pragma unroll
     for (int r = 0; r < kRowsPerStep; ++r) {
       const int i = rb * kRowsPerStep + r;
       A z[NC];
-      A m = neg_inf<A>();
+      A m = -INFINITY;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         const int j = lane + 32 * c;                     // past keys are visible to every query
         const bool ok = (j < Pk) && (!p.causal || j - n_past <= i);
-        z[c] = ok ? fma_acc(acc[r][c], scale, acc[r][c] * scale_lo) : neg_inf<A>();
+        z[c] = ok ? fmaf(acc[r][c], scale, acc[r][c] * scale_lo) : -INFINITY;
         m = z[c] > m ? z[c] : m;
       }
       m = warp_max(m);
       A l = (A)0;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
-        z[c] = (z[c] == neg_inf<A>()) ? (A)0 : exp_acc(z[c] - m);
+        z[c] = (z[c] == -INFINITY) ? (A)0 : expf(z[c] - m);
         l += z[c];
       }
       l = warp_sum(l);
@@ -413,14 +470,14 @@ __device__ __forceinline__ void score_frame_block(const ScoreParams& p, int hv, 
   if (tid < P) {                                       // the importance is that of the frame's own tokens
     A t = (A)0;
     for (int w = 0; w < kScoreWarps; ++w) t += red[w * 256 + n_past + tid];
-    reinterpret_cast<A*>(p.colsum_part)[(((long long)sf * HqV + hv) * RS + q) * P + tid] = t;
+    reinterpret_cast<A*>(p.colsum_part)[((long long)f * HqV + hv) * P + tid] = t;
   }
 
   // ---- Eq. 2-3: sum over the D bins of |DFT(k_j)| for this block's share of head g's tokens
   {
-    const int hg = (h % G) * RS + q;                 // the G * RS blocks that hold key head g share its tokens
+    const int hg = h % G;                            // the G blocks that hold key head g share its tokens
     const int half = D / 2;
-    for (int j = hg + warp * G * RS; j < P; j += kScoreWarps * G * RS) {
+    for (int j = hg + warp * G; j < P; j += kScoreWarps * G) {
       const T* kr = Ks + (size_t)(n_past + j) * DS;
       A total = (A)0;
       // bins 1 .. D/2-1 (twice, by conjugate symmetry) and bin 0
@@ -432,7 +489,7 @@ __device__ __forceinline__ void score_frame_block(const ScoreParams& p, int hv, 
           re += x * tw[2 * m];
           im -= x * tw[2 * m + 1];
         }
-        const A mag = sqrt_acc(re * re + im * im);
+        const A mag = sqrtf(re * re + im * im);
         total += (b == 0) ? mag : (A)2 * mag;
       }
       // bin D/2: alternating sum
@@ -444,75 +501,20 @@ __device__ __forceinline__ void score_frame_block(const ScoreParams& p, int hv, 
       total = warp_sum(total);
       alt = warp_sum(alt);
       if (lane == 0)
-        reinterpret_cast<A*>(p.ifft_part)[((long long)sf * HkvV + layer * Hkv + g) * P + j] = total + (alt < (A)0 ? -alt : alt);
+        reinterpret_cast<A*>(p.ifft_part)[((long long)f * HkvV + layer * Hkv + g) * P + j] = total + (alt < (A)0 ? -alt : alt);
     }
   }
 
-  // ---- last block of the frame finishes Eq. 1 / Eq. 3 and selects
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) {
-    const int old = atomicAdd(p.frame_counter + f, 1);
-    s_int[63] = (old == HqV * RS - 1);
-    if (old == HqV * RS - 1) p.frame_counter[f] = 0;  // ready for the next launch
-  }
-  __syncthreads();
-  if (!s_int[63] || p.no_select) return;
-  __threadfence();
-  double att[1] = {0.0}, fft[1] = {0.0};
-  if (tid < P) {
-    const A* cp = reinterpret_cast<const A*>(p.colsum_part) + (long long)sf * HqV * RS * P + tid;
-    if constexpr (sizeof(A) == 8) att[0] = ordered_sum(cp, HqV * RS, P);
-    else for (int hh = 0; hh < HqV * RS; ++hh) att[0] += (double)__ldcg(cp + (long long)hh * P);
-    att[0] = att[0] / (double)((long long)HqV * P);
-    const A* fp = reinterpret_cast<const A*>(p.ifft_part) + (long long)sf * HkvV * P + tid;
-    if constexpr (sizeof(A) == 8) fft[0] = ordered_sum(fp, HkvV, P);
-    else for (int gg = 0; gg < HkvV; ++gg) fft[0] += (double)__ldcg(fp + (long long)gg * P);
-    fft[0] = fft[0] / (double)((long long)HkvV * D);
-  }
-  __syncthreads();
-  select_frame<1>(p, f, att, fft, s_sc, s_int, s_misc);
+  finish_frame(p, reinterpret_cast<const A*>(p.colsum_part), reinterpret_cast<const A*>(p.ifft_part), f, f, 1, false, fin);
 }
 
-// Grid (Hq * row_split, frames).  Normal pass: block row = frame slot of the chunk.  Double-precision
-// pass (p.refine): a one-dimensional grid walks the (flagged frame, head, part) units; with
-// nothing flagged its blocks return at once.
-template <typename T, typename A, int NC>
+// Grid (query heads of all scoring layers, frames).
+template <typename T, int NC>
 __global__ void __launch_bounds__(kScoreThreads) score_kernel(const ScoreParams p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pdl_wait();
   pdl_trigger();
-  if (!p.refine) {
-    if (p.seg_gate) {
-      // A small one-dimensional grid walks the segments and scores the frames of flagged ones (rarely any).  The words of 32
-      // segments are read at once: read frame by frame they were 6 us of a call of 16 frames.
-      const int units = p.Ls * p.Hq * p.row_split, n_seg = (p.n_frames + p.gate_fseg - 1) / p.gate_fseg;
-      const int lane = threadIdx.x & 31;
-      for (int s0 = 0; s0 < n_seg; s0 += 32) {
-        unsigned set = __ballot_sync(kFull, s0 + lane < n_seg && __ldcg(p.seg_gate + s0 + lane) != 0);
-        for (; set; set &= set - 1) {
-          const int seg = s0 + __ffs(set) - 1, f1 = min((seg + 1) * p.gate_fseg, p.n_frames);
-          for (int f = seg * p.gate_fseg; f < f1; ++f) {
-            for (int u = blockIdx.x; u < units; u += gridDim.x) {
-              score_frame_block<T, A, NC>(p, u / p.row_split, u % p.row_split, p.row_split, f, f, smem_raw);
-              __syncthreads();
-            }
-          }
-        }
-      }
-      return;
-    }
-    score_frame_block<T, A, NC>(p, blockIdx.x / p.row_split, blockIdx.x % p.row_split, p.row_split, blockIdx.y, blockIdx.y,
-                                smem_raw);
-    return;
-  }
-  const int n = *p.n_flagged, heads = p.Ls * p.Hq;
-  const int rs = n * heads * p.row_split <= p.scratch_units ? p.row_split : 1, units = heads * rs;
-  for (int w = blockIdx.x; w < n * units; w += gridDim.x) {
-    const int slot = w / units, u = w - slot * units;
-    score_frame_block<T, A, NC>(p, u / rs, u % rs, rs, p.flagged[slot], slot, smem_raw);
-    __syncthreads();
-  }
+  score_frame_block<T, NC>(p, blockIdx.x, blockIdx.y, smem_raw);
 }
 
 }  // namespace mukv
