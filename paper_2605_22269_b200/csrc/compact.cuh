@@ -565,7 +565,7 @@ __device__ inline void compact_plane_part(const CompactParams& p, int plane, int
 // whole block; the kept rows are first grouped by super patch, then every thread sums its channels
 // of each group in ascending row order.  sc->red is used as scratch.
 template <typename T>
-__device__ inline void pool_patches(const CompactParams& p, int f, CompactScratch* sc) {
+__device__ __noinline__ void pool_patches(const CompactParams& p, int f, CompactScratch* sc) {
   constexpr int EW = ElemTraits<T>::kPerWord;
   const int tid = threadIdx.x;
   const int S = p.patch_split * p.patch_split, C = p.C, kappa = p.kappa;
@@ -702,12 +702,14 @@ __device__ __noinline__ void redo_flagged(const CompactParams& p, int e, int blo
   }
 }
 
-template <typename T>
+// PARTS: two or four blocks share a plane (p.parts).  SELECT: sel_mode 1; else the mode is looked up.  (A kernel for each, so that
+// none carries the code of the others: a block's first pass through its code is instruction fetch more than anything else.)
+template <typename T, bool PARTS, bool SELECT>
 __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __grid_constant__ CompactParams p) {
   __shared__ CompactScratch cs;
   __shared__ SelectScratch ss;
-  __shared__ unsigned s_seen;
   const int tid = threadIdx.x;
+  const int parts = PARTS ? p.parts : 1, sel_mode = SELECT ? 1 : p.sel_mode;
   // frame is the fast block index: the blocks that start first cover the low planes of every frame,
   // the plane-0 blocks among them
   const int f = blockIdx.x;
@@ -718,7 +720,7 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __gri
     if (row >= 1 && row <= p.prev_rows) {
       // nothing of this call is needed for the entries of the previous one: no wait for the scoring kernel (which has
       // itself waited for the previous call's kernels; without a scoring kernel the wait is here)
-      if (p.sel_mode == 2) pdl_wait();
+      if (sel_mode == 2) pdl_wait();
       const int pl = (row - 1) * gridDim.x + blockIdx.x;
       if (pl < 2 * p.prev.L) compact_segment_plane(p.prev, pl >> 1, pl & 1);
       return;
@@ -726,7 +728,7 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __gri
     if (row > p.prev_rows) row -= p.prev_rows;
   }
   if constexpr (sizeof(T) == 2) {
-    const int first = 2 * p.L * p.parts + (p.patch_split > 0 ? 1 : 0);     // row of the first block for flagged frames
+    const int first = 2 * p.L * parts + (p.patch_split > 0 ? 1 : 0);     // row of the first block for flagged frames
     if (p.redo_blocks > 0 && row >= first) {
       const int e = (row - first) * gridDim.x + blockIdx.x;
       if (e >= p.redo_blocks) return;
@@ -734,7 +736,7 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __gri
       pdl_trigger();
       // Nothing is flagged any more once every frame's ids are out.  The blocks that publish them are earlier ones of the grid
       // and wait for nobody.
-      if (p.sel_mode == 1) {
+      if (sel_mode == 1) {
         bool ok = true;
         for (int i = tid; i < p.n_frames; i += kCompactThreads) {
           const volatile unsigned* flag = p.sel_flag + i;
@@ -752,7 +754,7 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __gri
   }
   const bool patches = p.patch_split > 0 && row == 1;
   if (p.patch_split > 0 && row > 1) --row;
-  const int plane = patches ? 2 * p.L : row / p.parts, part = patches ? 0 : row % p.parts;
+  const int plane = patches ? 2 * p.L : row / parts, part = patches ? 0 : row % parts;
   const bool writes = plane == 0 && part == 0;           // this block writes the ids and the index of its frame
   pdl_wait();
   pdl_trigger();
@@ -763,7 +765,8 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __gri
   int kappa_f = p.kappa;
   unsigned char* page = p.store + p.sp.pages_off + f_abs * p.sp.page_bytes;
   bool risky;
-  if (p.sel_mode == 1) {
+  if (sel_mode == 1) {
+    __shared__ unsigned s_seen;
     // A block that starts after its frame's plane-0 block has published the ids (the blocks beyond
     // the first wave do) reads them; every other block selects itself.  Nobody waits.
     if (tid == 0) {
@@ -788,7 +791,7 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __gri
         if (tid == 0) *reinterpret_cast<volatile unsigned*>(p.sel_flag + f) = (p.epoch << 1) | (risky ? 1u : 0u);
       }
     }
-  } else if (p.sel_mode == 2) {
+  } else if (sel_mode == 2) {
     // Ranking by numbers the caller supplies (no Eq. 1-4): every block ranks its frame itself, in
     // double precision on exact inputs, so nothing is ever too close to call; plane 0 writes the ids.
     double sx[1] = {tid < p.P ? (double)__ldg(p.ext_scores + (long long)f * p.P + tid) : 0.0};
@@ -799,7 +802,7 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __gri
     if (bad && writes && tid == 0 && p.sp.status) atomicCAS(p.sp.status, 0, kStatusNonFinite);
     risky = false;
     __syncthreads();
-  } else if (p.sel_mode == 3) {
+  } else if (sel_mode == 3) {
     kappa_f = __ldcg(p.kept_count + f_abs);
     kappa_f = kappa_f < 0 ? 0 : (kappa_f > p.P ? p.P : kappa_f);
     page = p.store + __ldcg(p.sp.page_table + f_abs);
@@ -813,8 +816,8 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __gri
   }
   if (risky) return;
   if (plane >= 2 * p.L) pool_patches<T>(p, f, &cs);
-  else if (p.parts == 1) compact_plane<T>(p, plane, f, &cs, kappa_f, page);
-  else compact_plane_part<T>(p, plane, f, &cs, kappa_f, page, part, p.parts);
+  else if constexpr (PARTS) compact_plane_part<T>(p, plane, f, &cs, kappa_f, page, part, parts);
+  else compact_plane<T>(p, plane, f, &cs, kappa_f, page);
 }
 
 // Selection alone (scoring without a store): one block per frame, behind the persistent scoring kernel.  A code in *scoring

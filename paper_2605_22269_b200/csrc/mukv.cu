@@ -42,7 +42,7 @@ struct StoreLayout {
 
 struct WorkLayout {
   size_t q_terms, k_terms; // fp32 chunks: queries and keys of the scoring layers as three bf16 terms
-  size_t colsum_f, ifft_f, colsum_d, ifft_d, frame_counter, flagged, n_flagged, tail_ctr, sel_flag,
+  size_t colsum_f, ifft_f, colsum_d, ifft_d, frame_counter, head_counter, flagged, n_flagged, tail_ctr, sel_flag,
       seg_flag, stat_refined, dev_status, att_acc;
   size_t q64, qnorm, s_frm, s_seg, s_pat, f_frm, f_seg, f_pat, wtab, total;
   size_t zero_begin, zero_end;          // region that must start as zeros
@@ -289,6 +289,7 @@ WorkLayout work_layout(const mukv_config& c) {
   w.ifft_d = off;         off = align_up(off + F * Ls * c.n_kv_heads * P * sizeof(double));
   w.zero_begin = off;
   w.frame_counter = off;  off = align_up(off + F * sizeof(int));
+  w.head_counter = off;   off = align_up(off + F * Ls * c.n_q_heads * sizeof(int));
   w.flagged = off;        off = align_up(off + F * sizeof(int));
   w.n_flagged = off;      off = align_up(off + 2 * sizeof(int));   // alternate between chunks
   w.tail_ctr = off;       off = align_up(off + 2 * sizeof(int));
@@ -368,21 +369,22 @@ cudaError_t raise_score_limits(int optin) {
 constexpr int kMaxDevices = 64;
 std::mutex g_dev_mutex;
 bool g_limits_raised[kMaxDevices];
+int g_redo_per_sm[kMaxDevices];
 
 // Once per device (that device current): the dynamic shared-memory limit of every kernel that
 // needs more than the default goes to the device's maximum.  The limit belongs to the kernel,
 // not to a context, so it is never set to one context's need: a second context of another
 // shape, or the allocation-free entry point, would otherwise find it too low.
-cudaError_t raise_kernel_limits(int* n_sms) {
+// redo_capacity: blocks of redo_flagged that may wait for one another, i.e. are resident at once, whichever kernel they are blocks of.
+cudaError_t raise_kernel_limits(int* n_sms, int* redo_capacity) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if (n_sms) {
-    e = cudaDeviceGetAttribute(n_sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-  }
+  e = cudaDeviceGetAttribute(n_sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(g_dev_mutex);
+  if (redo_capacity) *redo_capacity = g_redo_per_sm[dev] * *n_sms;
   if (g_limits_raised[dev]) return cudaSuccess;
   int optin = 0;
   e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -393,6 +395,20 @@ cudaError_t raise_kernel_limits(int* n_sms) {
   if (e == cudaSuccess) e = raise_smem_limit((const void*)score_ps_kernel<false, false>, optin);
   if (e == cudaSuccess) e = raise_smem_limit((const void*)score_ps_kernel<true, false>, optin);
   if (e == cudaSuccess) e = raise_smem_limit((const void*)score_ps_kernel<false, true>, optin);
+  if (e == cudaSuccess) {
+    typedef __nv_bfloat16 B16;
+    int least = 1 << 30;
+    for (const void* fn : {(const void*)compact_kernel<B16, false, false>, (const void*)compact_kernel<B16, false, true>,
+                           (const void*)compact_kernel<B16, true, false>, (const void*)compact_kernel<B16, true, true>,
+                           (const void*)tail_kernel<float>}) {
+      int per_sm = 0;
+      if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kCompactThreads, 0);
+      least = std::min(least, per_sm);
+    }
+    if (e == cudaSuccess && least < 1) e = cudaErrorInvalidConfiguration;
+    g_redo_per_sm[dev] = least;
+    if (redo_capacity) *redo_capacity = least * *n_sms;
+  }
   if (e == cudaSuccess) g_limits_raised[dev] = true;
   return e;
 }
@@ -645,6 +661,7 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
   sp.colsum_part = ctx->ws + ctx->wl.colsum_f;
   sp.ifft_part = ctx->ws + ctx->wl.ifft_f;
   sp.frame_counter = reinterpret_cast<int*>(ctx->ws + ctx->wl.frame_counter);
+  sp.head_counter = reinterpret_cast<int*>(ctx->ws + ctx->wl.head_counter);
   sp.flagged = reinterpret_cast<int*>(ctx->ws + ctx->wl.flagged);
   sp.n_flagged = reinterpret_cast<int*>(ctx->ws + ctx->wl.n_flagged) + ctx->parity;
   sp.kept_store = reinterpret_cast<int*>(ctx->store + ctx->sl.kept);
@@ -808,13 +825,15 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
   // 300 with parts; calls of 7 frames and 24 layers, which get two parts: no difference.)
   cp.parts = 1;
   while (cp.parts < 4 && 4LL * n * L * cp.parts <= 3LL * ctx->n_sms && C * ctx->esize / (2 * cp.parts) >= 256) cp.parts *= 2;
-  // Flagged frames (frame-level selection by Eq. 1-4 only): blocks that redo them, one per SM, fewer when a frame has less work.
+  // Flagged frames (frame-level selection by Eq. 1-4 only): blocks that redo them, as many as are resident at once, fewer
+  // when a frame has less work (one per SM: they start wherever a place comes free, three of them on some SMs, none on others).
   // They are blocks of the compaction kernel, which spares the calls that flag nothing a launch.  fp32 calls keep the launch:
   // a hundredth of their time, behind a kernel of twice the bytes.
   int redo = 0;
   if (!seg_scope && !d_ext) {
     const int units = ctx->Ls * c.n_q_heads * ((P + 7) / 8), planes = 4 * L + 1;
-    redo = std::min(std::min(std::max(units, planes), ctx->redo_capacity), ctx->n_sms);
+    const int others = n * (L * 2 * cp.parts + (c.patch_split > 0 ? 1 : 0) + cp.prev_rows), room = ctx->redo_capacity - others;
+    redo = std::min(std::max(units, planes), room <= 0 ? ctx->redo_capacity : std::max(room, ctx->n_sms));
     cp.colsum_d = reinterpret_cast<double*>(ctx->ws + ctx->wl.colsum_d);
     cp.ifft_d = reinterpret_cast<double*>(ctx->ws + ctx->wl.ifft_d);
     cp.sp.scratch_rows = (int)std::min<size_t>(refine_rows(c), 0x7fffffff);
@@ -823,7 +842,10 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
   {
     ProfScope ps(ctx, 2, st);
     const int rows = L * 2 * cp.parts + (c.patch_split > 0 ? 1 : 0) + cp.prev_rows + (cp.redo_blocks + n - 1) / n;
-    e = launch_k(compact_kernel<T>, dim3(n, rows), kCompactThreads, 0, st, !ctx->prof_on, cp);
+    const bool sel = cp.sel_mode == 1;
+    e = launch_k(cp.parts > 1 ? (sel ? compact_kernel<T, true, true> : compact_kernel<T, true, false>)
+                              : (sel ? compact_kernel<T, false, true> : compact_kernel<T, false, false>),
+                 dim3(n, rows), kCompactThreads, 0, st, !ctx->prof_on, cp);
   }
   if (e != cudaSuccess) return broke_off(ctx, "compact kernel", e);
   ctx->seg_pending = false;
@@ -1090,15 +1112,7 @@ mukv_status create_impl(const mukv_config* cfg, void* d_store, size_t store_byte
   ctx->flag_margin = kFlagMargin;
   ctx->flat_ratio = kFlatRatio;
   const int D = cfg->head_dim;
-  cudaError_t e = raise_kernel_limits(&ctx->n_sms);
-  if (e == cudaSuccess) {
-    // the blocks of redo_flagged wait for one another: all of them must be resident
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, cfg->dtype == MUKV_BF16 ? (const void*)compact_kernel<__nv_bfloat16> : (const void*)tail_kernel<float>, kCompactThreads, 0);
-    if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
-    ctx->redo_capacity = per_sm * ctx->n_sms;
-  }
+  cudaError_t e = raise_kernel_limits(&ctx->n_sms, &ctx->redo_capacity);
   if (e == cudaSuccess && (ctx->tcs.ok || ctx->tcs.split)) {
     e = cudaMemcpy(ctx->ws + ctx->wl.wtab, dft_terms(D), dft_bytes(D), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !encode_map2(&ctx->wmap, ctx->ws + ctx->wl.wtab, D, 3LL * D, D)) e = cudaErrorInvalidValue;
@@ -1449,8 +1463,8 @@ constexpr size_t kNaTs = kNaKept + (size_t)kNaFrames * kNaP * sizeof(int);
 constexpr size_t kNaPt = kNaTs + 256;
 constexpr size_t kNaW128 = kNaPt + 256;                  // DFT matrix terms, D = 128 and D = 64
 constexpr size_t kNaW64 = kNaW128 + 3 * 128 * 128 * 2;
-constexpr size_t kNaCtrl = kNaW64 + 3 * 64 * 64 * 2;     // frame_counter[16], flagged[16], n_flagged, status
-constexpr size_t kNaCtrlBytes = 256;
+constexpr size_t kNaCtrl = kNaW64 + 3 * 64 * 64 * 2;     // frame_counter[16], flagged[16], n_flagged, status; at 256: head_counter
+constexpr size_t kNaCtrlBytes = 256 + (size_t)kNaFrames * kNaHq * sizeof(int);
 constexpr size_t kNaAtt = kNaCtrl + kNaCtrlBytes;        // column sums of the tensor-core path: zeroed together with the words
 constexpr size_t kNaTotal = kNaAtt + (size_t)kNaFrames * kNaP * sizeof(unsigned long long);
 
@@ -1473,7 +1487,7 @@ cudaError_t noalloc_setup(int dev, const NoallocDevice** out) {
     if (d.ptr) { *out = &d; return cudaSuccess; }
   }
   int n_sms = 0;
-  cudaError_t e = raise_kernel_limits(&n_sms);
+  cudaError_t e = raise_kernel_limits(&n_sms, nullptr);
   if (e != cudaSuccess) return e;
   std::lock_guard<std::mutex> lock(g_dev_mutex);
   if (!d.ptr) {
@@ -1524,6 +1538,7 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
   sp.colsum_part = base + kNaColF;
   sp.ifft_part = base + kNaFftF;
   sp.frame_counter = reinterpret_cast<int*>(base + kNaCtrl);
+  sp.head_counter = reinterpret_cast<int*>(base + kNaCtrl + 256);
   sp.flagged = reinterpret_cast<int*>(base + kNaCtrl) + kNaFrames;
   sp.n_flagged = reinterpret_cast<int*>(base + kNaCtrl) + 2 * kNaFrames;
   sp.kept_store = d_kept_out ? d_kept_out : reinterpret_cast<int*>(base + kNaKept);

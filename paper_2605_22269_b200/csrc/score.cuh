@@ -37,6 +37,7 @@ struct ScoreParams {
   void* colsum_part;            // A [F][Ls * Hq * row_split][P]
   void* ifft_part;              // A [F][Ls * Hkv][P]
   int* frame_counter;           // [F], zero between launches
+  int* head_counter;            // [places][heads], too: see finish_frame
   int* flagged;                 // [F] frame slots needing the double pass
   int* n_flagged;               // count (written by the float pass, read by the double pass)
   // outputs
@@ -282,13 +283,14 @@ __device__ inline void select_frame(const ScoreParams& p, int f, const double (&
   }
 }
 
-// Sums over n rows of P values, rows in order inside an eighth, then the eighths in order: thread t < P of a block of
-// kScoreThreads gets column t.  A warp takes an eighth of the rows, a lane of it every 32nd column: all loads of a thread are
-// independent (one thread per column walks n round trips to L2: 6 us for 112 rows).  part: [kScoreWarps][256].
+// Sums over n rows of P values (`stride` rows apart), rows in order inside an eighth, then the eighths in order: thread t < P of a
+// block of kScoreThreads gets column t.  A warp takes an eighth of the rows, a lane of it every 32nd column: all loads of a
+// thread are independent (one thread per column walks n round trips to L2: 6 us for 112 rows).  part: [kScoreWarps][256].
 template <typename A>
-__device__ inline double column_sums(const A* rows, int n, int P, double (*part)[256]) {
+__device__ __noinline__ double column_sums(const A* rows, int n, int stride, int P, double (*part)[256]) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int per = (n + kScoreWarps - 1) / kScoreWarps, r0 = min(n, warp * per), r1 = min(n, r0 + per);
+#pragma unroll 1
   for (int c0 = lane; c0 < P; c0 += 64) {                  // two columns at a time, eight rows in flight
     double t0 = 0.0, t1 = 0.0;
     const bool two = c0 + 32 < P;
@@ -296,8 +298,8 @@ __device__ inline double column_sums(const A* rows, int n, int P, double (*part)
       A x0[8], x1[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        x0[i] = r + i < r1 ? __ldcg(rows + (long long)(r + i) * P + c0) : (A)0;
-        x1[i] = two && r + i < r1 ? __ldcg(rows + (long long)(r + i) * P + c0 + 32) : (A)0;
+        x0[i] = r + i < r1 ? __ldcg(rows + (long long)(r + i) * stride * P + c0) : (A)0;
+        x1[i] = two && r + i < r1 ? __ldcg(rows + (long long)(r + i) * stride * P + c0 + 32) : (A)0;
       }
 #pragma unroll
       for (int i = 0; i < 8; ++i) { t0 += (double)x0[i]; t1 += (double)x1[i]; }
@@ -313,26 +315,42 @@ __device__ inline double column_sums(const A* rows, int n, int P, double (*part)
   return t;
 }
 
-// Every block that has written its share of a frame's partial sums (column sums [heads * RS][P] and frequency sums [key
-// heads][P], at place sf) calls this; the one that arrives last finishes Eq. 1 / Eq. 3 and selects, unless no_select.  Run by
-// a whole block.  refined: the selection is final (see select_frame).
-template <typename A>
-__device__ inline void finish_frame(const ScoreParams& p, const A* colsum, const A* ifft, int f, int sf, int RS, bool refined,
-                                    FinishScratch* s) {
-  const int tid = threadIdx.x, P = p.P, HqV = p.Ls * p.Hq, HkvV = p.Ls * p.Hkv;
+// true in every thread of the block that arrives last of n at *ctr, which is then zero again; what the others wrote before
+// is visible to it
+__device__ inline bool arrives_last(int* ctr, int n, int* s_flag) {
   __threadfence();
   __syncthreads();
-  if (tid == 0) {
-    const int old = atomicAdd(p.frame_counter + f, 1);
-    s->ints[63] = (old == HqV * RS - 1);
-    if (old == HqV * RS - 1) p.frame_counter[f] = 0;  // ready for the next launch
+  if (threadIdx.x == 0) {
+    const int old = atomicAdd(ctr, 1);
+    *s_flag = old == n - 1;
+    if (old == n - 1) *ctr = 0;                            // ready for the next launch
   }
   __syncthreads();
-  if (!s->ints[63] || p.no_select) return;
-  __threadfence();
+  const bool last = *s_flag != 0;
+  if (last) __threadfence();
+  __syncthreads();
+  return last;
+}
+
+// Every block that has written its share of a frame's partial sums (column sums [heads][RS][P] and frequency sums [key
+// heads][P], at place sf) calls this.  The last block of a head adds up its parts (in the row of the first; 392 rows of a frame
+// split over the device took one block 15 us), the last one of the frame finishes Eq. 1 / Eq. 3 and selects.  Run by a whole
+// block.  refined: the selection is final (see select_frame).
+template <typename A>
+__device__ inline void finish_frame(const ScoreParams& p, A* colsum, const A* ifft, int f, int sf, int hv, int RS, bool refined,
+                                    FinishScratch* s) {
+  if (p.no_select) return;
+  const int tid = threadIdx.x, P = p.P, HqV = p.Ls * p.Hq, HkvV = p.Ls * p.Hkv;
+  A* rows = colsum + (long long)sf * HqV * RS * P;
+  if (RS > 1) {
+    if (!arrives_last(p.head_counter + sf * HqV + hv, RS, s->ints)) return;
+    const double t = column_sums(rows + (long long)hv * RS * P, RS, 1, P, s->part);
+    if (tid < P) rows[(long long)hv * RS * P + tid] = (A)t;
+  }
+  if (!arrives_last(p.frame_counter + f, HqV, s->ints)) return;
   double att[1], fft[1];
-  att[0] = column_sums(colsum + (long long)sf * HqV * RS * P, HqV * RS, P, s->part) / (double)((long long)HqV * P);
-  fft[0] = column_sums(ifft + (long long)sf * HkvV * P, HkvV, P, s->part) / (double)((long long)HkvV * p.D);
+  att[0] = column_sums(rows, HqV, RS, P, s->part) / (double)((long long)HqV * P);
+  fft[0] = column_sums(ifft + (long long)sf * HkvV * P, HkvV, 1, P, s->part) / (double)((long long)HkvV * p.D);
   select_frame<1>(p, f, att, fft, refined, s->sc, s->ints, s->misc);
 }
 
@@ -505,7 +523,7 @@ __device__ __forceinline__ void score_frame_block(const ScoreParams& p, int hv, 
     }
   }
 
-  finish_frame(p, reinterpret_cast<const A*>(p.colsum_part), reinterpret_cast<const A*>(p.ifft_part), f, f, 1, false, fin);
+  finish_frame(p, reinterpret_cast<A*>(p.colsum_part), reinterpret_cast<const A*>(p.ifft_part), f, f, hv, 1, false, fin);
 }
 
 // Grid (query heads of all scoring layers, frames).

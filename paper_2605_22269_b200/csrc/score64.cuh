@@ -7,9 +7,10 @@
 // from global memory (a key head of 50 KB stays in L1), keeps their column sums in registers over the row tiles and exchanges
 // (maximum, sum) with the others once per row tile.
 // Bound by the fp64 tensor instruction and the conversions: the 138 M multiply-adds of a frame of 28 heads x 196 tokens x 128
-// channels are 7.6 us of the whole device.  (One multiply-add per lane and 32-bit word out of shared memory, with a conversion for
-// each, took 110 us a frame.)  No more than 80 registers and no dynamic shared memory, so that the blocks of this pass can be
-// blocks of compact_kernel: as a launch of its own behind every call it cost the calls that flag nothing 1 to 2 us.
+// channels are 7.6 us of the whole device; a flagged frame takes a call 75 us all the same, most of it code that comes from device
+// memory.  (One multiply-add per lane and 32-bit word out of shared memory, with a conversion for each: 130 us.)  No more
+// than 80 registers and no dynamic shared memory, so that the blocks of this pass can be blocks of compact_kernel: as a launch of
+// its own behind every call it cost the calls that flag nothing 1 to 2 us (sixteen calls of one frame 297 us, now 271).
 #pragma once
 #include "common.cuh"
 #include "score.cuh"
@@ -32,6 +33,10 @@ __device__ __forceinline__ double elem64(const uint4& x, int e) {
   if constexpr (sizeof(T) == 2) return (double)((e & 1) ? bf16_hi(w[e >> 1]) : bf16_lo(w[e >> 1]));
   else return (double)__uint_as_float(w[e]);
 }
+
+// (Out of line, like the other long pieces of this pass: it runs for one call in fifty, and its instructions come from device
+// memory then, a microsecond for every two or three hundred bytes in a row.)
+__device__ __noinline__ double exp64(double x) { return exp(x); }
 
 // The work of one block: part q (of RS) of the query rows of head hv of frame f (a frame slot of the chunk); hv counts the
 // query heads of all scoring layers, layer-major.  The partial sums go to place sf of colsum [places][heads * RS][P] and ifft
@@ -99,17 +104,12 @@ __device__ __noinline__ void score64_frame_block(const ScoreParams& p, double* c
         if (t < my) {
           const uint4 y0 = xb[t], y1 = xb[t + 1];
           xb[t] = __ldg(reinterpret_cast<const uint4*>(krow[t] + nb * 4 * VE));
-          if (t + 1 < my) {
-            xb[t + 1] = __ldg(reinterpret_cast<const uint4*>(krow[t + 1] + nb * 4 * VE));
+          if (t + 1 < my) xb[t + 1] = __ldg(reinterpret_cast<const uint4*>(krow[t + 1] + nb * 4 * VE));
 #pragma unroll
-            for (int s = 0; s < VE; ++s) {
-              const double a = elem64<T>(ya, s);
-              dmma_m8n8k4(acc[t], a, elem64<T>(y0, s));
-              dmma_m8n8k4(acc[t + 1], a, elem64<T>(y1, s));
-            }
-          } else {
-#pragma unroll
-            for (int s = 0; s < VE; ++s) dmma_m8n8k4(acc[t], elem64<T>(ya, s), elem64<T>(y0, s));
+          for (int s = 0; s < VE; ++s) {
+            const double a = elem64<T>(ya, s);
+            dmma_m8n8k4(acc[t], a, elem64<T>(y0, s));
+            if (t + 1 < my) dmma_m8n8k4(acc[t + 1], a, elem64<T>(y1, s));
           }
         }
       }
@@ -138,7 +138,7 @@ __device__ __noinline__ void score64_frame_block(const ScoreParams& p, double* c
       if (t < my) {
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-          acc[t][e] = acc[t][e] == -(double)INFINITY ? 0.0 : exp(acc[t][e] - m);
+          acc[t][e] = acc[t][e] == -(double)INFINITY ? 0.0 : exp64(acc[t][e] - m);
           l += acc[t][e];
         }
       }
@@ -157,12 +157,12 @@ __device__ __noinline__ void score64_frame_block(const ScoreParams& p, double* c
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       const double2 v = x[2 * fk + c][fr];
-      sum += v.y * (v.x == -(double)INFINITY ? 1.0 : exp(v.x - mm));   // (a share without a visible key has the sum 0)
+      sum += v.y * (v.x == -(double)INFINITY ? 1.0 : exp64(v.x - mm));   // (a share without a visible key has the sum 0)
     }
     __syncwarp();
     sum += __shfl_xor_sync(kFull, sum, 1);
     sum += __shfl_xor_sync(kFull, sum, 2);
-    const double w = (m == -(double)INFINITY ? 1.0 : exp(m - mm)) / sum;
+    const double w = (m == -(double)INFINITY ? 1.0 : exp64(m - mm)) / sum;
 #pragma unroll
     for (int t = 0; t < kScore64Tiles; ++t) {
       if (t < my) {
@@ -227,7 +227,7 @@ __device__ __noinline__ void score64_frame_block(const ScoreParams& p, double* c
     }
     __syncthreads();
   }
-  finish_frame(p, colsum, ifft, f, sf, RS, true, &sc->fin);
+  finish_frame(p, colsum, ifft, f, sf, hv, RS, true, &sc->fin);
 }
 
 // Parts into which the query rows of a head are split: as many as give every one of `blocks` blocks something to do, while
