@@ -320,22 +320,35 @@ WorkLayout work_layout(const mukv_config& c) {
 int pick_nc(int P) { return P <= 64 ? 2 : P <= 128 ? 4 : P <= 224 ? 7 : 8; }
 
 // Launches a kernel; with `dependent` it may be scheduled while the previous kernel of the stream
-// still runs (programmatic dependent launch: the kernel itself waits in pdl_wait()).
+// still runs (programmatic dependent launch: the kernel itself waits in pdl_wait()).  cluster > 1: that many
+// neighbouring blocks form a cluster.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t st,
-                     bool dependent, Args... args) {
+cudaError_t launch_c(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t st,
+                     bool dependent, unsigned cluster, Args... args) {
   cudaLaunchConfig_t cfg;
   memset(&cfg, 0, sizeof cfg);
   cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
+  if (dependent) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = cluster;
+    attr[cfg.numAttrs].val.clusterDim.y = attr[cfg.numAttrs].val.clusterDim.z = 1;
+    ++cfg.numAttrs;
+  }
   cfg.attrs = attr;
-  cfg.numAttrs = dependent ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t st,
+                     bool dependent, Args... args) {
+  return launch_c(kernel, grid, block, smem, st, dependent, 1u, args...);
 }
 
 template <typename T>
@@ -987,13 +1000,18 @@ mukv_status retrieve_impl(mukv_ctx* ctx, const void* d_qtok, const int32_t* h_q_
       rp.f_frm = reinterpret_cast<const float*>(ctx->ws + ctx->wl.f_frm); rp.f_frm_stride = pad4(c.max_frames);
       rp.f_seg = reinterpret_cast<const float*>(ctx->ws + ctx->wl.f_seg); rp.f_seg_stride = pad4(ctx->sl.max_segs);
       rp.f_pat = reinterpret_cast<const float*>(ctx->ws + ctx->wl.f_pat); rp.f_pat_stride = pad4((long long)c.max_frames * S);
+      // (of each granularity the copies that fit, in its own block; none where a question sees too few for it)
       const size_t room = (size_t)kRankStageBytes - rank_smem;
-      const size_t b1 = (size_t)(pad4(n_seg) + pad4(n_frm)) * sizeof(float);
-      const size_t b2 = (size_t)(pad4(n_seg) + pad4(n_pat)) * sizeof(float);
-      if (b1 <= room) rp.stage |= 1;
-      if (n_pat > 0 && b2 <= room) rp.stage |= 2;
-      rank_smem += rp.stage == 3 ? (b1 > b2 ? b1 : b2) : rp.stage == 2 ? b2 : rp.stage == 1 ? b1 : 0;
-      e = launch_k(rank_kernel, dim3(nq, k_pat > 0 ? 2 : 1), kRankThreads, rank_smem, st, !ctx->prof_on, rp, meta);
+      size_t stage = 0;
+      const long long counts[3] = {n_seg, n_frm, n_pat};
+      for (int i = 0; i < 3; ++i) {
+        const size_t b = (size_t)pad4(counts[i]) * sizeof(float);
+        if (counts[i] <= kRankFew || b > room || (i > 0 && mode == MUKV_RETR_HIER)) continue;
+        rp.stage |= 1 << i;
+        stage = std::max(stage, b);
+      }
+      const unsigned roles = k_pat > 0 ? 3 : 2;
+      e = launch_c(rank_kernel, dim3(nq * roles), kRankThreads, rank_smem + stage, st, !ctx->prof_on, roles, rp, meta);
     }
     if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "rank kernel: %s", cudaGetErrorString(e));
     ctx->launches += 4;

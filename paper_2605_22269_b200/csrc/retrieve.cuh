@@ -8,8 +8,7 @@
 //   scan_kernel     Eq. 7   cosine of every question with every frame, segment and patch-level key (a skinny
 //                           double-precision product on the fp64 tensor-core instruction)
 //   scan_few_kernel         the same for at most eight questions, a warp per row or two
-//   rank_kernel     stage-1 candidates, Eq. 8 rerank, final top-k; one block per question, a second one for its
-//                   patch-level blocks
+//   rank_kernel     stage-1 candidates, Eq. 8 rerank, final top-k; per question a cluster of blocks, one for each granularity
 //   gather_kernel   Eq. 9   copies the selected pages into the per-question decode buffers
 //   gather3_kernel          the same with summary tokens and the rows of patch-level blocks
 #pragma once
@@ -757,8 +756,7 @@ struct RankParams {
   int* counts; int counts_stride;         // 2 or 3 ints per question
   const float* f_frm; const float* f_seg; const float* f_pat;     // single-precision copies of the scores
   long long f_frm_stride, f_seg_stride, f_pat_stride;
-  int stage;                              // bit 0: the copies of segments and frames fit in shared memory, bit 1: those of
-                                          // segments and patch-level blocks
+  int stage;                              // bits 0, 1, 2: the copies of segments, frames, patch-level blocks fit in shared memory
 };
 
 constexpr int kRankThreads = 512;
@@ -776,19 +774,32 @@ struct RankShared {
   int pick[MUKV_MAX_TOPK];
   double pick_score[MUKV_MAX_TOPK];
   double gn[kRankThreads / 32];
+  // what the block of the segments finds for the others
+  double gnorm;
+  int have_g, c_seg;
 };
 
 // Stage 1 + stage 2 of one granularity for one question, run by the whole block: top-2k candidates
 // by cosine among the members, Eq. 8 against the global query gq (norm gnorm; have_g false: gamma = 0),
 // then the k best by the calibrated score.  PARALLEL / HIER callers pass semi = false: the k best by
 // cosine among the members.  Results (ascending ids) in sh->pick / sh->pick_score; returns the count.
+// remote: the global query is fetched from the block of the segments between the stages, see rank_kernel.
 __device__ __noinline__ int rank_level(const double* scores, const int* cnt, int n, int k, bool semi, double lambda,
-                                       double delta, const float* keys, int C, const double* gq, double gnorm,
-                                       bool have_g, RankShared* sh, float* buf) {
+                                       double delta, const float* keys, int C, double* gq, bool remote, RankShared* sh,
+                                       float* buf) {
   const int tid = threadIdx.x;
   const int n_cand = topk_set(scores, cnt, n, semi ? 2 * k : k, delta, semi ? sh->cand : sh->pick,
                               semi ? sh->cand_score : sh->pick_score, buf, &sh->sc);
   if (!semi) return n_cand;
+  if (remote) {
+    tc::cluster_wait();
+    for (int c = tid; c < C; c += kRankThreads) gq[c] = tc::cluster_ld_double(gq + c, 0);
+    if (tid == 0) { sh->gnorm = tc::cluster_ld_double(&sh->gnorm, 0); sh->have_g = tc::cluster_ld_int(&sh->have_g, 0); }
+    tc::cluster_arrive();                                    // that block may leave
+    __syncthreads();
+  }
+  const double gnorm = sh->gnorm;
+  const bool have_g = sh->have_g != 0;
   // Eq. 8 for every candidate: one warp per candidate
   const int lane = tid & 31, warp = tid >> 5;
   for (int ci = warp; ci < n_cand; ci += kRankThreads / 32) {
@@ -836,16 +847,20 @@ __device__ __forceinline__ void rank_emit(int* idx, float* score, long long base
   }
 }
 
-// Grid (questions, 1 or 2): with patch-level blocks a second block per question ranks them beside the frames; it finds the
-// segments again, which both need.  (One block for all: 42 us for eight questions on 1,800 frames; so: 28.)
+// A cluster of two or three blocks per question, one for each granularity: block 0 ranks the segments and works out the global
+// query, block 1 the frames, block 2 (k_pat > 0) the patch-level blocks.  Stage 1 needs nothing of the other blocks, stage 2 the
+// global query, which is read from block 0's shared memory behind a cluster barrier.  (One block after the other: 14.5 us for
+// one question on an hour of video, of which the segments and the global query were 5; bound by a chain of barriers, round
+// trips to L2 and instruction fetch, so that blocks beside one another are what helps.)
 __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, const QMeta meta) {
   __shared__ RankShared sh;
-  __shared__ __align__(8) uint64_t s_bar[3];
+  __shared__ __align__(8) uint64_t s_bar[1];
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* gq = reinterpret_cast<double*>(smem_raw);               // [C] global query
 
-  const int qi = blockIdx.x, tid = threadIdx.x;
-  const bool do_frm = blockIdx.y == 0, do_pat = p.k_pat > 0 && blockIdx.y + 1 == gridDim.y;
+  const int role = (int)tc::cluster_rank(), roles = p.k_pat > 0 ? 3 : 2;
+  const int qi = blockIdx.x / roles, tid = threadIdx.x;
+  if (role > 0) tc::cluster_arrive();                        // (phase 1: block 0 arrives when the others may go on)
   pdl_wait();                                                // the scores of the scan are complete
   if (p.nq <= kScanFew) pdl_trigger();                       // (many of these blocks would leave the gather an uneven start)
   const int C = p.C;
@@ -860,146 +875,127 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
   const double* sf = p.s_frm + (long long)qi * p.frm_stride;
   const double* ss = p.s_seg + (long long)qi * p.seg_stride;
   const double* sp = p.s_pat + (long long)qi * p.pat_stride;
-  // Single-precision copies of the scores, on their way while the segments are ranked.  (n4 values each: what lies
-  // behind the n-th belongs to this question's row, too)
-  float *buf_s = nullptr, *buf_f = nullptr, *buf_p = nullptr;
-  const int s4 = (n_seg + 3) & ~3, f4 = do_frm ? (n_frm + 3) & ~3 : 0, p4 = do_pat ? (n_frm * p.S + 3) & ~3 : 0;
-  const uint32_t bar0 = tc::smem_u32(s_bar);
-  auto load = [&](float* dst, const float* src, int n4, int bar) {
-    tc::mbar_expect_tx(bar0 + 8u * bar, 4u * (uint32_t)n4);
-    tc::bulk_load(tc::smem_u32(dst), src, 4u * (uint32_t)n4, bar0 + 8u * bar);
-  };
-  if (p.stage) {
-    buf_s = reinterpret_cast<float*>(gq + C);
-    if (do_frm && (p.stage & 1)) buf_f = buf_s + s4;
-    if (do_pat && (p.stage & 2)) buf_p = buf_s + s4;       // (in a block of its own)
+  const bool semi = p.mode == MUKV_RETR_SEMI, hier = p.mode == MUKV_RETR_HIER;
+  // Single-precision copies of this block's scores.  (n4 values: what lies behind the n-th belongs to this question's row, too)
+  const int n = role == 0 ? n_seg : role == 1 ? n_frm : n_frm * p.S, n4 = (n + 3) & ~3;
+  float* buf = nullptr;
+  // (few scores are all read as they are; HIER looks at the selected segments' frames only)
+  if (((p.stage >> role) & 1) && n > kRankFew && !(hier && role > 0)) {
+    buf = reinterpret_cast<float*>(gq + C);
+    const float* src = role == 0 ? p.f_seg + (long long)qi * p.f_seg_stride
+                       : role == 1 ? p.f_frm + (long long)qi * p.f_frm_stride : p.f_pat + (long long)qi * p.f_pat_stride;
+    const uint32_t bar = tc::smem_u32(s_bar);
     if (tid == 0) {
-      for (int b = 0; b < 3; ++b) tc::mbar_init(bar0 + 8u * b, 1);
+      tc::mbar_init(bar, 1);
       tc::fence_mbar_init();
       tc::fence_proxy_async_smem();
-      if (s4) load(buf_s, p.f_seg + (long long)qi * p.f_seg_stride, s4, 0);
-      if (buf_f && f4) load(buf_f, p.f_frm + (long long)qi * p.f_frm_stride, f4, 1);
-      if (buf_p && p4) load(buf_p, p.f_pat + (long long)qi * p.f_pat_stride, p4, 2);
+      tc::mbar_expect_tx(bar, 4u * (uint32_t)n4);
+      tc::bulk_load(tc::smem_u32(buf), src, 4u * (uint32_t)n4, bar);
     }
     __syncthreads();
+    // a wait that runs out (it cannot, the copy needs nothing else) leaves the doubles in global memory to rank by
+    if (!__syncthreads_and(tc::mbar_wait(bar, 0u))) buf = nullptr;
   }
-  // a wait that runs out (it cannot, the copies need nothing else) leaves the doubles in global memory to rank by
-  auto landed = [&](float* buf, int n4, int bar) -> float* {
-    if (!buf || !n4) return nullptr;
-    const bool ok = tc::mbar_wait(bar0 + 8u * bar, 0u);
-    return __syncthreads_and(ok) ? buf : nullptr;
-  };
-  float* const seg_buf = landed(buf_s, s4, 0);
-  const bool semi = p.mode == MUKV_RETR_SEMI;
 
-  // ---- global query = mean of the top-N segment keys (stage 1 order)
-  bool have_g = false;
-  double gnorm = 0.0;
-  int c_seg = -1;
-  if (semi) {
-    const int N = p.top_n > 0 ? p.top_n : p.k_seg;
-    // (without a lambda for segments the N = k_seg best are also the result: one ranking serves both)
-    const bool same = N == p.k_seg && !(p.lam_seg > 0.0);
-    int* top = same ? sh.pick : sh.top;
-    double* top_score = same ? sh.pick_score : sh.cand_score;
-    const int n_top = topk_set(ss, nullptr, n_seg, N, p.delta, top, top_score, seg_buf, &sh.sc);
-    if (same) c_seg = n_top;
-    const int n_use = __syncthreads_count(tid < n_top && !no_score(top_score[tid]));      // (N <= threads of the block)
-    if (n_use < n_top) {                                     // the list without those that have no score
-      if (tid == 0)
-        for (int i = 0, c = 0; i < n_top; ++i)
-          if (!no_score(top_score[i])) sh.top[c++] = top[i];
-      __syncthreads();
-      top = sh.top;
-    }
-    double part = 0.0;
-    for (int c = tid; c < C; c += kRankThreads) {
-      double t = 0.0;
-      for (int i = 0; i < n_use; i += 8) {                   // (eight loads in flight, added in order)
-        float x[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-          x[u] = i + u < n_use ? p.seg_key[(long long)top[i + u] * C + c] : 0.f;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) t += (double)x[u];
+  if (role == 0) {
+    int c_seg = -1;
+    if (semi) {
+      // ---- global query = mean of the top-N segment keys (stage 1 order)
+      const int N = p.top_n > 0 ? p.top_n : p.k_seg;
+      // (without a lambda for segments the N = k_seg best are also the result: one ranking serves both)
+      const bool same = N == p.k_seg && !(p.lam_seg > 0.0);
+      int* top = same ? sh.pick : sh.top;
+      double* top_score = same ? sh.pick_score : sh.cand_score;
+      const int n_top = topk_set(ss, nullptr, n_seg, N, p.delta, top, top_score, buf, &sh.sc);
+      if (same) c_seg = n_top;
+      const int n_use = __syncthreads_count(tid < n_top && !no_score(top_score[tid]));    // (N <= threads of the block)
+      if (n_use < n_top) {                                   // the list without those that have no score
+        if (tid == 0)
+          for (int i = 0, c = 0; i < n_top; ++i)
+            if (!no_score(top_score[i])) sh.top[c++] = top[i];
+        __syncthreads();
+        top = sh.top;
       }
-      t = n_use > 0 ? t / (double)n_use : 0.0;
-      gq[c] = t;
-      part += t * t;
-    }
-    __syncwarp();
-    part = warp_sum(part);
-    if ((tid & 31) == 0) sh.gn[tid >> 5] = part;
-    __syncthreads();
-    double gn = 0.0;
+      double part = 0.0;
+      for (int c = tid; c < C; c += kRankThreads) {
+        double t = 0.0;
+        for (int i = 0; i < n_use; i += 8) {                 // (eight loads in flight, added in order)
+          float x[8];
 #pragma unroll
-    for (int w = 0; w < kRankThreads / 32; ++w) gn += sh.gn[w];
-    gnorm = sqrt(gn);
-    have_g = n_use > 0;
+          for (int u = 0; u < 8; ++u)
+            x[u] = i + u < n_use ? p.seg_key[(long long)top[i + u] * C + c] : 0.f;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) t += (double)x[u];
+        }
+        t = n_use > 0 ? t / (double)n_use : 0.0;
+        gq[c] = t;
+        part += t * t;
+      }
+      __syncwarp();
+      part = warp_sum(part);
+      if ((tid & 31) == 0) sh.gn[tid >> 5] = part;
+      __syncthreads();
+      double gn = 0.0;
+#pragma unroll
+      for (int w = 0; w < kRankThreads / 32; ++w) gn += sh.gn[w];
+      if (tid == 0) { sh.gnorm = sqrt(gn); sh.have_g = n_use > 0; }
+    }
+    if (!hier) tc::cluster_arrive();
+    __syncthreads();
+    // ---- segments (the paper's lambda for them is 0: final = stage-1 top-k)
+    if (c_seg < 0)
+      c_seg = rank_level(ss, nullptr, n_seg, p.k_seg, semi && p.lam_seg > 0.0, p.lam_seg, p.delta, p.seg_key, C, gq, false, &sh, buf);
+    rank_emit(p.seg_idx, p.seg_score, (long long)qi * p.k_seg, p.k_seg, c_seg, &sh);
+    if (tid == 0) p.counts[p.counts_stride * qi] = c_seg;
+    if (hier) {
+      for (int i = tid; i < c_seg; i += kRankThreads) sh.sel_seg[i] = sh.pick[i];
+      if (tid == 0) sh.c_seg = c_seg;
+      tc::cluster_arrive();
+    }
+    tc::cluster_wait();
+    tc::cluster_arrive();                                    // phase 2: the others have read what they need
+    tc::cluster_wait();
+    return;
   }
 
-  // ---- segments (the paper's lambda for them is 0: final = stage-1 top-k)
-  if (c_seg < 0)
-    c_seg = rank_level(ss, nullptr, n_seg, p.k_seg, semi && p.lam_seg > 0.0, p.lam_seg, p.delta, p.seg_key, C, gq, gnorm,
-                       have_g, &sh, seg_buf);
-  if (do_frm) rank_emit(p.seg_idx, p.seg_score, (long long)qi * p.k_seg, p.k_seg, c_seg, &sh);
-  for (int i = tid; i < c_seg; i += kRankThreads) sh.sel_seg[i] = sh.pick[i];
-  __syncthreads();
-
-  // ---- frames
-  // HIER: only what lies inside the selected segments is a candidate.  Those are few, so the ranking
-  // runs over positions in the list "selected segments (ascending) x their frames" and maps the
-  // winners back (ascending position = ascending frame).
-  const int fseg = p.fseg;
-  int c_frm = 0;
-  float* const frm_buf = landed(buf_f, f4, 1);               // (waited for in every mode: the copy must land before the block leaves)
-  if (!do_frm) {
-  } else if (p.mode == MUKV_RETR_HIER) {
-    auto frame_of = [&](int i) { return sh.sel_seg[i / fseg] * fseg + i % fseg; };
-    auto score_h = [&](int i) { return sf[frame_of(i)]; };
-    auto member_h = [&](int i) { return frame_of(i) < n_frm; };
-    c_frm = block_topk_set(score_h, member_h, c_seg * fseg, p.k_frm, p.delta, sh.pick, sh.pick_score, &sh.sc);
-    for (int i = tid; i < c_frm; i += kRankThreads) sh.pick[i] = frame_of(sh.pick[i]);
+  // ---- frames, or patch-level blocks: (frame, super patch) pairs that kept at least one token
+  const double* sc = role == 1 ? sf : sp;
+  const int* cnt = role == 1 ? nullptr : p.patch_cnt;
+  const int k = role == 1 ? p.k_frm : p.k_pat;
+  int c = 0;
+  if (hier) {
+    // Only what lies inside the selected segments is a candidate.  Those are few, so the ranking runs over positions in the
+    // list "selected segments (ascending) x their blocks" and maps the winners back (ascending position = ascending block).
+    tc::cluster_wait();
+    const int c_seg = tc::cluster_ld_int(&sh.c_seg, 0);
+    for (int i = tid; i < c_seg; i += kRankThreads) sh.sel_seg[i] = tc::cluster_ld_int(sh.sel_seg + i, 0);
+    tc::cluster_arrive();
+    __syncthreads();
+    const int per_seg = p.fseg * (role == 1 ? 1 : p.S);
+    auto block_of = [&](int i) { return sh.sel_seg[i / per_seg] * per_seg + i % per_seg; };
+    auto score_h = [&](int i) { return sc[block_of(i)]; };
+    auto member_h = [&](int i) {
+      const int b = block_of(i);
+      return b < n && (!cnt || cnt[b] > 0);
+    };
+    c = block_topk_set(score_h, member_h, c_seg * per_seg, k, p.delta, sh.pick, sh.pick_score, &sh.sc);
+    for (int i = tid; i < c; i += kRankThreads) sh.pick[i] = block_of(sh.pick[i]);
     __syncthreads();
   } else {
-    c_frm = rank_level(sf, nullptr, n_frm, p.k_frm, semi, p.lam_frm, p.delta, p.frame_key, C, gq, gnorm, have_g, &sh,
-                       frm_buf);
-  }
-  if (do_frm) rank_emit(p.frm_idx, p.frm_score, (long long)qi * p.k_frm, p.k_frm, c_frm, &sh);
-  __syncthreads();
-
-  // ---- patch-level blocks: (frame, super patch) pairs that kept at least one token
-  int c_pat = 0;
-  float* const pat_buf = landed(buf_p, p4, 2);
-  if (do_pat) {
-    const int S = p.S;
-    const int* cnt = p.patch_cnt;
-    if (S > 0) {
-      if (p.mode == MUKV_RETR_HIER) {
-        const int per_seg = fseg * S;
-        auto block_of = [&](int i) { return sh.sel_seg[i / per_seg] * per_seg + i % per_seg; };
-        auto score_h = [&](int i) { return sp[block_of(i)]; };
-        auto member_h = [&](int i) {
-          const int b = block_of(i);
-          return b < n_frm * S && cnt[b] > 0;
-        };
-        c_pat = block_topk_set(score_h, member_h, c_seg * per_seg, p.k_pat, p.delta, sh.pick, sh.pick_score, &sh.sc);
-        for (int i = tid; i < c_pat; i += kRankThreads) sh.pick[i] = block_of(sh.pick[i]);
-        __syncthreads();
-      } else {
-        c_pat = rank_level(sp, cnt, n_frm * S, p.k_pat, semi, p.lam_pat, p.delta, p.patch_key, C, gq, gnorm, have_g, &sh,
-                           pat_buf);
-      }
+    c = rank_level(sc, cnt, n, k, semi, role == 1 ? p.lam_frm : p.lam_pat, p.delta, role == 1 ? p.frame_key : p.patch_key, C, gq,
+                   true, &sh, buf);
+    if (!semi) {
+      tc::cluster_wait();
+      tc::cluster_arrive();
     }
-    rank_emit(p.pat_idx, p.pat_score, (long long)qi * p.k_pat, p.k_pat, c_pat, &sh);
   }
+  if (role == 1) rank_emit(p.frm_idx, p.frm_score, (long long)qi * p.k_frm, p.k_frm, c, &sh);
+  else rank_emit(p.pat_idx, p.pat_score, (long long)qi * p.k_pat, p.k_pat, c, &sh);
   if (tid == 0) {
-    if (do_frm) {
-      p.counts[p.counts_stride * qi] = c_seg;
-      p.counts[p.counts_stride * qi + 1] = c_frm;
-    }
-    if (p.counts_stride > 2 && blockIdx.y + 1 == gridDim.y) p.counts[p.counts_stride * qi + 2] = c_pat;
+    p.counts[p.counts_stride * qi + role] = c;
+    if (roles == 2 && p.counts_stride > 2) p.counts[p.counts_stride * qi + 2] = 0;
   }
+  tc::cluster_wait();
 }
 
 // ------------------------------------------------------------------------------ Eq. 9
