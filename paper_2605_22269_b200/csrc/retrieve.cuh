@@ -734,6 +734,14 @@ __device__ __noinline__ int staged_topk_set(const double* scores, const int* cnt
 // the one of the two that fits (buf: null where there are no copies)
 __device__ __forceinline__ int topk_set(const double* scores, const int* cnt, int n, int k, double delta, int* out_idx,
                                         double* out_score, float* buf, RankScratch* sc) {
+  const int tid = threadIdx.x;
+  if (n <= kRankFew && !cnt) {                               // every score is a candidate
+    __syncthreads();                                         // (the scratch may still be read from a previous call)
+    if (tid < n) { sc->cand_key[tid] = order_key(scores[tid]); sc->cand_idx[tid] = tid; }
+    __syncthreads();
+    k = min(k, n);
+    return k > 0 ? rank_candidates(n, k, k == n, delta, out_idx, out_score, sc) : 0;
+  }
   if (n > kRankFew && buf) return staged_topk_set(scores, cnt, n, k, delta, out_idx, out_score, buf, sc);
   return block_topk_set(ArrScore{scores}, Members{cnt}, n, k, delta, out_idx, out_score, sc);
 }
@@ -770,7 +778,6 @@ struct RankShared {
   int top[MUKV_MAX_TOPK];
   int cand[kMaxCand];
   double cand_score[kMaxCand];
-  double s_new[kMaxCand];
   int pick[MUKV_MAX_TOPK];
   double pick_score[MUKV_MAX_TOPK];
   double gn[kRankThreads / 32];
@@ -829,11 +836,14 @@ __device__ __noinline__ int rank_level(const double* scores, const int* cnt, int
         gamma = dot / den;
       }
       const double s1 = sh->cand_score[ci];
-      sh->s_new[ci] = no_score(s1) ? kScoreNone : (1.0 - lambda) * s1 + lambda * gamma;
+      sh->sc.cand_key[ci] = order_key(no_score(s1) ? kScoreNone : (1.0 - lambda) * s1 + lambda * gamma);
+      sh->sc.cand_idx[ci] = ci;
     }
   }
   __syncthreads();
-  const int c = topk_set(sh->s_new, nullptr, n_cand, k, delta, sh->pick, sh->pick_score, (float*)nullptr, &sh->sc);
+  // (at most 2 k candidates: no more than a thread each)
+  const int c = min(k, n_cand);
+  if (c > 0) rank_candidates(n_cand, c, c == n_cand, delta, sh->pick, sh->pick_score, &sh->sc);
   // pick holds positions in the candidate list (ascending position = ascending block id)
   for (int i = tid; i < c; i += kRankThreads) sh->pick[i] = sh->cand[sh->pick[i]];
   __syncthreads();
