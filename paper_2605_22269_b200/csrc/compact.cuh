@@ -76,6 +76,7 @@ struct CompactParams {
   const unsigned long long* att_acc;  // [F][P] column sums of the persistent scoring kernel (sel_mode 1)
   unsigned long long* att_clear;  // sums of the call before, cleared for the next one
   long long n_clear;
+  int later_blocks;               // 1: the grid is larger than what is resident at once
   unsigned* sel_flag;             // [F] (epoch << 1 | risky) once the plane-0 block has published its frame's ids
   unsigned epoch;                 // number of this call, never repeated
   ScoreParams sp;                 // partial sums, Eq. 4 parameters, index and flag outputs
@@ -769,16 +770,21 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __gri
     __shared__ unsigned s_seen;
     // A block that starts after its frame's plane-0 block has published the ids (the blocks beyond
     // the first wave do) reads them; every other block selects itself.  Nobody waits.
-    if (tid == 0) {
-      unsigned v = 0u;
-      if (!writes) {
-        v = *reinterpret_cast<volatile unsigned*>(p.sel_flag + f);
-        __threadfence();
+    // (A grid that is resident as a whole has no such blocks, and the look costs a round trip to L2: 0.5 us of a one-frame
+    // call of 16.)
+    unsigned seen = 0u;
+    if (p.later_blocks) {
+      if (tid == 0) {
+        unsigned v = 0u;
+        if (!writes) {
+          v = *reinterpret_cast<volatile unsigned*>(p.sel_flag + f);
+          __threadfence();
+        }
+        s_seen = v;
       }
-      s_seen = v;
+      __syncthreads();
+      seen = s_seen;
     }
-    __syncthreads();
-    const unsigned seen = s_seen;
     if ((seen >> 1) == p.epoch) {
       risky = (seen & 1u) != 0u;
       for (int r = tid; r < p.kappa; r += kCompactThreads) cs.kept[r] = token_id(__ldcg(p.sp.kept_store + f_abs * p.kappa + r), p.P);

@@ -856,6 +856,7 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
     ProfScope ps(ctx, 2, st);
     const int rows = L * 2 * cp.parts + (c.patch_split > 0 ? 1 : 0) + cp.prev_rows + (cp.redo_blocks + n - 1) / n;
     const bool sel = cp.sel_mode == 1;
+    cp.later_blocks = (long long)n * rows > ctx->redo_capacity;
     e = launch_k(cp.parts > 1 ? (sel ? compact_kernel<T, true, true> : compact_kernel<T, true, false>)
                               : (sel ? compact_kernel<T, false, true> : compact_kernel<T, false, false>),
                  dim3(n, rows), kCompactThreads, 0, st, !ctx->prof_on, cp);
