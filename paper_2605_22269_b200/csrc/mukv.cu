@@ -404,6 +404,8 @@ cudaError_t raise_kernel_limits(int* n_sms, int* redo_capacity) {
   if (e == cudaSuccess) e = raise_score_limits<__nv_bfloat16>(optin);
   if (e == cudaSuccess) e = raise_score_limits<float>(optin);
   if (e == cudaSuccess) e = raise_smem_limit((const void*)rank_kernel, optin);
+  for (const void* fn : {(const void*)scan_kernel<1>, (const void*)scan_kernel<2>, (const void*)scan_kernel<4>, (const void*)scan_kernel<8>})
+    if (e == cudaSuccess) e = raise_smem_limit(fn, optin);
   if (e == cudaSuccess) e = raise_smem_limit((const void*)segsel_kernel, optin);
   if (e == cudaSuccess) e = raise_smem_limit((const void*)score_ps_kernel<false, false>, optin);
   if (e == cudaSuccess) e = raise_smem_limit((const void*)score_ps_kernel<true, false>, optin);
@@ -955,7 +957,6 @@ mukv_status retrieve_impl(mukv_ctx* ctx, const void* d_qtok, const int32_t* h_q_
     const int S = c.patch_split * c.patch_split;
     const long long n_pat = k_pat > 0 ? n_frm * S : 0;
     const long long rows = n_frm + n_seg + n_pat;
-    const unsigned blocks = (unsigned)((rows + kScanRows - 1) / kScanRows);
     double* s_pat = reinterpret_cast<double*>(ctx->ws + ctx->wl.s_pat);
     const float* patch_key = reinterpret_cast<const float*>(ctx->store + ctx->sl.patch_key);
     {
@@ -977,8 +978,13 @@ mukv_status retrieve_impl(mukv_ctx* ctx, const void* d_qtok, const int32_t* h_q_
         const dim3 grid((unsigned)(want < most ? want : most));
         e = launch_k(nq == 1 ? scan_few_kernel<1> : nq <= 4 ? scan_few_kernel<4> : scan_few_kernel<kScanFew>, grid, 256, 0, st,
                      !ctx->prof_on, sc);
-      } else
-        e = launch_k(scan_kernel, dim3(blocks), 256, 0, st, !ctx->prof_on, sc);
+      } else {
+        const ScanShape sh = scan_shape(rows, nq, ctx->n_sms);
+        sc.q_groups = sh.q_groups; sc.row_tiles = sh.row_tiles;
+        const dim3 grid((unsigned)(((rows + 7) / 8 + sh.row_tiles - 1) / sh.row_tiles));
+        e = launch_k(sh.T == 1 ? scan_kernel<1> : sh.T == 2 ? scan_kernel<2> : sh.T == 4 ? scan_kernel<4> : scan_kernel<8>, grid,
+                     32u * sh.q_groups * sh.row_tiles, sh.smem, st, !ctx->prof_on, sc);
+      }
     }
     if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "scan kernel: %s", cudaGetErrorString(e));
     RankParams rp;

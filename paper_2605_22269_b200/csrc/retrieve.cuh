@@ -97,17 +97,50 @@ __global__ void __launch_bounds__(kPoolThreads) qpool_kernel(const T* __restrict
 
 // ------------------------------------------------------------------------------ Eq. 7
 // Rows 0..n_frm-1 are frame keys, rows n_frm..n_frm+n_seg-1 segment keys, then n_pat patch-level
-// keys (n_pat = 0 without a patch level).  A block owns
-// kScanRows rows and walks the feature axis in chunks of kScanCC: the rows' chunk (float) and the
-// chunk of up to kScanQB pooled queries (double) are staged in shared memory.  The product itself
-// is a dense double-precision contraction [rows x C] . [C x questions] and runs on the
-// double-precision tensor-core instruction (mma.sync m8n8k4 f64): warp w owns rows 8*(w%4).. and
-// questions 32*(w/4).., four 8 x 8 accumulator tiles.  (Plain double-precision FMAs are slow on
-// this part; the scores have to be double because indices are ranked on them.)
-constexpr int kScanRows = 32;
-constexpr int kScanCC = 64;
-constexpr int kScanQB = 64;
-constexpr int kScanQPad = kScanQB + 4;
+// keys (n_pat = 0 without a patch level).  The product [rows x C] . [C x questions] runs on the double-precision tensor-core
+// instruction (mma.sync m8n8k4 f64; the scores have to be double because indices are ranked on them): a block owns
+// row_tiles x 8 rows and all questions, a warp eight rows and T tiles of eight questions.  It walks the feature axis in
+// chunks of 32 channels, the next chunk of the rows (float) and of the pooled questions (double) on its way to shared memory while
+// one is multiplied.
+// Bound by the fp64 tensor instruction, 64 multiply-adds per clock and SM: 21 us for 64 questions and the 11,475 rows of three
+// hours.  scan_shape() picks the tiles so that all schedulers get about the same share of them: with fixed blocks of 32
+// rows x 64 questions that case took SCAN_BEFORE us (three blocks on some SMs and two on others), now SCAN_NOW, and 1,913 rows (60 blocks
+// for 148 SMs) SCAN2_BEFORE, now SCAN2_NOW.
+constexpr int kScanCC = 32;                                  // channels of a chunk (C is a multiple of it)
+constexpr int kScanRowPad = kScanCC + 4;                     // floats of a row, doubles of a question row: + 4 keeps the
+constexpr int kScanQPad = 4;                                 // fragments' loads on different banks
+constexpr int kScanMaxWarps = 20;
+
+struct ScanShape {
+  int T, q_groups, row_tiles;                                // tiles of a warp; warps side by side: question groups x row tiles
+  size_t smem;
+};
+__host__ inline size_t scan_smem_bytes(int T, int q_groups, int row_tiles) {
+  return 2 * ((size_t)kScanCC * (8 * T * q_groups + kScanQPad) * sizeof(double) + (size_t)8 * row_tiles * kScanRowPad * sizeof(float));
+}
+// Least time of a chunk: the tiles of the busiest scheduler at 128 clocks each (8 instructions of 16), or the chunk's bytes at 64
+// a clock.
+__host__ inline ScanShape scan_shape(long long rows, int nq, int n_sms) {
+  const int nt = (nq + 7) / 8;
+  const long long tiles = (rows + 7) / 8;
+  ScanShape best{0, 0, 0, 0};
+  long long least = -1;
+  for (int T = 1; T <= 8; T *= 2) {
+    const int qg = (nt + T - 1) / T;
+    if (qg > 4) continue;
+    for (int rt = 1; rt * qg <= kScanMaxWarps; ++rt) {
+      const long long blocks = (tiles + rt - 1) / rt, per_sm = (blocks + n_sms - 1) / n_sms;
+      const long long mma = per_sm * ((rt * qg + 3) / 4) * T * 128;
+      const long long load = per_sm * (kScanCC * 8LL * 8 * T * qg + 8LL * rt * kScanCC * 4) / 64;
+      const long long t = (mma > load ? mma : load) + 32 * per_sm;
+      if (least < 0 || t < least) {
+        least = t;
+        best = {T, qg, rt, scan_smem_bytes(T, qg, rt)};
+      }
+    }
+  }
+  return best;
+}
 
 struct ScanParams {
   const float* frame_key; const float* seg_key; const float* patch_key;
@@ -120,6 +153,7 @@ struct ScanParams {
   float* f_frm; float* f_seg; float* f_pat;
   long long f_frm_stride, f_seg_stride, f_pat_stride;         // multiples of four
   const int* patch_cnt;
+  int q_groups, row_tiles;                                    // scan_kernel, see ScanShape
 };
 #define kScanAbsent (-INFINITY)
 // The score of a block whose key, or of a question whose pooled vector, holds Inf or NaN: below every cosine and every mix
@@ -148,101 +182,87 @@ __device__ __forceinline__ void scan_store(const ScanParams& sp, int qi, long lo
   }
 }
 
-__global__ void __launch_bounds__(256, 3) scan_kernel(const ScanParams sp) {
-  const float* __restrict__ frame_key = sp.frame_key;
-  const float* __restrict__ seg_key = sp.seg_key;
-  const long long n_frm = sp.n_frm, n_seg = sp.n_seg;
-  const int C = sp.C, nq = sp.nq, Hkv = sp.Hkv;
-  const double* __restrict__ q64t = sp.q64t;
-  const double* __restrict__ qn2 = sp.qn2;
-  __shared__ float rows[kScanRows][kScanCC + 1];
-  __shared__ __align__(16) double qs[kScanCC][kScanQPad];
-  __shared__ double s_knorm[kScanRows];
+template <int T>
+__global__ void __launch_bounds__(32 * kScanMaxWarps) scan_kernel(const ScanParams sp) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double s_qn[MUKV_MAX_QUESTIONS];
+  const int C = sp.C, nq = sp.nq, nt = blockDim.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int QB = 8 * T * sp.q_groups, q_stride = QB + kScanQPad, R = 8 * sp.row_tiles;
+  double* const s_q = reinterpret_cast<double*>(smem_raw);                        // [2][kScanCC][q_stride]
+  float* const s_rows = reinterpret_cast<float*>(s_q + 2 * kScanCC * q_stride);   // [2][R][kScanRowPad]
+  const long long row0 = (long long)blockIdx.x * R, n_rows = sp.n_frm + sp.n_seg + sp.n_pat;
+  auto copy16 = [](void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
+  };
+  auto row_ptr = [&](long long row) {
+    return row < sp.n_frm ? sp.frame_key + row * C
+           : (row < sp.n_frm + sp.n_seg ? sp.seg_key + (row - sp.n_frm) * C
+                                        : sp.patch_key + (row - sp.n_frm - sp.n_seg) * C);
+  };
+  auto fetch_rows = [&](int c0, int buf) {                   // (rows behind the last one repeat it: nobody stores their scores)
+    for (int v = tid; v < R * (kScanCC / 4); v += nt) {
+      const int r = v / (kScanCC / 4), c = v % (kScanCC / 4) * 4;
+      copy16(s_rows + ((long long)buf * R + r) * kScanRowPad + c, row_ptr(min(row0 + r, n_rows - 1)) + c0 + c);
+    }
+  };
+  auto fetch_questions = [&](int c0, int buf) {              // (columns behind the last question hold anything: a column of the
+    for (int v = tid; v < kScanCC * (QB / 2); v += nt) {     // product depends on its own question only)
+      const int c = v / (QB / 2), q = v % (QB / 2) * 2;
+      copy16(s_q + ((long long)buf * kScanCC + c) * q_stride + q, sp.q64t + (long long)(c0 + c) * MUKV_MAX_QUESTIONS + q);
+    }
+  };
+  // (The first keys are on their way before the wait: the kernel in front is qpool_kernel, which lets this one start only when
+  // everything before it is complete.)
+  fetch_rows(0, 0);
   pdl_wait();                                                // the pooled questions are complete
   pdl_trigger();
-  for (int qq = tid; qq < nq; qq += 256) {                   // norms of the pooled questions (read after the barriers below)
+  fetch_questions(0, 0);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  for (int qq = tid; qq < nq; qq += nt) {                    // norms of the pooled questions (read after the barriers below)
     double t = 0.0;
-    for (int gg = 0; gg < Hkv; ++gg) t += qn2[(long long)qq * Hkv + gg];
+    for (int g = 0; g < sp.Hkv; ++g) t += sp.qn2[(long long)qq * sp.Hkv + g];
     s_qn[qq] = sqrt(t);
   }
-  const long long row0 = (long long)blockIdx.x * kScanRows;
-  const long long n_rows = n_frm + n_seg + sp.n_pat;
-  const int lr = tid >> 3, lc = (tid & 7) * 8;               // staging: row, first column of 8
-  const long long my_row = row0 + lr;
-  const float* src = my_row < n_frm ? frame_key + my_row * C
-                     : (my_row < n_frm + n_seg ? seg_key + (my_row - n_frm) * C
-                     : (my_row < n_rows ? sp.patch_key + (my_row - n_frm - n_seg) * C : nullptr));
-  const int wr = (warp & 3) * 8, wq = (warp >> 2) * 32;      // this warp's rows and questions
+  const int rt = warp / sp.q_groups, q0 = warp % sp.q_groups * 8 * T;        // this warp's rows and questions
   const int fr = lane >> 2, fk = lane & 3;                   // fragment row / k (A), k / column (B)
-  for (int qb = 0; qb < nq; qb += kScanQB) {
-    double acc[4][2];
+  double acc[T][2], kk = 0.0;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) { acc[i][0] = 0.0; acc[i][1] = 0.0; }
-    double kk = 0.0;
-    // the chunk after the one being multiplied is already on its way into registers
-    float xr[8];
-    double xq[kScanCC * kScanQB / 256];
-    auto fetch = [&](int c0) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int cc = lc + i;
-        xr[i] = (src && c0 + cc < C) ? src[c0 + cc] : 0.f;
-      }
-#pragma unroll
-      for (int i = 0; i < kScanCC * kScanQB / 256; ++i) {
-        const int idx = tid + i * 256;
-        const int cc = idx / kScanQB, qq = idx % kScanQB;
-        xq[i] = (c0 + cc < C && qb + qq < nq) ? q64t[(long long)(c0 + cc) * MUKV_MAX_QUESTIONS + qb + qq] : 0.0;
-      }
-    };
-    fetch(0);
-    for (int c0 = 0; c0 < C; c0 += kScanCC) {
-      __syncthreads();                                       // the previous chunk has been consumed
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        rows[lr][lc + i] = xr[i];
-        kk = fma((double)xr[i], (double)xr[i], kk);
-      }
-#pragma unroll
-      for (int i = 0; i < kScanCC * kScanQB / 256; ++i) {
-        const int idx = tid + i * 256;
-        qs[idx / kScanQB][idx % kScanQB] = xq[i];
-      }
-      __syncthreads();
-      if (c0 + kScanCC < C) fetch(c0 + kScanCC);
-#pragma unroll 4
-      for (int cc = 0; cc < kScanCC; cc += 4) {
-        const double a = (double)rows[wr + fr][cc + fk];     // A[row fr][k fk]
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) dmma_m8n8k4(acc[nt], a, qs[cc + fk][wq + nt * 8 + fr]);   // B[k fk][col fr]
-      }
+  for (int i = 0; i < T; ++i) { acc[i][0] = 0.0; acc[i][1] = 0.0; }
+  for (int c0 = 0, buf = 0; c0 < C; c0 += kScanCC, buf ^= 1) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();                                         // this chunk is there, the one before has been consumed
+    if (c0 + kScanCC < C) {
+      fetch_rows(c0 + kScanCC, buf ^ 1);
+      fetch_questions(c0 + kScanCC, buf ^ 1);
+      asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    if (qb == 0) {
-      // the 8 staging threads of a row hold the parts of its squared norm
-      kk += __shfl_xor_sync(kFull, kk, 1);
-      kk += __shfl_xor_sync(kFull, kk, 2);
-      kk += __shfl_xor_sync(kFull, kk, 4);
-      if ((tid & 7) == 0) s_knorm[lr] = sqrt(kk);
+    const float* a_src = s_rows + ((long long)buf * R + rt * 8 + fr) * kScanRowPad + fk;
+    const double* b_src = s_q + ((long long)buf * kScanCC + fk) * q_stride + q0 + fr;
+#pragma unroll
+    for (int k = 0; k < kScanCC; k += 4) {
+      const double a = (double)a_src[k];                     // A[row fr][k fk]
+      kk = fma(a, a, kk);
+#pragma unroll
+      for (int t = 0; t < T; ++t) dmma_m8n8k4(acc[t], a, b_src[k * q_stride + t * 8]);   // B[k fk][col fr]
     }
-    __syncthreads();
-    // accumulator tile: row fr, columns 2*fk and 2*fk + 1
-    const int r = wr + fr;
-    const long long row = row0 + r;
-    if (row < n_rows) {
-      const double knorm = s_knorm[r];
+  }
+  // the four lanes of a row hold the parts of its squared norm
+  kk += __shfl_xor_sync(kFull, kk, 1);
+  kk += __shfl_xor_sync(kFull, kk, 2);
+  const double knorm = sqrt(kk);
+  // accumulator tile: row fr, columns 2*fk and 2*fk + 1
+  const long long row = row0 + rt * 8 + fr;
+  if (row < n_rows) {
 #pragma unroll
-      for (int nt = 0; nt < 4; ++nt) {
+    for (int t = 0; t < T; ++t) {
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int qi = qb + wq + nt * 8 + 2 * fk + j;
-          if (qi >= nq) continue;
-          double den = knorm * s_qn[qi];
-          den = den > 1e-12 ? den : 1e-12;
-          const double sc = acc[nt][j] / den;
-          scan_store(sp, qi, row, sc);
-        }
+      for (int e = 0; e < 2; ++e) {
+        const int qi = q0 + t * 8 + 2 * fk + e;
+        if (qi >= nq) continue;
+        double den = knorm * s_qn[qi];
+        den = den > 1e-12 ? den : 1e-12;
+        scan_store(sp, qi, row, acc[t][e] / den);
       }
     }
   }
