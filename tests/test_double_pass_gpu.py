@@ -18,6 +18,7 @@ pytestmark = pytest.mark.gpu
     (4, 2, 64, 9, False, {}),                              # a row more than a tile
     (2, 2, 64, 63, False, dict(attn_causal=1)),            # eight tiles, the last one ragged
     (6, 2, 64, 65, True, dict(attn_causal=1)),             # two tiles in one warp; causal: shares without a visible key
+    (6, 2, 64, 65, True, dict(path=1)),                    # flagged by the multiply-add kernel
     (28, 4, 128, 196, True, {}),
     (16, 2, 128, 256, False, dict(keep_low_freq=1)),       # all tiles full
     (4, 4, 64, 100, True, dict(past_frames=3)),            # 175 keys, the cached ones first
@@ -25,8 +26,9 @@ pytestmark = pytest.mark.gpu
 def test_flagged_frames(n, q_heads, kv_heads, head_dim, tokens, bf16, over):
     spec = StreamSpec(seed=91, n_layers=2, n_q_heads=q_heads, n_kv_heads=kv_heads, head_dim=head_dim, tokens_per_frame=tokens,
                       bf16=bf16, n_outlier=1, n_frames=6, scene_sigma=1.0, frame_sigma=0.5, scene_min=2, scene_max=4)
-    run = H.GpuRun(dict(spec=spec, keep=max(1, tokens // 4), fseg=4, chunk=n, alpha=0.7), options={B.OPT_FLAG_MARGIN: 4.0},
-                   **over).compress()
+    options = {B.OPT_FLAG_MARGIN: 4.0, B.OPT_SCORE_PATH: over.get("path", 0)}
+    over = {k: v for k, v in over.items() if k != "path"}
+    run = H.GpuRun(dict(spec=spec, keep=max(1, tokens // 4), fseg=4, chunk=n, alpha=0.7), options=options, **over).compress()
     st = O.Store(H.oracle_cfg(run.cfg))
     for t0 in range(0, 6, n):
         kv = [spec.frame_kv(t) for t in range(t0, t0 + n)]
