@@ -342,8 +342,8 @@ mukv_status mukv_get_stats(mukv_ctx* ctx, mukv_stats* out, mukv_stream stream);
  * context is bracketed by a pair of CUDA events on the call's stream (host objects; no device
  * memory).  mukv_profile_read waits for the recorded events, adds up the elapsed milliseconds
  * and the launch counts per kernel kind since the last read, and forgets them.
- * Kinds: 0 score, 1 tail (double-precision pass of flagged frames; segment-level selection),
- *        2 compact+pool, 3 segment pool, 4 question pool, 5 index scan, 6 rank, 7 gather. */
+ * Kinds: 0 score, 1 tail (double-precision pass of flagged frames of fp32 calls; segment-level selection),
+ *        2 compact+pool (bf16 calls: flagged frames, too), 3 segment pool, 4 question pool, 5 index scan, 6 rank, 7 gather. */
 #define MUKV_PROF_KINDS 8
 mukv_status mukv_profile_enable(mukv_ctx* ctx, int32_t on);
 mukv_status mukv_profile_read(mukv_ctx* ctx, double* ms, int64_t* launches);
@@ -372,8 +372,8 @@ mukv_status mukv_profile_read(mukv_ctx* ctx, double* ms, int64_t* launches);
  * list of frames that need the double-precision pass, the DFT matrix terms) is a fixed array inside the
  * library; every device that loads the library holds it until the process exits.  The call performs no
  * cudaMalloc / cudaFree and uses no allocating routine.  A call enqueues one small memset on `stream` (counters and
- * column sums must start at zero; the rest of the array is overwritten before it is read), then a bf16 call, scored on the
- * tensor cores, three kernels and an fp32 call two.  The first call on each device
+ * column sums must start at zero; the rest of the array is overwritten before it is read), then either
+ * two kernels.  The first call on each device
  * also looks up the array's device address, copies the matrix terms into it and raises the kernels'
  * shared-memory limit; make that first call outside any stream capture.
  * All calls on a device share the one array: two calls whose kernels may overlap on the device

@@ -826,22 +826,48 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __gri
   else compact_plane<T>(p, plane, f, &cs, kappa_f, page);
 }
 
-// Selection alone (scoring without a store): one block per frame, behind the persistent scoring kernel.  A code in *scoring
-// (one of that kernel's bounded waits ran out) leaves no sums to trust: the ids are then -1 and the scores NaN.
-__global__ void __launch_bounds__(kCompactThreads) select_kernel(const CompactParams p, const int* scoring) {
-  __shared__ SelectScratch ss;
-  __shared__ int s_kept[MUKV_MAX_TOKENS];
+// Selection alone (scoring without a store, bf16): one block per frame, behind the persistent scoring kernel; the blocks behind
+// those score the flagged frames again in double precision, once every frame's ids are out (a launch of its own for that cost
+// calls that flag nothing 0.4 us of 31).  A code in *scoring (one of that kernel's bounded waits ran out) leaves no sums to trust:
+// the ids are then -1 and the scores NaN.
+__global__ void __launch_bounds__(kCompactThreads, 3) select_kernel(const __grid_constant__ CompactParams p, const int* scoring) {
+  __shared__ union {
+    struct {
+      SelectScratch ss;
+      int kept[MUKV_MAX_TOKENS];
+    };
+    Score64Scratch s64;
+  } sh;
+  const ScoreParams& sp = p.sp;
+  const int n = sp.n_frames, tid = threadIdx.x;
   pdl_wait();
   pdl_trigger();
-  if (*scoring == 0) {
-    select_from_partials(p, blockIdx.x, true, s_kept, &ss);
+  const int failed = *scoring;
+  if ((int)blockIdx.x < n) {
+    const int f = blockIdx.x;
+    select_from_partials(p, f, true, sh.kept, &sh.ss);
+    const long long np = (long long)n * sp.P;
+    for (int t = tid; failed && t < sp.P; t += kCompactThreads) {
+      if (t < sp.kappa) sp.kept_store[(long long)f * sp.kappa + t] = -1;
+      for (int s = 0; s < 3 && sp.scores_out; ++s) sp.scores_out[s * np + (long long)f * sp.P + t] = __int_as_float(0x7fffffff);
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) *reinterpret_cast<volatile unsigned*>(p.sel_flag + f) = 1u;
     return;
   }
-  const ScoreParams& sp = p.sp;
-  const long long np = (long long)sp.n_frames * sp.P;
-  for (int t = threadIdx.x; t < sp.P; t += kCompactThreads) {
-    if (t < sp.kappa) sp.kept_store[(long long)blockIdx.x * sp.kappa + t] = -1;
-    for (int s = 0; s < 3 && sp.scores_out; ++s) sp.scores_out[s * np + (long long)blockIdx.x * sp.P + t] = __int_as_float(0x7fffffff);
+  if (failed) return;
+  const volatile unsigned* flag = p.sel_flag + tid;        // (n <= MUKV_NOALLOC_MAX_FRAMES)
+  const bool ok = tid >= n || wait_until([&] { return *flag != 0u; });
+  __threadfence();
+  if (!__syncthreads_and(ok)) return;                      // (never seen; the frames keep their single-precision ids)
+  const int n_fl = *reinterpret_cast<volatile int*>(sp.n_flagged), blocks = gridDim.x - n, heads = sp.Ls * sp.Hq;
+  if (n_fl == 0) return;
+  const int rs = score64_split(n_fl, heads, sp.P, blocks, sp.scratch_rows), units = heads * rs;
+  for (int w = blockIdx.x - n; w < n_fl * units; w += blocks) {
+    const int slot = w / units, u = w % units;
+    score64_frame_block<__nv_bfloat16>(sp, p.colsum_d, p.ifft_d, u / rs, u % rs, rs, __ldcg(sp.flagged + slot), slot, &sh.s64);
+    __syncthreads();
   }
 }
 

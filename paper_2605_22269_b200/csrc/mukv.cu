@@ -848,7 +848,7 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
   if (!seg_scope && !d_ext) {
     const int units = ctx->Ls * c.n_q_heads * ((P + 7) / 8), planes = 4 * L + 1;
     const int others = n * (L * 2 * cp.parts + (c.patch_split > 0 ? 1 : 0) + cp.prev_rows), room = ctx->redo_capacity - others;
-    redo = std::min(std::max(units, planes), room <= 0 ? ctx->redo_capacity : std::max(room, ctx->n_sms));
+    redo = std::min(std::max(units, planes), sizeof(T) == 4 ? ctx->n_sms : room <= 0 ? ctx->redo_capacity : std::max(room, ctx->n_sms));
     cp.colsum_d = reinterpret_cast<double*>(ctx->ws + ctx->wl.colsum_d);
     cp.ifft_d = reinterpret_cast<double*>(ctx->ws + ctx->wl.ifft_d);
     cp.sp.scratch_rows = (int)std::min<size_t>(refine_rows(c), 0x7fffffff);
@@ -1488,8 +1488,9 @@ constexpr size_t kNaTs = kNaKept + (size_t)kNaFrames * kNaP * sizeof(int);
 constexpr size_t kNaPt = kNaTs + 256;
 constexpr size_t kNaW128 = kNaPt + 256;                  // DFT matrix terms, D = 128 and D = 64
 constexpr size_t kNaW64 = kNaW128 + 3 * 128 * 128 * 2;
-constexpr size_t kNaCtrl = kNaW64 + 3 * 64 * 64 * 2;     // frame_counter[16], flagged[16], n_flagged, status; at 256: head_counter
-constexpr size_t kNaCtrlBytes = 256 + (size_t)kNaFrames * kNaHq * sizeof(int);
+constexpr size_t kNaCtrl = kNaW64 + 3 * 64 * 64 * 2;     // frame_counter[16], flagged[16], n_flagged, status; at 256: sel_flag, at 512:
+                                                         // head_counter
+constexpr size_t kNaCtrlBytes = 512 + (size_t)kNaFrames * kNaHq * sizeof(int);
 constexpr size_t kNaAtt = kNaCtrl + kNaCtrlBytes;        // column sums of the tensor-core path: zeroed together with the words
 constexpr size_t kNaTotal = kNaAtt + (size_t)kNaFrames * kNaP * sizeof(unsigned long long);
 
@@ -1563,7 +1564,7 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
   sp.colsum_part = base + kNaColF;
   sp.ifft_part = base + kNaFftF;
   sp.frame_counter = reinterpret_cast<int*>(base + kNaCtrl);
-  sp.head_counter = reinterpret_cast<int*>(base + kNaCtrl + 256);
+  sp.head_counter = reinterpret_cast<int*>(base + kNaCtrl + 512);
   sp.flagged = reinterpret_cast<int*>(base + kNaCtrl) + kNaFrames;
   sp.n_flagged = reinterpret_cast<int*>(base + kNaCtrl) + 2 * kNaFrames;
   sp.kept_store = d_kept_out ? d_kept_out : reinterpret_cast<int*>(base + kNaKept);
@@ -1594,8 +1595,15 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
     memset(&cp, 0, sizeof cp);
     cp.sp = sp;
     cp.att_acc = pl.att_acc;
-    e = launch_k(select_kernel, dim3(n), kCompactThreads, 0, st, true, cp, (const int*)pl.status);
+    cp.sel_flag = reinterpret_cast<unsigned*>(base + kNaCtrl + 256);
+    cp.colsum_d = reinterpret_cast<double*>(base + kNaColD);
+    cp.ifft_d = reinterpret_cast<double*>(base + kNaFftD);
+    cp.sp.scratch_rows = kNaFrames * kNaHq;
+    // (blocks for the flagged frames: three per SM are resident beside one another; they wait for the first n only)
+    const int units = n * c.n_q_heads * ((P + 7) / 8);
+    e = launch_k(select_kernel, dim3(n + std::min(units, 3 * nd->n_sms)), kCompactThreads, 0, st, true, cp, (const int*)pl.status);
     if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "select kernel: %s", cudaGetErrorString(e));
+    return MUKV_OK;
   } else {
     e = launch_score<T>(sp, nc, dim3(c.n_q_heads, n), score_smem_bytes<T>(P, D), st);
     if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "score kernel: %s", cudaGetErrorString(e));
