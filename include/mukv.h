@@ -128,7 +128,8 @@ typedef struct {
   int64_t store_bytes_used;      /* pages written so far, in bytes                      */
   int64_t refined_frames;        /* frames whose selection was redone in double         */
   int64_t refined_questions;     /* reserved (retrieval always scores in double)        */
-  int64_t kernel_launches;       /* kernels launched by this context since creation     */
+  int64_t kernel_launches;       /* kernels launched by this context since creation (without
+                                    the one that mukv_reset clears the counters with)     */
   int32_t device_status;         /* 0, or the first device-side event code recorded:
                                     3, 4, 5  a bounded wait inside the tensor-core scoring kernel
                                              ran out (producer, MMA issuer, epilogue): the chunk's
@@ -157,7 +158,7 @@ void mukv_destroy(mukv_ctx* ctx);
 
 /* Forgets every stored frame (capacity and buffers are kept) and clears the counters behind
  * mukv_get_stats (refined_frames, device_status).  The host-side frame counter is reset at once;
- * the device-side counters are cleared by a memset enqueued on `stream`, so the call must be
+ * the device-side counters are cleared by a small kernel enqueued on `stream`, so the call must be
  * ordered after the context's earlier work like any other call. */
 mukv_status mukv_reset(mukv_ctx* ctx, mukv_stream stream);
 
@@ -371,10 +372,9 @@ mukv_status mukv_profile_read(mukv_ctx* ctx, double* ms, int64_t* launches);
  * The scratch (about 2 MB: per-head partial sums in float and double, arrival counters, the
  * list of frames that need the double-precision pass, the DFT matrix terms) is a fixed array inside the
  * library; every device that loads the library holds it until the process exits.  The call performs no
- * cudaMalloc / cudaFree and uses no allocating routine.  A call enqueues one small memset on `stream` (counters and
- * column sums must start at zero; the rest of the array is overwritten before it is read), then either
- * two kernels.  The first call on each device
- * also looks up the array's device address, copies the matrix terms into it and raises the kernels'
+ * cudaMalloc / cudaFree and uses no allocating routine.  A call enqueues three kernels on `stream`; the first one
+ * is small and zeros counters and column sums (the rest of the array is overwritten before it is read).  The first call on
+ * each device also looks up the array's device address, copies the matrix terms into it and raises the kernels'
  * shared-memory limit; make that first call outside any stream capture.
  * All calls on a device share the one array: two calls whose kernels may overlap on the device
  * (different streams without an ordering between them) race; what such calls return is undefined, later calls

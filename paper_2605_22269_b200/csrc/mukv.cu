@@ -351,6 +351,18 @@ cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, unsigned block, size_t
   return launch_c(kernel, grid, block, smem, st, dependent, 1u, args...);
 }
 
+// Zeros `bytes` (a multiple of eight, below 16 GB) on the stream.  Where no kernel can be launched (a stream of another device than
+// the current one) it is a memset, which can.
+cudaError_t zero_async(void* p, size_t bytes, cudaStream_t st, bool dependent) {
+  const int n = (int)(bytes / 8), blocks = (n + kCompactThreads - 1) / kCompactThreads;
+  if (n <= 0) return cudaSuccess;
+  cudaError_t e = launch_k(zero_kernel, dim3(blocks < 148 ? blocks : 148), kCompactThreads, 0, st, dependent,
+                           static_cast<unsigned long long*>(p), n);
+  if (e == cudaSuccess) return e;
+  cudaGetLastError();
+  return cudaMemsetAsync(p, 0, bytes, st);
+}
+
 template <typename T>
 cudaError_t launch_score(const ScoreParams& sp, int nc, dim3 grid, size_t smem, cudaStream_t st) {
   switch (nc) {
@@ -1194,8 +1206,8 @@ mukv_status mukv_reset(mukv_ctx* ctx, mukv_stream stream) {
   // Arrival counters, flagged lists, selection flags, statistics, the event word and the column sums start over, and so does
   // the alternation between the two sets: calls captured into a graph behind a reset are replayed with the sets that they were
   // captured with, so the reset has to leave both in the same state every time.
-  cudaError_t e = cudaMemsetAsync(ctx->ws + ctx->wl.zero_begin, 0, ctx->wl.zero_end - ctx->wl.zero_begin,
-                                  static_cast<cudaStream_t>(stream));
+  cudaError_t e = zero_async(ctx->ws + ctx->wl.zero_begin, ctx->wl.zero_end - ctx->wl.zero_begin, static_cast<cudaStream_t>(stream),
+                             !ctx->prof_on);
   if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "mukv_reset: %s", cudaGetErrorString(e));
   ctx->frames = 0;
   ctx->parity = 0;
@@ -1575,10 +1587,10 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
   sp.refine = 0;
   sp.row_split = 1;
   // The array keeps what the last call left, be it one that broke off or raced with another: the arrival counters, the flagged
-  // count, the status word and (tensor-core path) the column sums start at zero in every call.  (2.6 us of 30.7 for sixteen
-  // frames of 28 heads x 196 tokens; left clean by the call before, they cost nothing and could be spoilt for good.)
-  e = cudaMemsetAsync(base + kNaCtrl, 0, kNaCtrlBytes + (ts.ok ? (size_t)n * P * sizeof(unsigned long long) : 0), st);
-  if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
+  // count, the status word and (tensor-core path) the column sums start at zero in every call.  (Left clean by the
+  // call before they could be spoilt for good.)
+  e = zero_async(base + kNaCtrl, kNaCtrlBytes + (ts.ok ? (size_t)n * P * sizeof(unsigned long long) : 0), st, true);
+  if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "clearing the scratch: %s", cudaGetErrorString(e));
   if (ts.ok) {
     // bf16: scored on the tensor cores like a chunk of a context, then one block per frame selects.
     PsLaunch pl;
