@@ -364,12 +364,12 @@ cudaError_t zero_async(void* p, size_t bytes, cudaStream_t st, bool dependent) {
 }
 
 template <typename T>
-cudaError_t launch_score(const ScoreParams& sp, int nc, dim3 grid, size_t smem, cudaStream_t st) {
+cudaError_t launch_score(const ScoreParams& sp, int nc, dim3 grid, size_t smem, cudaStream_t st, bool dependent) {
   switch (nc) {
-    case 2: return launch_k(score_kernel<T, 2>, grid, kScoreThreads, smem, st, false, sp);
-    case 4: return launch_k(score_kernel<T, 4>, grid, kScoreThreads, smem, st, false, sp);
-    case 7: return launch_k(score_kernel<T, 7>, grid, kScoreThreads, smem, st, false, sp);
-    default: return launch_k(score_kernel<T, 8>, grid, kScoreThreads, smem, st, false, sp);
+    case 2: return launch_k(score_kernel<T, 2>, grid, kScoreThreads, smem, st, dependent, sp);
+    case 4: return launch_k(score_kernel<T, 4>, grid, kScoreThreads, smem, st, dependent, sp);
+    case 7: return launch_k(score_kernel<T, 7>, grid, kScoreThreads, smem, st, dependent, sp);
+    default: return launch_k(score_kernel<T, 8>, grid, kScoreThreads, smem, st, dependent, sp);
   }
 }
 
@@ -575,7 +575,7 @@ cudaError_t flush_segments(const mukv_ctx* ctx, cudaStream_t st) {
   cp.L = a.L; cp.kappa = a.kappa; cp.C = a.C; cp.fseg = a.fseg; cp.n_frames = a.n_frames; cp.first_frame = a.first_frame;
   cp.frame_entry = const_cast<float*>(a.frame_entry); cp.frame_ksum = const_cast<double*>(a.frame_ksum);
   cp.seg_entry = a.seg_entry; cp.seg_key = a.seg_key; cp.kept_count = a.kept_count;
-  const cudaError_t e = launch_k(segment_kernel, dim3(2 * a.L), kCompactThreads, 0, st, false, cp);
+  const cudaError_t e = launch_k(segment_kernel, dim3(2 * a.L), kCompactThreads, 0, st, !ctx->prof_on, cp);
   if (e == cudaSuccess) ctx->seg_pending = false;
   return e;
 }
@@ -800,7 +800,7 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
       ctx->att_dirty[ctx->parity] = (long long)n * P;
       on_tc = true;
     } else
-      e = launch_score<T>(sp, ctx->nc, grid, score_smem_bytes<T>(ctx->key_rows, c.head_dim), st);
+      e = launch_score<T>(sp, ctx->nc, grid, score_smem_bytes<T>(ctx->key_rows, c.head_dim), st, !ctx->prof_on);
     ++n_launch;
   }
   if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "%s: %s", what, cudaGetErrorString(e));
@@ -1617,7 +1617,7 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
     if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "select kernel: %s", cudaGetErrorString(e));
     return MUKV_OK;
   } else {
-    e = launch_score<T>(sp, nc, dim3(c.n_q_heads, n), score_smem_bytes<T>(P, D), st);
+    e = launch_score<T>(sp, nc, dim3(c.n_q_heads, n), score_smem_bytes<T>(P, D), st, true);
     if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "score kernel: %s", cudaGetErrorString(e));
   }
   // Flagged frames in double precision.  The scratch holds the partial sums of 16 frames with one block per head; while
