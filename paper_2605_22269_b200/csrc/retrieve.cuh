@@ -103,9 +103,10 @@ __global__ void __launch_bounds__(kPoolThreads) qpool_kernel(const T* __restrict
 // chunks of 32 channels, the next chunk of the rows (float) and of the pooled questions (double) on its way to shared memory while
 // one is multiplied.
 // Bound by the fp64 tensor instruction, 64 multiply-adds per clock and SM: 21 us for 64 questions and the 11,475 rows of three
-// hours.  scan_shape() picks the tiles so that all schedulers get about the same share of them: with fixed blocks of 32
-// rows x 64 questions that case took SCAN_BEFORE us (three blocks on some SMs and two on others), now SCAN_NOW, and 1,913 rows (60 blocks
-// for 148 SMs) SCAN2_BEFORE, now SCAN2_NOW.
+// hours.  scan_shape() picks the tiles so that all SMs get about the same share of them.  From launch to end, in the chain of
+// dependent launches behind the pooling of the questions: 53 us with fixed blocks of 32 rows x 64 questions for that case, now 42;
+// 1,913 rows (60 blocks for 148 SMs, which went in twos to what the pooling had left free; alone on the device both take 23)
+// 51, now 26; 24 questions, padded to 64 then, and 5,313 rows 46, now 24.
 constexpr int kScanCC = 32;                                  // channels of a chunk (C is a multiple of it)
 constexpr int kScanRowPad = kScanCC + 4;                     // floats of a row, doubles of a question row: + 4 keeps the
 constexpr int kScanQPad = 4;                                 // fragments' loads on different banks
