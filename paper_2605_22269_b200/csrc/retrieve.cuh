@@ -30,6 +30,7 @@ struct QMeta {
 // scan_kernel, which stages it, a row per question (cs = 1) for scan_few_kernel; the head's share of the squared
 // norm goes to qn2[question][key head] (the scans add the shares in head order).
 constexpr int kPoolThreads = 512;
+constexpr int kScanFew = 8;        // questions up to which scan_few_kernel scans
 constexpr int kPoolSmemDoubles = 4096;
 
 template <typename T>
@@ -42,7 +43,10 @@ __global__ void __launch_bounds__(kPoolThreads) qpool_kernel(const T* __restrict
   const int qi = blockIdx.x, g = blockIdx.y;
   const int G = Hq / Hkv;
   pdl_wait();
-  pdl_trigger();
+  // (Only for few questions: the scan's blocks would pile up on the SMs that the many blocks of this kernel leave free.  With the
+  // trigger 38 questions on 169 frames took 174 us with their gather, without it 161; 21 over three levels of 1,795 frames 47.5,
+  // now 45.1; 64 on three hours 910.7, now 910.1.)
+  if (gridDim.x <= kScanFew) pdl_trigger();
   const int n0 = meta.off[qi], n1 = meta.off[qi + 1];
   const int DV = D / VE;                                    // vectors per head
   int nsl = kPoolThreads / DV;                              // token slices whose partial sums fit
@@ -273,7 +277,6 @@ __global__ void __launch_bounds__(32 * kScanMaxWarps) scan_kernel(const ScanPara
 // too thin for the tile above (64 questions wide, 32 rows in a block: 60 blocks of mostly padding for one question
 // and an hour of frames, 18 us); a row is one round trip to memory, its 16 doubles per lane and a butterfly: 4 us.
 // At eight questions and 9,100 rows the two take about the same time, which is where the line lies.
-constexpr int kScanFew = 8;
 
 template <int NQ>
 __global__ void __launch_bounds__(256) scan_few_kernel(const ScanParams sp) {
