@@ -34,6 +34,7 @@
 namespace mukv {
 
 constexpr int kCompactThreads = 256;
+constexpr int kTailWords = 1;
 static_assert(kCompactThreads == kScoreThreads, "redo_flagged runs the scoring and the compaction code in one block");
 
 struct CompactParams {
@@ -47,8 +48,11 @@ struct CompactParams {
   float* frame_key;               // [max_frames][C]
   double* frame_ksum;             // [max_frames][C]  exact sums of the last-layer kept keys
   long long* stat_refined;        // device counter
-  int* n_flagged_next;            // the flagged count of the next chunk (the two chunks' counts alternate)
-  int* tail_ctr;                  // [2] redo_flagged: blocks done with the double-precision scores / with everything
+  // Words of redo_flagged.  Two sets of them (and of the flagged count) alternate from call to call, and a call clears those of
+  // the next one: whatever a call leaves behind, a wait that ran out included, is nothing that a later one starts from.
+  int* n_flagged_next;            // the flagged count of the next call
+  int* tail_ctr;                  // [kTailWords] blocks done with the double-precision scores
+  int* tail_next;                 // the next call's
   int redo_blocks;                // compact_kernel: blocks at the end of the grid that redo flagged frames (0: none)
   double *colsum_d, *ifft_d;      // their partial sums, see score64_frame_block
   // segment entries (Eq. 5 at segment level)
@@ -79,6 +83,7 @@ struct CompactParams {
   int later_blocks;               // 1: the grid is larger than what is resident at once
   unsigned* sel_flag;             // [F] (epoch << 1 | risky) once the plane-0 block has published its frame's ids
   unsigned epoch;                 // number of this call, never repeated
+  unsigned long long wait_ns;     // limit of a wait for other blocks of the grid
   ScoreParams sp;                 // partial sums, Eq. 4 parameters, index and flag outputs
 };
 
@@ -630,17 +635,19 @@ __device__ __forceinline__ bool frame_is_flagged(const int* flagged, int n, int 
   return hit;
 }
 
-// Bounded wait until done() holds (other blocks of the same grid bring it about).  False after about 1.5 s.
+// Bounded wait until done() holds (other blocks of the same grid bring it about).  False after limit_ns; 0: one look.
+constexpr unsigned long long kWaitNs = 1500000000ull;
 template <typename Done>
-__device__ __forceinline__ bool wait_until(Done done) {
+__device__ __forceinline__ bool wait_until(unsigned long long limit_ns, Done done) {
   unsigned long long t0 = 0;
   for (long long spin = 0;; ++spin) {
     if (done()) return true;
+    if (limit_ns == 0) return false;
     if ((spin & 63) == 63) {
       unsigned long long now;
       asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
       if (t0 == 0) t0 = now;
-      else if (now - t0 > 1500000000ull) return false;
+      else if (now - t0 > limit_ns) return false;
     }
     __nanosleep(100);
   }
@@ -667,9 +674,9 @@ __device__ __noinline__ void redo_flagged(const CompactParams& p, int e, int blo
   __threadfence();
   __syncthreads();
   if (tid == 0) {
-    atomicAdd(p.tail_ctr, 1);
+    if (atomicAdd(p.tail_ctr, 1) == 0) *p.stat_refined += n_fl;
     const volatile int* ctr = p.tail_ctr;
-    s_ok = wait_until([&] { return *ctr >= blocks; }) ? 1 : 0;
+    s_ok = wait_until(p.wait_ns, [&] { return *ctr >= blocks; }) ? 1 : 0;
     __threadfence();
   }
   __syncthreads();
@@ -689,16 +696,6 @@ __device__ __noinline__ void redo_flagged(const CompactParams& p, int e, int blo
       if (x >= 2 * p.L * parts) pool_patches<T>(p, f, cs);
       else if (parts == 1) compact_plane<T>(p, x, f, cs, p.kappa, page);
       else compact_plane_part<T>(p, x >> 1, f, cs, p.kappa, page, x & 1, 2);
-    }
-  }
-  // ---- the block that leaves last resets the counters and adds to the statistics
-  __syncthreads();
-  if (tid == 0) {
-    const int old = atomicAdd(p.tail_ctr + 1, 1);
-    if (old == blocks - 1) {
-      *p.stat_refined += n_fl;
-      p.tail_ctr[0] = 0;
-      p.tail_ctr[1] = 0;
     }
   }
 }
@@ -741,7 +738,7 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __gri
         bool ok = true;
         for (int i = tid; i < p.n_frames; i += kCompactThreads) {
           const volatile unsigned* flag = p.sel_flag + i;
-          ok = wait_until([&] { return (*flag >> 1) == p.epoch; }) && ok;
+          ok = wait_until(p.wait_ns, [&] { return (*flag >> 1) == p.epoch; }) && ok;
         }
         __threadfence();
         if (!__syncthreads_and(ok)) {
@@ -759,7 +756,7 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __gri
   const bool writes = plane == 0 && part == 0;           // this block writes the ids and the index of its frame
   pdl_wait();
   pdl_trigger();
-  if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *p.n_flagged_next = 0;
+  if (blockIdx.x == 0 && blockIdx.y == 0 && tid <= kTailWords) *(tid < kTailWords ? p.tail_next + tid : p.n_flagged_next) = 0;
   if (writes)
     for (long long i = (long long)f * kCompactThreads + tid; i < p.n_clear; i += (long long)gridDim.x * kCompactThreads) p.att_clear[i] = 0ull;
   const long long f_abs = p.first_frame + f;
@@ -866,7 +863,7 @@ __global__ void __launch_bounds__(kCompactThreads, 3) select_kernel(const __grid
   }
   if (failed) return;
   const volatile unsigned* flag = p.sel_flag + tid;        // (n <= MUKV_NOALLOC_MAX_FRAMES)
-  const bool ok = tid >= n || wait_until([&] { return *flag != 0u; });
+  const bool ok = tid >= n || wait_until(p.wait_ns, [&] { return *flag != 0u; });
   __threadfence();
   if (!__syncthreads_and(ok)) return;                      // (never seen; the frames keep their single-precision ids)
   const int n_fl = *reinterpret_cast<volatile int*>(sp.n_flagged), blocks = gridDim.x - n, heads = sp.Ls * sp.Hq;

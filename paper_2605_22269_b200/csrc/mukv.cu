@@ -81,6 +81,7 @@ struct mukv_ctx {
   bool failed = false;                   // a compress call broke off half way: only reset / stats / destroy
   TcShape tcs;                           // tcs.ok: the chunk is scored on the tensor cores
   int n_sms;
+  unsigned long long wait_ns = kWaitNs;  // limit of the waits inside compact_kernel and tail_kernel
   int redo_capacity = 1;                 // blocks of redo_flagged that are resident at once on this device
   CUtensorMap wmap;                      // DFT matrix terms [3*D][D] bf16
   CUtensorMap pmap;                      // the page region as [frame][plane][kept row][key head][D] (past_frames > 0)
@@ -292,7 +293,7 @@ WorkLayout work_layout(const mukv_config& c) {
   w.head_counter = off;   off = align_up(off + F * Ls * c.n_q_heads * sizeof(int));
   w.flagged = off;        off = align_up(off + F * sizeof(int));
   w.n_flagged = off;      off = align_up(off + 2 * sizeof(int));   // alternate between chunks
-  w.tail_ctr = off;       off = align_up(off + 2 * sizeof(int));
+  w.tail_ctr = off;       off = align_up(off + 2 * kTailWords * sizeof(int));   // alternate, too
   w.sel_flag = off;       off = align_up(off + F * sizeof(unsigned));
   w.seg_flag = off;       off = align_up(off + F * sizeof(int));
   w.stat_refined = off;   off = align_up(off + sizeof(long long));
@@ -816,7 +817,9 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
   cp.frame_key = reinterpret_cast<float*>(ctx->store + ctx->sl.frame_key);
   cp.frame_ksum = reinterpret_cast<double*>(ctx->store + ctx->sl.frame_ksum);
   cp.stat_refined = reinterpret_cast<long long*>(ctx->ws + ctx->wl.stat_refined);
-  cp.tail_ctr = reinterpret_cast<int*>(ctx->ws + ctx->wl.tail_ctr);
+  cp.tail_ctr = reinterpret_cast<int*>(ctx->ws + ctx->wl.tail_ctr) + ctx->parity * kTailWords;
+  cp.tail_next = reinterpret_cast<int*>(ctx->ws + ctx->wl.tail_ctr) + (ctx->parity ^ 1) * kTailWords;
+  cp.wait_ns = ctx->wait_ns;
   cp.sel_flag = reinterpret_cast<unsigned*>(ctx->ws + ctx->wl.sel_flag);
   cp.epoch = (++ctx->epoch) & 0x7fffffffu;
   cp.n_flagged_next = reinterpret_cast<int*>(ctx->ws + ctx->wl.n_flagged) + (ctx->parity ^ 1);
@@ -1611,6 +1614,7 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
     cp.colsum_d = reinterpret_cast<double*>(base + kNaColD);
     cp.ifft_d = reinterpret_cast<double*>(base + kNaFftD);
     cp.sp.scratch_rows = kNaFrames * kNaHq;
+    cp.wait_ns = kWaitNs;
     // (blocks for the flagged frames: three per SM are resident beside one another; they wait for the first n only)
     const int units = n * c.n_q_heads * ((P + 7) / 8);
     e = launch_k(select_kernel, dim3(n + std::min(units, 3 * nd->n_sms)), kCompactThreads, 0, st, true, cp, (const int*)pl.status);

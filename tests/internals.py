@@ -1,0 +1,25 @@
+"""Builds and loads tests/internals.cu: the library with a few more entry points."""
+import ctypes as C
+import os
+import subprocess
+
+from paper_2605_22269_b200 import binding as B
+from paper_2605_22269_b200 import build as BUILD
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+_LIB = None
+
+
+def load():
+    global _LIB
+    if _LIB is None:
+        out, src = os.path.join(HERE, "_build", "libinternals.so"), os.path.join(HERE, "internals.cu")
+        main, deps = BUILD.TARGETS["libmukv.so"]
+        if BUILD._stale(out, [src, main] + deps):
+            os.makedirs(os.path.dirname(out), exist_ok=True)
+            r = subprocess.run([os.environ.get("NVCC", "nvcc")] + BUILD.NVCC_FLAGS + ["-o", out, src], capture_output=True, text=True)
+            assert r.returncode == 0, r.stderr
+        _LIB = B.load_library(out)
+        _LIB.internals_wait_limit.restype = None
+        _LIB.internals_wait_limit.argtypes = [C.c_void_p, C.c_ulonglong]
+    return _LIB

@@ -1,0 +1,53 @@
+"""Waits between blocks of one kernel: what is left when one runs out."""
+import numpy as np
+import pytest
+
+from oracle import mukv_oracle as O
+from paper_2605_22269_b200 import binding as B
+from paper_2605_22269_b200.synth.cpu import StreamSpec
+from tests import harness as H
+from tests import internals as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture
+def lib(monkeypatch):
+    monkeypatch.setattr(B, "_LIB", I.load())
+    return B._LIB
+
+
+@pytest.mark.parametrize("bf16", [True, False])
+def test_a_wait_that_ran_out_does_not_reach_the_next_calls(lib, bf16):
+    # Every frame is flagged.  The waits of the first and of the fourth call are given no time, those of the others the usual one:
+    # these store what the oracle stores.
+    spec = StreamSpec(seed=84, n_layers=2, n_q_heads=8, n_kv_heads=2, head_dim=64, tokens_per_frame=40, bf16=bf16, n_outlier=1,
+                      n_frames=18, scene_sigma=1.0, frame_sigma=0.5, scene_min=2, scene_max=4)
+    run = H.GpuRun(dict(spec=spec, keep=10, fseg=3, chunk=3, alpha=0.7), options={B.OPT_FLAG_MARGIN: 4.0})
+    dev = run.device
+    kept = H.torch.full((18, 10), -7, dtype=H.torch.int32, device=dev)
+    scores = H.torch.zeros((6, 3, 3, 40), device=dev)
+    for call in range(6):
+        lib.internals_wait_limit(run.ctx.handle, 0 if call in (0, 3) else 1_500_000_000)
+        run.ctx.mukv_compress_chunk(*run.gs.chunk(3 * call, 3), 3, 3 * call, kept[3 * call:3 * call + 3], scores[call])
+        assert run.ctx.mukv_get_stats().device_status == 6
+    st = H.oracle_stream(spec, H.oracle_cfg(run.cfg), range(18), last_only=False, workers=1)
+    run.kept = kept.cpu().numpy()
+    run.scores = scores.permute(1, 0, 2, 3).reshape(3, 18, 40).cpu().numpy()
+    good = [t for t in range(18) if t // 3 not in (0, 3)]
+    sub = O.Store(H.oracle_cfg(run.cfg))
+    for name in ("kept", "page_k", "page_v", "sum_k", "sum_v", "scores"):
+        getattr(sub, name).extend(getattr(st, name)[t] for t in good)
+    H.check_frames_against_oracle(run, sub, good, full_layers=True)
+    seg = run.ctx.region(3).cpu().numpy()
+    for u in (1, 2, 4, 5):                                 # (segment u holds the frames of call u)
+        sk, sv = st.segment_entry(u)
+        H.close(seg[u][:, 0], sk, f"segment entry K {u}")
+        H.close(seg[u][:, 1], sv, f"segment entry V {u}")
+    assert run.ctx.mukv_get_stats().refined_frames >= 12
+    # a reset forgets it
+    run.ctx.mukv_reset()
+    run.compress()
+    H.check_frames_against_oracle(run, st, range(18), full_layers=True)
+    stats = run.ctx.mukv_get_stats()
+    assert stats.device_status == 0 and stats.refined_frames == 18
