@@ -20,7 +20,9 @@
 // Flagged frames (about one chunk in fifty on the synthetic streams): redo_flagged.  Blocks behind those of the copies (bf16
 // calls; p.redo_blocks of them) wait until the ids of every frame of the chunk are published or the frame is on the list, and
 // leave if the list is empty; else they score its frames in double precision (score64.cuh), and when the selections have all been
-// made they compact those frames.  fp32 calls have tail_kernel<T> for it, a launch behind compact_kernel.
+// made they compact those frames.  Units of both are taken by ticket: a block waits for units that other blocks have taken, never
+// for a block that has not started, so nothing depends on how many of them the device has a place for (another context's blocks,
+// or a kernel of the caller's, may hold places).  fp32 calls have tail_kernel<T> for it, a launch behind compact_kernel.
 // The segment entries (Eq. 5 at segment level; one (layer, K|V) plane per block, mean over the frames
 // present) of the common case are not written by the call itself.  The next call pools them with a row
 // of compact_kernel blocks that does not wait for its scoring kernel (CompactParams::prev), or the first
@@ -34,7 +36,7 @@
 namespace mukv {
 
 constexpr int kCompactThreads = 256;
-constexpr int kTailWords = 1;
+constexpr int kTailWords = 2;
 static_assert(kCompactThreads == kScoreThreads, "redo_flagged runs the scoring and the compaction code in one block");
 
 struct CompactParams {
@@ -51,7 +53,7 @@ struct CompactParams {
   // Words of redo_flagged.  Two sets of them (and of the flagged count) alternate from call to call, and a call clears those of
   // the next one: whatever a call leaves behind, a wait that ran out included, is nothing that a later one starts from.
   int* n_flagged_next;            // the flagged count of the next call
-  int* tail_ctr;                  // [kTailWords] blocks done with the double-precision scores
+  int* tail_ctr;                  // [kTailWords] next unit, frames selected (sp.n_selected)
   int* tail_next;                 // the next call's
   int redo_blocks;                // compact_kernel: blocks at the end of the grid that redo flagged frames (0: none)
   double *colsum_d, *ifft_d;      // their partial sums, see score64_frame_block
@@ -655,48 +657,56 @@ __device__ __forceinline__ bool wait_until(unsigned long long limit_ns, Done don
 
 constexpr int kStatusTailWait = 6;   // the wait for another block's ids or double-precision scores ran out
 
-// The flagged frames of a call: block e of `blocks` that run this (no more than are resident at once, see mukv_create: they
-// wait for one another).
+// The flagged frames of a call, run by any number of blocks.  `blocks`: how many were launched for it; it sets the size of the
+// units only.  One counter hands out the units of both phases, so the first ticket of the second one is also the news that
+// every scoring unit has been taken.  (A barrier of all blocks in place of the tickets was as fast with the device to itself: a
+// flagged frame of a sixteen-frame call 75 us on top of it either way; all 64 frames of four calls 2,350 us, now 2,236.)
 template <typename T>
-__device__ __noinline__ void redo_flagged(const CompactParams& p, int e, int blocks, CompactScratch* cs) {
-  __shared__ int s_ok;
+__device__ __noinline__ void redo_flagged(const CompactParams& p, int blocks, CompactScratch* cs) {
+  __shared__ int s_word;
   const ScoreParams& sp = p.sp;
   const int tid = threadIdx.x;
   const int n_fl = *reinterpret_cast<volatile int*>(sp.n_flagged);
+  auto next_unit = [&] {
+    __syncthreads();                                       // (the last unit is done with what the block shares)
+    if (tid == 0) s_word = atomicAdd(p.tail_ctr, 1);
+    __syncthreads();
+    return s_word;
+  };
   // ---- scores in double precision; the block that finishes a frame last selects
   const int heads = sp.Ls * sp.Hq, rs = score64_split(n_fl, heads, sp.P, blocks, sp.scratch_rows), units = heads * rs;
-  for (int w = e; w < n_fl * units; w += blocks) {
+  int w = next_unit();
+  for (; w < n_fl * units; w = next_unit()) {
+    if (w == 0 && tid == 0) *p.stat_refined += n_fl;
     const int slot = w / units, u = w % units;
     score64_frame_block<T>(sp, p.colsum_d, p.ifft_d, u / rs, u % rs, rs, __ldcg(sp.flagged + slot), slot, &cs->s64);
-    __syncthreads();
   }
-  // ---- every block waits for all selections
-  __threadfence();
+  // ---- the flagged frames' compaction, plane by plane; two blocks share one by columns while there are enough
+  const int parts = n_fl * 4 * p.L <= blocks && p.C * (int)sizeof(T) >= 512 ? 2 : 1;
+  const int per = 2 * p.L * parts + (p.patch_split > 0 ? 1 : 0);
+  w -= n_fl * units;
+  if (w >= n_fl * per) return;
+  // every scoring unit has been taken by a block that runs: all selections are made before long
   __syncthreads();
   if (tid == 0) {
-    if (atomicAdd(p.tail_ctr, 1) == 0) *p.stat_refined += n_fl;
-    const volatile int* ctr = p.tail_ctr;
-    s_ok = wait_until(p.wait_ns, [&] { return *ctr >= blocks; }) ? 1 : 0;
+    const volatile int* done = sp.n_selected;
+    s_word = wait_until(p.wait_ns, [&] { return *done >= n_fl; }) ? 1 : 0;
     __threadfence();
   }
   __syncthreads();
-  if (!s_ok) {
+  if (!s_word) {
     if (tid == 0 && sp.status) atomicCAS(sp.status, 0, kStatusTailWait);
-  } else {
-    // ---- the flagged frames' compaction, plane by plane; two blocks share one by columns while there are enough
-    const int parts = n_fl * 4 * p.L <= blocks && p.C * (int)sizeof(T) >= 512 ? 2 : 1;
-    const int per = 2 * p.L * parts + (p.patch_split > 0 ? 1 : 0);
-    for (int u = e; u < n_fl * per; u += blocks) {
-      const int f = __ldcg(sp.flagged + u / per), x = u % per;
-      const long long f_abs = p.first_frame + f;
-      unsigned char* page = p.store + sp.pages_off + f_abs * sp.page_bytes;
-      __syncthreads();
-      for (int r = tid; r < p.kappa; r += kCompactThreads) cs->kept[r] = token_id(__ldcg(sp.kept_store + f_abs * p.kappa + r), p.P);
-      __syncthreads();
-      if (x >= 2 * p.L * parts) pool_patches<T>(p, f, cs);
-      else if (parts == 1) compact_plane<T>(p, x, f, cs, p.kappa, page);
-      else compact_plane_part<T>(p, x >> 1, f, cs, p.kappa, page, x & 1, 2);
-    }
+    return;
+  }
+  for (; w < n_fl * per; w = next_unit() - n_fl * units) {
+    const int f = __ldcg(sp.flagged + w / per), x = w % per;
+    const long long f_abs = p.first_frame + f;
+    unsigned char* page = p.store + sp.pages_off + f_abs * sp.page_bytes;
+    for (int r = tid; r < p.kappa; r += kCompactThreads) cs->kept[r] = token_id(__ldcg(sp.kept_store + f_abs * p.kappa + r), p.P);
+    __syncthreads();
+    if (x >= 2 * p.L * parts) pool_patches<T>(p, f, cs);
+    else if (parts == 1) compact_plane<T>(p, x, f, cs, p.kappa, page);
+    else compact_plane_part<T>(p, x >> 1, f, cs, p.kappa, page, x & 1, 2);
   }
 }
 
@@ -728,8 +738,7 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __gri
   if constexpr (sizeof(T) == 2) {
     const int first = 2 * p.L * parts + (p.patch_split > 0 ? 1 : 0);     // row of the first block for flagged frames
     if (p.redo_blocks > 0 && row >= first) {
-      const int e = (row - first) * gridDim.x + blockIdx.x;
-      if (e >= p.redo_blocks) return;
+      if ((row - first) * gridDim.x + blockIdx.x >= p.redo_blocks) return;
       pdl_wait();
       pdl_trigger();
       // Nothing is flagged any more once every frame's ids are out.  The blocks that publish them are earlier ones of the grid
@@ -746,7 +755,7 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __gri
           return;
         }
       }
-      if (*reinterpret_cast<volatile int*>(p.sp.n_flagged) != 0) redo_flagged<T>(p, e, p.redo_blocks, &cs);
+      if (*reinterpret_cast<volatile int*>(p.sp.n_flagged) != 0) redo_flagged<T>(p, p.redo_blocks, &cs);
       return;
     }
   }
@@ -893,7 +902,7 @@ __global__ void __launch_bounds__(kCompactThreads, 3) tail_kernel(const __grid_c
   pdl_trigger();                                // the next call's scoring kernel may be scheduled (it waits for this one itself)
   pdl_wait();
   if (*p.sp.n_flagged == 0) return;             // the common case
-  redo_flagged<T>(p, blockIdx.x, gridDim.x, &cs);
+  redo_flagged<T>(p, gridDim.x, &cs);
 }
 
 }  // namespace mukv

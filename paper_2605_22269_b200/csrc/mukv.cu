@@ -82,7 +82,7 @@ struct mukv_ctx {
   TcShape tcs;                           // tcs.ok: the chunk is scored on the tensor cores
   int n_sms;
   unsigned long long wait_ns = kWaitNs;  // limit of the waits inside compact_kernel and tail_kernel
-  int redo_capacity = 1;                 // blocks of redo_flagged that are resident at once on this device
+  int places = 1;                        // blocks of compact_kernel that an empty device holds at once
   CUtensorMap wmap;                      // DFT matrix terms [3*D][D] bf16
   CUtensorMap pmap;                      // the page region as [frame][plane][kept row][key head][D] (past_frames > 0)
   // Segment entries a compress call left to whoever comes next (see flush_segments): the frames whose
@@ -395,14 +395,14 @@ cudaError_t raise_score_limits(int optin) {
 constexpr int kMaxDevices = 64;
 std::mutex g_dev_mutex;
 bool g_limits_raised[kMaxDevices];
-int g_redo_per_sm[kMaxDevices];
+int g_compact_per_sm[kMaxDevices];
 
 // Once per device (that device current): the dynamic shared-memory limit of every kernel that
 // needs more than the default goes to the device's maximum.  The limit belongs to the kernel,
 // not to a context, so it is never set to one context's need: a second context of another
 // shape, or the allocation-free entry point, would otherwise find it too low.
-// redo_capacity: blocks of redo_flagged that may wait for one another, i.e. are resident at once, whichever kernel they are blocks of.
-cudaError_t raise_kernel_limits(int* n_sms, int* redo_capacity) {
+// places: blocks of compact_kernel, whichever form of it, that the device holds at once when nothing else runs.
+cudaError_t raise_kernel_limits(int* n_sms, int* places) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -410,7 +410,7 @@ cudaError_t raise_kernel_limits(int* n_sms, int* redo_capacity) {
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(g_dev_mutex);
-  if (redo_capacity) *redo_capacity = g_redo_per_sm[dev] * *n_sms;
+  if (places) *places = g_compact_per_sm[dev] * *n_sms;
   if (g_limits_raised[dev]) return cudaSuccess;
   int optin = 0;
   e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
@@ -427,15 +427,14 @@ cudaError_t raise_kernel_limits(int* n_sms, int* redo_capacity) {
     typedef __nv_bfloat16 B16;
     int least = 1 << 30;
     for (const void* fn : {(const void*)compact_kernel<B16, false, false>, (const void*)compact_kernel<B16, false, true>,
-                           (const void*)compact_kernel<B16, true, false>, (const void*)compact_kernel<B16, true, true>,
-                           (const void*)tail_kernel<float>}) {
+                           (const void*)compact_kernel<B16, true, false>, (const void*)compact_kernel<B16, true, true>}) {
       int per_sm = 0;
       if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kCompactThreads, 0);
       least = std::min(least, per_sm);
     }
     if (e == cudaSuccess && least < 1) e = cudaErrorInvalidConfiguration;
-    g_redo_per_sm[dev] = least;
-    if (redo_capacity) *redo_capacity = least * *n_sms;
+    g_compact_per_sm[dev] = least;
+    if (places) *places = least * *n_sms;
   }
   if (e == cudaSuccess) g_limits_raised[dev] = true;
   return e;
@@ -855,25 +854,27 @@ mukv_status compress_impl(mukv_ctx* ctx, const void* d_q, const float* d_ext, co
   // 300 with parts; calls of 7 frames and 24 layers, which get two parts: no difference.)
   cp.parts = 1;
   while (cp.parts < 4 && 4LL * n * L * cp.parts <= 3LL * ctx->n_sms && C * ctx->esize / (2 * cp.parts) >= 256) cp.parts *= 2;
-  // Flagged frames (frame-level selection by Eq. 1-4 only): blocks that redo them, as many as are resident at once, fewer
-  // when a frame has less work (one per SM: they start wherever a place comes free, three of them on some SMs, none on others).
+  // Flagged frames (frame-level selection by Eq. 1-4 only): blocks that redo them, as many as an empty device has places for
+  // beside the copies, or has in all (any number of them does the work, see redo_flagged; a block per SM would find its
+  // places three on some SMs and none on others), and no more than a frame has units.
   // They are blocks of the compaction kernel, which spares the calls that flag nothing a launch.  fp32 calls keep the launch:
   // a hundredth of their time, behind a kernel of twice the bytes.
   int redo = 0;
   if (!seg_scope && !d_ext) {
     const int units = ctx->Ls * c.n_q_heads * ((P + 7) / 8), planes = 4 * L + 1;
-    const int others = n * (L * 2 * cp.parts + (c.patch_split > 0 ? 1 : 0) + cp.prev_rows), room = ctx->redo_capacity - others;
-    redo = std::min(std::max(units, planes), sizeof(T) == 4 ? ctx->n_sms : room <= 0 ? ctx->redo_capacity : std::max(room, ctx->n_sms));
+    const int others = n * (L * 2 * cp.parts + (c.patch_split > 0 ? 1 : 0) + cp.prev_rows), room = ctx->places - others;
+    redo = std::min(std::max(units, planes), sizeof(T) == 4 ? ctx->n_sms : room <= 0 ? ctx->places : std::max(room, ctx->n_sms));
     cp.colsum_d = reinterpret_cast<double*>(ctx->ws + ctx->wl.colsum_d);
     cp.ifft_d = reinterpret_cast<double*>(ctx->ws + ctx->wl.ifft_d);
     cp.sp.scratch_rows = (int)std::min<size_t>(refine_rows(c), 0x7fffffff);
+    cp.sp.n_selected = cp.tail_ctr + 1;
     if (sizeof(T) == 2) cp.redo_blocks = redo;
   }
   {
     ProfScope ps(ctx, 2, st);
     const int rows = L * 2 * cp.parts + (c.patch_split > 0 ? 1 : 0) + cp.prev_rows + (cp.redo_blocks + n - 1) / n;
     const bool sel = cp.sel_mode == 1;
-    cp.later_blocks = (long long)n * rows > ctx->redo_capacity;
+    cp.later_blocks = (long long)n * rows > ctx->places;
     e = launch_k(cp.parts > 1 ? (sel ? compact_kernel<T, true, true> : compact_kernel<T, true, false>)
                               : (sel ? compact_kernel<T, false, true> : compact_kernel<T, false, false>),
                  dim3(n, rows), kCompactThreads, 0, st, !ctx->prof_on, cp);
@@ -1152,7 +1153,7 @@ mukv_status create_impl(const mukv_config* cfg, void* d_store, size_t store_byte
   ctx->flag_margin = kFlagMargin;
   ctx->flat_ratio = kFlatRatio;
   const int D = cfg->head_dim;
-  cudaError_t e = raise_kernel_limits(&ctx->n_sms, &ctx->redo_capacity);
+  cudaError_t e = raise_kernel_limits(&ctx->n_sms, &ctx->places);
   if (e == cudaSuccess && (ctx->tcs.ok || ctx->tcs.split)) {
     e = cudaMemcpy(ctx->ws + ctx->wl.wtab, dft_terms(D), dft_bytes(D), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !encode_map2(&ctx->wmap, ctx->ws + ctx->wl.wtab, D, 3LL * D, D)) e = cudaErrorInvalidValue;

@@ -47,6 +47,7 @@ struct ScoreParams {
   long long* frame_ts;          // [max_frames]
   long long* page_table;        // [max_frames]
   long long pages_off, page_bytes;
+  int* n_selected;              // double-precision pass: counts the frames it has selected; or null
   int* status;                  // device event word (0 = nothing recorded); see mukv_stats.device_status
   // cached keys the queries also attend to (Sec. 3.2): the kept keys of the n_past_frames frames stored
   // just before the chunk, kappa rows each, read from their pages; n_past_frames = 0: none
@@ -352,6 +353,11 @@ __device__ inline void finish_frame(const ScoreParams& p, A* colsum, const A* if
   att[0] = column_sums(rows, HqV, RS, P, s->part) / (double)((long long)HqV * P);
   fft[0] = column_sums(ifft + (long long)sf * HkvV * P, HkvV, 1, P, s->part) / (double)((long long)HkvV * p.D);
   select_frame<1>(p, f, att, fft, refined, s->sc, s->ints, s->misc);
+  if (p.n_selected) {
+    __threadfence();                                       // this thread's ids are visible before the frame counts
+    __syncthreads();
+    if (tid == 0) atomicAdd(p.n_selected, 1);
+  }
 }
 
 // The work of one block: query head hv of frame f (a frame slot of the chunk); hv counts the query heads of all scoring

@@ -51,3 +51,38 @@ def test_a_wait_that_ran_out_does_not_reach_the_next_calls(lib, bf16):
     H.check_frames_against_oracle(run, st, range(18), full_layers=True)
     stats = run.ctx.mukv_get_stats()
     assert stats.device_status == 0 and stats.refined_frames == 18
+
+
+@pytest.mark.parametrize("bf16", [True, False])
+def test_two_contexts_on_two_streams_with_every_frame_flagged(bf16):
+    # Calls whose copies alone fill the device.  Each context's flagged frames find places held by the other's.
+    spec = StreamSpec(seed=85, n_layers=14, n_q_heads=28, n_kv_heads=4, head_dim=128, tokens_per_frame=196, bf16=bf16, n_outlier=2,
+                      n_frames=64, scene_sigma=1.0, frame_sigma=0.5, scene_min=10, scene_max=20)
+    wl = dict(spec=spec, keep=49, fseg=16, chunk=16, alpha=0.7)
+    runs = [H.GpuRun(wl, options={B.OPT_FLAG_MARGIN: 4.0}) for _ in range(3)]
+    dev = runs[0].device
+    kept = H.torch.full((3, 64, 49), -7, dtype=H.torch.int32, device=dev)
+    chunks = []
+    for t0 in range(0, 64, 16):
+        chunks.append(runs[0].gs.alloc(16))
+        runs[0].gs.fill(t0, 16, *chunks[-1])
+    for c, x in enumerate(chunks):                         # alone
+        runs[2].ctx.mukv_compress_chunk(*x, 16, 16 * c, kept[2, 16 * c:16 * c + 16])
+    H.torch.cuda.synchronize()
+    streams = [H.torch.cuda.Stream() for _ in range(2)]
+    for rep in range(3):
+        for i, s in enumerate(streams):
+            runs[i].ctx.mukv_reset(stream=s)
+        for c, x in enumerate(chunks):
+            for i, s in enumerate(streams):
+                runs[i].ctx.mukv_compress_chunk(*x, 16, 16 * c, kept[i, 16 * c:16 * c + 16], stream=s)
+        H.torch.cuda.synchronize()
+        for i in range(2):
+            stats = runs[i].ctx.mukv_get_stats()
+            assert stats.device_status == 0 and stats.refined_frames == 64
+            assert H.torch.equal(kept[i], kept[2])
+            for region in (0, 1, 2, 3, 4, 5):
+                assert H.torch.equal(runs[i].ctx.region(region), runs[2].ctx.region(region)), region
+        kept[:2] = -7
+    st = H.oracle_stream(spec, H.oracle_cfg(runs[2].cfg), range(2), last_only=True, workers=1)
+    assert kept[2, :2].tolist() == [x.tolist() for x in st.kept]
