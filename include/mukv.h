@@ -380,7 +380,8 @@ mukv_status mukv_profile_read(mukv_ctx* ctx, double* ms, int64_t* launches);
  * All calls on a device share the one array: two calls whose kernels may overlap on the device
  * (different streams without an ordering between them) race; what such calls return is undefined, later calls
  * are not affected.  If a bounded wait inside the tensor-core scoring kernel runs out (codes 3, 4, 5 of mukv_stats; never
- * seen), every id of the call is -1 and every score NaN.  Messages of failures are read
+ * seen), every id of the call is -1 and every score NaN; if a block of the double-precision pass waits in vain for a
+ * frame's selection (never seen either), those of that frame and of all frames that need this pass are.  Messages of failures are read
  * with mukv_last_error(NULL). */
 #define MUKV_NOALLOC_MAX_FRAMES 16
 #define MUKV_NOALLOC_MAX_Q_HEADS 32

@@ -841,9 +841,14 @@ __global__ void __launch_bounds__(kCompactThreads) zero_kernel(unsigned long lon
 }
 
 // Selection alone (scoring without a store, bf16): one block per frame, behind the persistent scoring kernel; the blocks behind
-// those score the flagged frames again in double precision, once every frame's ids are out (a launch of its own for that cost
+// those score the flagged frames again in double precision, once every frame's selection is out (a launch of its own for that cost
 // calls that flag nothing 0.4 us of 31).  A code in *scoring (one of that kernel's bounded waits ran out) leaves no sums to trust:
 // the ids are then -1 and the scores NaN.
+// Nor does a block that waits too long for a frame leave ids that single precision could not decide: it gives the frame up, in
+// the word that the frame's own block would publish in, and whoever finds that word so, all blocks behind the selection and the
+// frame's own one, takes back what is not final: that frame, and the flagged ones.  (Either every one of these blocks
+// finds all frames published, or none does.)
+constexpr unsigned kSelDone = 1u, kSelGivenUp = 2u, kSelRisky = 3u;
 __global__ void __launch_bounds__(kCompactThreads, 3) select_kernel(const __grid_constant__ CompactParams p, const int* scoring) {
   __shared__ union {
     struct {
@@ -852,29 +857,45 @@ __global__ void __launch_bounds__(kCompactThreads, 3) select_kernel(const __grid
     };
     Score64Scratch s64;
   } sh;
+  __shared__ unsigned s_word;
   const ScoreParams& sp = p.sp;
   const int n = sp.n_frames, tid = threadIdx.x;
   pdl_wait();
   pdl_trigger();
   const int failed = *scoring;
-  if ((int)blockIdx.x < n) {
-    const int f = blockIdx.x;
-    select_from_partials(p, f, true, sh.kept, &sh.ss);
+  auto take_back = [&](int f) {
     const long long np = (long long)n * sp.P;
-    for (int t = tid; failed && t < sp.P; t += kCompactThreads) {
+    for (int t = tid; t < sp.P; t += kCompactThreads) {
       if (t < sp.kappa) sp.kept_store[(long long)f * sp.kappa + t] = -1;
       for (int s = 0; s < 3 && sp.scores_out; ++s) sp.scores_out[s * np + (long long)f * sp.P + t] = __int_as_float(0x7fffffff);
     }
+  };
+  if ((int)blockIdx.x < n) {
+    const int f = blockIdx.x;
+    const bool risky = select_from_partials(p, f, true, sh.kept, &sh.ss);
+    if (failed) take_back(f);
     __threadfence();
     __syncthreads();
-    if (tid == 0) *reinterpret_cast<volatile unsigned*>(p.sel_flag + f) = 1u;
+    if (tid == 0) s_word = atomicCAS(p.sel_flag + f, 0u, risky ? kSelRisky : kSelDone);
+    __syncthreads();
+    if (s_word == kSelGivenUp) take_back(f);
     return;
   }
   if (failed) return;
-  const volatile unsigned* flag = p.sel_flag + tid;        // (n <= MUKV_NOALLOC_MAX_FRAMES)
-  const bool ok = tid >= n || wait_until(p.wait_ns, [&] { return *flag != 0u; });
+  unsigned word = kSelDone;
+  if (tid < n) {                                           // (n <= MUKV_NOALLOC_MAX_FRAMES)
+    const volatile unsigned* flag = p.sel_flag + tid;
+    if (!wait_until(p.wait_ns, [&] { return (word = *flag) != 0u; })) {
+      word = atomicCAS(p.sel_flag + tid, 0u, kSelGivenUp);
+      if (word == 0u) word = kSelGivenUp;
+    }
+  }
   __threadfence();
-  if (!__syncthreads_and(ok)) return;                      // (never seen; the frames keep their single-precision ids)
+  if (__syncthreads_or(word == kSelGivenUp)) {
+    for (int f = 0; f < n; ++f)                            // (no word changes any more)
+      if (*reinterpret_cast<volatile unsigned*>(p.sel_flag + f) == kSelRisky) take_back(f);
+    return;
+  }
   const int n_fl = *reinterpret_cast<volatile int*>(sp.n_flagged), blocks = gridDim.x - n, heads = sp.Ls * sp.Hq;
   if (n_fl == 0) return;
   const int rs = score64_split(n_fl, heads, sp.P, blocks, sp.scratch_rows), units = heads * rs;

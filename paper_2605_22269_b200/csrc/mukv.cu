@@ -1555,7 +1555,7 @@ cudaError_t noalloc_setup(int dev, const NoallocDevice** out) {
 
 template <typename T>
 mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_last, int n, int* d_kept_out,
-                         float* d_scores_out, cudaStream_t st) {
+                         float* d_scores_out, cudaStream_t st, unsigned long long wait_ns) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
@@ -1615,7 +1615,7 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
     cp.colsum_d = reinterpret_cast<double*>(base + kNaColD);
     cp.ifft_d = reinterpret_cast<double*>(base + kNaFftD);
     cp.sp.scratch_rows = kNaFrames * kNaHq;
-    cp.wait_ns = kWaitNs;
+    cp.wait_ns = wait_ns;
     // (blocks for the flagged frames: three per SM are resident beside one another; they wait for the first n only)
     const int units = n * c.n_q_heads * ((P + 7) / 8);
     e = launch_k(select_kernel, dim3(n + std::min(units, 3 * nd->n_sms)), kCompactThreads, 0, st, true, cp, (const int*)pl.status);
@@ -1637,11 +1637,9 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
   return MUKV_OK;
 }
 
-}  // namespace
-
-extern "C" mukv_status mukv_score_frames_noalloc(const mukv_config* cfg, const void* d_q, const void* d_k_last,
-                                                 int32_t n_frames, int32_t* d_kept_out, float* d_scores_out,
-                                                 mukv_stream stream) {
+// wait_ns: limit of the waits inside select_kernel
+mukv_status score_frames_noalloc(const mukv_config* cfg, const void* d_q, const void* d_k_last, int32_t n_frames,
+                                 int32_t* d_kept_out, float* d_scores_out, mukv_stream stream, unsigned long long wait_ns) {
   try {
     if (!cfg || !d_q || !d_k_last) return fail(nullptr, MUKV_E_INVALID, "null argument");
     if (!d_kept_out && !d_scores_out) return fail(nullptr, MUKV_E_INVALID, "no output requested");
@@ -1667,9 +1665,17 @@ extern "C" mukv_status mukv_score_frames_noalloc(const mukv_config* cfg, const v
       return fail(nullptr, MUKV_E_ALIGN, "d_q, d_k_last must be 16-byte aligned, the outputs 4-byte aligned");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (c.dtype == MUKV_BF16)
-      return noalloc_impl<__nv_bfloat16>(c, d_q, d_k_last, n_frames, d_kept_out, d_scores_out, st);
-    return noalloc_impl<float>(c, d_q, d_k_last, n_frames, d_kept_out, d_scores_out, st);
+      return noalloc_impl<__nv_bfloat16>(c, d_q, d_k_last, n_frames, d_kept_out, d_scores_out, st, wait_ns);
+    return noalloc_impl<float>(c, d_q, d_k_last, n_frames, d_kept_out, d_scores_out, st, wait_ns);
   } catch (...) {
     return fail(nullptr, MUKV_E_INVALID, "unexpected exception");
   }
+}
+
+}  // namespace
+
+extern "C" mukv_status mukv_score_frames_noalloc(const mukv_config* cfg, const void* d_q, const void* d_k_last,
+                                                 int32_t n_frames, int32_t* d_kept_out, float* d_scores_out,
+                                                 mukv_stream stream) {
+  return score_frames_noalloc(cfg, d_q, d_k_last, n_frames, d_kept_out, d_scores_out, stream, kWaitNs);
 }

@@ -22,4 +22,6 @@ def load():
         _LIB = B.load_library(out)
         _LIB.internals_wait_limit.restype = None
         _LIB.internals_wait_limit.argtypes = [C.c_void_p, C.c_ulonglong]
+        _LIB.internals_score_noalloc.restype = C.c_int32
+        _LIB.internals_score_noalloc.argtypes = _LIB.mukv_score_frames_noalloc.argtypes + [C.c_ulonglong]
     return _LIB

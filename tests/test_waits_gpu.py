@@ -86,3 +86,30 @@ def test_two_contexts_on_two_streams_with_every_frame_flagged(bf16):
         kept[:2] = -7
     st = H.oracle_stream(spec, H.oracle_cfg(runs[2].cfg), range(2), last_only=True, workers=1)
     assert kept[2, :2].tolist() == [x.tolist() for x in st.kept]
+
+
+def test_scoring_without_a_workspace_takes_back_what_it_could_not_decide(lib):
+    # frames 3 and 9 hold every token twice and keep an odd number: only double precision decides them
+    spec = StreamSpec(seed=86, n_layers=1, n_q_heads=28, n_kv_heads=4, head_dim=128, tokens_per_frame=196, bf16=True, n_outlier=1,
+                      n_frames=16, scene_sigma=1.0, frame_sigma=0.5, scene_min=2, scene_max=4)
+    q, k, _ = spec.chunk(0, 16)
+    for f in (3, 9):
+        q[f, 1::2], k[0, f, 1::2] = q[f, ::2], k[0, f, ::2]
+    cfg = H.spec_config(spec, dict(keep=49, fseg=1, chunk=16, alpha=0.7))
+    ref = [O.score_frame(q[f], k[0, f], float(cfg.alpha)) for f in range(16)]
+    ids = [O.select_tokens(r[2], 49).tolist() for r in ref]
+    dq, dk = H.to_device(q, True), H.to_device(k[0], True)
+    kept = H.torch.full((16, 49), -7, dtype=H.torch.int32, device="cuda:0")
+    scores = H.torch.zeros((3, 16, 196), device="cuda:0")
+    for ns in (0, 1_500_000_000, 0, 1_500_000_000):
+        kept.fill_(-7)
+        assert lib.internals_score_noalloc(B.C.byref(cfg), dq.data_ptr(), dk.data_ptr(), 16, kept.data_ptr(), scores.data_ptr(),
+                                           B._stream(None), ns) == 0
+        got, sc = kept.tolist(), scores.cpu().numpy()
+        back = [f for f in range(16) if got[f] == [-1] * 49 and np.isnan(sc[:, f]).all()]
+        assert bool(back) == (ns == 0)
+        for f in range(16):
+            if f not in back:
+                assert got[f] == ids[f], f
+                for i in range(3):
+                    H.close(sc[i, f], ref[f][i], f"score[{i}] frame {f}")
