@@ -1033,8 +1033,8 @@ mukv_status retrieve_impl(mukv_ctx* ctx, const void* d_qtok, const int32_t* h_q_
         rp.stage |= 1 << i;
         stage = std::max(stage, b);
       }
-      const unsigned roles = k_pat > 0 ? 3 : 2;
-      e = launch_c(rank_kernel, dim3(nq * roles), kRankThreads, rank_smem + stage, st, !ctx->prof_on, roles, rp, meta);
+      rp.roles = rank_roles(mode, k_pat);
+      e = launch_c(rank_kernel, dim3(nq * rp.roles), kRankThreads, rank_smem + stage, st, !ctx->prof_on, rp.roles, rp, meta);
     }
     if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "rank kernel: %s", cudaGetErrorString(e));
     ctx->launches += 4;

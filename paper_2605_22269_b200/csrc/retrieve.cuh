@@ -776,6 +776,7 @@ __device__ __forceinline__ int topk_set(const double* scores, const int* cnt, in
 struct RankParams {
   int nq, C, fseg;
   int k_seg, k_frm, k_pat, top_n, mode;
+  int roles;                              // blocks per question, see rank_roles
   int S;                                  // patch-level blocks per frame (0: none)
   double lam_seg, lam_frm, lam_pat, delta;
   long long n_frm, n_seg;                 // stored
@@ -889,13 +890,17 @@ __device__ __forceinline__ void rank_emit(int* idx, float* score, long long base
 // global query, which is read from block 0's shared memory behind a cluster barrier.  (One block after the other: 14.5 us for
 // one question on an hour of video, of which the segments and the global query were 5; bound by a chain of barriers, round
 // trips to L2 and instruction fetch, so that blocks beside one another are what helps.)
+// HIER looks at the frames of the selected segments only, so a block of the frames would wait for that of the segments from the
+// start: block 0 ranks both, block 1 (k_pat > 0) the patch-level blocks beside its frames.  (With a block each, the hand-over cost
+// one question on three hours of video 25.8 us with its gather, now 24.4; 64 on half an hour 65.2, now 64.3.)
+__host__ __device__ inline int rank_roles(int mode, int k_pat) { return (mode == MUKV_RETR_HIER ? 1 : 2) + (k_pat > 0 ? 1 : 0); }
 __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, const QMeta meta) {
   __shared__ RankShared sh;
   __shared__ __align__(8) uint64_t s_bar[1];
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double* gq = reinterpret_cast<double*>(smem_raw);               // [C] global query
 
-  const int role = (int)tc::cluster_rank(), roles = p.k_pat > 0 ? 3 : 2;
+  const int role = (int)tc::cluster_rank(), roles = p.roles;
   const int qi = blockIdx.x / roles, tid = threadIdx.x;
   if (role > 0) tc::cluster_arrive();                        // (phase 1: block 0 arrives when the others may go on)
   pdl_wait();                                                // the scores of the scan are complete
@@ -984,55 +989,64 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
       c_seg = rank_level(ss, nullptr, n_seg, p.k_seg, semi && p.lam_seg > 0.0, p.lam_seg, p.delta, p.seg_key, C, gq, false, &sh, buf);
     rank_emit(p.seg_idx, p.seg_score, (long long)qi * p.k_seg, p.k_seg, c_seg, &sh);
     if (tid == 0) p.counts[p.counts_stride * qi] = c_seg;
-    if (hier) {
-      for (int i = tid; i < c_seg; i += kRankThreads) sh.sel_seg[i] = sh.pick[i];
-      if (tid == 0) sh.c_seg = c_seg;
-      tc::cluster_arrive();
+    if (!hier) {
+      tc::cluster_wait();
+      tc::cluster_arrive();                                  // phase 2: the others have read what they need
+      tc::cluster_wait();
+      return;
     }
-    tc::cluster_wait();
-    tc::cluster_arrive();                                    // phase 2: the others have read what they need
-    tc::cluster_wait();
-    return;
+    for (int i = tid; i < c_seg; i += kRankThreads) sh.sel_seg[i] = sh.pick[i];
+    if (tid == 0) sh.c_seg = c_seg;
+    if (roles > 1) tc::cluster_arrive();
+    __syncthreads();
   }
 
   // ---- frames, or patch-level blocks: (frame, super patch) pairs that kept at least one token
-  const double* sc = role == 1 ? sf : sp;
-  const int* cnt = role == 1 ? nullptr : p.patch_cnt;
-  const int k = role == 1 ? p.k_frm : p.k_pat;
+  const bool frames = hier ? role == 0 : role == 1;
+  const double* sc = frames ? sf : sp;
+  const int* cnt = frames ? nullptr : p.patch_cnt;
+  const int k = frames ? p.k_frm : p.k_pat;
   int c = 0;
   if (hier) {
     // Only what lies inside the selected segments is a candidate.  Those are few, so the ranking runs over positions in the
     // list "selected segments (ascending) x their blocks" and maps the winners back (ascending position = ascending block).
-    tc::cluster_wait();
-    const int c_seg = tc::cluster_ld_int(&sh.c_seg, 0);
-    for (int i = tid; i < c_seg; i += kRankThreads) sh.sel_seg[i] = tc::cluster_ld_int(sh.sel_seg + i, 0);
-    tc::cluster_arrive();
-    __syncthreads();
-    const int per_seg = p.fseg * (role == 1 ? 1 : p.S);
+    if (role > 0) {
+      tc::cluster_wait();
+      const int c_seg = tc::cluster_ld_int(&sh.c_seg, 0);
+      for (int i = tid; i < c_seg; i += kRankThreads) sh.sel_seg[i] = tc::cluster_ld_int(sh.sel_seg + i, 0);
+      if (tid == 0) sh.c_seg = c_seg;
+      tc::cluster_arrive();
+      __syncthreads();
+    }
+    const int per_seg = p.fseg * (frames ? 1 : p.S), n_blocks = frames ? n_frm : n_frm * p.S;
     auto block_of = [&](int i) { return sh.sel_seg[i / per_seg] * per_seg + i % per_seg; };
     auto score_h = [&](int i) { return sc[block_of(i)]; };
     auto member_h = [&](int i) {
       const int b = block_of(i);
-      return b < n && (!cnt || cnt[b] > 0);
+      return b < n_blocks && (!cnt || cnt[b] > 0);
     };
-    c = block_topk_set(score_h, member_h, c_seg * per_seg, k, p.delta, sh.pick, sh.pick_score, &sh.sc);
+    c = block_topk_set(score_h, member_h, sh.c_seg * per_seg, k, p.delta, sh.pick, sh.pick_score, &sh.sc);
     for (int i = tid; i < c; i += kRankThreads) sh.pick[i] = block_of(sh.pick[i]);
     __syncthreads();
   } else {
-    c = rank_level(sc, cnt, n, k, semi, role == 1 ? p.lam_frm : p.lam_pat, p.delta, role == 1 ? p.frame_key : p.patch_key, C, gq,
+    c = rank_level(sc, cnt, n, k, semi, frames ? p.lam_frm : p.lam_pat, p.delta, frames ? p.frame_key : p.patch_key, C, gq,
                    true, &sh, buf);
     if (!semi) {
       tc::cluster_wait();
       tc::cluster_arrive();
     }
   }
-  if (role == 1) rank_emit(p.frm_idx, p.frm_score, (long long)qi * p.k_frm, p.k_frm, c, &sh);
+  if (frames) rank_emit(p.frm_idx, p.frm_score, (long long)qi * p.k_frm, p.k_frm, c, &sh);
   else rank_emit(p.pat_idx, p.pat_score, (long long)qi * p.k_pat, p.k_pat, c, &sh);
   if (tid == 0) {
-    p.counts[p.counts_stride * qi + role] = c;
-    if (roles == 2 && p.counts_stride > 2) p.counts[p.counts_stride * qi + 2] = 0;
+    p.counts[p.counts_stride * qi + (frames ? 1 : 2)] = c;
+    if (p.k_pat == 0 && p.counts_stride > 2) p.counts[p.counts_stride * qi + 2] = 0;
   }
-  tc::cluster_wait();
+  if (roles > 1) tc::cluster_wait();
+  if (roles > 1 && role == 0) {                              // (HIER) phase 2: the other has read what it needs
+    tc::cluster_arrive();
+    tc::cluster_wait();
+  }
 }
 
 // ------------------------------------------------------------------------------ Eq. 9

@@ -150,3 +150,17 @@ def test_paper_k_and_lambda_on_the_one_hour_stream():
         retrieve3_check(run, st, qtok, offs, (20, 32, 12), (0.3, 0.3, 0.0), mode, full_layers=False)
     retrieve3_check(run, st, qtok, offs, (20, 32, 12), (0.3, 0.3, 0.0), B.RETR_SEMI, full_layers=False,
                     t_limit=np.array([900, 1, 17, 1799, 1800, 16, 450, 1000]))
+
+
+@pytest.mark.parametrize("n_q", [1, 9])
+def test_segments_first_with_and_without_the_patch_level(n_q):
+    # HIER ranks the frames in the block of the segments and the patch-level blocks beside them: no cluster without the
+    # patch level; questions that see no segment, some, all; more than the ranking reads directly (128) of each granularity
+    spec = StreamSpec(seed=43, n_layers=1, n_q_heads=4, n_kv_heads=1, head_dim=64, tokens_per_frame=16, bf16=True, n_outlier=1,
+                      n_frames=600, scene_sigma=1.0, frame_sigma=0.5, scene_min=2, scene_max=4)
+    run = H.GpuRun(dict(spec=spec, keep=4, fseg=4, chunk=60, alpha=0.7), patch_split=2, grid_width=4).compress()
+    st = H.oracle_stream(spec, H.oracle_cfg(run.cfg), range(600), last_only=False, workers=1)
+    qtok, offs, _ = spec.questions(n_q, 1, 6)
+    for limit in (None, np.resize(np.array([0, 3, 4, 37, 599, 600]), n_q)):
+        for k in ((0, 5, 3), (7, 5, 3), (0, 200, 140), (250, 200, 140)):
+            retrieve3_check(run, st, qtok, offs, k, (0.3, 0.3, 0.0), B.RETR_HIER, t_limit=limit, full_layers=False)
