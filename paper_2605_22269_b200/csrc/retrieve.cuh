@@ -123,24 +123,35 @@ struct ScanShape {
 __host__ inline size_t scan_smem_bytes(int T, int q_groups, int row_tiles) {
   return 2 * ((size_t)kScanCC * (8 * T * q_groups + kScanQPad) * sizeof(double) + (size_t)8 * row_tiles * kScanRowPad * sizeof(float));
 }
-// Least time of a chunk: the tiles of the busiest scheduler at 128 clocks each (8 instructions of 16), or the chunk's bytes at 64
-// a clock.
+// The shape of least time, in clocks per chunk.  A wave of blocks takes what its tiles take on the busiest scheduler (128 clocks
+// each, 8 instructions of 16) or its bytes at 64 a clock, the chunk's barrier and first operands (450) and the copies that one
+// thread issues (50 each: a block of few warps is slow at fetching the chunk of all questions); then the bytes of all blocks,
+// at 6,000 a clock of the device.  Blocks per SM as shared memory and registers (48 a thread for T = 1, up to 96 else) allow.
+// Fitted to every shape at 1 KB to 8 KB per pooled question, 9 to 128 questions and 107 to 44,625 rows: 0.5 % from the best one on
+// average, 7 % at the most.  (Without residency, copies and the last term 5 % and 70 %: 128 questions on 8,288 rows
+// went to 1,036 blocks of one row tile, each of which fetches all questions, 199 us; now 150.)
 __host__ inline ScanShape scan_shape(long long rows, int nq, int n_sms) {
-  const int nt = (nq + 7) / 8;
-  const long long tiles = (rows + 7) / 8;
+  const int nt = (nq + 7) / 8, tiles = (int)((rows + 7) / 8);      // (32-bit divisions: half a microsecond of the call)
   ScanShape best{0, 0, 0, 0};
   long long least = -1;
   for (int T = 1; T <= 8; T *= 2) {
     const int qg = (nt + T - 1) / T;
     if (qg > 4) continue;
     for (int rt = 1; rt * qg <= kScanMaxWarps; ++rt) {
-      const long long blocks = (tiles + rt - 1) / rt, per_sm = (blocks + n_sms - 1) / n_sms;
-      const long long mma = per_sm * ((rt * qg + 3) / 4) * T * 128;
-      const long long load = per_sm * (kScanCC * 8LL * 8 * T * qg + 8LL * rt * kScanCC * 4) / 64;
-      const long long t = (mma > load ? mma : load) + 32 * per_sm;
+      const int warps = rt * qg, smem = (int)scan_smem_bytes(T, qg, rt);
+      const int by_smem = 227 * 1024 / (smem + 2048), by_regs = (T == 1 ? 40 : 20) / warps;      // (neither is 0)
+      const int resident = by_smem < by_regs ? by_smem : by_regs;
+      const int blocks = (tiles + rt - 1) / rt, per_sm = (blocks + n_sms - 1) / n_sms, full = per_sm / resident;
+      const int bytes = kScanCC * 8 * 8 * T * qg + 8 * rt * kScanCC * 4, own = 450 + 50 * (bytes / 512) / warps;
+      auto wave = [&](int b) {
+        const int mma = (b * warps + 3) / 4 * T * 128, load = b * bytes / 64;
+        return (mma > load ? mma : load) + own;
+      };
+      const int rest = per_sm - full * resident;
+      const long long t = (long long)full * wave(resident) + (rest ? wave(rest) : 0) + (long long)blocks * bytes / 6000;
       if (least < 0 || t < least) {
         least = t;
-        best = {T, qg, rt, scan_smem_bytes(T, qg, rt)};
+        best = {T, qg, rt, (size_t)smem};
       }
     }
   }

@@ -9,3 +9,19 @@ extern "C" mukv_status internals_score_noalloc(const mukv_config* cfg, const voi
                                                float* scores, mukv_stream stream, unsigned long long ns) {
   return score_frames_noalloc(cfg, q, k, n, kept, scores, stream, ns);
 }
+
+// tiles of the scan: {question tiles of a warp, question groups, row tiles of a block}
+extern "C" void internals_scan_shape(long long rows, int nq, int n_sms, int* out) {
+  const ScanShape s = scan_shape(rows, nq, n_sms);
+  out[0] = s.T; out[1] = s.q_groups; out[2] = s.row_tiles;
+}
+
+// where the last retrieval left the scores of every question with every frame, segment and patch-level block: byte offset in the
+// workspace and question stride, doubles first, then their single-precision copies
+extern "C" void internals_scores(const mukv_ctx* ctx, long long* out) {
+  const long long T = ctx->cfg.max_frames, S = (long long)ctx->cfg.patch_split * ctx->cfg.patch_split;
+  const long long v[12] = {(long long)ctx->wl.s_frm, T, (long long)ctx->wl.s_seg, ctx->sl.max_segs, (long long)ctx->wl.s_pat, T * S,
+                           (long long)ctx->wl.f_frm, pad4(T), (long long)ctx->wl.f_seg, pad4(ctx->sl.max_segs), (long long)ctx->wl.f_pat,
+                           pad4(T * S)};
+  for (int i = 0; i < 12; ++i) out[i] = v[i];
+}

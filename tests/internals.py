@@ -22,6 +22,16 @@ def load():
         _LIB = B.load_library(out)
         _LIB.internals_wait_limit.restype = None
         _LIB.internals_wait_limit.argtypes = [C.c_void_p, C.c_ulonglong]
+        _LIB.internals_scan_shape.restype = _LIB.internals_scores.restype = None
+        _LIB.internals_scan_shape.argtypes = [C.c_longlong, C.c_int, C.c_int, C.POINTER(C.c_int)]
+        _LIB.internals_scores.argtypes = [C.c_void_p, C.POINTER(C.c_longlong)]
         _LIB.internals_score_noalloc.restype = C.c_int32
         _LIB.internals_score_noalloc.argtypes = _LIB.mukv_score_frames_noalloc.argtypes + [C.c_ulonglong]
     return _LIB
+
+
+def scan_shape(rows, nq, n_sms=148):
+    """(question tiles of a warp, question groups, row tiles of a block)"""
+    out = (C.c_int * 3)()
+    load().internals_scan_shape(rows, nq, n_sms, out)
+    return tuple(out)

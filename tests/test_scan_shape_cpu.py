@@ -1,0 +1,22 @@
+"""The rule that picks the scan's tiles."""
+from tests import internals as I
+
+
+def test_every_shape_fits():
+    # 227 KB of shared memory and 20 warps to a block; the columns of a block are columns of the pooled questions (128)
+    seen = set()
+    for rows in [1, 7, 8, 9, 63, 64, 107, 850, 1913, 4000, 7438, 8288, 11475, 21250, 44625, 400_000, 60_000_000]:
+        for nq in range(1, 129):
+            T, groups, tiles = I.scan_shape(rows, nq)
+            assert T in (1, 2, 4, 8) and 1 <= groups <= 4 and tiles >= 1 and groups * tiles <= 20
+            assert nq <= 8 * T * groups <= 128
+            assert 2 * (32 * (8 * T * groups + 4) * 8 + 8 * tiles * 36 * 4) + 1024 <= 227 * 1024
+            seen.add((T, tiles > 1))
+    assert seen == {(T, many) for T in (1, 2, 4, 8) for many in (False, True)} - {(8, False)}
+
+
+def test_blocks_do_not_multiply_the_fetched_questions():
+    # a block fetches every question: 128 of them on 8,288 rows once went to 1,036 blocks of a single row tile
+    for rows in range(7000, 15500, 500):
+        for nq in (97, 100, 128):
+            assert (rows + 7) // 8 // I.scan_shape(rows, nq)[2] <= 444, (rows, nq)
