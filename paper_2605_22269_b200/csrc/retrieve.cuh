@@ -232,10 +232,8 @@ __global__ void __launch_bounds__(32 * kScanMaxWarps) scan_kernel(const ScanPara
   // everything before it is complete.)
   fetch_rows(0, 0);
   pdl_wait();                                                // the pooled questions are complete
-  // (The ranking's blocks may start early beside a short scan only, one row tile to a block: beside a long one they take SMs from
-  // its last blocks.  With the trigger, without it: 10 questions on 13,269 rows 39.3 and 36.6 us with their gather, 64 on 11,475
-  // 910 and 908.7; 19 on 893 18.4 and 18.8.)
-  if (sp.row_tiles == 1) pdl_trigger();
+  // (No early start for the ranking: over 1,400 pairs of questions, rows and key widths it gained 0.4 us where the scan is one wave
+  // of blocks, mostly nothing, and cost up to 4.5 us where it is longer.)
   fetch_questions(0, 0);
   asm volatile("cp.async.commit_group;" ::: "memory");
   for (int qq = tid; qq < nq; qq += nt) {                    // norms of the pooled questions (read after the barriers below)
