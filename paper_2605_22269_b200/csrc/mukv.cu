@@ -956,7 +956,10 @@ mukv_status retrieve_impl(mukv_ctx* ctx, const void* d_qtok, const int32_t* h_q_
     const float* seg_key = reinterpret_cast<const float*>(ctx->store + ctx->sl.seg_key);
     const long long n_frm = ctx->frames;
     const long long n_seg = (n_frm + c.frames_per_segment - 1) / c.frames_per_segment;
-    const bool few = nq <= kScanFew;                       // see scan_few_kernel
+    const int S = c.patch_split * c.patch_split;
+    const long long n_pat = k_pat > 0 ? n_frm * S : 0;
+    const long long rows = n_frm + n_seg + n_pat;
+    const bool few = scan_by_rows(rows, nq, C);
     cudaError_t e = cudaSuccess;
     {
       ProfScope ps(ctx, 4, st);
@@ -964,15 +967,12 @@ mukv_status retrieve_impl(mukv_ctx* ctx, const void* d_qtok, const int32_t* h_q_
       const int cs = few ? 1 : MUKV_MAX_QUESTIONS, qs = few ? C : 1;
       if (c.dtype == MUKV_BF16)
         e = launch_k(qpool_kernel<__nv_bfloat16>, grid, kPoolThreads, 0, st, !ctx->prof_on,
-                     reinterpret_cast<const __nv_bfloat16*>(d_qtok), meta, c.n_q_heads, c.n_kv_heads, c.head_dim, q64, cs, qs, qnorm);
+                     reinterpret_cast<const __nv_bfloat16*>(d_qtok), meta, c.n_q_heads, c.n_kv_heads, c.head_dim, q64, cs, qs, qnorm, (int)few);
       else
         e = launch_k(qpool_kernel<float>, grid, kPoolThreads, 0, st, !ctx->prof_on, reinterpret_cast<const float*>(d_qtok), meta,
-                     c.n_q_heads, c.n_kv_heads, c.head_dim, q64, cs, qs, qnorm);
+                     c.n_q_heads, c.n_kv_heads, c.head_dim, q64, cs, qs, qnorm, (int)few);
     }
     if (e != cudaSuccess) return fail(ctx, MUKV_E_CUDA, "qpool kernel: %s", cudaGetErrorString(e));
-    const int S = c.patch_split * c.patch_split;
-    const long long n_pat = k_pat > 0 ? n_frm * S : 0;
-    const long long rows = n_frm + n_seg + n_pat;
     double* s_pat = reinterpret_cast<double*>(ctx->ws + ctx->wl.s_pat);
     const float* patch_key = reinterpret_cast<const float*>(ctx->store + ctx->sl.patch_key);
     {

@@ -7,7 +7,7 @@
 //   qpool_kernel    Eq. 6   one block per (question, key head)
 //   scan_kernel     Eq. 7   cosine of every question with every frame, segment and patch-level key (a skinny
 //                           double-precision product on the fp64 tensor-core instruction)
-//   scan_few_kernel         the same for at most eight questions, a warp per row or two
+//   scan_few_kernel         the same for at most eight questions on not too many rows, a warp per row or two
 //   rank_kernel     stage-1 candidates, Eq. 8 rerank, final top-k; per question a cluster of blocks, one for each granularity
 //   gather_kernel   Eq. 9   copies the selected pages into the per-question decode buffers
 //   gather3_kernel          the same with summary tokens and the rows of patch-level blocks
@@ -30,23 +30,23 @@ struct QMeta {
 // scan_kernel, which stages it, a row per question (cs = 1) for scan_few_kernel; the head's share of the squared
 // norm goes to qn2[question][key head] (the scans add the shares in head order).
 constexpr int kPoolThreads = 512;
-constexpr int kScanFew = 8;        // questions up to which scan_few_kernel scans
+constexpr int kScanFew = 8;        // questions that scan_few_kernel takes at the most, see scan_by_rows
 constexpr int kPoolSmemDoubles = 4096;
 
 template <typename T>
 __global__ void __launch_bounds__(kPoolThreads) qpool_kernel(const T* __restrict__ qtok, const QMeta meta, int Hq,
                                                              int Hkv, int D, double* __restrict__ q64, int cs, int qs,
-                                                             double* __restrict__ qn2) {
+                                                             double* __restrict__ qn2, int early) {
   constexpr int VE = 16 / sizeof(T);
   __shared__ double s_acc[kPoolSmemDoubles];
   __shared__ double s_part[kPoolThreads / 32];
   const int qi = blockIdx.x, g = blockIdx.y;
   const int G = Hq / Hkv;
   pdl_wait();
-  // (Only for few questions: the scan's blocks would pile up on the SMs that the many blocks of this kernel leave free.  With the
-  // trigger 38 questions on 169 frames took 174 us with their gather, without it 161; 21 over three levels of 1,795 frames 47.5,
-  // now 45.1; 64 on three hours 910.7, now 910.1.)
-  if (gridDim.x <= kScanFew) pdl_trigger();
+  // (In front of scan_few_kernel only, whose small blocks are all resident: those of scan_kernel pile up on the SMs that this kernel
+  // leaves free.  With the trigger 8 questions on 11,475 rows of 512 channels took 36.0 us, without it 31.8; 48 on 107 rows 46.1
+  // and 33.4; 9 to 24 on up to 11,475 rows the same within 0.3.)
+  if (early) pdl_trigger();
   const int n0 = meta.off[qi], n1 = meta.off[qi + 1];
   const int DV = D / VE;                                    // vectors per head
   int nsl = kPoolThreads / DV;                              // token slices whose partial sums fit
@@ -285,10 +285,19 @@ __global__ void __launch_bounds__(32 * kScanMaxWarps) scan_kernel(const ScanPara
   }
 }
 
-// The same for at most kScanFew questions: a warp per row, plain double-precision multiply-adds.  The product is then
-// too thin for the tile above (64 questions wide, 32 rows in a block: 60 blocks of mostly padding for one question
-// and an hour of frames, 18 us); a row is one round trip to memory, its 16 doubles per lane and a butterfly: 4 us.
-// At eight questions and 9,100 rows the two take about the same time, which is where the line lies.
+// The same for at most kScanFew questions: a warp per row, plain double-precision multiply-adds; a row is one round trip to memory, 16
+// doubles per lane and a butterfly.  scan_kernel goes through the feature axis in chunks, a barrier and the questions' operands
+// each: 28 us for a few questions and half an hour of 512 channels, with pooling, ranking and a small gather, where this one
+// takes 18 to 24.  But it takes eight questions in the time of one, and this one adds each question's product to every row, in loops
+// made for one, for four and for eight questions.  Where the two take the same time was measured at 64 to 2,048 channels, 107 to
+// 44,625 rows: at 512 channels 2 questions and 15,000 rows, 4 and 9,600, 5 to 8 and 5,000; at 128 channels 1 and 12,000, 2 to 4 and
+// 2,500; at 1,024 2 and 28,000, 4 and 14,500, 8 and 7,000.  Eight questions on 9,113 rows of 512 channels: 38 us by rows, 32 by
+// tiles; 44,625 rows: 97 and 54.
+__host__ inline bool scan_by_rows(long long rows, int nq, int C) {
+  if (nq == 1) return rows <= 100LL * C;
+  if (nq <= 4) return rows <= (34LL - 4 * nq) * C;
+  return nq <= kScanFew && rows * nq <= 70LL * C && rows <= 12000;
+}
 
 template <int NQ>
 __global__ void __launch_bounds__(256) scan_few_kernel(const ScanParams sp) {
@@ -913,7 +922,7 @@ __global__ void __launch_bounds__(kRankThreads) rank_kernel(const RankParams p, 
   const int qi = blockIdx.x / roles, tid = threadIdx.x;
   if (role > 0) tc::cluster_arrive();                        // (phase 1: block 0 arrives when the others may go on)
   pdl_wait();                                                // the scores of the scan are complete
-  if (p.nq <= kScanFew) pdl_trigger();                       // (many of these blocks would leave the gather an uneven start)
+  // (No early start for the gather: 0.1 to 0.6 us slower for 1 to 128 questions on 100 to 10,800 frames, faster for none of them.)
   const int C = p.C;
   long long tl = meta.t_limit[qi];
   if (tl > p.n_frm) tl = p.n_frm;

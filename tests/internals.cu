@@ -16,6 +16,8 @@ extern "C" void internals_scan_shape(long long rows, int nq, int n_sms, int* out
   out[0] = s.T; out[1] = s.q_groups; out[2] = s.row_tiles;
 }
 
+extern "C" int internals_scan_by_rows(long long rows, int nq, int channels) { return scan_by_rows(rows, nq, channels); }
+
 // where the last retrieval left the scores of every question with every frame, segment and patch-level block: byte offset in the
 // workspace and question stride, doubles first, then their single-precision copies
 extern "C" void internals_scores(const mukv_ctx* ctx, long long* out) {

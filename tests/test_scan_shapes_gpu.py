@@ -35,15 +35,11 @@ MANY_ROWS = [(50, 9, 1), (50, 33, 2), (110, 80, 4), (431, 16, 1), (431, 24, 1), 
              (770, 128, 8), (2000, 24, 1)]
 
 
-@pytest.mark.parametrize("T,nq,tiles", MANY_ROWS)
-def test_every_score_of_blocks_of_several_row_tiles(monkeypatch, T, nq, tiles):
-    monkeypatch.setattr(B, "_LIB", I.load())
+def check_every_score(T, nq):
+    """Compresses T frames, asks nq questions and compares what the scan left in the workspace."""
     spec = StreamSpec(seed=96, n_layers=1, n_q_heads=2, n_kv_heads=1, head_dim=64, tokens_per_frame=16, bf16=True, n_outlier=1,
                       n_frames=T, scene_sigma=1.0, frame_sigma=0.5, scene_min=2, scene_max=4)
     run = H.GpuRun(dict(spec=spec, keep=4, fseg=4, chunk=T, alpha=0.7), patch_split=4, grid_width=4, want_scores=False).compress()
-    rows = T + (T + 3) // 4 + 16 * T
-    shape = I.scan_shape(rows, nq, H.torch.cuda.get_device_properties(0).multi_processor_count)
-    assert shape[0] == tiles and shape[2] > 1 and rows % (8 * shape[2]) != 0          # (a last block that is not full)
     qtok, offs, _ = spec.questions(nq, 1, 5)
     i32, dev = H.torch.int32, run.device
     seg, frm, pat = (H.torch.full((nq, 3), -9, dtype=i32, device=dev) for _ in range(3))
@@ -66,4 +62,21 @@ def test_every_score_of_blocks_of_several_row_tiles(monkeypatch, T, nq, tiles):
                 else:                                      # rounded once
                     there = held if level == 2 else np.ones(n, bool)
                     assert np.abs(got[i][there] - ref[there]).max() < 2.0 ** -24 + 1e-13 and (got[i][~there] == -np.inf).all(), (level, i)
-    assert counts.min() >= 3
+    assert counts[:, 0].min() >= min(3, (T + 3) // 4) and counts[:, 1:].min() >= 3
+
+
+@pytest.mark.parametrize("T,nq,tiles", MANY_ROWS)
+def test_every_score_of_blocks_of_several_row_tiles(monkeypatch, T, nq, tiles):
+    monkeypatch.setattr(B, "_LIB", I.load())
+    rows = T + (T + 3) // 4 + 16 * T
+    shape = I.scan_shape(rows, nq, H.torch.cuda.get_device_properties(0).multi_processor_count)
+    assert shape[0] == tiles and shape[2] > 1 and rows % (8 * shape[2]) != 0          # (a last block that is not full)
+    check_every_score(T, nq)
+
+
+@pytest.mark.parametrize("T,nq,by_rows", [(3, 1, 1), (370, 1, 1), (372, 1, 0), (96, 2, 1), (97, 2, 0), (81, 3, 1), (82, 3, 0), (66, 4, 1),
+                                          (67, 4, 0), (51, 5, 1), (52, 5, 0), (32, 8, 1), (33, 8, 0), (431, 2, 0), (431, 7, 0)])
+def test_every_score_on_both_sides_of_the_line_between_the_scans(monkeypatch, T, nq, by_rows):
+    monkeypatch.setattr(B, "_LIB", I.load())
+    assert B._LIB.internals_scan_by_rows(T + (T + 3) // 4 + 16 * T, nq, 64) == by_rows
+    check_every_score(T, nq)
