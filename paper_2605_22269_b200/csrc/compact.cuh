@@ -806,11 +806,9 @@ __global__ void __launch_bounds__(kCompactThreads, 3) compact_kernel(const __gri
   } else if (sel_mode == 2) {
     // Ranking by numbers the caller supplies (no Eq. 1-4): every block ranks its frame itself, in
     // double precision on exact inputs, so nothing is ever too close to call; plane 0 writes the ids.
-    double sx[1] = {tid < p.P ? (double)__ldg(p.ext_scores + (long long)f * p.P + tid) : 0.0};
-    const bool bad = __syncthreads_or(tid < p.P && !isfinite(sx[0])) != 0;
-    if (bad) sx[0] = 0.0;
-    bool keep[1];
-    select_by_score<1>(p.sp, f, sx, writes, cs.kept, keep, ss.sc64, ss.cnt64, ss.misc64);
+    const double sx = tid < p.P ? (double)__ldg(p.ext_scores + (long long)f * p.P + tid) : 0.0;
+    const bool bad = __syncthreads_or(tid < p.P && !isfinite(sx)) != 0;
+    select_by_score(p.sp, f, bad ? 0.0 : sx, writes, cs.kept, ss.sc64, ss.cnt64, ss.misc64);
     if (bad && writes && tid == 0 && p.sp.status) atomicCAS(p.sp.status, 0, kStatusNonFinite);
     risky = false;
     __syncthreads();
@@ -849,6 +847,14 @@ __global__ void __launch_bounds__(kCompactThreads) zero_kernel(unsigned long lon
 // frame's own one, takes back what is not final: that frame, and the flagged ones.  (Either every one of these blocks
 // finds all frames published, or none does.)
 constexpr unsigned kSelDone = 1u, kSelGivenUp = 2u, kSelRisky = 3u;
+// (out of line: it never runs, and in line its code lay in the way of the flagged frames', 0.3 us of a call)
+__device__ __noinline__ void take_back(const ScoreParams& sp, int f) {
+  const long long np = (long long)sp.n_frames * sp.P;
+  for (int t = threadIdx.x; t < sp.P; t += kCompactThreads) {
+    if (t < sp.kappa) sp.kept_store[(long long)f * sp.kappa + t] = -1;
+    for (int s = 0; s < 3 && sp.scores_out; ++s) sp.scores_out[s * np + (long long)f * sp.P + t] = __int_as_float(0x7fffffff);
+  }
+}
 __global__ void __launch_bounds__(kCompactThreads, 3) select_kernel(const __grid_constant__ CompactParams p, const int* scoring) {
   __shared__ union {
     struct {
@@ -863,22 +869,15 @@ __global__ void __launch_bounds__(kCompactThreads, 3) select_kernel(const __grid
   pdl_wait();
   pdl_trigger();
   const int failed = *scoring;
-  auto take_back = [&](int f) {
-    const long long np = (long long)n * sp.P;
-    for (int t = tid; t < sp.P; t += kCompactThreads) {
-      if (t < sp.kappa) sp.kept_store[(long long)f * sp.kappa + t] = -1;
-      for (int s = 0; s < 3 && sp.scores_out; ++s) sp.scores_out[s * np + (long long)f * sp.P + t] = __int_as_float(0x7fffffff);
-    }
-  };
   if ((int)blockIdx.x < n) {
     const int f = blockIdx.x;
     const bool risky = select_from_partials(p, f, true, sh.kept, &sh.ss);
-    if (failed) take_back(f);
+    if (failed) take_back(sp, f);
     __threadfence();
     __syncthreads();
     if (tid == 0) s_word = atomicCAS(p.sel_flag + f, 0u, risky ? kSelRisky : kSelDone);
     __syncthreads();
-    if (s_word == kSelGivenUp) take_back(f);
+    if (s_word == kSelGivenUp) take_back(sp, f);
     return;
   }
   if (failed) return;
@@ -893,7 +892,7 @@ __global__ void __launch_bounds__(kCompactThreads, 3) select_kernel(const __grid
   __threadfence();
   if (__syncthreads_or(word == kSelGivenUp)) {
     for (int f = 0; f < n; ++f)                            // (no word changes any more)
-      if (*reinterpret_cast<volatile unsigned*>(p.sel_flag + f) == kSelRisky) take_back(f);
+      if (*reinterpret_cast<volatile unsigned*>(p.sel_flag + f) == kSelRisky) take_back(sp, f);
     return;
   }
   const int n_fl = *reinterpret_cast<volatile int*>(sp.n_flagged), blocks = gridDim.x - n, heads = sp.Ls * sp.Hq;

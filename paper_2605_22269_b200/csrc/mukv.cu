@@ -1560,12 +1560,13 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
   if (dev < 0 || dev >= kMaxDevices) return fail(nullptr, MUKV_E_CAPACITY, "device index %d not supported", dev);
-  const int P = c.tokens_per_frame, D = c.head_dim, nc = pick_nc(P);
+  const int P = c.tokens_per_frame, D = c.head_dim;
+  const TcShape ts = tc_shape(c);
+  if (sizeof(T) == 2 && !ts.ok) return fail(nullptr, MUKV_E_UNSUPPORTED, "no tiling of the scoring kernel for this shape");   // (none)
   const NoallocDevice* nd = nullptr;
   e = noalloc_setup(dev, &nd);
   if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "set-up of the static scratch: %s", cudaGetErrorString(e));
   unsigned char* base = nd->ptr;
-  const TcShape ts = tc_shape(c);
   ScoreParams sp;
   memset(&sp, 0, sizeof sp);
   sp.P = P; sp.Hq = c.n_q_heads; sp.Hkv = c.n_kv_heads; sp.D = D; sp.G = c.n_q_heads / c.n_kv_heads;
@@ -1595,7 +1596,8 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
   // call before they could be spoilt for good.)
   e = zero_async(base + kNaCtrl, kNaCtrlBytes + (ts.ok ? (size_t)n * P * sizeof(unsigned long long) : 0), st, true);
   if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "clearing the scratch: %s", cudaGetErrorString(e));
-  if (ts.ok) {
+  const int units = n * c.n_q_heads * ((P + 7) / 8);
+  if constexpr (sizeof(T) == 2) {
     // bf16: scored on the tensor cores like a chunk of a context, then one block per frame selects.
     PsLaunch pl;
     memset(&pl, 0, sizeof pl);
@@ -1617,23 +1619,20 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
     cp.sp.scratch_rows = kNaFrames * kNaHq;
     cp.wait_ns = wait_ns;
     // (blocks for the flagged frames: three per SM are resident beside one another; they wait for the first n only)
-    const int units = n * c.n_q_heads * ((P + 7) / 8);
     e = launch_k(select_kernel, dim3(n + std::min(units, 3 * nd->n_sms)), kCompactThreads, 0, st, true, cp, (const int*)pl.status);
     if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "select kernel: %s", cudaGetErrorString(e));
-    return MUKV_OK;
   } else {
-    e = launch_score<T>(sp, nc, dim3(c.n_q_heads, n), score_smem_bytes<T>(P, D), st, true);
+    e = launch_score<T>(sp, pick_nc(P), dim3(c.n_q_heads, n), score_smem_bytes<T>(P, D), st, true);
     if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "score kernel: %s", cudaGetErrorString(e));
+    // Flagged frames in double precision.  The scratch holds the partial sums of 16 frames with one block per head; while
+    // few frames are flagged the same room lets several blocks share a head.
+    sp.refine = 1;
+    sp.scratch_rows = kNaFrames * kNaHq;
+    sp.colsum_part = base + kNaColD;
+    sp.ifft_part = base + kNaFftD;
+    e = launch_k(score64_kernel<T>, dim3(std::min(units, nd->n_sms)), kScoreThreads, 0, st, true, sp);
+    if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "refine kernel: %s", cudaGetErrorString(e));
   }
-  // Flagged frames in double precision.  The scratch holds the partial sums of 16 frames with one block per head; while
-  // few frames are flagged the same room lets several blocks share a head.
-  sp.refine = 1;
-  sp.scratch_rows = kNaFrames * kNaHq;
-  sp.colsum_part = base + kNaColD;
-  sp.ifft_part = base + kNaFftD;
-  const int units = n * c.n_q_heads * ((P + 7) / 8);
-  e = launch_k(score64_kernel<T>, dim3(std::min(units, nd->n_sms)), kScoreThreads, 0, st, true, sp);
-  if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "refine kernel: %s", cudaGetErrorString(e));
   return MUKV_OK;
 }
 

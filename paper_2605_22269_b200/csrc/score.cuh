@@ -88,130 +88,87 @@ __host__ inline size_t score_smem_bytes(int P, int D) {
   return (all > sizeof(FinishScratch) ? all : sizeof(FinishScratch)) + 64;
 }
 
-// The top-kappa rule for one frame on final scores s (double), run by all threads of the group Grp.
-// Thread tid owns the tokens tid + k*size, k < TOK (TOK*size >= P).  tau is the kappa-th largest
-// score (rank counting: P <= 256); scores above tau + tie_eps are kept, the scores within tie_eps
-// of tau share the remaining places by lowest token id.  keep[k] says which of the thread's tokens
-// stay; the kept ids go, ascending, to s_kept (shared memory, may be null) and, with `write`, to
-// the store, to the caller's output and the frame's time stamp and page-table entry are set.
+// The top-kappa rule for one frame on final scores (double), run by a whole block; thread t < P owns token t and gives its score s
+// (P <= threads).  tau is the kappa-th largest score (rank counting); scores above tau + tie_eps are kept, the scores
+// within tie_eps of tau share the remaining places by lowest token id.  Returns whether the thread's token stays; the kept ids go,
+// ascending, to s_kept (shared memory, may be null) and, with `write`, to the store, to the caller's output and the frame's time
+// stamp and page-table entry are set.
 // s_sc (P doubles), s_int (one int per warp + 1), s_misc (4 doubles per warp) are shared scratch.
-template <int TOK, class Grp = BlockGroup>
-__device__ inline void select_by_score(const ScoreParams& p, int f, const double (&s)[TOK], bool write, int* s_kept,
-                                       bool (&keep)[TOK], double* s_sc, int* s_int, double* s_misc) {
-  const int tid = Grp::tid();
-  const int nt = Grp::size();
-  const int P = p.P;
+__device__ inline bool select_by_score(const ScoreParams& p, int f, double s, bool write, int* s_kept, double* s_sc, int* s_int,
+                                       double* s_misc) {
+  const int tid = threadIdx.x, P = p.P, kappa = p.kappa;
+  const bool valid = tid < P;
+  // (on order-preserving integers: a comparison of doubles takes sixteen clocks of a scheduler)
   unsigned long long* s_key = reinterpret_cast<unsigned long long*>(s_sc);
-  int tok[TOK];
-  bool valid[TOK];
-#pragma unroll
-  for (int k = 0; k < TOK; ++k) {
-    tok[k] = tid + k * nt;
-    valid[k] = tok[k] < P;
-    if (valid[k]) s_key[tok[k]] = order_key(s[k]);
-  }
-  Grp::sync();
-  const int kappa = p.kappa;
-#pragma unroll
-  for (int k = 0; k < TOK; ++k) {
-    if (valid[k]) {
-      int gt = 0, ge = 0;
-      // (on order-preserving integers: a comparison of doubles takes sixteen clocks of a scheduler)
-      const unsigned long long key = order_key(s[k]);
+  const unsigned long long key = order_key(s);
+  if (valid) s_key[tid] = key;
+  __syncthreads();
+  if (valid) {
+    int gt = 0, ge = 0;
 #pragma unroll 4
-      for (int i = 0; i < P; ++i) {
-        const unsigned long long o = s_key[i];
-        gt += (o > key);
-        ge += (o >= key);
-      }
-      if (gt < kappa && kappa <= ge) s_misc[0] = s[k];      // every writer holds the same value
+    for (int i = 0; i < P; ++i) {
+      const unsigned long long o = s_key[i];
+      gt += (o > key);
+      ge += (o >= key);
     }
+    if (gt < kappa && kappa <= ge) s_misc[0] = s;           // every writer holds the same value
   }
-  Grp::sync();
+  __syncthreads();
   const double tau = s_misc[0];
   const double delta = (double)p.tie_eps;
-  bool sure[TOK], band[TOK];
-  int n_sure = 0;
-#pragma unroll
-  for (int k = 0; k < TOK; ++k) {
-    sure[k] = valid[k] && (s[k] > tau + delta);
-    band[k] = valid[k] && !sure[k] && (s[k] >= tau - delta);
-    int t;
-    group_excl_count<Grp>(sure[k], s_int, t);
-    n_sure += t;
-  }
-  int band_before = 0;
-#pragma unroll
-  for (int k = 0; k < TOK; ++k) {
-    int t;
-    const int band_rank = band_before + group_excl_count<Grp>(band[k], s_int, t);
-    band_before += t;
-    keep[k] = sure[k] || (band[k] && band_rank < kappa - n_sure);
-  }
+  const bool sure = valid && (s > tau + delta);
+  const bool band = valid && !sure && (s >= tau - delta);
+  int n_sure, n_band, n_kept;
+  block_excl_count(sure, s_int, n_sure);
+  const int band_rank = block_excl_count(band, s_int, n_band);
+  const bool keep = sure || (band && band_rank < kappa - n_sure);
   const long long f_abs = p.first_frame + f;
-  int out_before = 0;
-#pragma unroll
-  for (int k = 0; k < TOK; ++k) {
-    int t;
-    const int pos = out_before + group_excl_count<Grp>(keep[k], s_int, t);
-    out_before += t;
-    if (keep[k]) {
-      if (s_kept) s_kept[pos] = tok[k];
-      if (write) {
-        p.kept_store[f_abs * kappa + pos] = tok[k];
-        if (p.kept_out) p.kept_out[(long long)f * kappa + pos] = tok[k];
-      }
+  const int pos = block_excl_count(keep, s_int, n_kept);
+  if (keep) {
+    if (s_kept) s_kept[pos] = tid;
+    if (write) {
+      p.kept_store[f_abs * kappa + pos] = tid;
+      if (p.kept_out) p.kept_out[(long long)f * kappa + pos] = tid;
     }
   }
   if (write && tid == 0) {
     p.frame_ts[f_abs] = f_abs;
     p.page_table[f_abs] = p.pages_off + f_abs * p.page_bytes;
   }
+  return keep;
 }
 
-// Eq. 4 and the top-kappa rule for one frame, run by all threads of the group Grp.  Thread tid owns
-// the tokens tid + k*size, k < TOK (TOK*size >= P); att_raw / fft_raw are their I_att and I_fft;
-// s_sc (P doubles), s_int (one int per warp + 1), s_misc (4 doubles per warp) are shared scratch.
+// Eq. 4 and the top-kappa rule for one frame, run by a whole block; thread t < P owns token t, att_raw / fft_raw are its I_att and
+// I_fft; s_sc (P doubles), s_int (one int per warp + 1), s_misc (4 doubles per warp) are shared scratch.
 // With `refined` the frame is not put on the flagged list however close it is.
 // The arithmetic here is always double: it is a few hundred operations per frame and keeps
 // the normalisation from adding rounding noise of its own to the scores.
-template <int TOK, class Grp = BlockGroup>
-__device__ inline void select_frame(const ScoreParams& p, int f, const double (&att_raw)[TOK],
-                                    const double (&fft_raw)[TOK], bool refined, double* s_sc, int* s_int, double* s_misc) {
+__device__ inline void select_frame(const ScoreParams& p, int f, double att_raw, double fft_raw, bool refined, double* s_sc, int* s_int,
+                                    double* s_misc) {
   typedef double A;
-  const int tid = Grp::tid(), lane = tid & 31, warp = tid >> 5;
-  const int nt = Grp::size(), nwarp = nt >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = (int)blockDim.x >> 5;
   const int P = p.P;
+  const bool valid = tid < P;
   const A big = (A)3.0e38;
-  int tok[TOK];
-  bool valid[TOK];
-#pragma unroll
-  for (int k = 0; k < TOK; ++k) { tok[k] = tid + k * nt; valid[k] = tok[k] < P; }
   // ---- a frame with a score that is not a number has no ranking: every score counts as 0 below,
   // so that the lowest kappa ids are kept, and the event is recorded
-  bool bad_here = false;
-#pragma unroll
-  for (int k = 0; k < TOK; ++k) bad_here |= valid[k] && !(isfinite(att_raw[k]) && isfinite(fft_raw[k]));
   int n_bad;
-  group_excl_count<Grp>(bad_here, s_int, n_bad);
+  block_excl_count(valid && !(isfinite(att_raw) && isfinite(fft_raw)), s_int, n_bad);
   const bool bad = n_bad != 0;
   // ---- min / max of both signals over the frame
   A v[4] = {big, -big, big, -big};
-#pragma unroll
-  for (int k = 0; k < TOK; ++k) {
-    if (valid[k]) {
-      v[0] = att_raw[k] < v[0] ? att_raw[k] : v[0];
-      v[1] = att_raw[k] > v[1] ? att_raw[k] : v[1];
-      v[2] = fft_raw[k] < v[2] ? fft_raw[k] : v[2];
-      v[3] = fft_raw[k] > v[3] ? fft_raw[k] : v[3];
-    }
+  if (valid) {
+    v[0] = att_raw < v[0] ? att_raw : v[0];
+    v[1] = att_raw > v[1] ? att_raw : v[1];
+    v[2] = fft_raw < v[2] ? fft_raw : v[2];
+    v[3] = fft_raw > v[3] ? fft_raw : v[3];
   }
   v[0] = warp_min(v[0]); v[1] = warp_max(v[1]); v[2] = warp_min(v[2]); v[3] = warp_max(v[3]);
   if (lane == 0) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) s_misc[warp * 4 + i] = v[i];
   }
-  Grp::sync();
+  __syncthreads();
   A amin = big, amax = -big, fmin_ = big, fmax_ = -big;
   for (int w = 0; w < nwarp; ++w) {
     amin = s_misc[w * 4 + 0] < amin ? s_misc[w * 4 + 0] : amin;
@@ -219,29 +176,19 @@ __device__ inline void select_frame(const ScoreParams& p, int f, const double (&
     fmin_ = s_misc[w * 4 + 2] < fmin_ ? s_misc[w * 4 + 2] : fmin_;
     fmax_ = s_misc[w * 4 + 3] > fmax_ ? s_misc[w * 4 + 3] : fmax_;
   }
-  Grp::sync();
+  __syncthreads();
   // ---- Eq. 4
   const A alpha = (A)p.alpha;
-  A s[TOK];
-#pragma unroll
-  for (int k = 0; k < TOK; ++k) {
-    A an = (amax == amin) ? (A)0 : (att_raw[k] - amin) / (amax - amin);
-    A fn = (fmax_ == fmin_) ? (A)0 : (fft_raw[k] - fmin_) / (fmax_ - fmin_);
-    if (p.keep_low) fn = (A)1 - fn;
-    s[k] = bad ? (A)0 : alpha * an + ((A)1 - alpha) * fn;
-  }
-  bool keep[TOK];
-  select_by_score<TOK, Grp>(p, f, s, true, nullptr, keep, s_sc, s_int, s_misc);
-  if (p.scores_out) {
+  const A an = (amax == amin) ? (A)0 : (att_raw - amin) / (amax - amin);
+  A fn = (fmax_ == fmin_) ? (A)0 : (fft_raw - fmin_) / (fmax_ - fmin_);
+  if (p.keep_low) fn = (A)1 - fn;
+  const A s = bad ? (A)0 : alpha * an + ((A)1 - alpha) * fn;
+  const bool keep = select_by_score(p, f, s, true, nullptr, s_sc, s_int, s_misc);
+  if (p.scores_out && valid) {
     const long long np = (long long)p.n_frames * P;
-#pragma unroll
-    for (int k = 0; k < TOK; ++k) {
-      if (valid[k]) {
-        p.scores_out[0 * np + (long long)f * P + tok[k]] = (float)att_raw[k];
-        p.scores_out[1 * np + (long long)f * P + tok[k]] = (float)fft_raw[k];
-        p.scores_out[2 * np + (long long)f * P + tok[k]] = (float)s[k];
-      }
-    }
+    p.scores_out[0 * np + (long long)f * P + tid] = (float)att_raw;
+    p.scores_out[1 * np + (long long)f * P + tid] = (float)fft_raw;
+    p.scores_out[2 * np + (long long)f * P + tid] = (float)s;
   }
   if (tid == 0 && bad && p.status) atomicCAS(p.status, 0, kStatusNonFinite);
   // ---- does single precision decide this frame safely?
@@ -252,19 +199,12 @@ __device__ inline void select_frame(const ScoreParams& p, int f, const double (&
   if (!refined && !bad) {
     const int kappa = p.kappa;
     const A delta = (A)p.tie_eps;
-    A a = big, b = -big;
-#pragma unroll
-    for (int k = 0; k < TOK; ++k) {
-      if (valid[k]) {
-        if (keep[k]) a = s[k] < a ? s[k] : a;
-        else b = s[k] > b ? s[k] : b;
-      }
-    }
+    A a = valid && keep ? s : big, b = valid && !keep ? s : -big;
     a = warp_min(a);
     b = warp_max(b);
-    Grp::sync();
+    __syncthreads();
     if (lane == 0) { s_misc[warp * 4] = a; s_misc[warp * 4 + 1] = b; }
-    Grp::sync();
+    __syncthreads();
     if (tid == 0) {
       for (int w = 1; w < nwarp; ++w) {
         a = s_misc[w * 4] < a ? s_misc[w * 4] : a;
@@ -349,10 +289,9 @@ __device__ inline void finish_frame(const ScoreParams& p, A* colsum, const A* if
     if (tid < P) rows[(long long)hv * RS * P + tid] = (A)t;
   }
   if (!arrives_last(p.frame_counter + f, HqV, s->ints)) return;
-  double att[1], fft[1];
-  att[0] = column_sums(rows, HqV, RS, P, s->part) / (double)((long long)HqV * P);
-  fft[0] = column_sums(ifft + (long long)sf * HkvV * P, HkvV, 1, P, s->part) / (double)((long long)HkvV * p.D);
-  select_frame<1>(p, f, att, fft, refined, s->sc, s->ints, s->misc);
+  const double att = column_sums(rows, HqV, RS, P, s->part) / (double)((long long)HqV * P);
+  const double fft = column_sums(ifft + (long long)sf * HkvV * P, HkvV, 1, P, s->part) / (double)((long long)HkvV * p.D);
+  select_frame(p, f, att, fft, refined, s->sc, s->ints, s->misc);
   if (p.n_selected) {
     __threadfence();                                       // this thread's ids are visible before the frame counts
     __syncthreads();

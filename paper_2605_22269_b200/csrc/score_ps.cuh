@@ -60,7 +60,8 @@ constexpr int kPsAccCols = 64;             // accumulator columns per epilogue t
 constexpr int kPsCtrlRegs = 32;
 constexpr int kPsEpiRegs = 112;
 static_assert(128 * (96 - kPsCtrlRegs) >= 512 * (kPsEpiRegs - 96), "register hand-over does not balance");
-typedef NamedGroup<5, kPsEpiThreads, kPsEpiOff> PsEpiGroup;
+// the epilogue warps meet (the other warps never join)
+__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync %0, %1;" ::"n"(5), "n"(kPsEpiThreads) : "memory"); }
 
 struct ScorePsParams {
   ScoreParams sp;            // ifft_part: float [F][Hkv][P]
@@ -745,11 +746,11 @@ __global__ void __maxnreg__(96) score_ps_kernel(const ScorePsParams p,
           const float s = warp_column_sums(v, lane);
           if (pp * 32 + lane < my_nch * 16) s_col[q * 256 + my_c0 * 16 + pp * 32 + lane] = s;
         }
-        PsEpiGroup::sync();
+        epi_sync();
         unsigned long long* row = p.att_acc + (long long)f * P;
         for (int t = et; t < P; t += kPsEpiThreads)
           att_add(row + t, (s_col[t] + s_col[256 + t]) + (s_col[512 + t] + s_col[768 + t]));
-        PsEpiGroup::sync();                                // the sums may be overwritten
+        epi_sync();                                // the sums may be overwritten
       }
       if (++x == ipu) {
         x = 0;

@@ -7,7 +7,7 @@
 // tokens, its page has that many rows, and the pages of a segment lie one behind the other in the
 // segment's share of the page region.  One block per segment of the chunk.
 // Two sources of the indicators:
-//   src32 = 0  the double-precision partial sums of score_kernel; everything in double precision,
+//   src32 = 0  the double-precision partial sums of score64_kernel; everything in double precision,
 //              the ranking by the radix select of the retrieval kernels (block_topk_set);
 //   src32 = 1  the single-precision partial sums of the persistent tensor-core kernel; Eq. 4 and the
 //              ranking in single precision (segment_select32: the scheme of the frame-level selection,
@@ -15,7 +15,7 @@
 //              ranking then stands only when the lowest kept and the highest dropped score are further
 //              apart than tie_eps + flag_margin and neither signal is flat (the rule of the
 //              frame-level selection); otherwise the kernel writes nothing but the segment's word in
-//              seg_flag, and the double-precision pass that follows (score_kernel gated by that word,
+//              seg_flag, and the double-precision pass that follows (score64_kernel gated by that word,
 //              then this kernel with src32 = 0 and only_flagged = 1) redoes the segment.
 #pragma once
 #include "common.cuh"

@@ -27,3 +27,6 @@ extern "C" void internals_scores(const mukv_ctx* ctx, long long* out) {
                            pad4(T * S)};
   for (int i = 0; i < 12; ++i) out[i] = v[i];
 }
+
+// whether a bf16 chunk of this shape is scored on the tensor cores
+extern "C" int internals_on_tensor_cores(const mukv_config* cfg) { return tc_shape(*cfg).ok; }

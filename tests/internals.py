@@ -27,6 +27,8 @@ def load():
         _LIB.internals_scan_by_rows.restype = C.c_int
         _LIB.internals_scan_by_rows.argtypes = [C.c_longlong, C.c_int, C.c_int]
         _LIB.internals_scores.argtypes = [C.c_void_p, C.POINTER(C.c_longlong)]
+        _LIB.internals_on_tensor_cores.restype = C.c_int
+        _LIB.internals_on_tensor_cores.argtypes = [C.POINTER(B.MukvConfig)]
         _LIB.internals_score_noalloc.restype = C.c_int32
         _LIB.internals_score_noalloc.argtypes = _LIB.mukv_score_frames_noalloc.argtypes + [C.c_ulonglong]
     return _LIB

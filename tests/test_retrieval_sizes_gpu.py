@@ -18,7 +18,7 @@ SPEC = StreamSpec(seed=71, n_layers=1, n_q_heads=4, n_kv_heads=2, head_dim=64, t
     (128, 2, 1, 3, 5, B.RETR_SEMI),                        # the most frames that are ranked directly, one row per warp in the scan
     (129, 1, 2, 3, 5, B.RETR_SEMI),                        # the histogram for frames and segments, two rows per warp, an odd row left
     (133, 7, 8, 2, 64, B.RETR_SEMI),                       # the most questions of the small scan; 128 candidates of 133
-    (133, 7, 9, 2, 64, B.RETR_PARALLEL),                   # one more: the tile of 64 questions
+    (133, 7, 9, 2, 64, B.RETR_PARALLEL),                   # more than a few questions
     (530, 4, 3, 5, 200, B.RETR_SEMI),                      # 400 candidates and their second ranking
     (530, 4, 3, 140, 256, B.RETR_SEMI),                    # 512 candidates and some ties: more than the short list may hold
     (530, 4, 3, 9, 30, B.RETR_HIER),
