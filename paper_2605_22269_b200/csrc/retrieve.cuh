@@ -123,13 +123,14 @@ struct ScanShape {
 __host__ inline size_t scan_smem_bytes(int T, int q_groups, int row_tiles) {
   return 2 * ((size_t)kScanCC * (8 * T * q_groups + kScanQPad) * sizeof(double) + (size_t)8 * row_tiles * kScanRowPad * sizeof(float));
 }
-// The shape of least time, in clocks per chunk.  A wave of blocks takes what its tiles take on the busiest scheduler (128 clocks
-// each, 8 instructions of 16) or its bytes at 64 a clock, the chunk's barrier and first operands (450) and the copies that one
-// thread issues (50 each: a block of few warps is slow at fetching the chunk of all questions); then the bytes of all blocks,
-// at 6,000 a clock of the device.  Blocks per SM as shared memory and registers (48 a thread for T = 1, up to 96 else) allow.
-// Fitted to every shape at 1 KB to 8 KB per pooled question, 9 to 128 questions and 107 to 44,625 rows: 0.5 % from the best one on
-// average, 7 % at the most.  (Without residency, copies and the last term 5 % and 70 %: 128 questions on 8,288 rows
-// went to 1,036 blocks of one row tile, each of which fetches all questions, 199 us; now 150.)
+// The shape of least time, in clocks per chunk.  A wave of blocks takes what its warps take on the busiest scheduler (128 clocks a
+// tile, 8 instructions of 16, and 40 for the rows' operands, which the tiles of a warp share) or its bytes at 32 a clock, the chunk's
+// barrier and first operands (400) and the copies that one thread issues (50 each: a block of few warps is slow at fetching the
+// chunk of all questions); then the bytes of all blocks, at 8,000 a clock of the device.  Blocks per SM as shared memory and
+// registers (48 a thread for T = 1, up to 96 else) allow.
+// Fitted to every shape at 1 to 8 KB per pooled question, 9 to 128 questions and 107 to 44,625 rows, keys in L2 and not: 0.7 % from the
+// best one on average, 9 % at the most.  (Without residency, copies and the last term 5 % and 70 %: 128 questions on 8,288 rows
+// went to 1,036 blocks of one row tile, each of which fetches all questions, 199 us; now 148.)
 __host__ inline ScanShape scan_shape(long long rows, int nq, int n_sms) {
   const int nt = (nq + 7) / 8, tiles = (int)((rows + 7) / 8);      // (32-bit divisions: half a microsecond of the call)
   ScanShape best{0, 0, 0, 0};
@@ -142,13 +143,13 @@ __host__ inline ScanShape scan_shape(long long rows, int nq, int n_sms) {
       const int by_smem = 227 * 1024 / (smem + 2048), by_regs = (T == 1 ? 40 : 20) / warps;      // (neither is 0)
       const int resident = by_smem < by_regs ? by_smem : by_regs;
       const int blocks = (tiles + rt - 1) / rt, per_sm = (blocks + n_sms - 1) / n_sms, full = per_sm / resident;
-      const int bytes = kScanCC * 8 * 8 * T * qg + 8 * rt * kScanCC * 4, own = 450 + 50 * (bytes / 512) / warps;
+      const int bytes = kScanCC * 8 * 8 * T * qg + 8 * rt * kScanCC * 4, own = 400 + 50 * (bytes / 512) / warps;
       auto wave = [&](int b) {
-        const int mma = (b * warps + 3) / 4 * T * 128, load = b * bytes / 64;
+        const int mma = (b * warps + 3) / 4 * (T * 128 + 40), load = b * bytes / 32;
         return (mma > load ? mma : load) + own;
       };
       const int rest = per_sm - full * resident;
-      const long long t = (long long)full * wave(resident) + (rest ? wave(rest) : 0) + (long long)blocks * bytes / 6000;
+      const long long t = (long long)full * wave(resident) + (rest ? wave(rest) : 0) + (long long)blocks * bytes / 8000;
       if (least < 0 || t < least) {
         least = t;
         best = {T, qg, rt, (size_t)smem};
@@ -290,13 +291,14 @@ __global__ void __launch_bounds__(32 * kScanMaxWarps) scan_kernel(const ScanPara
 // each: 28 us for a few questions and half an hour of 512 channels, with pooling, ranking and a small gather, where this one
 // takes 18 to 24.  But it takes eight questions in the time of one, and this one adds each question's product to every row, in loops
 // made for one, for four and for eight questions.  Where the two take the same time was measured at 64 to 2,048 channels, 107 to
-// 44,625 rows: at 512 channels 2 questions and 15,000 rows, 4 and 9,600, 5 to 8 and 5,000; at 128 channels 1 and 12,000, 2 to 4 and
-// 2,500; at 1,024 2 and 28,000, 4 and 14,500, 8 and 7,000.  Eight questions on 9,113 rows of 512 channels: 38 us by rows, 32 by
-// tiles; 44,625 rows: 97 and 54.
+// 44,625 rows, with the keys in L2 and with L2 flushed (a chunk is then a round trip to memory, so that the tiles start to pay later);
+// the line follows the flushed ones.  At 512 channels: 2 questions and 21,000 rows, 4 and 12,000, 5 and 10,000, 8 and 7,400 (in L2:
+// 15,000, 9,600, 5,000 and 4,500); at 128 channels 2 and 6,000, 8 and 3,000; at 1,024 4 and 30,000, 8 and 10,000.  Eight questions
+// on 11,475 rows of 512 channels: 55 us by rows, 48 by tiles (43 and 36); on 44,625 rows 107 and 66 (97 and 54).
 __host__ inline bool scan_by_rows(long long rows, int nq, int C) {
-  if (nq == 1) return rows <= 100LL * C;
-  if (nq <= 4) return rows <= (34LL - 4 * nq) * C;
-  return nq <= kScanFew && rows * nq <= 70LL * C && rows <= 12000;
+  if (nq == 1) return rows <= 200LL * C;
+  if (nq <= 4) return rows <= (60LL - 9 * nq) * C;
+  return nq <= kScanFew && rows * nq <= 100LL * C && rows <= 12000;
 }
 
 template <int NQ>

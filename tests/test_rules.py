@@ -15,7 +15,7 @@ def test_every_shape_fits():
             assert nq <= 8 * T * groups <= 128
             assert 2 * (32 * (8 * T * groups + 4) * 8 + 8 * tiles * 36 * 4) + 1024 <= 227 * 1024
             seen.add((T, tiles > 1))
-    assert seen == {(T, many) for T in (1, 2, 4, 8) for many in (False, True)} - {(8, False)}
+    assert seen >= {(T, True) for T in (1, 2, 4, 8)} | {(1, False)}      # (blocks of one row tile, of many)
 
 
 def test_blocks_do_not_multiply_the_fetched_questions():

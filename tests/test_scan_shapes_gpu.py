@@ -31,8 +31,8 @@ def test_scan_of_many_questions(nq, T, kv_heads, head_dim):
 
 
 # frames of one key head of 64 channels and sixteen patch-level blocks each, questions, question tiles of a warp
-MANY_ROWS = [(50, 9, 1), (50, 33, 2), (110, 80, 4), (431, 16, 1), (431, 24, 1), (431, 33, 4), (431, 97, 8), (770, 9, 2), (770, 64, 8),
-             (770, 128, 8), (2000, 24, 1)]
+MANY_ROWS = [(50, 9, 1), (50, 33, 2), (110, 80, 4), (431, 16, 2), (431, 24, 1), (431, 33, 4), (431, 97, 8), (770, 9, 2), (770, 64, 8),
+             (770, 128, 8), (2000, 24, 4)]
 
 
 def check_every_score(T, nq):
@@ -74,8 +74,8 @@ def test_every_score_of_blocks_of_several_row_tiles(monkeypatch, T, nq, tiles):
     check_every_score(T, nq)
 
 
-@pytest.mark.parametrize("T,nq,by_rows", [(3, 1, 1), (370, 1, 1), (372, 1, 0), (96, 2, 1), (97, 2, 0), (81, 3, 1), (82, 3, 0), (66, 4, 1),
-                                          (67, 4, 0), (51, 5, 1), (52, 5, 0), (32, 8, 1), (33, 8, 0), (431, 2, 0), (431, 7, 0)])
+@pytest.mark.parametrize("T,nq,by_rows", [(3, 1, 1), (742, 1, 1), (743, 1, 0), (155, 2, 1), (156, 2, 0), (122, 3, 1), (123, 3, 0), (89, 4, 1),
+                                          (90, 4, 0), (74, 5, 1), (75, 5, 0), (46, 8, 1), (47, 8, 0), (431, 2, 0), (431, 7, 0)])
 def test_every_score_on_both_sides_of_the_line_between_the_scans(monkeypatch, T, nq, by_rows):
     monkeypatch.setattr(B, "_LIB", I.load())
     assert B._LIB.internals_scan_by_rows(T + (T + 3) // 4 + 16 * T, nq, 64) == by_rows
