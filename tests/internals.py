@@ -2,6 +2,7 @@
 import ctypes as C
 import os
 import subprocess
+import tempfile
 
 from paper_2605_22269_b200 import binding as B
 from paper_2605_22269_b200 import build as BUILD
@@ -10,15 +11,27 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 _LIB = None
 
 
+def build():
+    """Path of the built library; in the tree where that can be written."""
+    src, (main, deps) = os.path.join(HERE, "internals.cu"), BUILD.TARGETS["libmukv.so"]
+    out = os.path.join(HERE, "_build", "libinternals.so")
+    if BUILD._stale(out, [src, main] + deps):
+        try:
+            os.makedirs(os.path.dirname(out), exist_ok=True)
+            writable = os.access(os.path.dirname(out), os.W_OK)
+        except OSError:
+            writable = False
+        if not writable:
+            out = os.path.join(tempfile.mkdtemp(prefix="internals"), "libinternals.so")
+        r = subprocess.run([os.environ.get("NVCC", "nvcc")] + BUILD.NVCC_FLAGS + ["-o", out, src], capture_output=True, text=True)
+        assert r.returncode == 0, r.stderr
+    return out
+
+
 def load():
     global _LIB
     if _LIB is None:
-        out, src = os.path.join(HERE, "_build", "libinternals.so"), os.path.join(HERE, "internals.cu")
-        main, deps = BUILD.TARGETS["libmukv.so"]
-        if BUILD._stale(out, [src, main] + deps):
-            os.makedirs(os.path.dirname(out), exist_ok=True)
-            r = subprocess.run([os.environ.get("NVCC", "nvcc")] + BUILD.NVCC_FLAGS + ["-o", out, src], capture_output=True, text=True)
-            assert r.returncode == 0, r.stderr
+        out = build()
         _LIB = B.load_library(out)
         _LIB.internals_wait_limit.restype = None
         _LIB.internals_wait_limit.argtypes = [C.c_void_p, C.c_ulonglong]
