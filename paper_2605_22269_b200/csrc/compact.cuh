@@ -846,16 +846,12 @@ __global__ void __launch_bounds__(kCompactThreads) zero_kernel(unsigned long lon
 // the word that the frame's own block would publish in, and whoever finds that word so, all blocks behind the selection and the
 // frame's own one, takes back what is not final: that frame, and the flagged ones.  (Either every one of these blocks
 // finds all frames published, or none does.)
+// Two blocks per SM: with three, 80 registers a thread, the double-precision scores spilled twice as much as in the compaction
+// kernel for what the ways out take, and a call with a flagged frame 83.4 us; with two and none spilled 77.5, two flagged frames 94.0
+// (106.8), eight 268 (369), sixteen 502 (587), nothing flagged 27.1 (27.8).  (Where the units of fewer blocks come out badly: three
+// 131 (119), six 268 (219), eleven 501 (370); one or two are what a call of sixteen frames sees, a quarter of the time.)
 constexpr unsigned kSelDone = 1u, kSelGivenUp = 2u, kSelRisky = 3u;
-// (out of line: it never runs, and in line its code lay in the way of the flagged frames', 0.3 us of a call)
-__device__ __noinline__ void take_back(const ScoreParams& sp, int f) {
-  const long long np = (long long)sp.n_frames * sp.P;
-  for (int t = threadIdx.x; t < sp.P; t += kCompactThreads) {
-    if (t < sp.kappa) sp.kept_store[(long long)f * sp.kappa + t] = -1;
-    for (int s = 0; s < 3 && sp.scores_out; ++s) sp.scores_out[s * np + (long long)f * sp.P + t] = __int_as_float(0x7fffffff);
-  }
-}
-__global__ void __launch_bounds__(kCompactThreads, 3) select_kernel(const __grid_constant__ CompactParams p, const int* scoring) {
+__global__ void __launch_bounds__(kCompactThreads, 2) select_kernel(const __grid_constant__ CompactParams p, const int* scoring) {
   __shared__ union {
     struct {
       SelectScratch ss;
@@ -869,39 +865,50 @@ __global__ void __launch_bounds__(kCompactThreads, 3) select_kernel(const __grid
   pdl_wait();
   pdl_trigger();
   const int failed = *scoring;
+  int f0 = 0, f1 = 0;                                      // frames to take back: all of these, or
+  bool only_risky = false;                                 // those that need the double-precision pass
   if ((int)blockIdx.x < n) {
     const int f = blockIdx.x;
     const bool risky = select_from_partials(p, f, true, sh.kept, &sh.ss);
-    if (failed) take_back(sp, f);
     __threadfence();
     __syncthreads();
     if (tid == 0) s_word = atomicCAS(p.sel_flag + f, 0u, risky ? kSelRisky : kSelDone);
     __syncthreads();
-    if (s_word == kSelGivenUp) take_back(sp, f);
-    return;
-  }
-  if (failed) return;
-  unsigned word = kSelDone;
-  if (tid < n) {                                           // (n <= MUKV_NOALLOC_MAX_FRAMES)
-    const volatile unsigned* flag = p.sel_flag + tid;
-    if (!wait_until(p.wait_ns, [&] { return (word = *flag) != 0u; })) {
-      word = atomicCAS(p.sel_flag + tid, 0u, kSelGivenUp);
-      if (word == 0u) word = kSelGivenUp;
+    if (!failed && s_word != kSelGivenUp) return;
+    f0 = f;
+    f1 = f + 1;
+  } else {
+    if (failed) return;
+    unsigned word = kSelDone;
+    if (tid < n) {                                         // (n <= MUKV_NOALLOC_MAX_FRAMES)
+      const volatile unsigned* flag = p.sel_flag + tid;
+      if (!wait_until(p.wait_ns, [&] { return (word = *flag) != 0u; })) {
+        word = atomicCAS(p.sel_flag + tid, 0u, kSelGivenUp);
+        if (word == 0u) word = kSelGivenUp;
+      }
     }
+    __threadfence();
+    if (!__syncthreads_or(word == kSelGivenUp)) {
+      const int n_fl = *reinterpret_cast<volatile int*>(sp.n_flagged), blocks = gridDim.x - n, heads = sp.Ls * sp.Hq;
+      if (n_fl == 0) return;
+      const int rs = score64_split(n_fl, heads, sp.P, blocks, sp.scratch_rows), units = heads * rs;
+      for (int w = blockIdx.x - n; w < n_fl * units; w += blocks) {
+        const int slot = w / units, u = w % units;
+        score64_frame_block<__nv_bfloat16>(sp, p.colsum_d, p.ifft_d, u / rs, u % rs, rs, __ldcg(sp.flagged + slot), slot, &sh.s64);
+        __syncthreads();
+      }
+      return;
+    }
+    f1 = n;
+    only_risky = true;
   }
-  __threadfence();
-  if (__syncthreads_or(word == kSelGivenUp)) {
-    for (int f = 0; f < n; ++f)                            // (no word changes any more)
-      if (*reinterpret_cast<volatile unsigned*>(p.sel_flag + f) == kSelRisky) take_back(sp, f);
-    return;
-  }
-  const int n_fl = *reinterpret_cast<volatile int*>(sp.n_flagged), blocks = gridDim.x - n, heads = sp.Ls * sp.Hq;
-  if (n_fl == 0) return;
-  const int rs = score64_split(n_fl, heads, sp.P, blocks, sp.scratch_rows), units = heads * rs;
-  for (int w = blockIdx.x - n; w < n_fl * units; w += blocks) {
-    const int slot = w / units, u = w % units;
-    score64_frame_block<__nv_bfloat16>(sp, p.colsum_d, p.ifft_d, u / rs, u % rs, rs, __ldcg(sp.flagged + slot), slot, &sh.s64);
-    __syncthreads();
+  const long long np = (long long)n * sp.P;
+  for (int f = f0; f < f1; ++f) {
+    if (only_risky && *reinterpret_cast<volatile unsigned*>(p.sel_flag + f) != kSelRisky) continue;   // (no word changes any more)
+    for (int t = tid; t < sp.P; t += kCompactThreads) {
+      if (t < sp.kappa) sp.kept_store[(long long)f * sp.kappa + t] = -1;
+      for (int s = 0; s < 3 && sp.scores_out; ++s) sp.scores_out[s * np + (long long)f * sp.P + t] = __int_as_float(0x7fffffff);
+    }
   }
 }
 

@@ -1618,8 +1618,8 @@ mukv_status noalloc_impl(const mukv_config& c, const void* d_q, const void* d_k_
     cp.ifft_d = reinterpret_cast<double*>(base + kNaFftD);
     cp.sp.scratch_rows = kNaFrames * kNaHq;
     cp.wait_ns = wait_ns;
-    // (blocks for the flagged frames: three per SM are resident beside one another; they wait for the first n only)
-    e = launch_k(select_kernel, dim3(n + std::min(units, 3 * nd->n_sms)), kCompactThreads, 0, st, true, cp, (const int*)pl.status);
+    // (blocks for the flagged frames: two per SM are resident beside one another; they wait for the first n only)
+    e = launch_k(select_kernel, dim3(n + std::min(units, 2 * nd->n_sms)), kCompactThreads, 0, st, true, cp, (const int*)pl.status);
     if (e != cudaSuccess) return fail(nullptr, MUKV_E_CUDA, "select kernel: %s", cudaGetErrorString(e));
   } else {
     e = launch_score<T>(sp, pick_nc(P), dim3(c.n_q_heads, n), score_smem_bytes<T>(P, D), st, true);
